@@ -1892,25 +1892,16 @@ long long hp_estimate_bytes(int nside, int lmax, wf_precision prec, bool staging
     long long b = 0;
     b += nalm * 16 + np * 16 + (lmax + 1) * 8 + ns * (4 + 16);  // A64, c64, x, st, log2 c, seeds
     if (f32) b += nalm * 8 + np * 8 + ns * 12;                   // A32, B32, x32, w32, FP32 seeds
-    // ring tables: roots per distinct length, Bluestein filters, twiddles, scratch
-    long long roots = 0, V = 0, nmaxF = 2, maxBlue = 1;
+    // ring tables: roots per distinct length, Bluestein filters and chirps, twiddles
+    long long roots = 0, V = 0;
     for (int k = 1; k <= nside; ++k) {
         const long long n = 4LL * k;
         roots += 2 * n;
-        if (n <= 32) continue;
-        if ((n & (n - 1)) == 0) {
-            nmaxF = std::max(nmaxF, n);
-        } else {
-            long long M = 1;
-            while (M < 2 * n - 1) M <<= 1;
-            V += M + n;  // filter and chirp
-            nmaxF = std::max(nmaxF, M);
-            maxBlue = std::max(maxBlue, n);
-        }
+        bool direct = false;
+        const int b2 = ring_fft_log((int)n, &direct);
+        if (!direct) V += (1LL << b2) + k;  // filter and chirp
     }
-    const long long zl = std::max(maxBlue, 32LL);
-    b += (roots + V + nmaxF) * ec + np * (48 + 4) + 64;
-    b += std::min<long long>(np, 8LL * 152) * 2 * zl * ec;
+    b += (roots + V + RING_TW) * ec + np * ((long long)sizeof(RingTab) + 4) + 64;
     // workspace
     b += nalm * 16 * (f32 ? 4 : 3);                              // a, a_new, b (+ b_low)
     b += 2 * np * (lmax + 1) * 2 * ec;                           // G, F

@@ -49,23 +49,24 @@ template <typename C, typename S> __host__ __device__ __forceinline__ C cscale(C
 // ---------------------------------------------------------------------------
 // ring table (one entry per north/south ring pair)
 // ---------------------------------------------------------------------------
-enum RingKind : int { RING_NAIVE = 0, RING_POW2 = 1, RING_BLUESTEIN = 2 };
+enum RingKind : int { RING_POW2 = 1, RING_BLUESTEIN = 2 };
 
 struct RingTab {
     int n;             // pixels in each ring of the pair
     int q;             // first-pixel longitude is q pi / n (q = 0 or 1)
     int kind;          // RingKind
-    int logF;          // log2 of the smem FFT length (pow2: n; Bluestein: M/2)
+    int logF;          // log2 of the FFT length N of its four length-n/4 DFTs (n/4, or 2^b >= n/2 - 1)
+    unsigned inv;      // ceil(2^32 / n): m / n = umulhi(m, inv) for the m of a band limit
     long long offN;    // first pixel of the north ring
     long long offS;    // first pixel of the south ring, -1 for the equator
     long long rootOff; // offset of e^{i pi p / n}, p < 2n, in the roots table
-    long long vOff;    // offset of the Bluestein filter (M entries: even half, odd half)
-    long long cOff;    // offset of the Bluestein chirp e^{-i pi j^2 / n}, j < n, in the chirp table
+    long long vOff;    // offset of the Bluestein filter spectrum of n/4 (N entries)
+    long long cOff;    // offset of the Bluestein chirp e^{-i pi j^2 / k}, j < k = n/4, in the chirp table
 };
 
-constexpr int NAIVE_MAX = 32;   // rings this short use a direct DFT
 constexpr int LEG_THREADS = 256;
-constexpr int RING_THREADS = 512;
+constexpr int RING_MAX_K = 2048;     // longest quarter ring (nside) of the ring kernel's FFTs
+constexpr int RING_TW = 2 * 4096 - 32;  // twiddles of the FFT lengths 32 .. 4096
 
 // ---------------------------------------------------------------------------
 // plan
@@ -100,7 +101,6 @@ struct Workspace {
     double2 *a = nullptr, *a_new = nullptr, *b = nullptr;
     void *G = nullptr, *F = nullptr;
     void *r = nullptr, *nu = nullptr, *t = nullptr;
-    void *scr = nullptr;          // per-CTA Bluestein scratch (2 * max Bluestein n complex per CTA)
     float2 *Glow = nullptr;       // mixed: FP64-block synthesis coefficients, rounded to FP32 [pair][glow_cap][hemisphere]
     double2 *b_low = nullptr;     // mixed: FP64-block analysis output (alm layout, m < lc)
     float2 *ca32 = nullptr;       // tensor-core plans: c a_lm in FP32, the synthesis B operand's source
@@ -144,12 +144,10 @@ struct HpTables {
     long long *lowrow = nullptr;  // first row of each m (lmax + 2 entries)
     int low_df = 0, np_pad = 0;
     int glow_cap = 0;      // row length of the FP64-block ring coefficients
-    int logNmax = 0;       // twiddle table is e^{-2 pi i t / 2^logNmax}, t < 2^logNmax
-    int bmax = 0;          // smem FFT buffer length (complex entries)
-    int maxBlue = 0;       // longest Bluestein ring
-    int ringGrid = 0;      // persistent grid of the ring kernels
+    int nmax = 0;          // longest ring
+    int ring_ctas = 2;     // ring kernel variant: CTAs per SM
+    int exmax = 0;         // exchange buffer of the ring FFTs (complex entries)
     int *order = nullptr;  // ring pairs by decreasing transform cost
-    int *ticket = nullptr; // work counter of the ring kernels (zeroed before each launch)
 };
 
 }  // namespace wf
@@ -268,6 +266,7 @@ wf_status hp_pol_tc_synthesis(wf_plan p, int ncols, const double2 *const *E, con
 
 // ring transforms (wf_ring.cu)
 wf_status hp_build_ring_tables(wf_plan p);
+int ring_fft_log(int n, bool *direct);
 // RS_BLEND_ANA: the blended ring goes straight into the forward DFT and the unfold to F
 enum RingSynMode { RS_BLEND = 0, RS_MAP = 1, RS_SYN = 2, RS_BLEND_ANA = 3 };
 wf_status hp_ring_synthesis(wf_plan p, int L, RingSynMode mode, double lam, double tau, double *out_map);

@@ -10,17 +10,17 @@
 // pair have the same n and q, so both are packed into one complex DFT
 // (z = f_N + i f_S).
 //
-// DFT engines, chosen per ring length at plan time:
-//   n <= 32            direct sum from shared memory;
-//   n a power of two   in-place radix-2 FFT in shared memory;
-//   otherwise          Bluestein: X_k = c_k sum_j (x_j c_j) conj(c_{k-j}),
-//                      c_j = e^{-i pi j^2 / n}, a circular convolution of
-//                      power-of-two length M >= 2n - 1.  Since the input is
-//                      zero beyond n <= M/2, the length-M transforms split
-//                      into two independent half-length ones (even and odd
-//                      outputs), so the shared buffer holds M/2 values and
-//                      the per-CTA global scratch holds the input and the
-//                      even-half result.
+// Every ring length is n = 4k.  A DFT of n splits into four DFTs of length k
+// and one radix-4 step with the twiddles w_n^{rq} (decimation in time for the
+// synthesis, in frequency for the analysis), and the radix-4 step of both
+// directions touches the pixels q, q + k, q + 2k, q + 3k of one thread: in the
+// messenger step a thread combines its four pixels, blends them (Eq. 3) and
+// splits them again in registers.  The four length-k DFTs run
+//   k = 2^b >= 16       as FFTs of length N = k;
+//   otherwise           by Bluestein's chirp convolution
+//                       X_p = c_p sum_j (x_j c_j) conj(c_{p-j}), c_j = e^{-i pi j^2 / k},
+//                       circular of length N = 2^b >= 2k - 1: FFT, product with the
+//                       tabulated filter spectrum, inverse FFT.
 //
 // Pixel blend (Eq. 3 solved for t with nu = N^-1, r = nu d):
 //     t = s + lambda tau (r - nu s) / (1 + (lambda - 1) tau nu)
@@ -73,653 +73,678 @@ void host_fft(std::vector<double2> &x)
 }
 
 // ---------------------------------------------------------------------------
-// device FFT helpers
+// register DFTs (forward, e^{-2 pi i nk / R}; the synthesis conjugates around
+// them), natural order in and out
 // ---------------------------------------------------------------------------
-// In-place power-of-two FFT in shared memory by all threads of the CTA:
-// Stockham autosort passes with radix-8 butterflies held in registers (one
-// radix-2 or radix-4 head pass when log2 N is not a multiple of 3).  Each
-// pass reads every element once into registers, waits at a barrier, and
-// writes every element once, so shared memory sees 2 log8(N) round trips
-// instead of 2 log2(N) for radix-2.  sign -1: e^{-2 pi i jk/N}; +1:
-// e^{+2 pi i jk/N} (unnormalised).  Twiddles come from a shared-memory table laid out
-// by pass: stw[Ns + k] = e^{-2 pi i k / (8 Ns)}, k < Ns, for every power of two
-// Ns <= 2^logB / 8 (2^logB / 4 entries: 16 KB in FP32 for the 8192-point rings).
-// A warp of one pass reads consecutive entries (Ns >= 32) or a few broadcast ones;
-// one table of the circle indexed k 2^logB / (8 Ns) put the lanes of the middle
-// passes on one bank.
-// Supports N <= 8192 with NT = 512 threads (two radix-8 butterflies per thread) or
-// NT = 1024 (one).
-template <typename T>
-__device__ __forceinline__ cx<T> mul_i(cx<T> a, int sign)
+template <typename T> __device__ __forceinline__ cx<T> mul_mi(cx<T> a) { return mk<T>(a.y, -a.x); }  // -i a
+
+template <typename T> __device__ __forceinline__ void dft4(cx<T> &a0, cx<T> &a1, cx<T> &a2, cx<T> &a3)
 {
-    return sign > 0 ? mk<T>(-a.y, a.x) : mk<T>(a.y, -a.x);  // (sign i) a
+    const cx<T> s02 = cadd(a0, a2), d02 = csub(a0, a2), s13 = cadd(a1, a3), d13 = mul_mi<T>(csub(a1, a3));
+    a0 = cadd(s02, s13);
+    a1 = cadd(d02, d13);
+    a2 = csub(s02, s13);
+    a3 = csub(d02, d13);
 }
 
-// Radix-R DFT in registers, in place, decimation in frequency: on return
-// v[k] holds output X[brev_R(k)] (bit-reversed index), which the caller
-// undoes at compile time when it stores.
-template <typename T>
-__device__ __forceinline__ void bfly(cx<T> &a, cx<T> &b)
+// the same with a2 = a3 = 0 on entry
+template <typename T> __device__ __forceinline__ void dft4_half(cx<T> &a0, cx<T> &a1, cx<T> &a2, cx<T> &a3)
 {
-    const cx<T> t = a;
-    a = cadd(t, b);
-    b = csub(t, b);
+    const cx<T> x = a0, y = a1, z = mul_mi<T>(a1);
+    a0 = cadd(x, y);
+    a1 = cadd(x, z);
+    a2 = csub(x, y);
+    a3 = csub(x, z);
 }
 
-template <typename T, int R> struct SmallDft;
-template <typename T> struct SmallDft<T, 2> {
-    static __device__ __forceinline__ void run(cx<T> (&v)[2], int) { bfly<T>(v[0], v[1]); }
-    static __device__ __forceinline__ constexpr int out(int k) { return k; }
-};
-template <typename T> struct SmallDft<T, 4> {
-    static __device__ __forceinline__ void run(cx<T> (&v)[4], int sign)
-    {
-        bfly<T>(v[0], v[2]);
-        bfly<T>(v[1], v[3]);
-        v[3] = mul_i<T>(v[3], sign);
-        bfly<T>(v[0], v[1]);
-        bfly<T>(v[2], v[3]);
-    }
-    static __device__ __forceinline__ constexpr int out(int k) { return ((k & 1) << 1) | ((k >> 1) & 1); }
-};
-template <typename T> struct SmallDft<T, 8> {
-    static __device__ __forceinline__ void run(cx<T> (&v)[8], int sign)
-    {
-        const T c = (T)0.70710678118654752440;
-        const T s = sign > 0 ? c : -c;
-        bfly<T>(v[0], v[4]);
-        bfly<T>(v[1], v[5]);
-        bfly<T>(v[2], v[6]);
-        bfly<T>(v[3], v[7]);
-        v[5] = cmul(v[5], mk<T>(c, s));
-        v[6] = mul_i<T>(v[6], sign);
-        v[7] = cmul(v[7], mk<T>(-c, s));
-        bfly<T>(v[0], v[2]);
-        bfly<T>(v[1], v[3]);
-        bfly<T>(v[4], v[6]);
-        bfly<T>(v[5], v[7]);
-        v[3] = mul_i<T>(v[3], sign);
-        v[7] = mul_i<T>(v[7], sign);
-        bfly<T>(v[0], v[1]);
-        bfly<T>(v[2], v[3]);
-        bfly<T>(v[4], v[5]);
-        bfly<T>(v[6], v[7]);
-    }
-    static __device__ __forceinline__ constexpr int out(int k)
-    {
-        return ((k & 1) << 2) | (k & 2) | ((k >> 2) & 1);
-    }
-};
-
-// Shared-memory FFT buffers are padded by one entry per 16: the Stockham
-// writes at small strides (8 Ns entries apart) would otherwise fall on one
-// or two banks for the whole warp.
-__device__ __forceinline__ int pidx(int i) { return i + (i >> 4); }
-inline size_t padded_len(int n) { return (size_t)n + (size_t)n / 16 + 1; }
-
-template <typename T, int R, int LOGR, int BPT>
-__device__ __forceinline__ void stockham_pass(cx<T> *x, int logN, int logNs, int sign, const cx<T> *stw)
+template <typename T, int R> __device__ __forceinline__ void dft_small(cx<T> *v)
 {
-    static_assert(R == 2 || R == 4 || R == 8, "radix 2, 4 or 8");
-    const int NR = (1 << logN) >> LOGR;
-    const int Ns = 1 << logNs;
-    // w1 = e^{-2 pi i k / (R Ns)} = stw[Ns + k]: radix 2 and 4 run only as the first pass
-    // (Ns = 1, k = 0, w1 = 1), so the table of R = 8 serves every pass
-    cx<T> v[BPT][R];
+    if constexpr (R == 2) {
+        const cx<T> a = v[0];
+        v[0] = cadd(a, v[1]);
+        v[1] = csub(a, v[1]);
+    } else if constexpr (R == 4) {
+        dft4<T>(v[0], v[1], v[2], v[3]);
+    } else if constexpr (R == 8) {
+        const T h = (T)0.70710678118654752440;
+        cx<T> e[4] = {v[0], v[2], v[4], v[6]}, o[4] = {v[1], v[3], v[5], v[7]};
+        dft4<T>(e[0], e[1], e[2], e[3]);
+        dft4<T>(o[0], o[1], o[2], o[3]);
+        o[1] = mk<T>(h * (o[1].x + o[1].y), h * (o[1].y - o[1].x));
+        o[2] = mul_mi<T>(o[2]);
+        o[3] = mk<T>(h * (o[3].y - o[3].x), -h * (o[3].x + o[3].y));
 #pragma unroll
-    for (int b = 0; b < BPT; ++b) {
-        const int j = b * blockDim.x + threadIdx.x;
-        if (j < NR) {
-            const int k = j & (Ns - 1);
-            // twiddles w^r, r < R, from one table entry w = e^{-+2 pi i k / (R Ns)} by products
-            // in a tree of depth log2 R (w^2 = w w, w^3 = w^2 w, w^4 = w^2 w^2, ...), not a
-            // chain of R - 2 dependent products
-            cx<T> w[R];
-            w[0] = mk<T>(1, 0);
-            w[1] = stw[Ns + k];
-            if (sign > 0) w[1].y = -w[1].y;
+        for (int k = 0; k < 4; ++k) {
+            v[k] = cadd(e[k], o[k]);
+            v[k + 4] = csub(e[k], o[k]);
+        }
+    }
+}
+
+// 16 = 4 x 4; HALF: v[8..15] are zero on entry (and need not be set)
+template <typename T, bool HALF> __device__ __forceinline__ void dft16(cx<T> (&v)[16])
+{
+    const T c1 = (T)0.92387953251128675613, s1 = (T)0.38268343236508977173, h = (T)0.70710678118654752440;
 #pragma unroll
-            for (int r = 2; r < R; ++r) {
-                const int hb = r >= 4 ? 4 : 2;  // highest power of two <= r (R <= 8)
-                w[r] = r == hb ? cmul(w[hb / 2], w[hb / 2]) : cmul(w[hb], w[r - hb]);
+    for (int n = 0; n < 4; ++n) {
+        if (HALF) dft4_half<T>(v[n], v[4 + n], v[8 + n], v[12 + n]);
+        else dft4<T>(v[n], v[4 + n], v[8 + n], v[12 + n]);
+    }
+    // v[4 k + n] *= w16^{k n}
+    auto w1 = [&](cx<T> a, T c, T s) { return mk<T>(a.x * c + a.y * s, a.y * c - a.x * s); };  // a e^{-i angle}
+    v[5] = w1(v[5], c1, s1);
+    v[6] = mk<T>(h * (v[6].x + v[6].y), h * (v[6].y - v[6].x));
+    v[7] = w1(v[7], s1, c1);
+    v[9] = mk<T>(h * (v[9].x + v[9].y), h * (v[9].y - v[9].x));
+    v[10] = mul_mi<T>(v[10]);
+    v[11] = mk<T>(h * (v[11].y - v[11].x), -h * (v[11].x + v[11].y));
+    v[13] = w1(v[13], s1, c1);
+    v[14] = mk<T>(h * (v[14].y - v[14].x), -h * (v[14].x + v[14].y));
+    v[15] = w1(v[15], -c1, -s1);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) dft4<T>(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
+    // slot 4 k1 + k2 holds output k1 + 4 k2: transpose (register renaming)
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int b = a + 1; b < 4; ++b) {
+            const cx<T> x = v[4 * a + b];
+            v[4 * a + b] = v[4 * b + a];
+            v[4 * b + a] = x;
+        }
+}
+
+// v[k] *= w_N^{t k} (conjugated for INV), N = 2^B, t < N/16, from the table of every
+// N: tw[N - 32 + k N/16 + t].  FP32 reads k = 1, 4, 8 and forms the other powers (three
+// products deep at most); FP64, whose arithmetic is the scarce part, reads all of them.
+template <typename T, int B, bool INV>
+__device__ __forceinline__ void tw16(cx<T> (&v)[16], int t, const cx<T> *__restrict__ tw)
+{
+    constexpr int st = 1 << (B - 4);
+    const cx<T> *p = tw + ((1 << B) - 32) + t;
+    auto ld = [&](int k) {
+        cx<T> w = __ldg(p + k * st);
+        if (INV) w.y = -w.y;
+        return w;
+    };
+    if constexpr (sizeof(T) == 4) {
+        const cx<T> a = ld(1), q = ld(4), o = ld(8);
+        const cx<T> b = cmul(a, a), c = cmul(b, a), e = cmul(o, q);
+        v[1] = cmul(v[1], a);
+        v[2] = cmul(v[2], b);
+        v[3] = cmul(v[3], c);
+        v[4] = cmul(v[4], q);
+        v[5] = cmul(v[5], cmul(q, a));
+        v[6] = cmul(v[6], cmul(q, b));
+        v[7] = cmul(v[7], cmul(q, c));
+        v[8] = cmul(v[8], o);
+        v[9] = cmul(v[9], cmul(o, a));
+        v[10] = cmul(v[10], cmul(o, b));
+        v[11] = cmul(v[11], cmul(o, c));
+        v[12] = cmul(v[12], e);
+        v[13] = cmul(v[13], cmul(e, a));
+        v[14] = cmul(v[14], cmul(e, b));
+        v[15] = cmul(v[15], cmul(e, c));
+    } else {
+#pragma unroll
+        for (int k = 1; k < 16; ++k) v[k] = cmul(v[k], ld(k));
+    }
+}
+
+// shared buffers are padded by one entry per 16: the strides of the exchanges
+// below (16, R, 16 R entries) would otherwise fall on a few banks
+__host__ __device__ __forceinline__ int pidx(int i) { return i + (i >> 4); }
+inline size_t padded_len(size_t n) { return n + n / 16 + 1; }
+
+// ---------------------------------------------------------------------------
+// One DFT of length N = 2^B by a team of N/16 threads, 16 values each, in
+// registers.  Thread t enters with x[e N/16 + t] in v[e].
+//   B <= 8:  radix 16, exchange, radix R = N/16
+//   B >= 9:  radix 16, exchange, radix 16, exchange, radix R = N/256
+// The last exchange (the only one for B <= 8) stays inside groups of R <= 16
+// consecutive threads: a warp barrier.  The first needs the team's barrier
+// (a warp barrier again for B = 9, whose team is one warp).  The forward
+// transform leaves X in the registers in the order fft_index gives; the
+// inverse starts from that order and runs the same steps backwards, so a
+// convolution needs no reordering and its shared-memory traffic is four
+// exchanges.  In the backward run every thread writes the addresses it read
+// last, so no barrier guards the buffer between steps.
+// ---------------------------------------------------------------------------
+template <int B> struct Team {
+    static constexpr int N = 1 << B, NT = N / 16;           // values, threads
+    static constexpr int R = B <= 8 ? N / 16 : N / 256;     // last radix (B = 4: none)
+};
+
+// frequency held in register e of thread t after the forward transform of length 2^B
+__host__ __device__ inline int fft_index(int B, int t, int e)
+{
+    if (B == 4) return e;
+    if (B <= 8) {
+        const int R = 1 << (B - 4), u = e / R, k2 = e % R;
+        return t * (16 / R) + u + 16 * k2;
+    }
+    const int R = 1 << (B - 8), u = e / R, k3 = e % R, k1 = t / R, t2 = t % R;
+    return k1 + 16 * (t2 * (16 / R) + u) + 256 * k3;
+}
+
+template <int B> __device__ __forceinline__ void team_sync(int slot, unsigned mask)
+{
+    if constexpr (B <= 9) __syncwarp(mask);
+    else asm volatile("bar.sync %0, %1;" ::"r"(1 + slot), "r"(Team<B>::NT) : "memory");
+}
+
+// The addresses split into a part of the thread and a compile-time offset: pidx(a + b) =
+// pidx(a) + pidx(b) wherever b is a multiple of a power of two above a mod 16.
+template <typename T, int B, bool HALF>
+__device__ __forceinline__ void fft_forward(cx<T> (&v)[16], cx<T> *ex, int t, int slot, unsigned mask,
+                                            const cx<T> *__restrict__ tw)
+{
+    constexpr int NT = Team<B>::NT, R = Team<B>::R;
+    dft16<T, HALF>(v);
+    if constexpr (B > 4) {
+        tw16<T, B, false>(v, t, tw);
+        cx<T> *e1 = ex + pidx(t);
+#pragma unroll
+        for (int k = 0; k < 16; ++k) e1[pidx(k * NT)] = v[k];
+        team_sync<B>(slot, mask);
+        if constexpr (B > 8) {
+            cx<T> *e2 = ex + pidx((t / R) * NT + t % R);
+#pragma unroll
+            for (int k = 0; k < 16; ++k) v[k] = e2[pidx(k * R)];
+            dft16<T, false>(v);
+            tw16<T, B - 4, false>(v, t % R, tw);
+#pragma unroll
+            for (int k = 0; k < 16; ++k) e2[pidx(k * R)] = v[k];
+            __syncwarp(mask);
+        }
+        const cx<T> *e3 = ex + 17 * t;  // pidx(16 t)
+#pragma unroll
+        for (int e = 0; e < 16; ++e) v[e] = e3[e];
+        if constexpr (R == 16) {
+            dft16<T, false>(v);
+        } else {
+#pragma unroll
+            for (int u = 0; u < 16; u += R) dft_small<T, R>(v + u);
+        }
+    }
+}
+
+// inverse (unnormalised) of fft_forward on the conjugate: takes conj X, returns conj x
+template <typename T, int B>
+__device__ __forceinline__ void fft_backward(cx<T> (&v)[16], cx<T> *ex, int t, int slot, unsigned mask,
+                                             const cx<T> *__restrict__ tw)
+{
+    constexpr int NT = Team<B>::NT, R = Team<B>::R;
+    if constexpr (B > 4) {
+        if constexpr (R == 16) {
+            dft16<T, false>(v);
+        } else {
+#pragma unroll
+            for (int u = 0; u < 16; u += R) dft_small<T, R>(v + u);
+        }
+        cx<T> *e3 = ex + 17 * t;
+#pragma unroll
+        for (int e = 0; e < 16; ++e) e3[e] = v[e];
+        if constexpr (B > 8) {
+            __syncwarp(mask);
+            cx<T> *e2 = ex + pidx((t / R) * NT + t % R);
+#pragma unroll
+            for (int k = 0; k < 16; ++k) v[k] = e2[pidx(k * R)];
+            tw16<T, B - 4, false>(v, t % R, tw);
+            dft16<T, false>(v);
+#pragma unroll
+            for (int k = 0; k < 16; ++k) e2[pidx(k * R)] = v[k];
+        }
+        team_sync<B>(slot, mask);
+        const cx<T> *e1 = ex + pidx(t);
+#pragma unroll
+        for (int k = 0; k < 16; ++k) v[k] = e1[pidx(k * NT)];
+        tw16<T, B, false>(v, t, tw);
+    }
+    dft16<T, false>(v);
+}
+
+// threads of a ring CTA, one ring pair each: a team of 256 holds the longest Bluestein FFT
+// (N = 4096) with 16 values per thread; shorter ones run up to four of the pair's sub-DFTs
+// side by side
+constexpr int RING_CTA = 256;
+
+// position of value j of a ring (or of frequency j) in the padded buffer: the four
+// length-k sequences j mod 4 one after another
+__device__ __forceinline__ int zpos(int j, int k) { return pidx((j & 3) * k + (j >> 2)); }
+
+template <typename P> __device__ __forceinline__ const P *opaque(const P *p)
+{
+    asm volatile("" : "+l"(p));
+    return p;
+}
+__device__ __forceinline__ int opaque(int t)
+{
+    asm volatile("" : "+r"(t));
+    return t;
+}
+
+// The four length-k DFTs (forward; FLIP conjugates in and out, i.e. the inverse) of the
+// sequences at zb[pidx(r k + j)], in place.
+template <typename T, int B, bool BLUE>
+__device__ __noinline__ void sub_dfts(cx<T> *zb, cx<T> *exch, int k, bool flip, const cx<T> *V0,
+                                      const cx<T> *chirp0, const cx<T> *tw0)
+{
+    constexpr int N = Team<B>::N, NT = Team<B>::NT, R = Team<B>::R;
+    constexpr int SLOTS = NT * 4 <= RING_CTA ? 4 : RING_CTA / NT;
+    const int slot = threadIdx.x / NT, t0 = threadIdx.x % NT;
+    if (slot >= SLOTS) return;  // whole warps, or the lanes that `mask` leaves out
+    const unsigned mask = SLOTS * NT >= 32 ? 0xffffffffu : (1u << (SLOTS * NT)) - 1u;
+    cx<T> *ex = exch + slot * (N + N / 16);
+    const T sg = flip ? (T)-1 : (T)1;
+#pragma unroll 1
+    for (int r = slot; r < 4; r += SLOTS) {
+        // opaque: addresses and table values are formed again in every round (tables from L1);
+        // held in registers across the rounds and the FFTs they spill
+        const int t = opaque(t0);
+        const cx<T> *__restrict__ tw = opaque(tw0);
+        cx<T> v[16];
+        if constexpr (BLUE) {
+            const cx<T> *__restrict__ V = opaque(V0), *__restrict__ chirp = opaque(chirp0);
+            // value j = e NT + t of sequence r
+            cx<T> *z = zb + pidx(r * k + t);
+            auto at = [&](int e) -> cx<T> & { return NT >= 16 ? z[pidx(e * NT)] : zb[pidx(r * k + e * NT + t)]; };
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const int j = e * NT + t;
+                v[e] = mk<T>(0, 0);
+                if (j < k) {
+                    cx<T> u = at(e);
+                    u.y *= sg;
+                    v[e] = cmul(u, __ldg(chirp + j));
+                }
             }
+            fft_forward<T, B, true>(v, ex, t, slot, mask, tw);
 #pragma unroll
-            for (int r = 0; r < R; ++r) v[b][r] = x[pidx(j + r * NR)];
-#pragma unroll
-            for (int r = 1; r < R; ++r) v[b][r] = cmul(v[b][r], w[r]);
-            SmallDft<T, R>::run(v[b], sign);
-        }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int b = 0; b < BPT; ++b) {
-        const int j = b * blockDim.x + threadIdx.x;
-        if (j < NR) {
-            const int k = j & (Ns - 1);
-            const int d = ((j >> logNs) << (logNs + LOGR)) + k;
-#pragma unroll
-            for (int r = 0; r < R; ++r) x[pidx(d + SmallDft<T, R>::out(r) * Ns)] = v[b][r];
-        }
-    }
-    __syncthreads();
-}
-
-// Threads of the ring kernels: FP32 plans run 1024 (32 warps per SM, one radix-8
-// butterfly per thread and pass at N = 8192: twice the warps of 512 threads to hide the
-// shared-memory and L2 latencies of one pair's chain of passes), FP64 plans 512 (their
-// butterflies need twice the registers).
-template <typename T> __host__ __device__ constexpr int ring_threads() { return sizeof(T) == 4 ? 1024 : 512; }
-
-template <typename T>
-__device__ __noinline__ void fft_pow2(cx<T> *x, int logN, int sign, const cx<T> *stw)
-{
-    constexpr int NT = ring_threads<T>();
-    int logNs = 0;
-    const int head = logN % 3;
-    if (head == 1) {
-        stockham_pass<T, 2, 1, 4096 / NT>(x, logN, 0, sign, stw);
-        logNs = 1;
-    } else if (head == 2) {
-        stockham_pass<T, 4, 2, 2048 / NT>(x, logN, 0, sign, stw);
-        logNs = 2;
-    }
-    while (logNs < logN) {
-        stockham_pass<T, 8, 3, 1024 / NT>(x, logN, logNs, sign, stw);
-        logNs += 3;
-    }
-}
-
-// The n outputs of a ring DFT: in the padded FFT buffer (power-of-two rings)
-// or in the plain zout buffer (direct and Bluestein rings).
-template <typename T> struct RingOut {
-    const cx<T> *p;
-    int padded;
-    __device__ __forceinline__ cx<T> operator[](int j) const { return p[padded ? pidx(j) : j]; }
-};
-
-// DFT of one ring pair.  Input: padded buf (direct / pow2) or plain zin (Bluestein).
-template <typename T>
-__device__ RingOut<T> ring_dft(const RingTab &R, cx<T> *buf, cx<T> *zin, cx<T> *zout, int sign,
-                               const cx<T> *__restrict__ roots, const cx<T> *__restrict__ V,
-                               const cx<T> *__restrict__ chirp, const cx<T> *__restrict__ tw, int logNmax,
-                               const cx<T> *stw)
-{
-    const int n = R.n;
-    const unsigned twon = 2u * (unsigned)n;
-    const cx<T> *root = roots + R.rootOff;
-    if (R.kind == RING_NAIVE) {
-        for (int j = threadIdx.x; j < n; j += blockDim.x) {
-            cx<T> acc = mk<T>(0, 0);
-            for (int k = 0; k < n; ++k) {
-                cx<T> w = root[(2u * (unsigned)(j * k)) % twon];
-                if (sign < 0) w.y = -w.y;
-                acc = cadd(acc, cmul(buf[pidx(k)], w));
+            for (int e = 0; e < 16; ++e) {
+                v[e] = cmul(v[e], __ldg(V + e * NT + t));
+                v[e].y = -v[e].y;
             }
-            zout[j] = acc;
+            fft_backward<T, B>(v, ex, t, slot, mask, opaque(tw0));
+            const cx<T> *__restrict__ chirp2 = opaque(chirp0);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const int j = e * NT + t;
+                if (j < k) {
+                    cx<T> y = cmul(cconj(v[e]), __ldg(chirp2 + j));
+                    y.y *= sg;
+                    at(e) = y;
+                }
+            }
+        } else {
+            cx<T> *zr = zb + pidx(r * N), *z = zr + pidx(t);
+#pragma unroll
+            for (int e = 0; e < 16; ++e) {
+                v[e] = z[pidx(e * NT)];
+                v[e].y *= sg;
+            }
+            if (r >= SLOTS) team_sync<B>(slot, mask);  // the exchange buffer's last readers are done
+            fft_forward<T, B, false>(v, ex, t, slot, mask, tw);
+            // outputs land where other threads of the team may still read inputs (B = 4: its own)
+            team_sync<B>(slot, mask);
+            // pidx(fft_index(B, t, e)) as a part of the thread and a constant
+            cx<T> *o = zr + (B == 4 ? 0 : B <= 8 ? t * (16 / R) : t / R + 17 * (t % R) * (16 / R));
+#pragma unroll
+            for (int e = 0; e < 16; ++e) {
+                v[e].y *= sg;
+                o[B == 4 ? e : B <= 8 ? e / R + 17 * (e % R) : 17 * (e / R + 16 * (e % R))] = v[e];
+            }
         }
-        __syncthreads();
-        return RingOut<T>{zout, 0};
     }
+}
+
+template <typename T>
+__device__ __forceinline__ void ring_sub_dfts(const RingTab &R, cx<T> *zb, cx<T> *ex, bool flip,
+                                              const cx<T> *__restrict__ V, const cx<T> *__restrict__ chirp,
+                                              const cx<T> *__restrict__ tw)
+{
+    const cx<T> *v = V + R.vOff, *c = chirp + R.cOff;
+    const int k = R.n >> 2;
     if (R.kind == RING_POW2) {
-        fft_pow2<T>(buf, R.logF, sign, stw);
-        return RingOut<T>{buf, 1};
-    }
-    // Bluestein, two half-length passes; the chirp c_j = e^{-i pi j^2 / n} is read
-    // from its own table in order (consecutive lanes, consecutive entries)
-    const int H = 1 << R.logF;                 // M / 2
-    const int mstep = logNmax - (R.logF + 1);  // index step of w_M in tw
-    const cx<T> *Vh = V + R.vOff;
-    const cx<T> *ch = chirp + R.cOff;
-    for (int h = 0; h < 2; ++h) {
-#pragma unroll 4
-        for (int j = threadIdx.x; j < H; j += blockDim.x) {
-            cx<T> v = mk<T>(0, 0);
-            if (j < n) {
-                cx<T> u = zin[j];
-                if (sign > 0) u.y = -u.y;
-                v = cmul(u, ch[j]);
-                if (h) v = cmul(v, tw[j << mstep]);
-            }
-            buf[pidx(j)] = v;
+        switch (R.logF) {
+        case 4: sub_dfts<T, 4, false>(zb, ex, k, flip, v, c, tw); break;
+        case 5: sub_dfts<T, 5, false>(zb, ex, k, flip, v, c, tw); break;
+        case 6: sub_dfts<T, 6, false>(zb, ex, k, flip, v, c, tw); break;
+        case 7: sub_dfts<T, 7, false>(zb, ex, k, flip, v, c, tw); break;
+        case 8: sub_dfts<T, 8, false>(zb, ex, k, flip, v, c, tw); break;
+        case 9: sub_dfts<T, 9, false>(zb, ex, k, flip, v, c, tw); break;
+        case 10: sub_dfts<T, 10, false>(zb, ex, k, flip, v, c, tw); break;
+        default: sub_dfts<T, 11, false>(zb, ex, k, flip, v, c, tw); break;
         }
-        __syncthreads();
-        fft_pow2<T>(buf, R.logF, -1, stw);
-        for (int k = threadIdx.x; k < H; k += blockDim.x) buf[pidx(k)] = cmul(buf[pidx(k)], Vh[h * H + k]);
-        __syncthreads();
-        fft_pow2<T>(buf, R.logF, +1, stw);
-#pragma unroll 4
-        for (int k = threadIdx.x; k < n; k += blockDim.x) {
-            if (h == 0) {
-                zout[k] = buf[pidx(k)];
-            } else {
-                cx<T> w = tw[k << mstep];
-                w.y = -w.y;  // w_M^{-k}
-                cx<T> y = cmul(cadd(zout[k], cmul(buf[pidx(k)], w)), ch[k]);
-                if (sign > 0) y.y = -y.y;
-                zout[k] = y;
-            }
+    } else {
+        switch (R.logF) {
+        case 4: sub_dfts<T, 4, true>(zb, ex, k, flip, v, c, tw); break;
+        case 5: sub_dfts<T, 5, true>(zb, ex, k, flip, v, c, tw); break;
+        case 6: sub_dfts<T, 6, true>(zb, ex, k, flip, v, c, tw); break;
+        case 7: sub_dfts<T, 7, true>(zb, ex, k, flip, v, c, tw); break;
+        case 8: sub_dfts<T, 8, true>(zb, ex, k, flip, v, c, tw); break;
+        case 9: sub_dfts<T, 9, true>(zb, ex, k, flip, v, c, tw); break;
+        case 10: sub_dfts<T, 10, true>(zb, ex, k, flip, v, c, tw); break;
+        case 11: sub_dfts<T, 11, true>(zb, ex, k, flip, v, c, tw); break;
+        default: sub_dfts<T, 12, true>(zb, ex, k, flip, v, c, tw); break;
         }
-        __syncthreads();
     }
-    return RingOut<T>{zout, 0};
+    __syncthreads();
 }
 
-template <typename T>
 __device__ __forceinline__ double block_sum(double v, double *red)
 {
 #pragma unroll
     for (int o = 16; o >= 1; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (lane == 0) red[warp] = v;
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
     __syncthreads();
     double s = 0.0;
     if (threadIdx.x == 0)
         for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[w];
-    __syncthreads();  // red is reused by the next call
     return s;
 }
 
-struct RingCommon {
-    int npairs, lmax, L, logNmax;
-    int logB;             // log2 of the longest FFT run (the shared twiddle table has 2^logB / 4 entries)
+template <typename T> struct RingArgs {
+    int lmax, L;
     const RingTab *rings;
-    const int *order;     // ring pairs by decreasing cost
-    int *ticket;          // work counter (zeroed before the launch)
-    long long scr_stride;
-    const float2 *Glow;   // mixed path: FP64-block coefficients for m < lc, rounded to FP32 (or null)
+    const int *order;      // ring pairs by decreasing cost: CTA i takes pair order[i]
+    const cx<T> *roots, *V, *chirp, *tw;
+    int zlen;              // padded length of the ring buffer; the exchange buffer follows it
+    const cx<T> *G;        // synthesis input
+    const float2 *Glow;    // mixed path: FP64-block coefficients for m < lc, rounded to FP32 (or null)
     int lc, glow_stride;
-    int bpad;             // padded shared FFT buffer length
-    int zsmem;            // 1: Bluestein / direct buffers follow the FFT buffer in shared memory
+    int mode;              // RingSynMode, or RS_ANA
+    const T *r, *nu;       // blend
+    T lam, tau;
+    T *tmap;               // synthesis: output map; analysis: null
+    double *omap;          // RS_MAP output
+    const T *amap;         // RS_ANA input
+    double *part;          // per ring pair: chi^2 pixel term
+    cx<T> *F;              // analysis output
 };
 
-__device__ __forceinline__ void prefetch_l2(const void *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+constexpr int RS_ANA = 16;  // analysis only (beside RingSynMode)
 
-// prefetch a byte range into L2, one 128-byte line per thread and step
-__device__ __forceinline__ void prefetch_range(const void *base, size_t bytes)
+// north and south coefficient of one m (adjacent in memory): one 16-byte load in FP32
+__device__ __forceinline__ void load_ns(const float2 *g, float2 &n, float2 &s)
 {
-    const char *b = reinterpret_cast<const char *>(base);
-    for (size_t off = (size_t)threadIdx.x * 128; off < bytes; off += (size_t)blockDim.x * 128) prefetch_l2(b + off);
+    const float4 v = *reinterpret_cast<const float4 *>(g);
+    n = make_float2(v.x, v.y);
+    s = make_float2(v.z, v.w);
+}
+__device__ __forceinline__ void load_ns(const double2 *g, double2 &n, double2 &s)
+{
+    n = g[0];
+    s = g[1];
+}
+__device__ __forceinline__ void store_ns(float2 *g, float2 n, float2 s)
+{
+    *reinterpret_cast<float4 *>(g) = make_float4(n.x, n.y, s.x, s.y);
+}
+__device__ __forceinline__ void store_ns(double2 *g, double2 n, double2 s)
+{
+    g[0] = n;
+    g[1] = s;
 }
 
-__device__ __forceinline__ bool aligned16(const void *p) { return ((size_t)p & 15) == 0; }
-
-// Eq. 3 blend of four pixels (float4 lanes), adding their chi^2 pixel terms to chi
-__device__ __forceinline__ float4 blend4(float4 s, float4 r, float4 nu, float lt, float lm1t, float &chi)
+// Fold H_k = sum_{m = k mod n} G_m e^{i pi m q / n} + conj terms of -m, for the packed
+// north/south pair.  e^{i pi m / n} at m = k + a n is (-1)^a e^{i pi k / n}: the aliases of a
+// bin are summed with alternating signs and take the phase once.  Rings longer than L have
+// at most one alias of each sign, independent bins with several loads in flight; shorter
+// rings sum each bin over S lanes of a warp (S up to 32 for the polar rings, whose bins
+// collect ~2L/n aliases), combined by shuffles in a fixed order.
+template <typename T>
+__device__ __forceinline__ void fold_ring(const RingArgs<T> &A, const RingTab &R, const cx<T> *__restrict__ g,
+                                          const float2 *__restrict__ gl, bool south, cx<T> *zb)
 {
-    auto one = [&](float sv, float rv, float nv) {
-        const float den = 1.f + lm1t * nv;
-        chi += (nv * sv * sv - 2.f * rv * sv) / den;
-        return sv + lt * (rv - nv * sv) / den;
+    const int n = R.n, q = R.q, L = A.L, k4 = n >> 2, lc = gl ? A.lc : 0;
+    const cx<T> *root = A.roots + R.rootOff;
+    auto coef = [&](int m, cx<T> &a, cx<T> &b) {
+        load_ns(g + 2 * m, a, b);
+        if (m < lc) {
+            const float2 x = gl[2 * m], y = gl[2 * m + 1];
+            a.x += (T)x.x;
+            a.y += (T)x.y;
+            b.x += (T)y.x;
+            b.y += (T)y.y;
+        }
     };
-    return make_float4(one(s.x, r.x, nu.x), one(s.y, r.y, nu.y), one(s.z, r.z, nu.z), one(s.w, r.w, nu.w));
-}
-
-// Shared twiddle table by pass: stw[Ns + k] = e^{-2 pi i k / (8 Ns)} = tw[k 2^logNmax / (8 Ns)]
-// for the powers of two Ns <= 2^logB / 8 (entry 0 unused).
-template <typename T>
-__device__ __forceinline__ void load_twiddles(cx<T> *stw, const cx<T> *__restrict__ tw, const RingCommon &rc)
-{
-    const int n = (1 << rc.logB) >> 2;
-    for (int u = threadIdx.x; u < n; u += blockDim.x) {
-        if (u == 0) continue;
-        const int logNs = 31 - __clz(u), k = u - (1 << logNs);
-        stw[u] = tw[(size_t)k << (rc.logNmax - 3 - logNs)];
+    if (n > L) {
+#pragma unroll 4
+        for (int k = threadIdx.x; k < n; k += RING_CTA) {
+            cx<T> hn = mk<T>(0, 0), hs = mk<T>(0, 0), a, b;
+            if (k <= L) {
+                coef(k, a, b);
+                const cx<T> ph = root[q ? k : 0];
+                hn = cmul(a, ph);
+                hs = cmul(b, ph);
+            }
+            const int mneg = n - k;
+            if (k > 0 && mneg <= L) {
+                coef(mneg, a, b);
+                const cx<T> ph = root[q ? mneg : 0];
+                hn = cadd(hn, cconj(cmul(a, ph)));
+                hs = cadd(hs, cconj(cmul(b, ph)));
+            }
+            if (!south) hs = mk<T>(0, 0);
+            zb[zpos(k, k4)] = mk<T>(hn.x - hs.y, hn.y + hs.x);
+        }
+        return;
     }
-}
-
-// The next pair's ring tables into L2: e^{i pi p / n} (fold phases and Bluestein chirps)
-// and, for a Bluestein ring, its filter spectrum (M entries).
-template <typename T>
-__device__ __forceinline__ void prefetch_ring_tables(const RingTab &Rn, const cx<T> *roots, const cx<T> *V,
-                                                     const cx<T> *chirp)
-{
-    if (Rn.kind == RING_BLUESTEIN) {
-        prefetch_range(roots + Rn.rootOff, (size_t)2 * Rn.n * sizeof(cx<T>));
-        prefetch_range(V + Rn.vOff, ((size_t)2 << Rn.logF) * sizeof(cx<T>));
-        prefetch_range(chirp + Rn.cOff, (size_t)Rn.n * sizeof(cx<T>));
-    } else if (Rn.q) {
-        prefetch_range(roots + Rn.rootOff, (size_t)2 * Rn.n * sizeof(cx<T>));
+    int S = 1;
+    while (S < 32 && 2 * S * n <= RING_CTA) S *= 2;
+    const int sub = threadIdx.x & (S - 1), nb = RING_CTA / S;
+    for (int base = 0; base < n; base += nb) {
+        const int k = base + threadIdx.x / S;
+        cx<T> pn = mk<T>(0, 0), ps = pn, mn = pn, ms = pn, a, b;
+        if (k < n) {
+            const int m0 = k == 0 ? n : n - k;
+            // alternating signs over the alias number (q = 1; the belt's q = 0 rings are longer than L
+            // or take no sign)
+#pragma unroll 2
+            for (int i = sub, m = k + sub * n; m <= L; i += S, m += S * n) {
+                coef(m, a, b);
+                const T s = (q && (i & 1)) ? (T)-1 : (T)1;
+                pn.x = fma(s, a.x, pn.x);
+                pn.y = fma(s, a.y, pn.y);
+                ps.x = fma(s, b.x, ps.x);
+                ps.y = fma(s, b.y, ps.y);
+            }
+#pragma unroll 2
+            for (int i = sub, m = m0 + sub * n; m <= L; i += S, m += S * n) {
+                coef(m, a, b);
+                const T s = (q && (i & 1)) ? (T)-1 : (T)1;
+                mn.x = fma(s, a.x, mn.x);
+                mn.y = fma(s, a.y, mn.y);
+                ms.x = fma(s, b.x, ms.x);
+                ms.y = fma(s, b.y, ms.y);
+            }
+            const cx<T> ph = root[q ? k : 0], pm = root[q ? m0 : 0];
+            pn = cadd(cmul(pn, ph), cconj(cmul(mn, pm)));
+            ps = cadd(cmul(ps, ph), cconj(cmul(ms, pm)));
+        }
+        for (int o = S >> 1; o >= 1; o >>= 1) {
+            pn.x += __shfl_xor_sync(0xffffffffu, pn.x, o);
+            pn.y += __shfl_xor_sync(0xffffffffu, pn.y, o);
+            ps.x += __shfl_xor_sync(0xffffffffu, ps.x, o);
+            ps.y += __shfl_xor_sync(0xffffffffu, ps.y, o);
+        }
+        if (k < n && sub == 0) {
+            if (!south) ps = mk<T>(0, 0);
+            zb[zpos(k, k4)] = mk<T>(pn.x - ps.y, pn.y + ps.x);
+        }
     }
-}
-
-// Work distribution: CTAs take ring pairs from a global counter in order of
-// decreasing cost (Bluestein rings first), one ticket ahead so that the next
-// pair's rows can be prefetched while this one is transformed.
-__device__ __forceinline__ int take_ticket(int *ticket, int *s_tick)
-{
-    if (threadIdx.x == 0) *s_tick = atomicAdd(ticket, 1);
-    __syncthreads();
-    const int t = *s_tick;
-    __syncthreads();
-    return t;
 }
 
 // Unfold a forward ring DFT of the packed pair (z = f_N + i f_S) to
-// F_m = e^{-i pi m q / n} DFT(f)[m mod n] for both rings, m <= L; ends with a barrier.
+// F_m = e^{-i pi m q / n} DFT(f)[m mod n] for both rings, m <= L.
 template <typename T>
-__device__ __forceinline__ void unfold_ring(const RingTab &R, const RingOut<T> &z, const cx<T> *__restrict__ root, int q,
-                                            unsigned twon, bool south, cx<T> *__restrict__ f, int L)
+__device__ __forceinline__ void unfold_ring(const RingArgs<T> &A, const RingTab &R, const cx<T> *zb, bool south,
+                                            cx<T> *__restrict__ f)
 {
-    const int n = R.n;
+    const int n = R.n, k4 = n >> 2, L = A.L;
+    const cx<T> *root = A.roots + R.rootOff;
 #pragma unroll 4
-    for (int m = threadIdx.x; m <= L; m += blockDim.x) {
-        const int k = m % n;
-        const int nk = (n - k) % n;
-        const cx<T> zk = z[k], znk = z[nk];
+    for (int m = threadIdx.x; m <= L; m += RING_CTA) {
+        const unsigned al = __umulhi((unsigned)m, R.inv);  // m / n
+        const int k = m - (int)al * n;
+        const int nk = k ? n - k : 0;
+        const cx<T> zk = zb[zpos(k, k4)], znk = zb[zpos(nk, k4)];
+        cx<T> ph = mk<T>(1, 0);
+        if (R.q) {
+            ph = root[k];
+            const T s = (al & 1) ? (T)-1 : (T)1;
+            ph = mk<T>(s * ph.x, -s * ph.y);
+        }
         const cx<T> tn = mk<T>((T)0.5 * (zk.x + znk.x), (T)0.5 * (zk.y - znk.y));
         const cx<T> ts = mk<T>((T)0.5 * (zk.y + znk.y), (T)-0.5 * (zk.x - znk.x));
-        cx<T> ph = root[q ? (unsigned)m % twon : 0u];
-        ph.y = -ph.y;
-        f[2 * m] = cmul(ph, tn);
-        f[2 * m + 1] = south ? cmul(ph, ts) : mk<T>(0, 0);
+        store_ns(f + 2 * m, cmul(ph, tn), south ? cmul(ph, ts) : mk<T>(0, 0));
     }
-    __syncthreads();
 }
 
-// ---------------------------------------------------------------------------
-// synthesis side: fold -> inverse ring DFT -> blend (or write the map)
-// ---------------------------------------------------------------------------
-// Fold H_k = sum_{m = k mod n} G_m e^{i pi m q / n} + conj terms of -m, for
-// the packed north/south pair.  Each bin is summed by S sub-lanes of one warp
-// (S = n > 256 ? 1 : up to 32), each taking every S-th alias of the bin, and
-// the S partial sums are combined by shuffles in a fixed order: small polar
-// rings, whose bins collect up to 2L/n aliases, no longer serialise the CTA.
-template <typename T>
-__global__ void __launch_bounds__(ring_threads<T>(), 1) k_ringsyn(RingCommon rc, const cx<T> *__restrict__ roots,
-                                                          const cx<T> *__restrict__ V,
-                                                          const cx<T> *__restrict__ chirp, const cx<T> *__restrict__ tw,
-                                                          cx<T> *__restrict__ scr, const cx<T> *__restrict__ G,
-                                                          int mode, const T *__restrict__ r, const T *__restrict__ nu,
-                                                          T lam, T tau, T *__restrict__ tmap,
-                                                          double *__restrict__ omap, double *__restrict__ part,
-                                                          cx<T> *__restrict__ F)
+// One ring pair per CTA: fold, four inverse sub-DFTs, radix-4 step with the pixels (blend, or a
+// map written or read), four forward sub-DFTs, unfold.
+//
+// What bounds it: the latency of one pair's chain of steps, covered by the SM's other CTAs.  An
+// earlier version gave a pair a 1024-thread CTA and in-place radix-8 passes in shared memory,
+// each between two CTA barriers (~60 barriers per Bluestein pair, the first stall).  Here a
+// pair takes 256 threads and keeps its values in registers between two exchanges per FFT.
+// Mean over the ring passes of one solve (cooling and full-band steps, output map), FP32: nside
+// 2048 1.28 -> 0.53 ms, nside 512 0.153 -> 0.057 ms, nside 128 0.042 -> 0.019 ms (cold caches);
+// FP64: nside 512 0.93 -> 0.55 ms and nside 100 0.21 -> 0.073 ms, bound by the FP64 pipe.
+//
+// MINB CTAs per SM set the register budget: FP32 at 128 registers (2) or 80 with a small spill
+// (3).  Three are faster where shared memory holds three and there are pairs for them (a map
+// pass at nside 1024 0.131 -> 0.112 ms, a step at nside 512 0.066 -> 0.057 ms), two where it does
+// not (nside 2048: 0.525 against 0.570 ms averaged over a solve) or where one wave holds every
+// pair (nside 128: 18.5 against 20.6 us).  FP64: two at 128 registers against one at 255:
+// nside 100 0.126 -> 0.073 ms, nside 512 0.60 -> 0.55 ms.
+template <typename T, int MINB>
+__global__ void __launch_bounds__(RING_CTA, MINB) k_ring(const RingArgs<T> A)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ double red[32];
-    __shared__ int s_tick;
-    cx<T> *buf = reinterpret_cast<cx<T> *>(smem_raw);
-    cx<T> *zin = rc.zsmem ? buf + rc.bpad : scr + (size_t)blockIdx.x * rc.scr_stride;
-    cx<T> *zout = zin + rc.scr_stride / 2;
-    cx<T> *stw = buf + rc.bpad + (rc.zsmem ? rc.scr_stride : 0);
-    load_twiddles<T>(stw, tw, rc);
-    const int L = rc.L;
-    const T lt = lam * tau, lm1t = (lam - (T)1) * tau;
-    int cur = take_ticket(rc.ticket, &s_tick);
-    while (cur < rc.npairs) {
-        if (threadIdx.x == 0) s_tick = atomicAdd(rc.ticket, 1);
+    __shared__ double red[RING_CTA / 32];
+    cx<T> *zb = reinterpret_cast<cx<T> *>(smem_raw), *ex = zb + A.zlen;
+    const int pair = A.order[blockIdx.x], mode = A.mode;
+    const RingTab R = A.rings[pair];
+    const int n = R.n, k = n >> 2;
+    const bool south = R.offS >= 0, syn = mode != RS_ANA, blend = mode == RS_BLEND || mode == RS_BLEND_ANA;
+    const bool ana = mode == RS_ANA || mode == RS_BLEND_ANA;
+    const cx<T> *root = A.roots + R.rootOff;
+    const size_t row = (size_t)pair * (A.lmax + 1) * 2;
+    if (syn) {
+        fold_ring<T>(A, R, A.G + row, A.Glow ? A.Glow + (size_t)pair * A.glow_stride * 2 : nullptr, south, zb);
         __syncthreads();
-        const int nxt = s_tick;
-        const int pair = rc.order[cur];
-        const RingTab R = rc.rings[pair];
-        const int n = R.n, q = R.q;
-        const unsigned twon = 2u * (unsigned)n;
-        const cx<T> *root = roots + R.rootOff;
-        const cx<T> *g = G + (size_t)pair * (rc.lmax + 1) * 2;
-        const bool blue = R.kind == RING_BLUESTEIN;
-        const bool south = R.offS >= 0;
-        if (nxt < rc.npairs) {  // next pair of this CTA: pull its rows into L2
-            const int pn = rc.order[nxt];
-            const RingTab Rn = rc.rings[pn];
-            prefetch_range(G + (size_t)pn * (rc.lmax + 1) * 2, (size_t)(L + 1) * 2 * sizeof(cx<T>));
-            prefetch_ring_tables<T>(Rn, roots, V, chirp);
-            if (mode == RS_BLEND) {
-                prefetch_range(r + Rn.offN, (size_t)Rn.n * sizeof(T));
-                prefetch_range(nu + Rn.offN, (size_t)Rn.n * sizeof(T));
-                if (Rn.offS >= 0) {
-                    prefetch_range(r + Rn.offS, (size_t)Rn.n * sizeof(T));
-                    prefetch_range(nu + Rn.offS, (size_t)Rn.n * sizeof(T));
-                }
-            }
-        }
-        const float2 *gl = rc.Glow ? rc.Glow + (size_t)pair * rc.glow_stride * 2 : nullptr;
-        auto coef = [&](int m, int h) -> cx<T> {
-            cx<T> v = g[2 * m + h];
-            if (gl && m < rc.lc) {
-                const float2 w = gl[2 * m + h];
-                v.x += (T)w.x;
-                v.y += (T)w.y;
-            }
-            return v;
-        };
-        int S = 1;
-        while (S < 32 && 2 * S * n <= (int)blockDim.x) S *= 2;
-        const int sub = threadIdx.x & (S - 1);
-        const int nb = blockDim.x / S;
-        // rings longer than L: each bin k has at most one alias of each sign (m = k and
-        // m = n - k), so the bins are independent and four of them are loaded at once
-        const bool single = n > L;
-        if (single) {
-#pragma unroll 4
-            for (int k = threadIdx.x; k < n; k += blockDim.x) {
-                cx<T> hn = mk<T>(0, 0), hs = mk<T>(0, 0);
-                if (k <= L) {
-                    const cx<T> ph = root[q ? k : 0];
-                    hn = cmul(coef(k, 0), ph);
-                    hs = cmul(coef(k, 1), ph);
-                }
-                const int mneg = n - k;
-                if (k > 0 && mneg <= L) {
-                    const cx<T> ph = root[q ? mneg : 0];
-                    hn = cadd(hn, cconj(cmul(coef(mneg, 0), ph)));
-                    hs = cadd(hs, cconj(cmul(coef(mneg, 1), ph)));
-                }
-                if (!south) hs = mk<T>(0, 0);
-                const cx<T> z = mk<T>(hn.x - hs.y, hn.y + hs.x);
-                if (blue) zin[k] = z;
-                else buf[pidx(k)] = z;
-            }
-        }
-        for (int base = 0; base < (single ? 0 : n); base += nb) {
-            const int k = base + threadIdx.x / S;
-            cx<T> hn = mk<T>(0, 0), hs = mk<T>(0, 0);
-            if (k < n) {
-                for (int m = k + sub * n; m <= L; m += S * n) {
-                    const cx<T> ph = root[q ? (unsigned)m % twon : 0u];
-                    hn = cadd(hn, cmul(coef(m, 0), ph));
-                    hs = cadd(hs, cmul(coef(m, 1), ph));
-                }
-                for (int m = (k == 0 ? n : n - k) + sub * n; m <= L; m += S * n) {
-                    const cx<T> ph = root[q ? (unsigned)m % twon : 0u];
-                    hn = cadd(hn, cconj(cmul(coef(m, 0), ph)));
-                    hs = cadd(hs, cconj(cmul(coef(m, 1), ph)));
-                }
-            }
-            for (int o = S >> 1; o >= 1; o >>= 1) {
-                hn.x += __shfl_xor_sync(0xffffffffu, hn.x, o);
-                hn.y += __shfl_xor_sync(0xffffffffu, hn.y, o);
-                hs.x += __shfl_xor_sync(0xffffffffu, hs.x, o);
-                hs.y += __shfl_xor_sync(0xffffffffu, hs.y, o);
-            }
-            if (k < n && sub == 0) {
-                if (!south) hs = mk<T>(0, 0);
-                const cx<T> z = mk<T>(hn.x - hs.y, hn.y + hs.x);
-                if (blue) zin[k] = z;
-                else buf[pidx(k)] = z;
-            }
-        }
-        __syncthreads();
-        const RingOut<T> z = ring_dft<T>(R, buf, zin, zout, +1, roots, V, chirp, tw, rc.logNmax, stw);
-        T chi_pair = 0;  // per-thread partial of this pair in the working precision
-        int j0 = threadIdx.x, jstep = blockDim.x;
+        ring_sub_dfts<T>(R, zb, ex, true, A.V, A.chirp, A.tw);
+    }
+    const T lt = A.lam * A.tau, lm1t = (A.lam - (T)1) * A.tau;
+    T chi = 0;
+    auto blend1 = [&](T s, T rv, T nv) {
+        const T id = (T)1 / ((T)1 + lm1t * nv);  // one division for both (FP64 divides are a dozen operations)
+        chi += (nv * s * s - (T)2 * rv * s) * id;
+        return s + lt * (rv - nv * s) * id;
+    };
+#pragma unroll 2
+    for (int p = threadIdx.x; p < k; p += RING_CTA) {
+        const int z0 = pidx(p), z1 = pidx(k + p), z2 = pidx(2 * k + p), z3 = pidx(3 * k + p);
+        cx<T> w1 = root[2 * p], w2, w3;
         if constexpr (sizeof(T) == 4) {
-            // four consecutive pixels per thread with 16-byte loads and stores (ring
-            // lengths and offsets are multiples of 4); the scalar loop below takes over
-            // for unaligned map views
-            const bool fused = mode == RS_BLEND_ANA, blend = mode == RS_BLEND || fused;
-            if (mode != RS_MAP && (fused || (aligned16(tmap + R.offN) && (!south || aligned16(tmap + R.offS)))) &&
-                (!blend ||
-                 (aligned16(r + R.offN) && aligned16(nu + R.offN) &&
-                  (!south || (aligned16(r + R.offS) && aligned16(nu + R.offS)))))) {
-                for (int j = 4 * threadIdx.x; j < n; j += 4 * blockDim.x) {
-                    const cx<T> z0 = z[j], z1 = z[j + 1], z2 = z[j + 2], z3 = z[j + 3];
-                    float4 sN = make_float4(z0.x, z1.x, z2.x, z3.x), sS = make_float4(z0.y, z1.y, z2.y, z3.y);
-                    if (blend) {
-                        sN = blend4(sN, *reinterpret_cast<const float4 *>(r + R.offN + j),
-                                    *reinterpret_cast<const float4 *>(nu + R.offN + j), lt, lm1t, chi_pair);
-                        if (south)
-                            sS = blend4(sS, *reinterpret_cast<const float4 *>(r + R.offS + j),
-                                        *reinterpret_cast<const float4 *>(nu + R.offS + j), lt, lm1t, chi_pair);
-                    }
-                    if (fused) {  // packed north/south input of the forward DFT (same indices as z)
-                        if (!south) sS = make_float4(0.f, 0.f, 0.f, 0.f);
-                        cx<T> *d = blue ? zin + j : nullptr;
-                        const cx<T> v0 = mk<T>(sN.x, sS.x), v1 = mk<T>(sN.y, sS.y), v2 = mk<T>(sN.z, sS.z),
-                                    v3 = mk<T>(sN.w, sS.w);
-                        if (d) {
-                            d[0] = v0;
-                            d[1] = v1;
-                            d[2] = v2;
-                            d[3] = v3;
-                        } else {
-                            buf[pidx(j)] = v0;
-                            buf[pidx(j + 1)] = v1;
-                            buf[pidx(j + 2)] = v2;
-                            buf[pidx(j + 3)] = v3;
-                        }
-                    } else {
-                        *reinterpret_cast<float4 *>(tmap + R.offN + j) = sN;
-                        if (south) *reinterpret_cast<float4 *>(tmap + R.offS + j) = sS;
-                    }
-                }
-                j0 = n;  // done
-            }
-        }
-        for (int j = j0; j < n; j += jstep) {
-            const cx<T> zz = z[j];
-            const long long iN = R.offN + j;
-            if (mode == RS_MAP) {
-                omap[iN] = (double)zz.x;
-                if (south) omap[R.offS + j] = (double)zz.y;
-            } else if (mode == RS_SYN) {
-                tmap[iN] = zz.x;
-                if (south) tmap[R.offS + j] = zz.y;
-            } else {
-                T tN, tS = 0;
-                {
-                    const T s = zz.x, nv = nu[iN], rv = r[iN];
-                    const T den = (T)1 + lm1t * nv;
-                    tN = s + lt * (rv - nv * s) / den;
-                    chi_pair += (nv * s * s - (T)2 * rv * s) / den;
-                }
-                if (south) {
-                    const long long iS = R.offS + j;
-                    const T s = zz.y, nv = nu[iS], rv = r[iS];
-                    const T den = (T)1 + lm1t * nv;
-                    tS = s + lt * (rv - nv * s) / den;
-                    chi_pair += (nv * s * s - (T)2 * rv * s) / den;
-                }
-                if (mode == RS_BLEND_ANA) {  // same index as z: read and written by this thread only
-                    if (blue) zin[j] = mk<T>(tN, tS);
-                    else buf[pidx(j)] = mk<T>(tN, tS);
-                } else {
-                    tmap[iN] = tN;
-                    if (south) tmap[R.offS + j] = tS;
-                }
-            }
-        }
-        if (mode == RS_BLEND || mode == RS_BLEND_ANA) {  // per-pair partial: the reduction order does not depend on the schedule
-            const double s = block_sum<T>((double)chi_pair, red);
-            if (threadIdx.x == 0) part[pair] = s;
+            w2 = cmul(w1, w1);
+            w3 = cmul(w2, w1);
         } else {
-            __syncthreads();
+            w2 = root[4 * p];
+            w3 = root[6 * p];
         }
-        if (mode == RS_BLEND_ANA) {  // forward DFT of the blended ring and unfold to F_m, m <= L
-            const RingOut<T> zf = ring_dft<T>(R, buf, zin, zout, -1, roots, V, chirp, tw, rc.logNmax, stw);
-            unfold_ring<T>(R, zf, root, q, twon, south, F + (size_t)pair * (rc.lmax + 1) * 2, L);
-        }
-        cur = nxt;
-    }
-}
-
-// ---------------------------------------------------------------------------
-// analysis side: pack -> forward ring DFT -> unfold to F_m, m <= L
-// ---------------------------------------------------------------------------
-template <typename T>
-__global__ void __launch_bounds__(ring_threads<T>(), 1) k_ringana(RingCommon rc, const cx<T> *__restrict__ roots,
-                                                          const cx<T> *__restrict__ V,
-                                                          const cx<T> *__restrict__ chirp, const cx<T> *__restrict__ tw,
-                                                          cx<T> *__restrict__ scr, const T *__restrict__ map,
-                                                          cx<T> *__restrict__ F)
-{
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ int s_tick;
-    cx<T> *buf = reinterpret_cast<cx<T> *>(smem_raw);
-    cx<T> *zin = rc.zsmem ? buf + rc.bpad : scr + (size_t)blockIdx.x * rc.scr_stride;
-    cx<T> *zout = zin + rc.scr_stride / 2;
-    cx<T> *stw = buf + rc.bpad + (rc.zsmem ? rc.scr_stride : 0);
-    load_twiddles<T>(stw, tw, rc);
-    const int L = rc.L;
-    int cur = take_ticket(rc.ticket, &s_tick);
-    while (cur < rc.npairs) {
-        if (threadIdx.x == 0) s_tick = atomicAdd(rc.ticket, 1);
-        __syncthreads();
-        const int nxt = s_tick;
-        const int pair = rc.order[cur];
-        const RingTab R = rc.rings[pair];
-        const int n = R.n, q = R.q;
-        const unsigned twon = 2u * (unsigned)n;
-        const cx<T> *root = roots + R.rootOff;
-        const bool blue = R.kind == RING_BLUESTEIN;
-        const bool south = R.offS >= 0;
-        if (nxt < rc.npairs) {
-            const RingTab Rn = rc.rings[rc.order[nxt]];
-            prefetch_ring_tables<T>(Rn, roots, V, chirp);
-            prefetch_range(map + Rn.offN, (size_t)Rn.n * sizeof(T));
-            if (Rn.offS >= 0) prefetch_range(map + Rn.offS, (size_t)Rn.n * sizeof(T));
-        }
-        int j0 = threadIdx.x;
-        if constexpr (sizeof(T) == 4) {
-            // four consecutive pixels per thread with 16-byte loads (aligned map views)
-            if (aligned16(map + R.offN) && (!south || aligned16(map + R.offS))) {
-                for (int j = 4 * threadIdx.x; j < n; j += 4 * blockDim.x) {
-                    const float4 a = *reinterpret_cast<const float4 *>(map + R.offN + j);
-                    const float4 b = south ? *reinterpret_cast<const float4 *>(map + R.offS + j) : make_float4(0, 0, 0, 0);
-                    cx<T> *d = blue ? zin + j : nullptr;
-                    const cx<T> v0 = mk<T>(a.x, b.x), v1 = mk<T>(a.y, b.y), v2 = mk<T>(a.z, b.z), v3 = mk<T>(a.w, b.w);
-                    if (d) {
-                        d[0] = v0;
-                        d[1] = v1;
-                        d[2] = v2;
-                        d[3] = v3;
-                    } else {
-                        buf[pidx(j)] = v0;
-                        buf[pidx(j + 1)] = v1;
-                        buf[pidx(j + 2)] = v2;
-                        buf[pidx(j + 3)] = v3;
-                    }
+        // x[s]: pixel p + s k of the north (re) and south (im) ring
+        cx<T> x[4];
+        const long long iN = R.offN + p, iS = R.offS + p;
+        if (syn) {
+            // the four sub-DFTs conjugated: x_s = conj sum_r (-i)^{rs} conj(w^{rp} X_r)
+            x[0] = cconj(zb[z0]);
+            x[1] = cconj(cmul(zb[z1], w1));
+            x[2] = cconj(cmul(zb[z2], w2));
+            x[3] = cconj(cmul(zb[z3], w3));
+            dft4<T>(x[0], x[1], x[2], x[3]);
+#pragma unroll
+            for (int s = 0; s < 4; ++s) x[s].y = -x[s].y;
+            if (mode == RS_MAP) {
+#pragma unroll
+                for (int s = 0; s < 4; ++s) {
+                    A.omap[iN + s * k] = (double)x[s].x;
+                    if (south) A.omap[iS + s * k] = (double)x[s].y;
                 }
-                j0 = n;
+            } else if (blend) {
+                T rN[4], nN[4], rS[4], nS[4];
+#pragma unroll
+                for (int s = 0; s < 4; ++s) {
+                    rN[s] = A.r[iN + s * k];
+                    nN[s] = A.nu[iN + s * k];
+                    rS[s] = south ? A.r[iS + s * k] : (T)0;
+                    nS[s] = south ? A.nu[iS + s * k] : (T)0;
+                }
+#pragma unroll
+                for (int s = 0; s < 4; ++s) {
+                    x[s].x = blend1(x[s].x, rN[s], nN[s]);
+                    x[s].y = south ? blend1(x[s].y, rS[s], nS[s]) : (T)0;
+                }
             }
+            if (mode == RS_SYN || mode == RS_BLEND) {
+#pragma unroll
+                for (int s = 0; s < 4; ++s) {
+                    A.tmap[iN + s * k] = x[s].x;
+                    if (south) A.tmap[iS + s * k] = x[s].y;
+                }
+            }
+        } else {
+#pragma unroll
+            for (int s = 0; s < 4; ++s) x[s] = mk<T>(A.amap[iN + s * k], south ? A.amap[iS + s * k] : (T)0);
         }
-        for (int j = j0; j < n; j += blockDim.x) {
-            const cx<T> v = mk<T>(map[R.offN + j], south ? map[R.offS + j] : (T)0);
-            if (blue) zin[j] = v;
-            else buf[pidx(j)] = v;
+        if (ana) {
+            dft4<T>(x[0], x[1], x[2], x[3]);
+            zb[z0] = x[0];
+            zb[z1] = cmul(x[1], cconj(w1));
+            zb[z2] = cmul(x[2], cconj(w2));
+            zb[z3] = cmul(x[3], cconj(w3));
         }
+    }
+    if (blend) {  // per-pair partial: the reduction order does not depend on the schedule
+        const double s = block_sum((double)chi, red);
+        if (threadIdx.x == 0) A.part[pair] = s;
+    }
+    if (ana) {
         __syncthreads();
-        const RingOut<T> z = ring_dft<T>(R, buf, zin, zout, -1, roots, V, chirp, tw, rc.logNmax, stw);
-        unfold_ring<T>(R, z, root, q, twon, south, F + (size_t)pair * (rc.lmax + 1) * 2, L);
-        cur = nxt;
+        ring_sub_dfts<T>(R, zb, ex, false, A.V, A.chirp, A.tw);
+        unfold_ring<T>(A, R, zb, south, A.F + row);
     }
 }
 
 template <typename T> struct RingLaunch {
-    static RingCommon common(wf_plan p, int L)
+    static RingArgs<T> args(wf_plan p, int L, int mode)
     {
         const HpTables &t = p->tab;
-        RingCommon rc{};
-        rc.npairs = p->npairs;
-        rc.lmax = p->lmax;
-        rc.L = L;
-        rc.logNmax = t.logNmax;
-        rc.rings = t.rings;
-        rc.order = t.order;
-        rc.ticket = t.ticket;
-        rc.scr_stride = 2LL * zlen(t);
-        rc.bpad = (int)padded_len(t.bmax);
-        rc.logB = ilog2(t.bmax);
-        rc.zsmem = zsmem();
-        return rc;
+        RingArgs<T> a{};
+        a.lmax = p->lmax;
+        a.L = L;
+        a.rings = t.rings;
+        a.order = t.order;
+        a.roots = (const cx<T> *)t.roots;
+        a.V = (const cx<T> *)t.V;
+        a.chirp = (const cx<T> *)t.chirp;
+        a.tw = (const cx<T> *)t.tw;
+        a.zlen = (int)padded_len(t.nmax);
+        a.mode = mode;
+        return a;
+    }
+    static wf_status launch(wf_plan p, const RingArgs<T> &a)
+    {
+        const size_t sm = smem_bytes(p->tab);
+        auto kernel = k_ring<T, 2>;
+        if constexpr (sizeof(T) == 4)
+            if (p->tab.ring_ctas == 3) kernel = k_ring<T, 3>;
+        kernel<<<p->npairs, RING_CTA, sm, p->stream>>>(a);
+        WF_COUNT_LAUNCH(p);
+        WF_CUDA(cudaGetLastError());
+        return WF_OK;
     }
     static wf_status syn(wf_plan p, int L, RingSynMode mode, double lam, double tau, double *omap)
     {
@@ -739,23 +764,22 @@ template <typename T> struct RingLaunch {
                                  const float2 *glow, int lc, int glow_stride, void *tmap, double *omap,
                                  void *F = nullptr)
     {
-        const HpTables &t = p->tab;
-        RingCommon rc = common(p, L);
+        RingArgs<T> a = args(p, L, (int)mode);
         if (glow && lc > 0) {
-            rc.Glow = glow;
-            rc.lc = lc;
-            rc.glow_stride = glow_stride;
+            a.Glow = glow;
+            a.lc = lc;
+            a.glow_stride = glow_stride;
         }
-        const size_t sm = smem_bytes(t);
-        WF_CUDA(cudaMemsetAsync(t.ticket, 0, sizeof(int), p->stream));
-        k_ringsyn<T><<<t.ringGrid, ring_threads<T>(), sm, p->stream>>>(
-            rc, (const cx<T> *)t.roots, (const cx<T> *)t.V, (const cx<T> *)t.chirp, (const cx<T> *)t.tw,
-            (cx<T> *)p->ws.scr,
-            (const cx<T> *)G, (int)mode, (const T *)p->ws.r, (const T *)p->ws.nu, (T)lam, (T)tau,
-            (T *)tmap, omap, p->ws.part_pix, (cx<T> *)F);
-        WF_COUNT_LAUNCH(p);
-        WF_CUDA(cudaGetLastError());
-        return WF_OK;
+        a.G = (const cx<T> *)G;
+        a.r = (const T *)p->ws.r;
+        a.nu = (const T *)p->ws.nu;
+        a.lam = (T)lam;
+        a.tau = (T)tau;
+        a.tmap = (T *)tmap;
+        a.omap = omap;
+        a.part = p->ws.part_pix;
+        a.F = (cx<T> *)F;
+        return launch(p, a);
     }
     // messenger step on the rings: fold, inverse DFT, Eq. 3, forward DFT, unfold into F
     static wf_status syn_ana(wf_plan p, int L, double lam, double tau)
@@ -769,44 +793,31 @@ template <typename T> struct RingLaunch {
     static wf_status ana(wf_plan p, int L, const void *map) { return ana_buf(p, L, map, p->ws.F); }
     static wf_status ana_buf(wf_plan p, int L, const void *map, void *F)
     {
-        const HpTables &t = p->tab;
-        RingCommon rc = common(p, L);
-        const size_t sm = smem_bytes(t);
-        WF_CUDA(cudaMemsetAsync(t.ticket, 0, sizeof(int), p->stream));
-        k_ringana<T><<<t.ringGrid, ring_threads<T>(), sm, p->stream>>>(rc, (const cx<T> *)t.roots, (const cx<T> *)t.V,
-                                                                  (const cx<T> *)t.chirp, (const cx<T> *)t.tw,
-                                                                  (cx<T> *)p->ws.scr,
-                                                                  (const T *)map, (cx<T> *)F);
-        WF_COUNT_LAUNCH(p);
-        WF_CUDA(cudaGetLastError());
-        return WF_OK;
+        RingArgs<T> a = args(p, L, RS_ANA);
+        a.amap = (const T *)map;
+        a.F = (cx<T> *)F;
+        return launch(p, a);
     }
-    // FP32: the Bluestein / direct buffers fit next to the FFT buffer (the kernel
-    // runs one CTA per SM anyway, bounded by registers); FP64 keeps them in
-    // per-CTA global scratch
-    static int zsmem() { return sizeof(T) == 4 ? 1 : 0; }
-    static long long zlen(const HpTables &t) { return t.maxBlue > NAIVE_MAX ? t.maxBlue : NAIVE_MAX; }
-    static size_t smem_bytes(const HpTables &t)
-    {
-        return (padded_len(t.bmax) + (zsmem() ? 2 * (size_t)zlen(t) : 0) + (size_t)t.bmax / 4) * sizeof(cx<T>);
-    }
+    static size_t smem_bytes(const HpTables &t) { return (padded_len(t.nmax) + padded_len(t.exmax)) * sizeof(cx<T>); }
     // The dynamic shared-memory limit is raised once per kernel and size, before
     // any launch that needs it, and never lowered: plans of several sizes may
     // launch concurrently from different host threads.
-    static wf_status grid(wf_plan p, int *out)
+    static wf_status prepare(wf_plan p)
     {
         const size_t sm = smem_bytes(p->tab);
-        wf_status st;
-        if ((st = raise_smem_limit((const void *)k_ringsyn<T>, sm)) != WF_OK) return st;
-        if ((st = raise_smem_limit((const void *)k_ringana<T>, sm)) != WF_OK) return st;
-        int b1 = 0, b2 = 0;
-        WF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b1, k_ringsyn<T>, ring_threads<T>(), sm));
-        WF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b2, k_ringana<T>, ring_threads<T>(), sm));
-        int b = b1 < b2 ? b1 : b2;
+        if (wf_status st = raise_smem_limit((const void *)k_ring<T, 2>, sm)) return st;
+        int b = 0;
+        WF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_ring<T, 2>, RING_CTA, sm));
         if (b < 1) return set_error(WF_EUNSUPPORTED, "ring kernel does not fit on an SM (smem %zu bytes)", sm);
-        long long g = (long long)b * p->nsm;
-        if (g > p->npairs) g = p->npairs;
-        *out = (int)g;
+        p->tab.ring_ctas = 2;
+        if constexpr (sizeof(T) == 4) {
+            if (p->npairs > 2 * p->nsm) {
+                int b3 = 0;
+                if (wf_status st = raise_smem_limit((const void *)k_ring<T, 3>, sm)) return st;
+                WF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b3, k_ring<T, 3>, RING_CTA, sm));
+                if (b3 >= 3) p->tab.ring_ctas = 3;
+            }
+        }
         return WF_OK;
     }
 };
@@ -824,10 +835,19 @@ wf_status upload_cx(wf_plan p, void **dst, const std::vector<double2> &src)
 
 }  // namespace
 
+// log2 of the FFT length that serves a ring of n = 4k pixels, and whether k itself is that length
+int ring_fft_log(int n, bool *direct)
+{
+    const int k = n / 4;
+    *direct = k >= 16 && is_pow2(k);
+    return *direct ? ilog2(k) : std::max(4, ilog2(2LL * k - 1));
+}
+
 wf_status hp_build_ring_tables(wf_plan p)
 {
     const int nside = p->nside, np = p->npairs;
     const int R = 4 * nside - 1;
+    if (nside > RING_MAX_K) return set_error(WF_EUNSUPPORTED, "rings longer than %d pixels (nside > %d)", 4 * RING_MAX_K, RING_MAX_K);
     // ring offsets (RING order)
     std::vector<long long> off(R + 1, 0);
     std::vector<int> nr(R), qr(R);
@@ -845,8 +865,7 @@ wf_status hp_build_ring_tables(wf_plan p)
     std::vector<RingTab> rt(np);
     std::map<int, long long> rootOff, vOff, cOff;
     std::vector<double2> roots, Vtab, chirp;
-    long long nmaxF = 2;  // largest full FFT length (pow2 n or Bluestein M)
-    int bmax = 2 * NAIVE_MAX, maxBlue = 1;
+    int exmax = 0;
     for (int pr = 0; pr < np; ++pr) {
         RingTab &t = rt[pr];
         const int i0 = pr;  // north ring, 0-based
@@ -854,7 +873,8 @@ wf_status hp_build_ring_tables(wf_plan p)
         t.q = qr[i0];
         t.offN = off[i0];
         t.offS = (pr < np - 1) ? off[R - 1 - pr] : -1;
-        const int n = t.n;
+        const int n = t.n, k = n / 4;
+        t.inv = (unsigned)((0x100000000ull + n - 1) / n);
         if (!rootOff.count(n)) {
             rootOff[n] = (long long)roots.size();
             for (int q = 0; q < 2 * n; ++q) {
@@ -865,58 +885,47 @@ wf_status hp_build_ring_tables(wf_plan p)
         t.rootOff = rootOff[n];
         t.vOff = 0;
         t.cOff = 0;
-        if (n <= NAIVE_MAX) {
-            t.kind = RING_NAIVE;
-            t.logF = 0;
-        } else if (is_pow2(n)) {
-            t.kind = RING_POW2;
-            t.logF = ilog2(n);
-            if (n > nmaxF) nmaxF = n;
-            if (n > bmax) bmax = n;
-        } else {
-            t.kind = RING_BLUESTEIN;
-            const int lgM = ilog2(2LL * n - 1);
-            const long long M = 1LL << lgM;
-            t.logF = lgM - 1;
-            if (M > nmaxF) nmaxF = M;
-            if (M / 2 > bmax) bmax = (int)(M / 2);
-            if (n > maxBlue) maxBlue = n;
-            if (!vOff.count(n)) {
-                vOff[n] = (long long)Vtab.size();
-                std::vector<double2> v(M, make_double2(0.0, 0.0));
-                for (long long j = 0; j < n; ++j) {
-                    const long long e = (j * j) % (2LL * n);
-                    const double a = M_PI * (double)e / (double)n;  // conj(c_j) = e^{+i pi j^2 / n}
+        bool direct = false;
+        t.logF = ring_fft_log(n, &direct);
+        t.kind = direct ? RING_POW2 : RING_BLUESTEIN;
+        const int N = 1 << t.logF, nt = N / 16;
+        exmax = std::max(exmax, N * std::min(4, RING_CTA / nt));
+        if (!direct) {
+            if (!vOff.count(k)) {
+                vOff[k] = (long long)Vtab.size();
+                std::vector<double2> v(N, make_double2(0.0, 0.0));
+                for (long long j = 0; j < k; ++j) {
+                    const long long e = (j * j) % (2LL * k);
+                    const double a = M_PI * (double)e / (double)k;  // conj(c_j) = e^{+i pi j^2 / k}
                     v[j] = make_double2(std::cos(a), std::sin(a));
-                    if (j > 0) v[M - j] = v[j];
+                    if (j > 0) v[N - j] = v[j];
                 }
                 host_fft(v);
-                for (long long k = 0; k < M / 2; ++k) Vtab.push_back(cscale(v[2 * k], 1.0 / (double)M));
-                for (long long k = 0; k < M / 2; ++k) Vtab.push_back(cscale(v[2 * k + 1], 1.0 / (double)M));
-            }
-            t.vOff = vOff[n];
-            if (!cOff.count(n)) {  // c_j = e^{-i pi j^2 / n}, j^2 reduced mod 2n exactly
-                cOff[n] = (long long)chirp.size();
-                for (long long j = 0; j < n; ++j) {
-                    const double a = -M_PI * (double)((j * j) % (2LL * n)) / (double)n;
+                // in the order the forward transform leaves the frequencies in, 1/N folded in
+                for (int e = 0; e < 16; ++e)
+                    for (int th = 0; th < nt; ++th) Vtab.push_back(cscale(v[fft_index(t.logF, th, e)], 1.0 / (double)N));
+                cOff[k] = (long long)chirp.size();
+                for (long long j = 0; j < k; ++j) {  // c_j = e^{-i pi j^2 / k}, j^2 reduced mod 2k exactly
+                    const double a = -M_PI * (double)((j * j) % (2LL * k)) / (double)k;
                     chirp.push_back(make_double2(std::cos(a), std::sin(a)));
                 }
             }
-            t.cOff = cOff[n];
+            t.vOff = vOff[k];
+            t.cOff = cOff[k];
         }
     }
-    const int logNmax = ilog2(nmaxF);
-    if (bmax > 8192) return set_error(WF_EUNSUPPORTED, "ring FFT longer than 8192 (nside > 2048)");
-    std::vector<double2> tw((size_t)1 << logNmax);
-    for (size_t t = 0; t < tw.size(); ++t) {
-        const double a = -2.0 * M_PI * (double)t / (double)(1LL << logNmax);
-        tw[t] = make_double2(std::cos(a), std::sin(a));
-    }
+    // twiddles of every FFT length N = 32 .. 4096: tw[N - 32 + k N/16 + t] = e^{-2 pi i t k / N}
+    std::vector<double2> tw(RING_TW);
+    for (int N = 32; N <= 4096; N *= 2)
+        for (int kk = 0; kk < 16; ++kk)
+            for (int t = 0; t < N / 16; ++t) {
+                const double a = -2.0 * M_PI * (double)(t * kk) / (double)N;
+                tw[N - 32 + kk * (N / 16) + t] = make_double2(std::cos(a), std::sin(a));
+            }
     if (Vtab.empty()) Vtab.push_back(make_double2(0, 0));
     if (chirp.empty()) chirp.push_back(make_double2(0, 0));
-    p->tab.logNmax = logNmax;
-    p->tab.bmax = bmax;
-    p->tab.maxBlue = maxBlue;
+    p->tab.nmax = 4 * nside;
+    p->tab.exmax = exmax;
     wf_status st;
     if ((st = plan_alloc(p, (void **)&p->tab.rings, rt.size() * sizeof(RingTab))) != WF_OK) return st;
     if ((st = to_device(p, p->tab.rings, rt.data(), rt.size() * sizeof(RingTab))) != WF_OK) return st;
@@ -926,31 +935,27 @@ wf_status hp_build_ring_tables(wf_plan p)
         if ((st = upload_cx<float>(p, &p->tab.V, Vtab)) != WF_OK) return st;
         if ((st = upload_cx<float>(p, &p->tab.chirp, chirp)) != WF_OK) return st;
         if ((st = upload_cx<float>(p, &p->tab.tw, tw)) != WF_OK) return st;
-        if ((st = RingLaunch<float>::grid(p, &p->tab.ringGrid)) != WF_OK) return st;
+        if ((st = RingLaunch<float>::prepare(p)) != WF_OK) return st;
     } else {
         if ((st = upload_cx<double>(p, &p->tab.roots, roots)) != WF_OK) return st;
         if ((st = upload_cx<double>(p, &p->tab.V, Vtab)) != WF_OK) return st;
         if ((st = upload_cx<double>(p, &p->tab.chirp, chirp)) != WF_OK) return st;
         if ((st = upload_cx<double>(p, &p->tab.tw, tw)) != WF_OK) return st;
-        if ((st = RingLaunch<double>::grid(p, &p->tab.ringGrid)) != WF_OK) return st;
+        if ((st = RingLaunch<double>::prepare(p)) != WF_OK) return st;
     }
-    // pairs by decreasing cost: Bluestein (four half-length FFTs), then the rest by length
+    // pairs by decreasing cost (two FFTs of N per Bluestein sub-DFT): the grid hands them out in
+    // this order, so the launch ends on its cheapest pairs
     std::vector<int> order(np);
     std::vector<double> cost(np);
     for (int i = 0; i < np; ++i) {
         order[i] = i;
         const RingTab &t = rt[i];
-        const double F = (double)(1LL << t.logF);
-        cost[i] = t.kind == RING_BLUESTEIN ? 4.0 * F * (t.logF + 2) : t.kind == RING_POW2 ? F * t.logF : (double)t.n * t.n / 8;
-        cost[i] += 2.0 * p->lmax / 64.0;
+        const double F = 4.0 * (double)(1LL << t.logF) * (t.logF + 2);
+        cost[i] = (t.kind == RING_BLUESTEIN ? 2.0 : 1.0) * F + 8.0 * t.n + 4.0 * p->lmax;
     }
     std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return cost[x] > cost[y]; });
     if ((st = plan_alloc(p, (void **)&p->tab.order, np * sizeof(int))) != WF_OK) return st;
-    if ((st = to_device(p, p->tab.order, order.data(), np * sizeof(int))) != WF_OK) return st;
-    if ((st = plan_alloc(p, (void **)&p->tab.ticket, 16)) != WF_OK) return st;
-    const size_t es = f32 ? sizeof(float2) : sizeof(double2);
-    const long long zl = maxBlue > NAIVE_MAX ? maxBlue : NAIVE_MAX;
-    return plan_alloc(p, &p->ws.scr, (size_t)p->tab.ringGrid * 2 * zl * es + 16);
+    return to_device(p, p->tab.order, order.data(), np * sizeof(int));
 }
 
 wf_status hp_ring_synthesis(wf_plan p, int L, RingSynMode mode, double lam, double tau, double *out_map)
