@@ -276,21 +276,22 @@ struct SumSpec {
     int n[5];
     int stride[5];
 };
-__global__ void k_sums(SumSpec sp, int nsum, double *__restrict__ out)
+__global__ void __launch_bounds__(512) k_sums(SumSpec sp, double *__restrict__ out)
 {
-    __shared__ double red[32];
-    for (int k = 0; k < nsum; ++k) {
-        double s = 0.0;
-        for (int i = threadIdx.x; i < sp.n[k]; i += blockDim.x) s += sp.in[k][(long long)i * sp.stride[k]];
-        for (int o = 16; o >= 1; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            double t = 0.0;
-            for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
-            out[k] = t;
-        }
-        __syncthreads();
+    __shared__ double red[16];
+    const int k = blockIdx.x;
+    const double *in = sp.in[k];
+    const int n = sp.n[k], stride = sp.stride[k];
+    double s = 0.0;
+#pragma unroll 4
+    for (int i = threadIdx.x; i < n; i += 512) s += in[(long long)i * stride];
+    for (int o = 16; o >= 1; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double t = 0.0;
+        for (int w = 0; w < 16; ++w) t += red[w];
+        out[k] = t;
     }
 }
 
@@ -474,14 +475,15 @@ __global__ void k_blend(long long npix, const T *__restrict__ r, const T *__rest
 
 int grid_for(long long n, int nsm) { return (int)std::min<long long>((n + 255) / 256, (long long)nsm * 8); }
 
-// reduce the partial sums in a fixed order into ws.scal and copy them to the
-// pinned host mirror ws.h_scal (enqueued only: valid after the stream syncs)
+// reduce the partial sums in a fixed order, a CTA each, into the pinned host
+// mirror ws.h_scal (enqueued only: valid after the stream syncs; the kernel
+// writes the host memory itself, a copy after it is one more operation on the
+// stream's critical path)
 wf_status sums_enqueue(wf_plan p, SumSpec sp, int nsum)
 {
-    k_sums<<<1, 256, 0, p->stream>>>(sp, nsum, p->ws.scal);
+    k_sums<<<nsum, 512, 0, p->stream>>>(sp, p->ws.h_scal);
     WF_COUNT_LAUNCH(p);
     WF_CUDA(cudaGetLastError());
-    WF_CUDA(cudaMemcpyAsync(p->ws.h_scal, p->ws.scal, nsum * sizeof(double), cudaMemcpyDeviceToHost, p->stream));
     return WF_OK;
 }
 
@@ -1008,7 +1010,8 @@ wf_status hp_launch(HpRun &R)
         pr.begin(WF_K_RING_SYN);
         void *r_src = p->ws.r;
         if (R.corr) p->ws.r = p->ws.r0;  // correction form: B delta, the iteration without its source
-        st = hp_ring_synthesis_analysis(p, R.L, R.lam, tau);
+        st = hp_ring_synthesis_analysis(p, R.L, R.lam, tau,
+                                        EpiArgs{p->lmax, R.C_ell, p->omega, R.lam * R.tau_h, R.tau_h, p->ws.epi});
         p->ws.r = r_src;
         if (st != WF_OK) return st;
         pr.end();
@@ -1025,6 +1028,8 @@ wf_status hp_launch(HpRun &R)
     ba.tauh = R.tau_h;
     ba.S = R.C_ell;
     ba.want_resid = full ? 1 : 0;
+    ba.want_norms = R.rigorous ? 1 : 0;
+    ba.epi_ready = R.rigorous ? 0 : 1;
     const double2 *a_old = p->ws.a;
     if (R.corr) {
         // the epilogue's residual compares its output B delta_k with delta_k - d0, i.e.
@@ -1891,7 +1896,9 @@ long long hp_estimate_bytes(int nside, int lmax, wf_precision prec, bool staging
     const long long es = f32 ? 4 : 8, ec = 2 * es;
     long long b = 0;
     b += nalm * 16 + np * 16 + (lmax + 1) * 8 + ns * (4 + 16);  // A64, c64, x, st, log2 c, seeds
-    if (f32) b += nalm * 8 + np * 8 + ns * 12;                   // A32, B32, x32, w32, FP32 seeds
+    // x32, w32, xw, FP32 seeds; two-step tables, partial sums of the analysis (per (m, k))
+    if (f32) b += np * 24 + ns * 12 + (nalm / 2 + 2 * lmax + 8) * (8 + 8 + 32 + 32) + (lmax + 1) * 8;
+    if (tc_prec(prec)) b += nalm * 8 + ns * 12;                  // A32, B32 and one-step seeds
     // ring tables: roots per distinct length, Bluestein filters and chirps, twiddles
     long long roots = 0, V = 0;
     for (int k = 1; k <= nside; ++k) {
@@ -2056,8 +2063,14 @@ wf_status wf_set_options(wf_plan p, const wf_options *opt)
         return set_error(WF_EINVAL, "tile_syn and tile_ana must be 2, 4 or 8 (0: keep)");
     const long long old_cap = p->opt.mixed_table_bytes;
     p->opt = opt ? *opt : wf_options{};
-    if (p->opt.tile_syn > 0) p->tile_syn = p->opt.tile_syn;
-    if (p->opt.tile_ana > 0) p->tile_ana = p->opt.tile_ana;
+    if (p->opt.tile_syn > 0) {
+        p->tile_syn = p->opt.tile_syn;
+        p->tile_syn_set = true;
+    }
+    if (p->opt.tile_ana > 0) {
+        p->tile_ana = p->opt.tile_ana;
+        p->tile_ana_set = true;
+    }
     if (p->g.kind == WF_GEOM_HEALPIX && p->prec == WF_PREC_FP64 && p->g.ncomp == 1)
         p->df_legendre = p->opt.fp64_emulation != 0;
     // mixed temperature tables: a forced block (or a changed table cap) takes effect now

@@ -131,9 +131,20 @@ struct HpTables {
     double *s0_64 = nullptr, *s1_64 = nullptr;
     double *x64 = nullptr;
     double *st64 = nullptr;  // sin(theta) per pair
-    // mixed precision: FP32 A and B = A - 2 per alm, x and w = 1 - x per pair,
-    // and the FP32 seeds that start the recurrence at max(l_s, l_c) (m < l_c)
-    float *A32 = nullptr, *B32 = nullptr, *x32 = nullptr, *w32 = nullptr;
+    // mixed precision: x and w = 1 - x per pair (FP32); ring variables and 1/x per pair and the
+    // two-step tables of the belt and cap forms per (m, k) (wf_legendre.cu); first k and starting
+    // state per (m, pair); the analysis' sums per part (zero between launches)
+    float *x32 = nullptr, *w32 = nullptr;
+    float4 *xw = nullptr;
+    float2 *tb = nullptr, *tp = nullptr;
+    double4 *kd = nullptr;
+    double *Atop = nullptr;       // per m: A at lmax + 1
+    int *k0_mx = nullptr;
+    float2 *seed_mx = nullptr;
+    float4 *psum = nullptr;
+    // tensor-core plans: FP32 A and B = A - 2 per alm, and the one-step forms' seeds (mu_l, mu_{l+1})
+    // at l = ls_mx = max(l_s, l_c)
+    float *A32 = nullptr, *B32 = nullptr;
     int *ls_mx = nullptr;
     float *s0_mx = nullptr, *s1_mx = nullptr;
     int lc_mx = 0;         // FP64 block l < lc_mx of the mixed path
@@ -178,6 +189,7 @@ struct wf_plan_s {
     double bnorm_given = 0;   // > 0: the next solve's residual norm |Y^T r| (the sweeps take their parent's)
     bool events_ready = false;
     int tile_syn = 4, tile_ana = 8;  // mixed Legendre tiles: ring pairs per thread / per lane
+    bool tile_syn_set = false, tile_ana_set = false;  // chosen by the user or the autotuner; else by size per launch
     bool tc_deferred = false;        // tensor-core plan in a batch step: its synthesis ran in the group launch
     cudaStream_t aux = nullptr;      // mixed precision: stream of the FP64 low-l block
     cudaEvent_t fork_ev = nullptr, join_ev = nullptr;
@@ -243,7 +255,31 @@ struct BlendArgs {
     const double *S = nullptr;  // C_ell (device)
     const double4 *epi = nullptr;  // per l: (Omega S/(S + lambda tau_h), 1/S, 1/S + 1/tau_h, S > 0); filled per launch
     int want_resid = 0;
+    int want_norms = 0;  // x^T S^-1 x and x^T S^-2 x of the result (the chi^2-bound schedule's; else 0)
+    int epi_ready = 0;   // the ring pass of this iteration has filled ws.epi (EpiArgs)
 };
+// per-l factors of the harmonic blend (Eq. 4) and of the chi^2 / residual sums, l <= lmax
+struct EpiArgs {
+    int lmax;
+    const double *S;
+    double omega, lam_tauh, tauh;
+    double4 *epi;
+};
+#ifdef __CUDACC__
+__device__ __forceinline__ void epi_entry(const EpiArgs &a, int l)
+{
+    if (l > a.lmax) return;
+    const double s = a.S[l];
+    double4 e = make_double4(0.0, 0.0, 0.0, 0.0);
+    if (s > 0.0) {
+        e.x = a.omega * s / (s + a.lam_tauh);
+        e.y = 1.0 / s;
+        e.z = 1.0 / s + 1.0 / a.tauh;
+        e.w = 1.0;
+    }
+    a.epi[l] = e;
+}
+#endif
 wf_status hp_set_low_block(wf_plan p, int lc);
 long long hp_low_table_bytes(int lmax, int npairs, int lc);
 wf_status hp_autotune(wf_plan p, int reps);
@@ -276,7 +312,8 @@ wf_status hp_ring_synthesis_buf(wf_plan p, int L, RingSynMode mode, double lam, 
                                 void *tmap, double *out_map);
 wf_status hp_ring_analysis_buf(wf_plan p, int L, const void *map_T, void *F);
 // mixed plans: the FP32 synthesis pass with an explicit FP64-block buffer (m < lc)
-wf_status hp_ring_synthesis_analysis(wf_plan p, int L, double lam, double tau);
+// (the messenger step's ring pass; it also fills the blend table of the analysis that follows)
+wf_status hp_ring_synthesis_analysis(wf_plan p, int L, double lam, double tau, const EpiArgs &epi);
 wf_status hp_ring_synthesis_buf_low(wf_plan p, int L, RingSynMode mode, double lam, double tau, const void *G,
                                     const float2 *glow, int lc, int glow_stride, void *tmap, double *out_map);
 // FP64 temperature Legendre transforms on explicit buffers (FP64 plans)

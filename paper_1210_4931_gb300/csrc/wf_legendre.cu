@@ -16,16 +16,10 @@
 //
 // Two precisions:
 //   FP64     k_legsyn<double>, k_legana<double,...>: one ring pair per thread.
-//   mixed    k_legsyn_mx<NP>, k_legana_mx<NP, CH>: FP32 recurrence and
+//   mixed    k_legsyn_mx<NP>, k_legana_mx<NP>: FP32 recurrence and
 //            contraction, NP ring pairs per thread (synthesis) or per lane
-//            (analysis) in packed f32x2 lanes (__ffma2_rn); NP is the plan's
-//            tile choice (4 and 8 by default, or what wf_plan_autotune timed).
-//            Near the poles the plain recurrence mu_l = A x mu_{l-1} - mu_{l-2}
-//            loses ~1/sin(theta) digits (its two characteristic roots merge
-//            at x = 1), so rings with x > 0.4 run the same recurrence in
-//            difference form (Reinsch's modification):
-//                D_l = D_{l-1} + (B_l - A_l w) mu_{l-1},  mu_l = mu_{l-1} + D_l,
-//            w = 1 - x exact from the grid, B_l = A_l - 2 tabulated in FP64.
+//            (analysis) in packed f32x2 lanes (__ffma2_rn), in the two-step
+//            forms of the belt and the polar cap described at MxPart below.
 //            The block l < l_c, where the messenger iteration's contraction
 //            margin tau_h / S_l is below the FP32 error, runs through the FP64
 //            kernels instead (the FP32 recurrence restarts at l_c from FP64
@@ -34,6 +28,7 @@
 #include <climits>
 #include <cmath>
 #include <cstdio>
+#include <type_traits>
 
 #include "wf_internal.cuh"
 
@@ -42,9 +37,6 @@ namespace wf {
 namespace {
 
 constexpr double SEED_LOG2_THRESHOLD = -80.0;
-// ring pairs per thread (mixed synthesis) and per lane (mixed analysis): the
-// plan's tile choice, 4 and 8 unless wf_plan_autotune measured better
-constexpr float X_DIFFERENCE_FORM = 0.4f;
 constexpr int BIG = INT_MAX / 2;
 
 __host__ __device__ inline long long mbase(int lmax, int m) { return (long long)m * (2 * lmax + 3 - m) / 2; }
@@ -105,49 +97,74 @@ __global__ void k_seeds(int lmax, int npairs, const double *__restrict__ xp, con
     s1_out[idx] = s1;
 }
 
-// FP32 seeds of the mixed kernels for a given FP64 block l < lc: for m < lc
-// the FP32 recurrence starts at max(l_s, lcm) from FP64-accurate values
-__global__ void k_restart_seeds(int lmax, int npairs, int lc, const double *__restrict__ xp,
-                                const double *__restrict__ A, const int *__restrict__ ls_in,
+// first entry of m in the tables per (m, k), k = (l - m) / 2: at least (lmax - m + 1)/2 + 1
+// entries before the next m's
+__host__ __device__ inline long long kbase(int lmax, int m) { return (mbase(lmax, m) + 4 * (long long)m) >> 1; }
+
+// Starting states of the mixed kernels for a given FP64 block l < lc.
+//
+// Two-step kernels: k0 (k = (l - m) / 2) is the first kept k rounded up to a multiple of four,
+// so that a pair starts between two blocks of four steps (the terms between, at most
+// three k after |lambda| first exceeds 2^-80, stay below 2^-50); k0 = lmax where nothing is
+// kept.  For m < lc the FP64-accurate values of l_c's multiple of four below start a ring
+// that has begun by then; the kernels leave out what lies below l_c.
+// seed, belt (p >= ncap): (mu_l, x mu_{l+1}); cap: (E, D) = (mu_l / e_k, mu_{l+2} / e_{k+1} - mu_l / e_k).
+//
+// Tensor-core synthesis (ls_out not null): the recurrence starts at l = max(l_s, lcm) from
+// s0, s1 = (mu_l, mu_{l+1}).
+__global__ void k_restart_seeds(int lmax, int npairs, int lc, int ncap, const double *__restrict__ xp,
+                                const double *__restrict__ A, const double *__restrict__ Atop,
+                                const double4 *__restrict__ kd, const int *__restrict__ ls_in,
                                 const double *__restrict__ s0_in, const double *__restrict__ s1_in,
-                                int *__restrict__ ls_out, float *__restrict__ s0_out, float *__restrict__ s1_out)
+                                int *__restrict__ k0_out, float2 *__restrict__ seed, int *__restrict__ ls_out,
+                                float *__restrict__ s0_out, float *__restrict__ s1_out)
 {
     const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= (long long)(lmax + 1) * npairs) return;
     const int m = (int)(idx / npairs);
     const int p = (int)(idx % npairs);
-    int ls = ls_in[idx];
-    double s0 = s0_in[idx], s1 = s1_in[idx];
-    if (m < lc && ls <= lmax) {
-        const int l1 = lcm_of(lc, m);
-        if (ls < l1) {
-            if (l1 > lmax) {
-                ls = lmax + 1;
-                s0 = s1 = 0.0;
-            } else {
-                const long long base = mbase(lmax, m);
-                const double x = xp[p];
-                double a = s0, b = s1;  // mu_l, mu_{l+1} at l = ls
-                for (int l = ls + 2; l <= l1 + 1 && l <= lmax; ++l) {
-                    const double c2 = A[base + (l - m)] * x * b - a;
-                    a = b;
-                    b = c2;
-                }
-                // now (a, b) = (mu_{l1}, mu_{l1+1}), or (mu_{lmax-1}, mu_{lmax}) if l1 = lmax
-                if (l1 == lmax && ls + 1 < lmax) {
-                    s0 = b;
-                    s1 = 0.0;
-                } else {
-                    s0 = a;
-                    s1 = b;
-                }
-                ls = l1;
+    const double *Am = A + mbase(lmax, m) - m;  // A_l = Am[l]
+    const double x = xp[p];
+    const int ls = ls_in[idx];
+    const int l1 = m < lc ? lcm_of(lc, m) : m;  // the FP64 block's end
+    // (mu_l, mu_{l+1}) from the seeds at ls up to l = la <= lmax (mu_{lmax+1} = 0 where la = lmax)
+    auto at = [&](int la, double &a, double &b) {
+        a = s0_in[idx];
+        b = s1_in[idx];
+        for (int l = ls; l < la; ++l) {
+            const double c = l + 2 <= lmax ? Am[l + 2] * x * b - a : 0.0;
+            a = b;
+            b = c;
+        }
+    };
+    double a = 0.0, b = 0.0;
+    if (ls_out) {
+        const int l = ls > lmax ? ls : l1 > ls ? (l1 > lmax ? lmax + 1 : l1) : ls;
+        if (l <= lmax) at(l, a, b);
+        ls_out[idx] = l;
+        s0_out[idx] = (float)a;
+        s1_out[idx] = (float)b;
+    }
+    int k0 = lmax;
+    float2 sd = make_float2(0.f, 0.f);
+    if (ls <= lmax) {
+        const int kn = (ls - m) >> 1, k1 = ((l1 - m) >> 1) & ~3;
+        const int k = kn <= k1 ? k1 : (kn + 3) & ~3, l = m + 2 * k;
+        if (l <= lmax && l1 <= lmax) {
+            k0 = k;
+            at(l, a, b);
+            sd = make_float2((float)a, (float)(x * b));
+            if (p < ncap) {
+                const long long kk = kbase(lmax, m) + k;
+                const double e0 = a * kd[kk].w;
+                double e1 = 0.0;
+                if (l + 2 <= lmax + 1) e1 = ((l + 2 <= lmax ? Am[l + 2] : Atop[m]) * x * b - a) * kd[kk + 1].w;
+                sd = make_float2((float)e0, (float)(e1 - e0));
             }
         }
     }
-    ls_out[idx] = ls;
-    s0_out[idx] = (float)s0;
-    s1_out[idx] = (float)s1;
+    k0_out[idx] = k0;
+    seed[idx] = sd;
 }
 
 template <typename T>
@@ -279,76 +296,69 @@ __device__ __forceinline__ void block_reduce4(double (&v)[4], double (*red)[LEG_
 
 // Eq. (4) epilogue shared by both precisions: t_hat = Omega (c acc + low),
 // a_new = S/(S + lam tau_h) t_hat, chi^2 of a_old, lambda = 1 residual.
-// per-l factors of the harmonic blend (Eq. 4) and of the chi^2 / residual sums
-__global__ void k_epi_table(int lmax, const double *__restrict__ S, double omega, double lam_tauh, double tauh,
-                            double4 *__restrict__ epi)
+__global__ void k_epi_table(EpiArgs a)
 {
-    const int l = blockIdx.x * blockDim.x + threadIdx.x;
-    if (l > lmax) return;
-    const double s = S[l];
-    double4 e = make_double4(0.0, 0.0, 0.0, 0.0);
-    if (s > 0.0) {
-        e.x = omega * s / (s + lam_tauh);
-        e.y = 1.0 / s;
-        e.z = 1.0 / s + 1.0 / tauh;
-        e.w = 1.0;
-    }
-    epi[l] = e;
+    epi_entry(a, blockIdx.x * blockDim.x + threadIdx.x);
 }
 
-template <typename ACC>
-__device__ __forceinline__ void blend_epilogue(int lmax, int L, int m, long long base, int mode, double omega,
-                                               const BlendArgs &ba, const double *__restrict__ c64,
-                                               const ACC *acc, const double2 *__restrict__ low, int low_lim,
-                                               const double2 *__restrict__ a_old, double2 *__restrict__ out,
+// sums of one thread over its a_lm: chi^2 of a_old, residual^2, x^T S^-1 x and x^T S^-2 x of a_new
+struct BlendSums {
+    double chi2 = 0.0, res2 = 0.0, hnew = 0.0, qnew = 0.0;
+};
+
+// one a_lm: b = c_lm times its ring sum, or 0 (l > L); the sums leave out the weight 2 of m > 0.
+// (Every FP64 operation counts here: at 1/64 of the FP32 rate the epilogue of the mixed analysis
+// is bound by the FP64 pipe.)
+__device__ __forceinline__ void blend_one(int l, int L, long long idx, int mode, const BlendArgs &ba, double2 b,
+                                          const double2 *__restrict__ a_old, double2 *__restrict__ out, BlendSums &v)
+{
+    if (mode == LEG_ADJOINT) {
+        out[idx] = b;
+        return;
+    }
+    // per-l factors tabulated once per launch (no FP64 division per a_lm)
+    const double4 e = ba.epi[l];
+    const double2 ao = a_old[idx];
+    double2 an = make_double2(0.0, 0.0);
+    if (l <= L && e.w > 0.0) {
+        an.x = e.x * b.x;
+        an.y = e.x * b.y;
+    }
+    if (e.w > 0.0) {
+        v.chi2 += (ao.x * ao.x + ao.y * ao.y) * e.y;
+        if (ba.want_norms) {
+            const double an2 = (an.x * an.x + an.y * an.y) * e.y;
+            v.hnew += an2;
+            v.qnew += an2 * e.y;
+        }
+        if (ba.want_resid) {
+            const double dx = e.z * (ao.x - an.x), dy = e.z * (ao.y - an.y);
+            v.res2 += dx * dx + dy * dy;
+        }
+    }
+    out[idx] = an;
+}
+
+__device__ __forceinline__ void blend_sums(const BlendSums &s, int m, double *__restrict__ part,
+                                           double (*red)[LEG_THREADS / 32])
+{
+    double v[4] = {s.chi2, s.res2, s.hnew, s.qnew};
+    block_reduce4(v, red);
+    if (threadIdx.x == 0)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) part[4 * m + k] = m ? 2.0 * v[k] : v[k];
+}
+
+// val(j): c_lm times the ring sum at l = m + j
+template <typename VAL>
+__device__ __forceinline__ void blend_epilogue(int lmax, int L, int m, long long base, int mode, const BlendArgs &ba,
+                                               VAL val, const double2 *__restrict__ a_old, double2 *__restrict__ out,
                                                double *__restrict__ part, double (*red)[LEG_THREADS / 32])
 {
-    double chi2 = 0.0, res2 = 0.0, hnew = 0.0, qnew = 0.0;
-    const double wm = (m == 0) ? 1.0 : 2.0;
-    for (int j = threadIdx.x; j <= lmax - m; j += blockDim.x) {
-        const int l = m + j;
-        const long long idx = base + j;
-        double2 b = make_double2(0.0, 0.0);
-        if (l <= L) {
-            b.x = c64[idx] * (double)acc[j].x;
-            b.y = c64[idx] * (double)acc[j].y;
-            if (low && l < low_lim) {
-                const double2 q = low[idx];
-                b.x += q.x;
-                b.y += q.y;
-            }
-        }
-        if (mode == LEG_ADJOINT) {
-            out[idx] = b;
-        } else {
-            // per-l factors tabulated once per launch (no FP64 division per a_lm)
-            const double4 e = ba.epi[l];
-            const double2 ao = a_old[idx];
-            double2 an = make_double2(0.0, 0.0);
-            if (l <= L && e.w > 0.0) {
-                an.x = e.x * b.x;
-                an.y = e.x * b.y;
-            }
-            if (e.w > 0.0) {
-                chi2 += wm * (ao.x * ao.x + ao.y * ao.y) * e.y;
-                const double an2 = wm * (an.x * an.x + an.y * an.y) * e.y;
-                hnew += an2;
-                qnew += an2 * e.y;
-                if (ba.want_resid) {
-                    const double dx = e.z * (ao.x - an.x), dy = e.z * (ao.y - an.y);
-                    res2 += wm * (dx * dx + dy * dy);
-                }
-            }
-            out[idx] = an;
-        }
-    }
-    if (mode == LEG_BLEND) {
-        double v[4] = {chi2, res2, hnew, qnew};
-        block_reduce4(v, red);
-        if (threadIdx.x == 0)
-#pragma unroll
-            for (int k = 0; k < 4; ++k) part[4 * m + k] = v[k];
-    }
+    BlendSums v;
+    for (int j = threadIdx.x; j <= lmax - m; j += blockDim.x)
+        blend_one(m + j, L, base + j, mode, ba, m + j <= L ? val(j) : make_double2(0.0, 0.0), a_old, out, v);
+    if (mode == LEG_BLEND) blend_sums(v, m, part, red);
 }
 
 // ---------------------------------------------------------------------------
@@ -441,7 +451,8 @@ __global__ void __launch_bounds__(LEG_THREADS) k_legana(int lmax, int L, int npa
         }
         return;
     }
-    blend_epilogue(lmax, Lm, m, base, mode, omega, ba, c64, acc, nullptr, 0, a_old, out, part, red);
+    auto val = [&](int j) { return cscale(acc[j], c64[base + j]); };
+    blend_epilogue(lmax, Lm, m, base, mode, ba, val, a_old, out, part, red);
 }
 
 // ---------------------------------------------------------------------------
@@ -910,12 +921,52 @@ __global__ void __launch_bounds__(LEG_THREADS, 2) k_legana_df(int lmax, int L, i
         }
     }
     __syncthreads();
-    blend_epilogue(lmax, L, m, base, mode, omega, ba, c64, acc, nullptr, 0, a_old, out, part, red);
+    auto val = [&](int j) { return cscale(acc[j], c64[base + j]); };
+    blend_epilogue(lmax, L, m, base, mode, ba, val, a_old, out, part, red);
 }
 
 // ---------------------------------------------------------------------------
-// mixed precision: FP32 kernels, four ring pairs per thread in two f32x2
-// packs, plain or difference-form recurrence by ring
+// Mixed precision: FP32 kernels, NP ring pairs per thread (synthesis) or lane
+// (analysis) in NP/2 f32x2 packs.
+//
+// Both kernels are bound by the FP32 FMA pipe, so what counts is the operations
+// per (l, m, ring pair): two for the complex contraction with lambda_lm and as
+// few as possible for the recurrence.  The ring pairs fall into two parts with
+// a form each, both of which advance two l at once (k = (l - m)/2) with three
+// operations:
+//
+//  belt (rings of 4 nside pixels below x = 2/3): the one-step recurrence
+//  mu_l = A_l x mu_{l-1} - mu_{l-2} with the odd values carried as x mu, so that
+//  the step from odd to even needs no product A_l x:
+//      E_k = mu_{m+2k},  O_k = x mu_{m+2k+1}
+//      E_{k+1} = A_{2k+2} O_k - E_k,  O_{k+1} = (A_{2k+3} x^2) E_{k+1} - O_k.
+//  The odd sum is divided by x at the end (analysis: its input is).  On the
+//  belt x = 2j / (3 nside), so x^2 enters as the integer j^2 (exact in FP32)
+//  with 4 / (9 nside^2) in the tabulated A_{2k+3}.
+//
+//  polar cap (x >= 2/3): the even values alone, by the recurrence in x^2 that
+//  follows from eliminating O (Ishioka, J. Met. Soc. Japan 96, 2018, has one
+//  recurrence of this kind), rescaled (mu_{m+2k} = e_k E_k) so that the
+//  coefficient of E_{k-1} is one, in difference form (Reinsch's modification,
+//  with w2 = 1 - x^2 = sin^2 theta, small near the pole):
+//      D_{k+1} = D_k + (gamma_k - alpha_k w2) E_k,  E_{k+1} = E_k + D_{k+1}.
+//  An odd value is the neighbouring even ones' sum over x,
+//      x mu_{m+2k+1} = (mu_{m+2k+2} + mu_{m+2k}) / A_{2k+2},
+//  so the odd coefficients fold into coefficients of the E_k once per m (FP64)
+//  and the contraction costs the same two operations.  1/x <= 1.5 here.
+//
+// 3.5 operations per (l, pair) (cap 3.6, see below), against 5 (difference form, x > 0.4)
+// and 4 of the one-step forms before.
+//
+// Accuracy.  A rounding of a ring's variable (x, w2) moves the ring: a phase error that
+// grows with l, the same in both directions.  The round trip of a smooth signal keeps of it
+// what does not average out over the rings, so the variable has to be better than one FP32
+// rounding: the belt's is exact; the cap's rounding error dw is made up for in every fourth
+// step (k = 3 mod 4) by D += -4 (4 dw) E, with the limit 4 of alpha (a quarter operation per k).
+// FP32 emulation against extended precision, nside 1024, one m, relative error of G and of
+// the analysis of a smooth exact G: belt 1.0 to 2.9e-6 and 6 to 10e-7 (one-step forms
+// 1.2e-5 and 14 to 33e-7); cap 0.8 to 3.1e-6 and 7 to 16e-7 (4 to 8e-6 and 14 to 25e-7; without
+// the correction 4 to 9e-6 and 26 to 50e-7).
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ float2 dup(float a) { return make_float2(a, a); }
 __device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
@@ -926,396 +977,396 @@ __device__ __forceinline__ void put(float2 &v, int k, float a)
     else v.x = a;
 }
 
+struct MxTables {
+    int lmax, L, npairs, ncap, lc;
+    const int *k0;            // per (m, pair): first k, a multiple of four
+    const float2 *seed;       // per (m, pair): state of the part's form at k0
+    const float4 *xw;         // per pair: belt (j^2, 0, 1/x), cap (w2, -16 times its rounding error, 1/x); 1/x = 0 for x = 0
+    const float2 *tb, *tp;    // per (m, k): (A_{2k+2}, A_{2k+3} 4 / (9 nside^2)); (-alpha_{k+1}, gamma_{k+1})
+    const double *c64;        // per a_lm: lambda = c mu
+    const double4 *kd;        // per (m, k): (c_2k e_k, c_{2k+1} e_k / A_{2k+2}, c_{2k-1} e_k / A_{2k}, 1 / e_k)
+};
+
+// the pairs of one thread: first k and starting state (needed until the last of the warp's
+// pairs has started), ring variable and the cap's correction of its rounding
 template <int NP> struct MxPairs {
-    static constexpr int NPK = NP / 2;
-    int ls[NP];
-    float s0[NP], s1[NP];
-    float2 X[NP / 2], W[NP / 2];
-    int lmin, lmaxs;
-    bool diff;
+    int k0[NP];
+    float2 sd[NP];
+    float2 X[NP / 2], C[NP / 2];
+    int kmin, kmaxs;
 };
 
 template <int NP>
-__device__ __forceinline__ void mx_load_pairs(MxPairs<NP> &P, int m, int L, int npairs, int p0,
-                                              const int *__restrict__ ls_tab, const float *__restrict__ s0_tab,
-                                              const float *__restrict__ s1_tab, const float *__restrict__ xp,
-                                              const float *__restrict__ wp)
+__device__ __forceinline__ void mx_load_pairs(MxPairs<NP> &P, const MxTables &t, int m, int nk, int p0, int pend)
 {
-    P.lmin = BIG;
-    P.lmaxs = -1;
-    float xs[NP], ws[NP];
+    P.kmin = BIG;
+    P.kmaxs = -1;
 #pragma unroll
-    for (int k = 0; k < NP; ++k) {
-        const int p = p0 + k;
-        int ls = BIG;
-        float s0 = 0.f, s1 = 0.f, x = 0.f, w = 1.f;
-        if (p < npairs) {
-            const size_t sidx = (size_t)m * npairs + p;
-            ls = ls_tab[sidx];
-            if (ls > L) ls = BIG;
-            else {
-                s0 = s0_tab[sidx];
-                s1 = s1_tab[sidx];
-            }
-            x = xp[p];
-            w = wp[p];
+    for (int i = 0; i < NP; ++i) {
+        const int p = p0 + i;
+        int k0 = BIG;
+        float2 sd = make_float2(0.f, 0.f);
+        float4 X = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (p < pend) {
+            const size_t idx = (size_t)m * t.npairs + p;
+            k0 = t.k0[idx];
+            if (k0 < nk) sd = t.seed[idx];
+            else k0 = BIG;
+            X = t.xw[p];
         }
-        P.ls[k] = ls;
-        P.s0[k] = s0;
-        P.s1[k] = s1;
-        xs[k] = x;
-        ws[k] = w;
-        if (ls < P.lmin) P.lmin = ls;
-        if (ls != BIG && ls > P.lmaxs) P.lmaxs = ls;
+        P.k0[i] = k0;
+        P.sd[i] = sd;
+        put(P.X[i >> 1], i & 1, X.x);
+        put(P.C[i >> 1], i & 1, X.y);
+        P.kmin = min(P.kmin, k0);
+        if (k0 != BIG) P.kmaxs = max(P.kmaxs, k0);
     }
-#pragma unroll
-    for (int pk = 0; pk < NP / 2; ++pk) {
-        P.X[pk] = make_float2(xs[2 * pk], xs[2 * pk + 1]);
-        P.W[pk] = make_float2(ws[2 * pk], ws[2 * pk + 1]);
-    }
-    P.diff = xs[0] > X_DIFFERENCE_FORM;
 }
 
-// one double step (l, l+1) of the recurrence for both packs.
-// plain state: (Sa, Sb) = (mu_{l-2}, mu_{l-1}); difference state: (Sa, Sb) =
-// (D_{l-1}, mu_{l-1}).  Outputs mu_l (V0) and mu_{l+1} (V1).
-template <bool DIFF, bool INJECT, int NP>
-__device__ __forceinline__ void mx_step(const MxPairs<NP> &P, int l, float A0, float B0, float A1, float B1,
-                                        float2 (&Sa)[NP / 2], float2 (&Sb)[NP / 2], float2 (&V0)[NP / 2],
-                                        float2 (&V1)[NP / 2])
+// advance from k to k + 1 with the table entry of k (CAP: O holds D_{k+1}); FIX: k = 3 mod 4.
+// (The two copies of a scalar operand and the signs cost nothing: with every value stored twice
+// in shared memory and the signs moved into the tables the synthesis ran 12 % longer.)
+template <bool CAP, bool FIX, int NPK>
+__device__ __forceinline__ void mx_advance(float2 t, const float2 (&X)[NPK], const float2 (&C)[NPK], float2 (&E)[NPK],
+                                           float2 (&O)[NPK])
 {
 #pragma unroll
-    for (int pk = 0; pk < NP / 2; ++pk) {
-        if (DIFF) {
-            float2 D = Sa[pk], mu = Sb[pk];
-            D = __ffma2_rn(__ffma2_rn(dup(-A0), P.W[pk], dup(B0)), mu, D);
-            const float2 v0 = __fadd2_rn(mu, D);
-            D = __ffma2_rn(__ffma2_rn(dup(-A1), P.W[pk], dup(B1)), v0, D);
-            const float2 v1 = __fadd2_rn(v0, D);
-            V0[pk] = v0;
-            V1[pk] = v1;
-            Sa[pk] = D;
-            Sb[pk] = v1;
+    for (int i = 0; i < NPK; ++i) {
+        if (CAP) {
+            E[i] = __fadd2_rn(E[i], O[i]);
+            O[i] = __ffma2_rn(__ffma2_rn(dup(t.x), X[i], dup(t.y)), E[i], O[i]);
+            if (FIX) O[i] = __ffma2_rn(C[i], E[i], O[i]);
         } else {
-            const float2 v0 = __ffma2_rn(__fmul2_rn(dup(A0), P.X[pk]), Sb[pk], neg2(Sa[pk]));
-            const float2 v1 = __ffma2_rn(__fmul2_rn(dup(A1), P.X[pk]), v0, neg2(Sb[pk]));
-            V0[pk] = v0;
-            V1[pk] = v1;
-            Sa[pk] = v0;
-            Sb[pk] = v1;
-        }
-        if (INJECT) {
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int k = 2 * pk + h;
-                if (l == P.ls[k]) {
-                    put(V0[pk], h, P.s0[k]);
-                    put(V1[pk], h, P.s1[k]);
-                    if (DIFF) {
-                        put(Sa[pk], h, P.s1[k] - P.s0[k]);
-                        put(Sb[pk], h, P.s1[k]);
-                    } else {
-                        put(Sa[pk], h, P.s0[k]);
-                        put(Sb[pk], h, P.s1[k]);
-                    }
-                }
-            }
+            E[i] = __ffma2_rn(dup(t.x), O[i], neg2(E[i]));
+            O[i] = __ffma2_rn(__fmul2_rn(dup(t.y), X[i]), E[i], neg2(O[i]));
         }
     }
 }
 
-// lmin, lmaxs: the warp's smallest first l and largest seeding l, so that the
-// warp runs one loop with one trip count (lanes not yet started add zeros)
-template <bool DIFF, int NP>
-__device__ __forceinline__ void mx_syn_run(const MxPairs<NP> &P, int m, int L, const float4 *__restrict__ sAB,
-                                           const float4 *__restrict__ sac, float2 (&ER)[NP / 2],
-                                           float2 (&EI)[NP / 2], float2 (&OR)[NP / 2], float2 (&OI)[NP / 2],
-                                           int lmin, int lmaxs)
+// Measured (nside 1024, one map): 0.608 ms with the one-step forms, 0.442 ms with these, the FMA
+// pipe 71 % busy; mean over the syntheses of an nside 2048 solve 2.93 -> 2.11 ms.
+// Synthesis of one (m, part): blockDim.x threads, NP pairs each, per pass.  Shared staging per
+// k: st[k] the recurrence entry, sac[k] = coefficients of E (re, im) and of O or folded odd
+// (re, im).  Control flow is warp-uniform: one first k and one seeding range per warp (lanes
+// not yet started add zeros).
+template <int NP, bool CAP>
+__device__ __forceinline__ void mx_synthesis(const MxTables &t, int m, const double2 *__restrict__ alm,
+                                             float2 *__restrict__ G, float4 *sac, float2 *st)
 {
-    float2 Sa[NP / 2], Sb[NP / 2], V0[NP / 2], V1[NP / 2];
-#pragma unroll
-    for (int pk = 0; pk < NP / 2; ++pk) Sa[pk] = Sb[pk] = dup(0.f);
-    int l = lmin;
-    for (; l <= L && l <= lmaxs; l += 2) {
-        const int j = (l - m) >> 1;
-        const float4 ab = sAB[j], ac = sac[j];
-        mx_step<DIFF, true, NP>(P, l, ab.x, ab.y, ab.z, ab.w, Sa, Sb, V0, V1);
-#pragma unroll
-        for (int pk = 0; pk < NP / 2; ++pk) {
-            ER[pk] = __ffma2_rn(dup(ac.x), V0[pk], ER[pk]);
-            EI[pk] = __ffma2_rn(dup(ac.y), V0[pk], EI[pk]);
-            OR[pk] = __ffma2_rn(dup(ac.z), V1[pk], OR[pk]);
-            OI[pk] = __ffma2_rn(dup(ac.w), V1[pk], OI[pk]);
+    constexpr int NPK = NP / 2;
+    const int nl = t.L - m + 1, nk = (nl >> 1) + 1;  // k with 2k <= L - m + 1
+    const long long base = mbase(t.lmax, m), kb = kbase(t.lmax, m);
+    const int i_lo = m < t.lc ? lcm_of(t.lc, m) - m : 0;  // coefficients below the FP64 block's end stay out
+    for (int k = threadIdx.x; k < nk + 3; k += blockDim.x) {  // steps run in fours: zeros past the end
+        const int i0 = 2 * k, i1 = 2 * k + 1;
+        double2 e = make_double2(0.0, 0.0), o = e;
+        if (k >= nk) {
+        } else if (CAP) {
+            const double4 d = t.kd[kb + k];
+            if (i0 >= i_lo && i0 < nl) e = cscale(alm[base + i0], d.x);
+            if (i1 >= i_lo && i1 < nl) o = cscale(alm[base + i1], d.y);
+            if (k > 0 && i0 - 1 >= i_lo) o = cadd(o, cscale(alm[base + i0 - 1], d.z));  // i0 - 1 < nl: k < nk
+        } else {
+            if (i0 >= i_lo && i0 < nl) e = cscale(alm[base + i0], t.c64[base + i0]);
+            if (i1 >= i_lo && i1 < nl) o = cscale(alm[base + i1], t.c64[base + i1]);
         }
+        sac[k] = make_float4((float)e.x, (float)e.y, (float)o.x, (float)o.y);
+        st[k] = k < nk ? (CAP ? t.tp : t.tb)[kb + k] : make_float2(0.f, 0.f);
     }
-    for (; l <= L; l += 2) {
-        const int j = (l - m) >> 1;
-        const float4 ab = sAB[j], ac = sac[j];
-        mx_step<DIFF, false, NP>(P, l, ab.x, ab.y, ab.z, ab.w, Sa, Sb, V0, V1);
+    __syncthreads();
+    const int pbeg = CAP ? 0 : t.ncap, pend = CAP ? t.ncap : t.npairs;
+    const size_t pstride = (size_t)(t.lmax + 1) * 2;
+    for (int w0 = (blockIdx.x * blockDim.x + (threadIdx.x & ~31)) * NP; pbeg + w0 < pend; w0 += gridDim.x * blockDim.x * NP) {
+        const int p0 = pbeg + w0 + (threadIdx.x & 31) * NP;
+        MxPairs<NP> P;
+        mx_load_pairs<NP>(P, t, m, nk, p0, pend);
+        float2 ER[NPK], EI[NPK], OR[NPK], OI[NPK], E[NPK], O[NPK];
 #pragma unroll
-        for (int pk = 0; pk < NP / 2; ++pk) {
-            ER[pk] = __ffma2_rn(dup(ac.x), V0[pk], ER[pk]);
-            EI[pk] = __ffma2_rn(dup(ac.y), V0[pk], EI[pk]);
-            OR[pk] = __ffma2_rn(dup(ac.z), V1[pk], OR[pk]);
-            OI[pk] = __ffma2_rn(dup(ac.w), V1[pk], OI[pk]);
+        for (int i = 0; i < NPK; ++i) ER[i] = EI[i] = OR[i] = OI[i] = E[i] = O[i] = dup(0.f);
+        int k = __reduce_min_sync(0xffffffffu, P.kmin);
+        const int kmaxs = __reduce_max_sync(0xffffffffu, P.kmaxs);
+        auto step = [&](int kk, auto fix) {
+            const float4 ac = sac[kk];
+            const float2 tt = st[kk];
+#pragma unroll
+            for (int i = 0; i < NPK; ++i) {
+                ER[i] = __ffma2_rn(dup(ac.x), E[i], ER[i]);
+                EI[i] = __ffma2_rn(dup(ac.y), E[i], EI[i]);
+                OR[i] = __ffma2_rn(dup(ac.z), CAP ? E[i] : O[i], OR[i]);
+                OI[i] = __ffma2_rn(dup(ac.w), CAP ? E[i] : O[i], OI[i]);
+            }
+            mx_advance<CAP, decltype(fix)::value, NPK>(tt, P.X, P.C, E, O);
+        };
+        auto four = [&]() {
+            step(k, std::false_type{});
+            step(k + 1, std::false_type{});
+            step(k + 2, std::false_type{});
+            step(k + 3, std::true_type{});
+        };
+        for (; k < nk && k <= kmaxs; k += 4) {
+#pragma unroll
+            for (int i = 0; i < NP; ++i)
+                if (k == P.k0[i]) {
+                    put(E[i >> 1], i & 1, P.sd[i].x);
+                    put(O[i >> 1], i & 1, P.sd[i].y);
+                }
+            four();
+        }
+        for (; k < nk; k += 4) four();
+#pragma unroll
+        for (int i = 0; i < NP; ++i) {
+            const int p = p0 + i;
+            if (p >= pend) break;
+            const int pk = i >> 1, h = i & 1;
+            const float ix = t.xw[p].z;
+            const float er = get(ER[pk], h), ei = get(EI[pk], h), orr = get(OR[pk], h) * ix, oi = get(OI[pk], h) * ix;
+            *reinterpret_cast<float4 *>(G + (size_t)p * pstride + 2 * (size_t)m) =
+                make_float4(er + orr, ei + oi, er - orr, ei - oi);
         }
     }
 }
 
-// shared-memory staging: per pair of l (l = m + 2j, l + 1):
-//   sAB[j] = (A_l, B_l, A_{l+1}, B_{l+1}),  sac[j] = (Re a'_l, Im a'_l, Re a'_{l+1}, Im a'_{l+1})
+// grid: (CTAs of a part, m, part), the belt's (more work per pair) first
 template <int NP>
-__global__ void __launch_bounds__(LEG_THREADS) k_legsyn_mx(int lmax, int L, int npairs,
-                                                           const double2 *__restrict__ alm,
-                                                           const float *__restrict__ A, const float *__restrict__ B,
-                                                           const double *__restrict__ c64,
-                                                           const int *__restrict__ ls_tab,
-                                                           const float *__restrict__ s0_tab,
-                                                           const float *__restrict__ s1_tab,
-                                                           const float *__restrict__ xp, const float *__restrict__ wp,
+__global__ void __launch_bounds__(LEG_THREADS) k_legsyn_mx(const MxTables t, const double2 *__restrict__ alm,
                                                            float2 *__restrict__ G)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int m = blockIdx.y;
-    const int nl = L - m + 1;
-    const int nj = (nl + 1) / 2 + 1;
-    const long long base = mbase(lmax, m);
-    float4 *sAB = reinterpret_cast<float4 *>(smem_raw);
-    float4 *sac = sAB + nj;
-    for (int j = threadIdx.x; j < nj; j += blockDim.x) {
-        float4 ab = make_float4(0.f, 0.f, 0.f, 0.f), ac = make_float4(0.f, 0.f, 0.f, 0.f);
-        const int i0 = 2 * j, i1 = 2 * j + 1;
-        if (i0 < nl) {
-            const double2 a = alm[base + i0];
-            const double cc = c64[base + i0];
-            ab.x = A[base + i0];
-            ab.y = B[base + i0];
-            ac.x = (float)(a.x * cc);
-            ac.y = (float)(a.y * cc);
-        }
-        if (i1 < nl) {
-            const double2 a = alm[base + i1];
-            const double cc = c64[base + i1];
-            ab.z = A[base + i1];
-            ab.w = B[base + i1];
-            ac.z = (float)(a.x * cc);
-            ac.w = (float)(a.y * cc);
-        }
-        sAB[j] = ab;
-        sac[j] = ac;
-    }
-    __syncthreads();
-    const size_t pstride = (size_t)(lmax + 1) * 2;
-    for (int p0 = (blockIdx.x * blockDim.x + threadIdx.x) * NP; p0 < npairs; p0 += gridDim.x * blockDim.x * NP) {
-        MxPairs<NP> P;
-        mx_load_pairs<NP>(P, m, L, npairs, p0, ls_tab, s0_tab, s1_tab, xp, wp);
-        float2 ER[NP / 2], EI[NP / 2], OR[NP / 2], OI[NP / 2];
-#pragma unroll
-        for (int pk = 0; pk < NP / 2; ++pk) ER[pk] = EI[pk] = OR[pk] = OI[pk] = dup(0.f);
-        // warp-uniform control flow: one first l, one seeding range and one recurrence
-        // form (the first active lane's) per warp -- per-lane forms split the warp across
-        // both loop bodies; measured 9 % faster at nside 2048
-        const unsigned am = __activemask();
-        const int lmin = __reduce_min_sync(am, P.lmin), lmaxs = __reduce_max_sync(am, P.lmaxs);
-        const bool diff = __shfl_sync(am, P.diff ? 1 : 0, __ffs(am) - 1) != 0;
-        if (lmin <= L) {
-            if (diff) mx_syn_run<true, NP>(P, m, L, sAB, sac, ER, EI, OR, OI, lmin, lmaxs);
-            else mx_syn_run<false, NP>(P, m, L, sAB, sac, ER, EI, OR, OI, lmin, lmaxs);
-        }
-#pragma unroll
-        for (int k = 0; k < NP; ++k) {
-            const int p = p0 + k;
-            if (p >= npairs) break;
-            const int pk = k >> 1, h = k & 1;
-            const float er = get(ER[pk], h), ei = get(EI[pk], h), orr = get(OR[pk], h), oi = get(OI[pk], h);
-            float2 *g = G + (size_t)p * pstride + 2 * (size_t)m;
-            g[0] = make_float2(er + orr, ei + oi);
-            g[1] = make_float2(er - orr, ei - oi);
-        }
-    }
+    const int m = blockIdx.y, nk = ((t.L - m + 1) >> 1) + 1;
+    float4 *sac = reinterpret_cast<float4 *>(smem_raw);
+    float2 *st = reinterpret_cast<float2 *>(sac + nk + 3);
+    if (blockIdx.z) mx_synthesis<NP, true>(t, m, alm, G, sac, st);
+    else mx_synthesis<NP, false>(t, m, alm, G, sac, st);
 }
 
-// analysis: CTA per m; a warp covers 32 lanes x NP pairs; chunks of CH
-// values of l accumulate the packs in f32x2 registers, then are summed across
-// the warp (through the swizzled shared stage for CH = 8, by a shuffle
-// reduce-scatter otherwise).  Eight pairs per lane halve the cross-lane sum
-// per (l, m, pair) against four; two CTAs per SM (128 registers) measured
-// faster than one CTA with no spills.
+constexpr int MX_TBLK = 64;  // table entries a warp stages at a time
 
+// shared memory of an analysis warp: two stages of the cross-lane sum (per lane and k of a block
+// E re, im, O re, im), table entries, and the pairs' first k (two to a word) and starting
+// states, read while pairs start
+template <int NP> struct __align__(16) MxAnaShared {
+    float4 stage[2][4 * 32];
+    float2 tab[MX_TBLK];
+    unsigned k0[NP / 2][32];
+    float2 sd[NP][32];
+};
 
-template <bool DIFF, int NP, int CH>
-__device__ __forceinline__ void mx_ana_run(const MxPairs<NP> &P, int m, int L, int lmin_w, int lmaxs_w,
-                                           const float4 *__restrict__ sAB,
-                                           const float2 (&FEr)[NP / 2], const float2 (&FEi)[NP / 2],
-                                           const float2 (&FOr)[NP / 2], const float2 (&FOi)[NP / 2],
-                                           float2 *acc, float4 *stage, int lane)
+// Analysis of one (m, part, group of 32 NP pairs) by one warp: blocks of four k (eight l) are
+// summed over the packs in registers, across the warp through a shared stage, and added to
+// sum[4 k + (0, 1)] (E re, im), sum[4 k + (2, 3)] (O, or the folded odd values' E / x) in global
+// memory.  The stage of one block is read while the next block's FMAs run (two stages), one
+// row per step, so that its latency is not waited for.
+//
+// What bounds it: the FMA pipe (about 270 cycles per block and warp) and, four warps to a
+// shared-memory port, the stage: with both halves of each packed sum staged (64 wavefronts per
+// block and 16 more additions when read) the cross-lane sum took 38 % of the time, the
+// port being busy as long as the pipe.  Adding the halves first leaves 32.
+template <int NP, bool CAP>
+__device__ __forceinline__ void mx_analysis(const MxTables &t, int m, int grp, const float2 *__restrict__ F,
+                                            float *sum, MxAnaShared<NP> &S, int nk)
 {
     constexpr int NPK = NP / 2;
-    float2 Sa[NPK], Sb[NPK], V0[NPK], V1[NPK];
+    const int lane = threadIdx.x;
+    const int pend = CAP ? t.ncap : t.npairs;
+    const int p0 = (CAP ? 0 : t.ncap) + grp * 32 * NP + lane * NP;
+    const size_t pstride = (size_t)(t.lmax + 1) * 2;
+    const float2 *tab = (CAP ? t.tp : t.tb) + kbase(t.lmax, m);
+    float2 X[NPK], C[NPK], FEr[NPK], FEi[NPK], FOr[NPK], FOi[NPK], E[NPK], O[NPK];
+    int kmin, kmaxs, knext;  // first and last starting k of the warp; next one of this lane
+    {
+        MxPairs<NP> P;
+        mx_load_pairs<NP>(P, t, m, nk, p0, pend);
+        knext = P.kmin;
+        kmin = __reduce_min_sync(0xffffffffu, P.kmin);
+        kmaxs = __reduce_max_sync(0xffffffffu, P.kmaxs);
+        if (kmin >= nk) return;
 #pragma unroll
-    for (int pk = 0; pk < NPK; ++pk) Sa[pk] = Sb[pk] = dup(0.f);
-    for (int l0 = lmin_w; l0 <= L; l0 += CH) {
-        float2 AR[CH], AI[CH];
-        const bool inj = l0 <= lmaxs_w;
-#pragma unroll
-        for (int i = 0; i < CH; i += 2) {
-            const float4 ab = sAB[(l0 - m + i) >> 1];  // l0 - m is even
-            if (inj) mx_step<DIFF, true, NP>(P, l0 + i, ab.x, ab.y, ab.z, ab.w, Sa, Sb, V0, V1);
-            else mx_step<DIFF, false, NP>(P, l0 + i, ab.x, ab.y, ab.z, ab.w, Sa, Sb, V0, V1);
-            AR[i] = __fmul2_rn(FEr[0], V0[0]);
-            AI[i] = __fmul2_rn(FEi[0], V0[0]);
-            AR[i + 1] = __fmul2_rn(FOr[0], V1[0]);
-            AI[i + 1] = __fmul2_rn(FOi[0], V1[0]);
-#pragma unroll
-            for (int pk = 1; pk < NPK; ++pk) {
-                AR[i] = __ffma2_rn(FEr[pk], V0[pk], AR[i]);
-                AI[i] = __ffma2_rn(FEi[pk], V0[pk], AI[i]);
-                AR[i + 1] = __ffma2_rn(FOr[pk], V1[pk], AR[i + 1]);
-                AI[i + 1] = __ffma2_rn(FOi[pk], V1[pk], AI[i + 1]);
+        for (int i = 0; i < NP; ++i) {
+            float4 f = make_float4(0.f, 0.f, 0.f, 0.f);
+            float ix = 0.f;
+            if (P.k0[i] != BIG) {
+                f = *reinterpret_cast<const float4 *>(F + (size_t)(p0 + i) * pstride + 2 * (size_t)m);
+                ix = t.xw[p0 + i].z;
             }
-            if constexpr (CH == 8) {
-                stage[stage_slot(i, lane)] = make_float4(AR[i].x, AR[i].y, AI[i].x, AI[i].y);
-                stage[stage_slot(i + 1, lane)] = make_float4(AR[i + 1].x, AR[i + 1].y, AI[i + 1].x, AI[i + 1].y);
-            }
+            put(FEr[i >> 1], i & 1, f.x + f.z);
+            put(FEi[i >> 1], i & 1, f.y + f.w);
+            put(FOr[i >> 1], i & 1, (f.x - f.z) * ix);
+            put(FOi[i >> 1], i & 1, (f.y - f.w) * ix);
+            S.sd[i][lane] = P.sd[i];
         }
-        if constexpr (CH == 8) {
-            __syncwarp();
-            const int i = lane >> 2, q = lane & 3;
-            const float4 *row = stage + 32 * i + 8 * q;
-            const int c = q + 4 * (i & 1);
-            // the eight stores summed as a tree of depth 3 (a chain of 7 dependent adds held
-            // each lane on its loads' latency)
-            float2 tr[8], ti[8];
 #pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const float4 v = row[j ^ c];
-                tr[j] = make_float2(v.x, v.y);
-                ti[j] = make_float2(v.z, v.w);
-            }
-#pragma unroll
-            for (int w = 4; w >= 1; w >>= 1)
-#pragma unroll
-                for (int j = 0; j < w; ++j) {
-                    tr[j] = __fadd2_rn(tr[j], tr[j + w]);
-                    ti[j] = __fadd2_rn(ti[j], ti[j + w]);
-                }
-            float vr = tr[0].x + tr[0].y, vi = ti[0].x + ti[0].y;
-            vr += __shfl_xor_sync(0xffffffffu, vr, 1);
-            vi += __shfl_xor_sync(0xffffffffu, vi, 1);
-            vr += __shfl_xor_sync(0xffffffffu, vr, 2);
-            vi += __shfl_xor_sync(0xffffffffu, vi, 2);
-            if (q == 0) {
-                const int l = l0 + i;
-                if (l <= L) {
-                    atomicAdd(&acc[l - m].x, vr);
-                    atomicAdd(&acc[l - m].y, vi);
-                }
-            }
-            __syncwarp();  // the next chunk rewrites the stage
-        } else {
-            float vr[CH], vi[CH];
-#pragma unroll
-            for (int i = 0; i < CH; ++i) {
-                vr[i] = AR[i].x + AR[i].y;
-                vi[i] = AI[i].x + AI[i].y;
-            }
-            warp_reduce_scatter<float, CH>(vr, vi, lane);
-            constexpr int sh = 5 - Log2<CH>::v;  // each l ends in 2^sh lanes
-            if ((lane & ((1 << sh) - 1)) == 0) {
-                const int l = l0 + (lane >> sh);
-                if (l <= L) {
-                    atomicAdd(&acc[l - m].x, vr[0]);
-                    atomicAdd(&acc[l - m].y, vi[0]);
-                }
-            }
+        for (int i = 0; i < NPK; ++i) {
+            X[i] = P.X[i];
+            C[i] = P.C[i];
+            S.k0[i][lane] = (unsigned)(P.k0[2 * i] & 0xffff) | (unsigned)P.k0[2 * i + 1] << 16;  // BIG: 0xffff, no k
+            E[i] = O[i] = dup(0.f);
         }
     }
+    auto load_table = [&](int k0) {
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < MX_TBLK / 32; ++i) {
+            const int k = k0 + i * 32 + lane;
+            S.tab[i * 32 + lane] = k < nk ? tab[k] : make_float2(0.f, 0.f);  // blocks run up to three k past the end
+        }
+        __syncwarp();
+    };
+    load_table(kmin & ~(MX_TBLK - 1));
+    // lane (r, q) = (lane / 8, lane % 8) reads k = r of a block, lanes 4q .. 4q + 3 (in an order that
+    // keeps the eight lanes of a phase on distinct banks); three shuffles' exchange then leaves
+    // component q & 3 summed over the warp
+    const int rr = lane >> 3, rq = lane & 7, rc = rq >> 1, rrow = 32 * rr + 4 * rq;
+    float *dst = sum + 4 * rr + (rq & 3);
+    auto finish = [&](int kc, float4 v) {
+        const bool odd = rq & 2, im = rq & 1;
+        float a = odd ? v.z : v.x, b = odd ? v.w : v.y;
+        a += __shfl_xor_sync(0xffffffffu, odd ? v.x : v.z, 2);
+        b += __shfl_xor_sync(0xffffffffu, odd ? v.y : v.w, 2);
+        float c = im ? b : a;
+        c += __shfl_xor_sync(0xffffffffu, im ? a : b, 1);
+        c += __shfl_xor_sync(0xffffffffu, c, 4);
+        if (rq < 4 && kc + rr < nk) atomicAdd(dst + 4 * kc, c);  // no value used: a native reduction in L2
+    };
+    int buf = 0, kc = kmin;
+    auto block = [&]() {
+        if ((kc & (MX_TBLK - 1)) == 0 && kc != kmin) load_table(kc);
+        const float2 *tk = S.tab + (kc & (MX_TBLK - 1));
+        float4 *stage = S.stage[buf] + lane;
+        const float4 *prev = S.stage[buf ^ 1] + rrow;
+        float4 v;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float4 w = prev[i ^ rc];
+            float2 er = __fmul2_rn(FEr[0], E[0]), ei = __fmul2_rn(FEi[0], E[0]);
+            float2 orr = __fmul2_rn(FOr[0], CAP ? E[0] : O[0]), oi = __fmul2_rn(FOi[0], CAP ? E[0] : O[0]);
+#pragma unroll
+            for (int q = 1; q < NPK; ++q) {
+                er = __ffma2_rn(FEr[q], E[q], er);
+                ei = __ffma2_rn(FEi[q], E[q], ei);
+                orr = __ffma2_rn(FOr[q], CAP ? E[q] : O[q], orr);
+                oi = __ffma2_rn(FOi[q], CAP ? E[q] : O[q], oi);
+            }
+            stage[32 * i] = make_float4(er.x + er.y, ei.x + ei.y, orr.x + orr.y, oi.x + oi.y);
+            if (i == 3) mx_advance<CAP, true, NPK>(tk[i], X, C, E, O);
+            else mx_advance<CAP, false, NPK>(tk[i], X, C, E, O);
+            v = i ? make_float4(v.x + w.x, v.y + w.y, v.z + w.z, v.w + w.w) : w;
+        }
+        if (kc != kmin) finish(kc - 4, v);
+        __syncwarp();
+        buf ^= 1;
+        kc += 4;
+    };
+    // two loops: the starting states' writes into halves of packed registers stay out of the second
+    while (kc < nk && kc <= kmaxs) {
+        if (knext == kc) {
+            knext = BIG;
+#pragma unroll
+            for (int i = 0; i < NPK; ++i) {
+                const unsigned w = S.k0[i][lane];
+                const int ka = (int)(w & 0xffff), kb = (int)(w >> 16);
+                if (ka == kc) {
+                    const float2 s = S.sd[2 * i][lane];
+                    E[i].x = s.x;
+                    O[i].x = s.y;
+                } else if (ka > kc) {
+                    knext = min(knext, ka);
+                }
+                if (kb == kc) {
+                    const float2 s = S.sd[2 * i + 1][lane];
+                    E[i].y = s.x;
+                    O[i].y = s.y;
+                } else if (kb > kc) {
+                    knext = min(knext, kb);
+                }
+            }
+        }
+        __syncwarp();
+        block();
+    }
+    while (kc < nk) block();
+    const float4 *prev = S.stage[buf ^ 1] + rrow;
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const float4 w = prev[i ^ rc];
+        v.x += w.x;
+        v.y += w.y;
+        v.z += w.z;
+        v.w += w.w;
+    }
+    finish(kmin + ((nk - 1 - kmin) & ~3), v);
 }
 
-template <int NP, int CH>
-__global__ void __launch_bounds__(LEG_THREADS, 2) k_legana_mx(int lmax, int L, int npairs, int lc,
-                                                           const float2 *__restrict__ F, const float *__restrict__ A,
-                                                           const float *__restrict__ B,
-                                                           const int *__restrict__ ls_tab,
-                                                           const float *__restrict__ s0_tab,
-                                                           const float *__restrict__ s1_tab,
-                                                           const float *__restrict__ xp, const float *__restrict__ wp,
-                                                           const double *__restrict__ c64, int mode, double omega,
-                                                           BlendArgs ba, const double2 *__restrict__ low,
-                                                           const double2 *__restrict__ a_old,
-                                                           double2 *__restrict__ out, double *__restrict__ part)
+// Measured with the epilogue below: nside 768 adjoint 0.443 -> 0.262 + 0.031 ms, mean over the
+// analyses of a solve at nside 2048 3.90 -> 2.72 + 0.30 ms, at nside 512 0.138 -> 0.068 + 0.031 ms,
+// at nside 128 0.027 -> 0.010 + 0.008 ms.
+// One warp per CTA and (group of pairs, part, m), grid (belt groups, cap groups; m): no barrier
+// joins warps of unequal work.  Before, a CTA summed an m in shared memory: its warps spent a
+// third of their time at the barrier before the epilogue (nside 768), and FP32 atomics in
+// shared memory are compare-and-swap loops.
+template <int NP>
+__global__ void __launch_bounds__(32, NP == 8 ? 17 : 16) k_legana_mx(const MxTables t, int ngroups, const float2 *__restrict__ F,
+                                                      float4 *__restrict__ psum)
 {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ MxAnaShared<NP> S;
+    const int m = blockIdx.y, nk = ((t.L - m + 1) >> 1) + 1;
+    const long long kb = kbase(t.lmax, m), nks = kbase(t.lmax, t.lmax + 1) + 2;  // nks: entries per part
+    // groups nearest the equator (most l above the first kept one) first
+    const int g = blockIdx.x;
+    if (g < ngroups) mx_analysis<NP, false>(t, m, ngroups - 1 - g, F, &psum[kb].x, S, nk);
+    else mx_analysis<NP, true>(t, m, 2 * ngroups - 1 - g, F, &psum[nks + kb].x, S, nk);
+}
+
+// (double)f for finite f in integer arithmetic: the conversion instruction runs at the FP64 rate
+__device__ __forceinline__ double widen(float f)
+{
+    const unsigned u = __float_as_uint(f), a = u & 0x7fffffffu;
+    if (a < 0x00800000u || a >= 0x7f800000u) return (double)f;  // zero, denormal, infinity, NaN
+    return __hiloint2double((int)((u & 0x80000000u) | ((a >> 3) + 0x38000000u)), (int)(a << 29));
+}
+
+// Eq. (4) epilogue of the mixed analysis, a CTA per m; clears the sums for the next launch.  Run
+// by the last warp at its m inside the kernel above it took 14 % of that kernel (one warp's
+// chain of loads per m, nside 768).
+__global__ void __launch_bounds__(128) k_ana_epilogue(const MxTables t, int mode, BlendArgs ba,
+                                                      const double2 *__restrict__ low,
+                                                      const double2 *__restrict__ a_old, double2 *__restrict__ out,
+                                                      double *__restrict__ part, float4 *__restrict__ psum)
+{
     __shared__ double red[4][LEG_THREADS / 32];
-    __shared__ int next_group;
-    const int m = blockIdx.x;
-    const int nl = L - m + 1;
-    const int nlp = nl + CH + 2;
-    const long long base = mbase(lmax, m);
-    // (A_l, B_l, A_l+1, B_l+1) per pair of l from l - m = 0; for CH = 8 the per-warp
-    // stages of the cross-lane sum; FP32 accumulators (each entry sums one cross-lane
-    // result per group of ring pairs; the epilogue converts to FP64)
-    const int nab = (nlp + 1) / 2;
-    float4 *sAB = reinterpret_cast<float4 *>(smem_raw);
-    float4 *stage = sAB + nab;
-    float2 *acc = reinterpret_cast<float2 *>(stage + (CH == 8 ? LEG_THREADS * 8 : 0));
-    for (int i = threadIdx.x; i < nab; i += blockDim.x) {
-        const int j = 2 * i;
-        sAB[i] = make_float4(j < nl ? A[base + j] : 0.f, j < nl ? B[base + j] : 0.f,
-                             j + 1 < nl ? A[base + j + 1] : 0.f, j + 1 < nl ? B[base + j + 1] : 0.f);
-    }
-    for (int i = threadIdx.x; i < nlp; i += blockDim.x) acc[i] = make_float2(0.f, 0.f);
-    if (threadIdx.x == 0) next_group = 0;
-    __syncthreads();
-    const int lane = threadIdx.x & 31;
-    const int per_group = 32 * NP;
-    const int ngroups = (npairs + per_group - 1) / per_group;
-    const size_t pstride = (size_t)(lmax + 1) * 2;
-    for (;;) {
-        // warps take groups of ring pairs dynamically (their work differs with latitude)
-        int grp = 0;
-        if (lane == 0) grp = atomicAdd(&next_group, 1);
-        grp = __shfl_sync(0xffffffffu, grp, 0);
-        if (grp >= ngroups) break;
-        // equator first: the work per pair grows towards the equator (more l above the
-        // first kept one), so handing out the largest groups first shortens the tail at the
-        // barrier before the epilogue
-        const int p0 = (ngroups - 1 - grp) * per_group + lane * NP;
-        MxPairs<NP> P;
-        mx_load_pairs<NP>(P, m, L, npairs, p0, ls_tab, s0_tab, s1_tab, xp, wp);
-        // one recurrence form per warp: the shuffles below need warp-uniform control flow
-        P.diff = __shfl_sync(0xffffffffu, P.diff ? 1 : 0, 0) != 0;
-        const int lmin_w = __reduce_min_sync(0xffffffffu, P.lmin);
-        const int lmaxs_w = __reduce_max_sync(0xffffffffu, P.lmaxs);  // one seeding range per warp
-        if (lmin_w > L) continue;
-        float fer[NP], fei[NP], forr[NP], foi[NP];
-#pragma unroll
-        for (int k = 0; k < NP; ++k) {
-            fer[k] = fei[k] = forr[k] = foi[k] = 0.f;
-            if (P.ls[k] != BIG) {
-                const float2 *f = F + (size_t)(p0 + k) * pstride + 2 * (size_t)m;
-                const float2 fn = f[0], fs = f[1];
-                fer[k] = fn.x + fs.x;
-                fei[k] = fn.y + fs.y;
-                forr[k] = fn.x - fs.x;
-                foi[k] = fn.y - fs.y;
+    const int m = blockIdx.x, nk = ((t.L - m + 1) >> 1) + 1;
+    const long long base = mbase(t.lmax, m), kb = kbase(t.lmax, m);
+    const long long nks = kbase(t.lmax, t.lmax + 1) + 2;
+    float4 *sb = psum + kb, *sc = psum + nks + kb;
+    // belt: c mu-sums; cap: even l from E_k, odd l from the fold over E_k and E_{k+1}; the FP64
+    // block's l take its values
+    const int low_lim = (low && m < t.lc) ? lcm_of(t.lc, m) : 0;
+    BlendSums v;
+    for (int k = threadIdx.x; 2 * k <= t.lmax - m; k += blockDim.x) {
+        const int l = m + 2 * k;
+        const long long i = base + 2 * k;
+        double2 e = make_double2(0.0, 0.0), o = e;
+        if (l < low_lim) {
+            if (l <= t.L) e = low[i];
+            if (l < t.L) o = low[i + 1];
+        } else if (l <= t.L) {
+            const float4 b = sb[k], c = sc[k];
+            const double4 d = t.kd[kb + k];
+            const double ce = t.c64[i];
+            e = make_double2(ce * widen(b.x) + d.x * widen(c.x), ce * widen(b.y) + d.x * widen(c.y));
+            if (l < t.L) {
+                const float4 c2 = sc[k + 1];
+                const double r = t.kd[kb + k + 1].z, co = t.c64[i + 1];
+                o = make_double2(co * widen(b.z) + (d.y * widen(c.z) + r * widen(c2.z)),
+                                 co * widen(b.w) + (d.y * widen(c.w) + r * widen(c2.w)));
             }
         }
-        float2 FEr[NP / 2], FEi[NP / 2], FOr[NP / 2], FOi[NP / 2];
-#pragma unroll
-        for (int pk = 0; pk < NP / 2; ++pk) {
-            FEr[pk] = make_float2(fer[2 * pk], fer[2 * pk + 1]);
-            FEi[pk] = make_float2(fei[2 * pk], fei[2 * pk + 1]);
-            FOr[pk] = make_float2(forr[2 * pk], forr[2 * pk + 1]);
-            FOi[pk] = make_float2(foi[2 * pk], foi[2 * pk + 1]);
-        }
-        float4 *wstage = stage + (threadIdx.x >> 5) * 256;
-        if (P.diff) mx_ana_run<true, NP, CH>(P, m, L, lmin_w, lmaxs_w, sAB, FEr, FEi, FOr, FOi, acc, wstage, lane);
-        else mx_ana_run<false, NP, CH>(P, m, L, lmin_w, lmaxs_w, sAB, FEr, FEi, FOr, FOi, acc, wstage, lane);
+        blend_one(l, t.L, i, mode, ba, e, a_old, out, v);
+        if (l < t.lmax) blend_one(l + 1, t.L, i + 1, mode, ba, o, a_old, out, v);
     }
+    if (mode == LEG_BLEND) blend_sums(v, m, part, red);
     __syncthreads();
-    const int low_lim = (low && m < lc) ? lcm_of(lc, m) : 0;
-    blend_epilogue(lmax, L, m, base, mode, omega, ba, c64, acc, low, low_lim, a_old, out, part, red);
+    for (int k = threadIdx.x; k < nk; k += blockDim.x) sb[k] = sc[k] = make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
 // ---------------------------------------------------------------------------
@@ -1327,12 +1378,7 @@ size_t syn_smem(int L) { return (size_t)(L + 3) * (sizeof(cx<T>) + sizeof(T)) + 
 template <typename T, int CH>
 size_t ana_smem(int L) { return (size_t)(L + 1 + CH + 2) * (sizeof(double2) + sizeof(T)) + 16; }
 
-size_t syn_mx_smem(int L) { return (size_t)((L + 2) / 2 + 2) * 2 * sizeof(float4) + 16; }
-size_t ana_mx_smem(int L, int ch)
-{
-    return (size_t)(L + 1 + ch + 2) * (sizeof(float2) + 2 * sizeof(float)) + 32 +
-           (ch == 8 ? (size_t)LEG_THREADS * 8 * sizeof(float4) : 0);
-}
+size_t syn_mx_smem(int L) { return (size_t)((L + 1) / 2 + 5) * (sizeof(float4) + sizeof(float2)) + 16; }
 
 template <typename TG>
 wf_status launch_syn64(wf_plan p, const double2 *alm, int L, int lcut, cx<TG> *G, int gstride, cudaStream_t s)
@@ -1474,7 +1520,12 @@ wf_status hp_build_legendre_tables(wf_plan p, const std::vector<double> &xpair, 
 {
     const int lmax = p->lmax, np = p->npairs;
     const long long nalm = p->nalm;
-    std::vector<double> A(nalm), c(nalm), Bm2(nalm), log2c(lmax + 1);
+    const bool f32 = p->prec != WF_PREC_FP64, tc = tc_prec(p->prec);
+    const long long nks = kbase(lmax, lmax + 1) + 2;  // entries of the tables per (m, k)
+    std::vector<double> A(nalm), c(nalm), Bm2(tc ? nalm : 0), log2c(lmax + 1), Atop(lmax + 1);
+    std::vector<double4> kd(f32 ? nks : 0, make_double4(0.0, 0.0, 0.0, 0.0));
+    std::vector<float2> tb(f32 ? nks : 0, make_float2(0.f, 0.f)), tp(f32 ? nks : 0, make_float2(0.f, 0.f));
+    std::vector<double> Ax(lmax + 8), cx_(lmax + 8), e(lmax / 2 + 8);
     for (int m = 0; m <= lmax; ++m) {
         const long long b = mbase(lmax, m);
         auto coef = [m](int l) { return std::sqrt((4.0 * l * l - 1.0) / ((double)l * l - (double)m * m)); };
@@ -1492,7 +1543,42 @@ wf_status hp_build_legendre_tables(wf_plan p, const std::vector<double> &xpair, 
         A[b] = 0.0;
         if (m + 1 <= lmax) A[b + 1] = std::sqrt(2.0 * m + 3.0) * c[b] / c[b + 1];
         for (int l = m + 2; l <= lmax; ++l) A[b + (l - m)] = coef(l) * c[b + (l - 1 - m)] / c[b + (l - m)];
-        for (int l = m; l <= lmax; ++l) Bm2[b + (l - m)] = A[b + (l - m)] - 2.0;
+        if (tc)
+            for (int l = m; l <= lmax; ++l) Bm2[b + (l - m)] = A[b + (l - m)] - 2.0;
+        if (f32) {
+            // A and c a few l past lmax (i = l - m), then the tables of the two-step forms
+            const int n = lmax - m + 1, K = n / 2 + 1;  // k = 0 .. K - 1: 2k <= lmax - m + 1
+            for (int i = 0; i < n; ++i) {
+                Ax[i] = A[b + i];
+                cx_[i] = c[b + i];
+            }
+            for (int i = n; i < n + 5; ++i) {
+                const int l = m + i;
+                if (i == 1) {
+                    cx_[i] = 1.0;
+                    Ax[i] = std::sqrt(2.0 * m + 3.0);
+                } else {
+                    cx_[i] = (coef(l) / coef(l - 1)) * cx_[i - 2];
+                    Ax[i] = coef(l) * cx_[i - 1] / cx_[i];
+                }
+            }
+            Atop[m] = Ax[n];
+            e[0] = e[1] = 1.0;
+            for (int k = 1; k <= K; ++k) e[k + 1] = e[k - 1] * (Ax[2 * k + 2] / Ax[2 * k]);
+            // one chain rescaled so that alpha - beta tends to 2 at the top, as A does above
+            const int kt = std::max(1, (n - 1) / 2);
+            const double r = e[kt] / e[kt - 1];
+            for (int k = 1; k <= K + 1; k += 2) e[k] *= (kt & 1) ? 1.0 / r : r;
+            const long long kb = kbase(lmax, m);
+            for (int k = 0; k < K; ++k) {
+                const double A2 = Ax[2 * k + 2], g = e[k + 1] / e[k + 2];
+                const double al = Ax[2 * k + 4] * Ax[2 * k + 3] * g, be = (Ax[2 * k + 4] / A2 + 1.0) * g;
+                tb[kb + k] = make_float2((float)A2, (float)(Ax[2 * k + 3] * (4.0 / 9.0) / ((double)p->nside * p->nside)));
+                tp[kb + k] = make_float2(-(float)al, (float)(al - be - 2.0));
+                kd[kb + k] = make_double4(2 * k < n ? cx_[2 * k] * e[k] : 0.0, 2 * k + 1 < n ? cx_[2 * k + 1] * e[k] / A2 : 0.0,
+                                          k > 0 && 2 * k - 1 < n ? cx_[2 * k - 1] * e[k] / Ax[2 * k] : 0.0, 1.0 / e[k]);
+            }
+        }
         // log2 of sqrt((2m+1)/(4 pi) (2m)! / (2^m m!)^2)
         log2c[m] = 0.5 * (std::log(2.0 * m + 1.0) - std::log(4.0 * M_PI) + std::lgamma(2.0 * m + 1.0) -
                           2.0 * std::lgamma(m + 1.0) - 2.0 * m * std::log(2.0)) / std::log(2.0);
@@ -1502,8 +1588,7 @@ wf_status hp_build_legendre_tables(wf_plan p, const std::vector<double> &xpair, 
     // 1 - x exactly for the polar-cap rings (1 - z = k^2 / (3 nside^2))
     for (int i = 0; i + 1 < p->nside && i < np; ++i)
         wpair[i] = (double)(i + 1) * (i + 1) / (3.0 * p->nside * p->nside);
-    const bool f32 = p->prec != WF_PREC_FP64;
-    double *dx64 = nullptr, *dst64 = nullptr, *dlog2c = nullptr;
+    double *dst64 = nullptr, *dlog2c = nullptr;
     wf_status st;
     HpTables &t = p->tab;
     if ((st = plan_alloc(p, (void **)&t.c64, nalm * sizeof(double))) != WF_OK) return st;
@@ -1530,26 +1615,53 @@ wf_status hp_build_legendre_tables(wf_plan p, const std::vector<double> &xpair, 
         WF_CUDA(cudaGetLastError());
     }
     if (f32) {
-        if ((st = plan_alloc(p, (void **)&t.A32, nalm * sizeof(float))) != WF_OK) return st;
-        if ((st = plan_alloc(p, (void **)&t.B32, nalm * sizeof(float))) != WF_OK) return st;
         if ((st = plan_alloc(p, (void **)&t.x32, np * sizeof(float))) != WF_OK) return st;
         if ((st = plan_alloc(p, (void **)&t.w32, np * sizeof(float))) != WF_OK) return st;
-        if ((st = plan_alloc(p, (void **)&t.ls_mx, ns * sizeof(int))) != WF_OK) return st;
-        if ((st = plan_alloc(p, (void **)&t.s0_mx, ns * sizeof(float))) != WF_OK) return st;
-        if ((st = plan_alloc(p, (void **)&t.s1_mx, ns * sizeof(float))) != WF_OK) return st;
-        std::vector<float> Af(nalm), Bf(nalm), xf(np), wf(np);
-        for (long long i = 0; i < nalm; ++i) {
-            Af[i] = (float)A[i];
-            Bf[i] = (float)Bm2[i];
-        }
+        if ((st = plan_alloc(p, (void **)&t.xw, np * sizeof(float4))) != WF_OK) return st;
+        if ((st = plan_alloc(p, (void **)&t.tb, nks * sizeof(float2))) != WF_OK) return st;
+        if ((st = plan_alloc(p, (void **)&t.tp, nks * sizeof(float2))) != WF_OK) return st;
+        if ((st = plan_alloc(p, (void **)&t.kd, nks * sizeof(double4))) != WF_OK) return st;
+        if ((st = plan_alloc(p, (void **)&t.Atop, (lmax + 1) * sizeof(double))) != WF_OK) return st;
+        if ((st = plan_alloc(p, (void **)&t.psum, 2 * nks * sizeof(float4))) != WF_OK) return st;
+        if ((st = plan_alloc(p, (void **)&t.k0_mx, ns * sizeof(int))) != WF_OK) return st;
+        if ((st = plan_alloc(p, (void **)&t.seed_mx, ns * sizeof(float2))) != WF_OK) return st;
+        std::vector<float> xf(np), wf(np);
+        std::vector<float4> xw(np);
         for (int i = 0; i < np; ++i) {
             xf[i] = (float)xpair[i];
             wf[i] = (float)wpair[i];
+            const float ix = i + 1 < np ? (float)(1.0 / xpair[i]) : 0.f;  // the equator's odd values vanish
+            if (i < p->nside) {
+                const double w2 = wpair[i] * (2.0 - wpair[i]);
+                const float w = (float)w2;
+                xw[i] = make_float4(w, (float)(-16.0 * (w2 - (double)w)), ix, 0.f);
+            } else {
+                const float j = (float)(np - 1 - i);
+                xw[i] = make_float4(j * j, 0.f, ix, 0.f);
+            }
         }
-        if ((st = to_device(p, t.A32, Af.data(), nalm * sizeof(float))) != WF_OK) return st;
-        if ((st = to_device(p, t.B32, Bf.data(), nalm * sizeof(float))) != WF_OK) return st;
+        WF_CUDA(cudaMemsetAsync(t.psum, 0, 2 * nks * sizeof(float4), p->stream));
         if ((st = to_device(p, t.x32, xf.data(), np * sizeof(float))) != WF_OK) return st;
         if ((st = to_device(p, t.w32, wf.data(), np * sizeof(float))) != WF_OK) return st;
+        if ((st = to_device(p, t.xw, xw.data(), np * sizeof(float4))) != WF_OK) return st;
+        if ((st = to_device(p, t.tb, tb.data(), nks * sizeof(float2))) != WF_OK) return st;
+        if ((st = to_device(p, t.tp, tp.data(), nks * sizeof(float2))) != WF_OK) return st;
+        if ((st = to_device(p, t.kd, kd.data(), nks * sizeof(double4))) != WF_OK) return st;
+        if ((st = to_device(p, t.Atop, Atop.data(), (lmax + 1) * sizeof(double))) != WF_OK) return st;
+        if (tc) {  // the tensor-core synthesis keeps the one-step forms
+            if ((st = plan_alloc(p, (void **)&t.A32, nalm * sizeof(float))) != WF_OK) return st;
+            if ((st = plan_alloc(p, (void **)&t.B32, nalm * sizeof(float))) != WF_OK) return st;
+            if ((st = plan_alloc(p, (void **)&t.ls_mx, ns * sizeof(int))) != WF_OK) return st;
+            if ((st = plan_alloc(p, (void **)&t.s0_mx, ns * sizeof(float))) != WF_OK) return st;
+            if ((st = plan_alloc(p, (void **)&t.s1_mx, ns * sizeof(float))) != WF_OK) return st;
+            std::vector<float> Af(nalm), Bf(nalm);
+            for (long long i = 0; i < nalm; ++i) {
+                Af[i] = (float)A[i];
+                Bf[i] = (float)Bm2[i];
+            }
+            if ((st = to_device(p, t.A32, Af.data(), nalm * sizeof(float))) != WF_OK) return st;
+            if ((st = to_device(p, t.B32, Bf.data(), nalm * sizeof(float))) != WF_OK) return st;
+        }
         t.lc_mx = -1;
         if ((st = hp_set_low_block(p, 0)) != WF_OK) return st;
     }
@@ -1559,9 +1671,6 @@ wf_status hp_build_legendre_tables(wf_plan p, const std::vector<double> &xpair, 
         const void *syn[] = {(const void *)k_legsyn_mx<2>, (const void *)k_legsyn_mx<4>, (const void *)k_legsyn_mx<8>};
         for (const void *f : syn)
             if ((st = raise_smem_limit(f, syn_mx_smem(lmax))) != WF_OK) return st;
-        if ((st = raise_smem_limit((const void *)k_legana_mx<2, 16>, ana_mx_smem(lmax, 16))) != WF_OK) return st;
-        if ((st = raise_smem_limit((const void *)k_legana_mx<4, 16>, ana_mx_smem(lmax, 16))) != WF_OK) return st;
-        if ((st = raise_smem_limit((const void *)k_legana_mx<8, 8>, ana_mx_smem(lmax, 8))) != WF_OK) return st;
         if ((st = raise_smem_limit((const void *)k_legsyn<double, float>, syn_smem<double>(lmax))) != WF_OK)
             return st;
         if ((st = raise_smem_limit((const void *)k_legana<double, float, 16, true>, ana_smem<double, 16>(lmax))) !=
@@ -1571,7 +1680,7 @@ wf_status hp_build_legendre_tables(wf_plan p, const std::vector<double> &xpair, 
             return st;
         if ((st = raise_smem_limit((const void *)k_lowana_df, (size_t)((np + 31) & ~31) * sizeof(float4))) != WF_OK)
             return st;
-        if (tc_prec(p->prec)) {
+        if (tc) {
             if ((st = tc_prepare(lmax)) != WF_OK) return st;
             if ((st = plan_alloc(p, (void **)&p->ws.ca32, nalm * sizeof(float2))) != WF_OK) return st;
         }
@@ -1599,8 +1708,9 @@ wf_status hp_set_low_block(wf_plan p, int lc)
     if (lc == t.lc_mx) return WF_OK;
     const long long ns = (long long)(p->lmax + 1) * p->npairs;
     const int th = 256;
-    k_restart_seeds<<<(unsigned)((ns + th - 1) / th), th, 0, p->stream>>>(p->lmax, p->npairs, lc, t.x64, t.A64, t.ls,
-                                                                        t.s0_64, t.s1_64, t.ls_mx, t.s0_mx, t.s1_mx);
+    k_restart_seeds<<<(unsigned)((ns + th - 1) / th), th, 0, p->stream>>>(
+        p->lmax, p->npairs, lc, p->nside, t.x64, t.A64, t.Atop, t.kd, t.ls, t.s0_64, t.s1_64, t.k0_mx, t.seed_mx,
+        t.ls_mx, t.s0_mx, t.s1_mx);
     WF_COUNT_LAUNCH(p);
     WF_CUDA(cudaGetLastError());
     if (lc > 0 && lc > t.glow_cap) {
@@ -1667,16 +1777,36 @@ wf_status join_aux(wf_plan p)
     return WF_OK;
 }
 
+MxTables mx_tables(wf_plan p, int L)
+{
+    const HpTables &t = p->tab;
+    return MxTables{p->lmax, L,    p->npairs, p->nside, t.lc_mx, t.k0_mx, t.seed_mx,
+                    t.xw,    t.tb, t.tp,      t.c64,    t.kd};
+}
+
+// threads of a CTA that gives one part of the ring pairs (nside of them) to 32 NP pairs per warp
+int mx_threads(wf_plan p, int np) { return std::min(LEG_THREADS, 32 * ((p->nside + 32 * np - 1) / (32 * np))); }
+
+// Ring pairs per thread or lane of one launch to band limit L.  A tile set by the user or timed by
+// wf_plan_autotune is kept; by default the largest tile that still gives min8 (8 pairs) or min4
+// (4 pairs) warps is taken.  The lines lie where the measured times cross (us, tiles 2 / 4 / 8):
+// synthesis nside 64 7 / 7 / 9, 128 8.3 / 9.9 / 11.9, 512 50 / 47 / 57, 1024 502 / 462 / 457; analysis
+// nside 256 21.8 / 20.6 / 23.1.
+constexpr int SYN_MIN_WARPS_8 = 8192, SYN_MIN_WARPS_4 = 4096, ANA_MIN_WARPS = 1824;
+int mx_tile(wf_plan p, int L, int tile, bool set, int min8, int min4)
+{
+    if (set) return tile;
+    auto warps = [&](int np) { return 2LL * (L + 1) * ((p->nside + 32 * np - 1) / (32 * np)); };
+    return warps(8) >= min8 ? 8 : warps(4) >= min4 ? 4 : 2;
+}
+
 template <int NP>
 wf_status launch_syn_mx(wf_plan p, const double2 *alm, int L)
 {
-    const HpTables &t = p->tab;
-    const int gx = (p->npairs + NP * LEG_THREADS - 1) / (NP * LEG_THREADS);
-    dim3 grid(gx, L + 1);
+    const int th = mx_threads(p, NP), gx = (p->nside + NP * th - 1) / (NP * th);
     const size_t sm = syn_mx_smem(L);
     if (wf_status st = raise_smem_limit((const void *)k_legsyn_mx<NP>, sm)) return st;
-    k_legsyn_mx<NP><<<grid, LEG_THREADS, sm, p->stream>>>(p->lmax, L, p->npairs, alm, t.A32, t.B32, t.c64, t.ls_mx,
-                                                           t.s0_mx, t.s1_mx, t.x32, t.w32, (float2 *)p->ws.G);
+    k_legsyn_mx<NP><<<dim3(gx, L + 1, 2), th, sm, p->stream>>>(mx_tables(p, L), alm, (float2 *)p->ws.G);
     WF_COUNT_LAUNCH(p);
     WF_CUDA(cudaGetLastError());
     return WF_OK;
@@ -1701,7 +1831,7 @@ wf_status hp_legendre_synthesis(wf_plan p, const double2 *alm, int L)
         float2 *G = (float2 *)p->ws.G;
         st = p->tc_deferred ? WF_OK : hp_tc_synthesis(p, 1, &alm, &p->ws.ca32, &G, &L, L, p->stream);
     } else {
-        switch (p->tile_syn) {
+        switch (mx_tile(p, L, p->tile_syn, p->tile_syn_set, SYN_MIN_WARPS_8, SYN_MIN_WARPS_4)) {
         case 2: st = launch_syn_mx<2>(p, alm, L); break;
         case 8: st = launch_syn_mx<8>(p, alm, L); break;
         default: st = launch_syn_mx<4>(p, alm, L); break;
@@ -1713,16 +1843,15 @@ wf_status hp_legendre_synthesis(wf_plan p, const double2 *alm, int L)
 }
 
 namespace {
-template <int NP, int CH>
+template <int NP>
 wf_status launch_ana_mx_t(wf_plan p, int L, LegMode mode, const BlendArgs &ba, const double2 *low,
                           const double2 *a_old, double2 *out)
 {
-    const HpTables &t = p->tab;
-    const size_t sm = ana_mx_smem(L, CH);
-    if (wf_status st = raise_smem_limit((const void *)k_legana_mx<NP, CH>, sm)) return st;
-    k_legana_mx<NP, CH><<<L + 1, LEG_THREADS, sm, p->stream>>>(
-        p->lmax, L, p->npairs, t.lc_mx, (const float2 *)p->ws.F, t.A32, t.B32, t.ls_mx, t.s0_mx, t.s1_mx, t.x32,
-        t.w32, t.c64, (int)mode, p->omega, ba, low, a_old, out, p->ws.part_harm);
+    const int ng = (p->nside + 32 * NP - 1) / (32 * NP);
+    const MxTables t = mx_tables(p, L);
+    k_legana_mx<NP><<<dim3(2 * ng, L + 1), 32, 0, p->stream>>>(t, ng, (const float2 *)p->ws.F, p->tab.psum);
+    WF_COUNT_LAUNCH(p);
+    k_ana_epilogue<<<L + 1, 128, 0, p->stream>>>(t, (int)mode, ba, low, a_old, out, p->ws.part_harm, p->tab.psum);
     WF_COUNT_LAUNCH(p);
     WF_CUDA(cudaGetLastError());
     return WF_OK;
@@ -1731,10 +1860,10 @@ wf_status launch_ana_mx_t(wf_plan p, int L, LegMode mode, const BlendArgs &ba, c
 wf_status launch_ana_mx(wf_plan p, int L, LegMode mode, const BlendArgs &ba, const double2 *low, const double2 *a_old,
                         double2 *out)
 {
-    switch (p->tile_ana) {
-    case 2: return launch_ana_mx_t<2, 16>(p, L, mode, ba, low, a_old, out);
-    case 4: return launch_ana_mx_t<4, 16>(p, L, mode, ba, low, a_old, out);
-    default: return launch_ana_mx_t<8, 8>(p, L, mode, ba, low, a_old, out);
+    switch (mx_tile(p, L, p->tile_ana, p->tile_ana_set, ANA_MIN_WARPS, ANA_MIN_WARPS)) {
+    case 2: return launch_ana_mx_t<2>(p, L, mode, ba, low, a_old, out);
+    case 4: return launch_ana_mx_t<4>(p, L, mode, ba, low, a_old, out);
+    default: return launch_ana_mx_t<8>(p, L, mode, ba, low, a_old, out);
     }
 }
 }  // namespace
@@ -1753,6 +1882,8 @@ wf_status hp_autotune(wf_plan p, int reps)
     WF_CUDA(cudaEventCreate(&e0));
     WF_CUDA(cudaEventCreate(&e1));
     const int saved_syn = p->tile_syn, saved_ana = p->tile_ana;
+    const bool set_syn = p->tile_syn_set, set_ana = p->tile_ana_set;
+    p->tile_syn_set = p->tile_ana_set = true;
     const int np[3] = {2, 4, 8};
     float best_syn = 1e30f, best_ana = 1e30f;
     int pick_syn = saved_syn, pick_ana = saved_ana;
@@ -1783,6 +1914,10 @@ wf_status hp_autotune(wf_plan p, int reps)
     cudaEventDestroy(e1);
     p->tile_syn = st == WF_OK ? pick_syn : saved_syn;
     p->tile_ana = st == WF_OK ? pick_ana : saved_ana;
+    if (st != WF_OK) {
+        p->tile_syn_set = set_syn;
+        p->tile_ana_set = set_ana;
+    }
     return st;
 }
 
@@ -1791,9 +1926,11 @@ wf_status hp_legendre_analysis(wf_plan p, int L, LegMode mode, const BlendArgs &
 {
     const HpTables &t = p->tab;
     BlendArgs ba = ba_in;
-    if (mode == LEG_BLEND) {
-        k_epi_table<<<(p->lmax + 256) / 256, 256, 0, p->stream>>>(p->lmax, ba.S, p->omega, ba.lam_tauh, ba.tauh,
-                                                                  p->ws.epi);
+    if (mode == LEG_BLEND && ba.epi_ready) {
+        ba.epi = p->ws.epi;  // the ring pass of this iteration has filled it
+    } else if (mode == LEG_BLEND) {
+        k_epi_table<<<(p->lmax + 256) / 256, 256, 0, p->stream>>>(
+            EpiArgs{p->lmax, ba.S, p->omega, ba.lam_tauh, ba.tauh, p->ws.epi});
         WF_COUNT_LAUNCH(p);
         WF_CUDA(cudaGetLastError());
         ba.epi = p->ws.epi;

@@ -461,6 +461,8 @@ template <typename T> struct RingArgs {
     const T *amap;         // RS_ANA input
     double *part;          // per ring pair: chi^2 pixel term
     cx<T> *F;              // analysis output
+    int npairs;
+    EpiArgs epi;           // messenger step: CTAs past the pairs fill the blend table of the analysis
 };
 
 constexpr int RS_ANA = 16;  // analysis only (beside RingSynMode)
@@ -624,6 +626,10 @@ __global__ void __launch_bounds__(RING_CTA, MINB) k_ring(const RingArgs<T> A)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ double red[RING_CTA / 32];
+    if ((int)blockIdx.x >= A.npairs) {  // (a launch of its own costs 3.5 us an iteration)
+        epi_entry(A.epi, (blockIdx.x - A.npairs) * RING_CTA + threadIdx.x);
+        return;
+    }
     cx<T> *zb = reinterpret_cast<cx<T> *>(smem_raw), *ex = zb + A.zlen;
     const int pair = A.order[blockIdx.x], mode = A.mode;
     const RingTab R = A.rings[pair];
@@ -732,6 +738,7 @@ template <typename T> struct RingLaunch {
         a.chirp = (const cx<T> *)t.chirp;
         a.tw = (const cx<T> *)t.tw;
         a.zlen = (int)padded_len(t.nmax);
+        a.npairs = p->npairs;
         a.mode = mode;
         return a;
     }
@@ -741,7 +748,8 @@ template <typename T> struct RingLaunch {
         auto kernel = k_ring<T, 2>;
         if constexpr (sizeof(T) == 4)
             if (p->tab.ring_ctas == 3) kernel = k_ring<T, 3>;
-        kernel<<<p->npairs, RING_CTA, sm, p->stream>>>(a);
+        const int extra = a.epi.epi ? (a.epi.lmax + RING_CTA) / RING_CTA : 0;
+        kernel<<<p->npairs + extra, RING_CTA, sm, p->stream>>>(a);
         WF_COUNT_LAUNCH(p);
         WF_CUDA(cudaGetLastError());
         return WF_OK;
@@ -762,9 +770,10 @@ template <typename T> struct RingLaunch {
     // glow_stride columns per pair) added to G, or none (glow null)
     static wf_status syn_buf_low(wf_plan p, int L, RingSynMode mode, double lam, double tau, const void *G,
                                  const float2 *glow, int lc, int glow_stride, void *tmap, double *omap,
-                                 void *F = nullptr)
+                                 void *F = nullptr, const EpiArgs *epi = nullptr)
     {
         RingArgs<T> a = args(p, L, (int)mode);
+        if (epi) a.epi = *epi;
         if (glow && lc > 0) {
             a.Glow = glow;
             a.lc = lc;
@@ -782,13 +791,13 @@ template <typename T> struct RingLaunch {
         return launch(p, a);
     }
     // messenger step on the rings: fold, inverse DFT, Eq. 3, forward DFT, unfold into F
-    static wf_status syn_ana(wf_plan p, int L, double lam, double tau)
+    static wf_status syn_ana(wf_plan p, int L, double lam, double tau, const EpiArgs &epi)
     {
         const HpTables &t = p->tab;
         if (p->prec != WF_PREC_FP64 && t.lc_mx > 0)
             return syn_buf_low(p, L, RS_BLEND_ANA, lam, tau, p->ws.G, p->ws.Glow, t.lc_mx, t.glow_cap, nullptr,
-                               nullptr, p->ws.F);
-        return syn_buf_low(p, L, RS_BLEND_ANA, lam, tau, p->ws.G, nullptr, 0, 0, nullptr, nullptr, p->ws.F);
+                               nullptr, p->ws.F, &epi);
+        return syn_buf_low(p, L, RS_BLEND_ANA, lam, tau, p->ws.G, nullptr, 0, 0, nullptr, nullptr, p->ws.F, &epi);
     }
     static wf_status ana(wf_plan p, int L, const void *map) { return ana_buf(p, L, map, p->ws.F); }
     static wf_status ana_buf(wf_plan p, int L, const void *map, void *F)
@@ -964,10 +973,10 @@ wf_status hp_ring_synthesis(wf_plan p, int L, RingSynMode mode, double lam, doub
                                    : RingLaunch<float>::syn(p, L, mode, lam, tau, out_map);
 }
 
-wf_status hp_ring_synthesis_analysis(wf_plan p, int L, double lam, double tau)
+wf_status hp_ring_synthesis_analysis(wf_plan p, int L, double lam, double tau, const EpiArgs &epi)
 {
-    return p->prec == WF_PREC_FP64 ? RingLaunch<double>::syn_ana(p, L, lam, tau)
-                                   : RingLaunch<float>::syn_ana(p, L, lam, tau);
+    return p->prec == WF_PREC_FP64 ? RingLaunch<double>::syn_ana(p, L, lam, tau, epi)
+                                   : RingLaunch<float>::syn_ana(p, L, lam, tau, epi);
 }
 
 wf_status hp_ring_synthesis_buf(wf_plan p, int L, RingSynMode mode, double lam, double tau, const void *G,
