@@ -330,7 +330,7 @@ wf_status wf_probe_fp32_fma(void *cuda_stream, int packed, double *tflops);
  * counterpart; it exists for callers that cannot allocate at solve time (a
  * solve inside another framework's memory pool, or where cudaMalloc is not
  * allowed).  Same arithmetic and results as wf_solve on a flat plan of the
- * same n, with the solver's scratch in one static device array (0.71 MiB,
+ * same n, with the solver's scratch in one static device array (0.97 MiB,
  * resident on every device that loads the library) instead of plan memory.
  * n: power of two in [16, 128]; opt: may be NULL (defaults), opt->maxiter <=
  * 20000; anything larger is rejected with WF_EINVAL.  d, noise_var, mask, S,

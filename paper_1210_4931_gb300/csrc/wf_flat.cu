@@ -2,52 +2,50 @@
 // unitary 2-D DFT (the "e.g. Fourier space" basis of Sect. 2.1).
 //
 // The whole solve -- every iteration of Eqs. (3)-(4), the chi^2 of Eq. (6),
-// the residual and the cooling schedule -- runs in ONE persistent launch of a
-// single thread-block cluster of CS CTAs (CS = 16 where the device co-schedules
-// that non-portable size, else 8; flat_cluster_size).  The grid never leaves the
-// cluster's shared memory:
-//   CTA c owns pixel rows [c n/CS, (c+1) n/CS) (source r, inverse noise nu)
-//   and spectrum columns kx in [c P, (c+1) P), P = ceil((n/2+1)/CS) (a, S).
-// One iteration:
-//   1. column inverse FFTs (ky) of the owned a columns          (local)
-//   2. cluster barrier; each CTA gathers its rows' spectra from every CTA's
-//      column buffer through distributed shared memory, c2r FFTs the rows,
-//      applies the pixel blend of Eq. (3) and r2c FFTs the result
-//   3. cluster barrier; each CTA gathers its columns from every CTA's row
-//      buffer, forward FFTs them (ky) and applies the harmonic blend of
-//      Eq. (4), accumulating chi^2 and the lambda = 1 residual
-//   4. cluster barrier; every CTA sums all CTAs' partials in the same order
-//      and takes the same schedule decision (no broadcast needed).
-// FFTs are radix-2, one warp per row/column, in shared memory.
-#include <cooperative_groups.h>
-
+// the residual and the cooling schedule -- runs in ONE cooperative launch of
+// n/2 + 1 CTAs of n threads.  CTA c owns spectrum column kx = c and (c < n/2)
+// the pixel rows 2c, 2c + 1; thread t keeps one mode (a, and the factors of
+// Eq. 4) and two pixels (r, nu, the factors of Eq. 3) in registers for the whole
+// solve.  One iteration:
+//   1. inverse FFT (ky) of the column, written to global memory (L2)
+//   2. grid barrier; every CTA sums all CTAs' partials of the previous iteration in
+//      the same order and takes the same schedule decision; inverse FFT of its
+//      two rows (packed, below), the pixel blend of Eq. (3), forward FFT
+//   3. grid barrier; forward FFT (ky) of the column, the harmonic blend of Eq. (4)
+//      with its chi^2 and lambda = 1 residual sums.
+// Two real rows go through one complex FFT: the inverse DFT of Xa + i Xb (both
+// Hermitian) is xa + i xb, and the forward DFT Z of ta + i tb gives
+// Ta = (Z_k + conj Z_-k) / 2 and Tb = (Z_k - conj Z_-k) / 2i.
+//
+// What bounds it: FP64 runs at 1/64 of the FP32 rate (a warp instruction takes 64 cycles
+// of its scheduler's FP64 unit), so an iteration wants many SMs: one FFT per SM, one
+// value per thread on all four schedulers, 32 FP64 operations per thread and FFT.  The
+// rest is two grid barriers and their exchanges through L2.  A cluster of 16 CTAs (the
+// largest) with four to five FFTs each in one warp took 42.5 us per iteration of the
+// 128 x 128 grid, 18 to 21 us of it FP64 issue, three cluster barriers;
+// this kernel takes 14.2 us (4.25 ms for 300 iterations against 12.6), and 11.3 against 18.5 us on
+// the 32 x 32 grid, where both are bound by the barriers.
 #include <algorithm>
-#include <mutex>
 #include <cmath>
 #include <cstdio>
 #include <vector>
 
 #include "wf_internal.cuh"
 
-namespace cg = cooperative_groups;
-
 namespace wf {
 
-constexpr int FLAT_CS = 8;      // portable cluster size; the smallest the solve runs on
-constexpr int FLAT_CS_MAX = 16; // non-portable cluster size, used where the device co-schedules it
-constexpr int FLAT_THREADS = 256;
-constexpr int FLAT_WARPS = FLAT_THREADS / 32;
 constexpr int FLAT_MAXN = 128;
+constexpr int FLAT_NP = 2;  // partial sums per CTA: chi^2, residual^2
 
 struct FlatStatus {
-    int iters, converged, levels, stop_reason;  // stop_reason: 0 schedule/replay end, 1 converged, 2 maxiter, 3 diverged
+    int iters, converged, levels, stop_reason;  // 0 schedule/replay end, 1 converged, 2 maxiter, 3 diverged, 4 barrier gave up
     double final_resid, chi2_final, bnorm;
 };
 
 struct FlatPlan {
-    int n = 0, logn = 0, nh = 0, P = 0, RP = 0, cs = 8;
-    size_t smem = 0;
+    int n = 0, nh = 0;
     double *r = nullptr, *nu = nullptr;  // device pixel maps
+    double2 *xch = nullptr;              // FlatScratch of the launch
     double *levels = nullptr;            // device lambda levels
     double *tr_lam = nullptr, *tr_chi2 = nullptr, *tr_res = nullptr;
     int tr_cap = 0;
@@ -58,8 +56,15 @@ struct FlatPlan {
 
 namespace {
 
+// exchange buffers (column layout, [kx][y]), two generations of partial sums, barrier counter
+inline size_t flat_scratch_bytes(int n)
+{
+    const size_t nh = n / 2 + 1;
+    return 2 * nh * n * sizeof(double2) + 2 * nh * FLAT_NP * sizeof(double) + 256;
+}
+
 struct FlatArgs {
-    int n, logn, nh, P, RP;
+    int n, nh;
     const double *r, *nu, *S;
     const double *g1;      // fluct: unit draws in pixel space (or null)
     const double2 *g2;     // fluct: unit harmonic draws (or null)
@@ -74,387 +79,357 @@ struct FlatArgs {
     double *tr_lam, *tr_chi2, *tr_res;
     int tr_cap;
     FlatStatus *status;
+    double2 *x1, *x2;      // columns after step 1, row spectra after step 2
+    double *part;
+    unsigned *bar;         // zero at launch
 };
 
-__device__ __forceinline__ double2 dmul(double2 a, double2 b) { return cmul(a, b); }
-
-// radix-2 DIT FFT of length 2^logn on x (shared memory) by one warp
-__device__ void warp_fft(double2 *x, int logn, int sign, const double2 *tw /* e^{-2 pi i t / n}, t < n/2 */)
+void flat_set_scratch(FlatArgs &A, void *base, int n)
 {
-    const int n = 1 << logn, lane = threadIdx.x & 31;
-    for (int i = lane; i < n; i += 32) {
-        const int j = (int)(__brev((unsigned)i) >> (32 - logn));
-        if (i < j) {
-            const double2 t = x[i];
-            x[i] = x[j];
-            x[j] = t;
-        }
-    }
-    __syncwarp();
-    for (int s = 1; s <= logn; ++s) {
-        const int half = 1 << (s - 1);
-        for (int b = lane; b < n / 2; b += 32) {
-            const int pos = b & (half - 1);
-            const int i0 = ((b >> (s - 1)) << s) + pos, i1 = i0 + half;
-            double2 w = tw[pos << (logn - s)];
-            if (sign > 0) w.y = -w.y;
-            const double2 u = x[i0], v = dmul(x[i1], w);
-            x[i0] = cadd(u, v);
-            x[i1] = csub(u, v);
-        }
-        __syncwarp();
-    }
+    const size_t nh = n / 2 + 1;
+    A.x1 = (double2 *)base;
+    A.x2 = A.x1 + nh * n;
+    A.part = (double *)(A.x2 + nh * n);
+    A.bar = (unsigned *)(A.part + 2 * nh * FLAT_NP);
 }
 
-enum FlatStep { FS_ITER = 0, FS_PROLOGUE = 1, FS_FLUCT_SRC = 2, FS_OUT = 3 };
-
-// dynamic shared memory of k_flat_solve: twiddles; a, column and row buffers; per-warp FFT
-// rows; S, 1/S and S / (S + lam tau) per owned mode; r, nu and 1 / (1 + (lam - 1) tau nu)
-// per owned pixel
-inline size_t flat_smem(int n, int P, int RP, int nh)
+__device__ __forceinline__ double flip(double v, bool neg)
 {
-    return (size_t)(n / 2) * 16 + (size_t)P * n * 16 * 2 + (size_t)RP * nh * 16 + (size_t)FLAT_WARPS * n * 16 +
-           (size_t)P * n * 8 * 3 + (size_t)RP * n * 8 * 3;
+    return __hiloint2double(__double2hiint(v) ^ (neg ? 0x80000000 : 0), __double2loint(v));
 }
 
-__global__ void __launch_bounds__(FLAT_THREADS) k_flat_solve(FlatArgs A)
+// FFT of length n = 2^logn over the CTA's first n threads, one value per thread, natural order in
+// and out (Stockham, decimation in frequency: radix 4, a last radix 2 where logn is odd; thread t
+// computes output t of every pass, six additions and one twiddle product).  sign -1:
+// e^{-2 pi i jk/n}, +1: conjugated.  buf: 2 n entries, used alternately, so one barrier a pass.
+__device__ double2 cta_fft(double2 v, int n, int sign, double2 *buf, const double2 *tw /* e^{-2 pi i j / n} */)
 {
-    cg::cluster_group cluster = cg::this_cluster();
-    const int c = (int)cluster.block_rank();
-    const int n = A.n, nh = A.nh, P = A.P, RP = A.RP, logn = A.logn;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int c0 = c * P;
-    const double inv_tau = 1.0 / A.tau;
-    const int ncol = max(0, min(nh, c0 + P) - c0);
-    const int y0 = c * RP;
-    const double sy = rsqrt((double)n), sx = rsqrt((double)n);
-
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    double2 *tw = reinterpret_cast<double2 *>(smem_raw);            // n/2
-    double2 *acol = tw + n / 2;                                      // P * n
-    double2 *colbuf = acol + (size_t)P * n;                          // P * n
-    double2 *rowbuf = colbuf + (size_t)P * n;                        // RP * nh
-    double2 *wscr = rowbuf + (size_t)RP * nh;                        // FLAT_WARPS * n
-    double *Scol = reinterpret_cast<double *>(wscr + (size_t)FLAT_WARPS * n);  // P * n
-    double *rpix = Scol + (size_t)P * n;                             // RP * n
-    double *nupix = rpix + (size_t)RP * n;                           // RP * n
-    double *invden = nupix + (size_t)RP * n;                         // RP * n: 1 / (1 + (lam - 1) tau nu)
-    double *Sinv = invden + (size_t)RP * n;                          // P * n: 1 / S (0 where S = 0)
-    double *fcol = Sinv + (size_t)P * n;                             // P * n: S / (S + lam tau)
-    __shared__ double part[4];   // pix chi2, harm chi2, resid^2, spare
-    __shared__ double red[FLAT_WARPS][3];
-
-    for (int t = tid; t < n / 2; t += blockDim.x) {
-        double s, co;
-        sincospi(-2.0 * t / n, &s, &co);
-        tw[t] = make_double2(co, s);
+    const int t = threadIdx.x;
+    int s = 1, nc = n;  // stride, remaining length
+    double2 *cur = buf, *nxt = buf + n;
+    while (nc > 1) {
+        if (t < n) cur[t] = v;
+        __syncthreads();
+        if (t < n) {
+            const int q = t & (s - 1), u = t / s;
+            if (nc == 2) {
+                const double2 x0 = cur[q], x1 = cur[q + s];
+                v = make_double2(x0.x + flip(x1.x, u & 1), x0.y + flip(x1.y, u & 1));
+            } else {
+                const int m = nc >> 2, r = u & 3, p = u >> 2, i0 = q + s * p, st = s * m;
+                const double2 x0 = cur[i0], x1 = cur[i0 + st], x2 = cur[i0 + 2 * st], x3 = cur[i0 + 3 * st];
+                const bool odd = r & 1;
+                const double ax = x0.x + flip(x2.x, odd), ay = x0.y + flip(x2.y, odd);
+                const double bx = x1.x + flip(x3.x, odd), by = x1.y + flip(x3.y, odd);
+                // b (sign i)^r: r = 2 negates; r odd swaps, one part negated
+                const bool pos = sign > 0;
+                const double rx = odd ? flip(by, (r == 1) == pos) : flip(bx, r == 2);
+                const double ry = odd ? flip(bx, (r == 3) == pos) : flip(by, r == 2);
+                v = make_double2(ax + rx, ay + ry);
+                if (m > 1) {
+                    double2 w = tw[p * r * s];
+                    w.y = flip(w.y, pos);
+                    v = cmul(v, w);
+                }
+            }
+        }
+        const int R = nc == 2 ? 2 : 4;
+        s *= R;
+        nc /= R;
+        double2 *x = cur;
+        cur = nxt;
+        nxt = x;
     }
-    for (int i = tid; i < P * n; i += blockDim.x) {
-        const int kl = i / n, ky = i % n;
-        const int kx = c0 + kl;
-        acol[i] = make_double2(0.0, 0.0);
-        const double S = (kl < ncol) ? A.S[(size_t)ky * nh + kx] : 0.0;
-        Scol[i] = S;
-        Sinv[i] = S > 0.0 ? 1.0 / S : 0.0;
+    __syncthreads();  // the buffers are free
+    return v;
+}
+
+// sum over a warp, in every lane (same order always)
+__device__ __forceinline__ double warp_sum(double v)
+{
+    for (int o = 16; o >= 1; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+constexpr int FLAT_MAX_POLLS = 1 << 22;  // seconds; the launch is cooperative, so a barrier takes microseconds
+
+// all CTAs have arrived (and their global writes are visible) when it returns true; false, in every
+// thread of the CTA, when the wait gave up
+__device__ __forceinline__ bool grid_barrier(unsigned *bar, unsigned target, int *ok)
+{
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        // (release and acquire carry the CTA's other threads' accesses through the CTA barriers)
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
+        unsigned v = 0;
+        int polls = 0;
+        do {
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
+        } while ((int)(v - target) < 0 && ++polls < FLAT_MAX_POLLS);  // (the count may wrap)
+        *ok = (int)(v - target) >= 0;
     }
-    for (int i = tid; i < RP * n; i += blockDim.x) {
-        const size_t g = (size_t)y0 * n + i;
-        rpix[i] = A.r[g];
-        nupix[i] = A.nu[g];
+    __syncthreads();
+    return *ok != 0;
+}
+
+__global__ void __launch_bounds__(FLAT_MAXN) k_flat_solve(const FlatArgs A)
+{
+    __shared__ double2 buf[2 * FLAT_MAXN], tw[FLAT_MAXN];
+    __shared__ double red[FLAT_MAXN / 32][FLAT_NP];
+    __shared__ int ok;
+    const int n = A.n, nh = A.nh, c = blockIdx.x, t = threadIdx.x;
+    const bool mode = t < n, row = mode && c < n / 2;
+    const int ya = 2 * c, yb = 2 * c + 1;
+    const double inv_tau = 1.0 / A.tau, dn = (double)n, wk = (c == 0 || 2 * c == n) ? 1.0 : 2.0;
+    unsigned arrivals = 0;
+    for (int i = t; i < n; i += blockDim.x) {
+        double sn, cs;
+        sincospi(-2.0 * i / n, &sn, &cs);
+        tw[i] = make_double2(cs, sn);
+    }
+    // this thread's mode (ky = t, kx = c); a is kept over n, so that neither FFT needs its 1/n
+    const double S = mode ? A.S[(size_t)t * nh + c] : 0.0;
+    const double si = S > 0.0 ? dn * dn / S : 0.0;                     // chi^2 of a: |a / n|^2 n^2 / S
+    const double kr = S > 0.0 ? dn * (1.0 / S + inv_tau) : 0.0;        // residual
+    double2 a = make_double2(0.0, 0.0);
+    double f = 0.0;                                                    // S / (S + lam tau) / (2 n^2)
+    // its two pixels (rows ya, yb; x = t)
+    double ra = 0.0, rb = 0.0, na = 0.0, nb = 0.0, ia = 1.0, ib = 1.0;  // r, nu, 1 / (1 + (lam - 1) tau nu)
+    double la = 0.0, lb = 0.0;                                          // lam tau ia, lam tau ib
+    if (row) {
+        ra = A.r[(size_t)ya * n + t];
+        rb = A.r[(size_t)yb * n + t];
+        na = A.nu[(size_t)ya * n + t];
+        nb = A.nu[(size_t)yb * n + t];
     }
     __syncthreads();
 
-    // the per-pixel and per-mode factors of Eqs. (3) and (4) for one lambda (FP64 divisions
-    // once per cooling level, not once per iteration)
-    double cur_lam = NAN;
-    auto set_level = [&](double lam) {
-        const double lm1t = (lam - 1.0) * A.tau, lt = lam * A.tau;
-        for (int i = tid; i < RP * n; i += blockDim.x) invden[i] = 1.0 / (1.0 + lm1t * nupix[i]);
-        for (int i = tid; i < P * n; i += blockDim.x) {
-            const double S = Scol[i];
-            fcol[i] = S > 0.0 ? S / (S + lt) : 0.0;
+    auto barrier = [&]() {
+        arrivals += gridDim.x;
+        return grid_barrier(A.bar, arrivals, &ok);
+    };
+    // step 1: the column's inverse FFT of v into x1
+    auto columns_out = [&](double2 v) {
+        v = cta_fft(v, n, +1, buf, tw);
+        if (mode) __stcg(A.x1 + (size_t)c * n + t, v);
+    };
+    // row spectra from x1: this thread's entry of the packed inverse FFT
+    auto rows_load = [&]() {
+        double2 z = make_double2(0.0, 0.0);
+        if (row) {
+            const bool up = t >= nh;
+            const double2 *x = A.x1 + (size_t)(up ? n - t : t) * n + ya;
+            const double2 va = __ldcg(x), vb = __ldcg(x + 1);
+            z = make_double2(va.x - flip(vb.y, up), flip(va.y, up) + vb.x);
         }
-        cur_lam = lam;
+        return z;
+    };
+    auto rows_in = [&](double2 z) { return c < n / 2 ? cta_fft(z, n, +1, buf, tw) : z; };
+    // rows to x2: twice the forward FFTs of the pixel values ta, tb
+    auto rows_out = [&](double ta, double tb) {
+        if (c >= n / 2) return;
+        const double2 z = cta_fft(make_double2(ta, tb), n, -1, buf, tw);
+        if (mode) buf[t] = z;
+        __syncthreads();
+        if (t < nh) {
+            const double2 y = buf[(n - t) & (n - 1)];  // conj Z_-k = (y.x, -y.y)
+            double2 *x = A.x2 + (size_t)t * n + ya;
+            __stcg(x, make_double2(z.x + y.x, z.y - y.y));
+            __stcg(x + 1, make_double2(z.y + y.y, y.x - z.x));
+        }
         __syncthreads();
     };
-
-    auto block_reduce3 = [&](double a, double b, double d) {
-        for (int o = 16; o >= 1; o >>= 1) {
-            a += __shfl_xor_sync(0xffffffffu, a, o);
-            b += __shfl_xor_sync(0xffffffffu, b, o);
-            d += __shfl_xor_sync(0xffffffffu, d, o);
-        }
-        if (lane == 0) { red[warp][0] = a; red[warp][1] = b; red[warp][2] = d; }
-        __syncthreads();
-        if (tid == 0) {
-            double s0 = 0, s1 = 0, s2 = 0;
-            for (int w = 0; w < FLAT_WARPS; ++w) { s0 += red[w][0]; s1 += red[w][1]; s2 += red[w][2]; }
-            part[0] = s0; part[1] = s1; part[2] = s2;
-        }
-        __syncthreads();
+    // column from x2: 2 n times this thread's mode of the pixel values
+    auto columns_in = [&]() {
+        const double2 v = mode ? __ldcg(A.x2 + (size_t)c * n + t) : make_double2(0.0, 0.0);
+        return cta_fft(v, n, -1, buf, tw);
     };
-
-    // ---- step 1: inverse column FFTs of acol into colbuf ----
-    auto step1 = [&]() {
-        for (int kl = warp; kl < ncol; kl += FLAT_WARPS) {
-            double2 *x = colbuf + (size_t)kl * n;
-            for (int ky = lane; ky < n; ky += 32) x[ky] = acol[(size_t)kl * n + ky];
-            __syncwarp();
-            warp_fft(x, logn, +1, tw);
-            for (int y = lane; y < n; y += 32) x[y] = cscale(x[y], sy);
-            __syncwarp();
-        }
-    };
-
-    // ---- step 2: rows: gather, c2r, blend (or other use), r2c into rowbuf ----
-    // Two real rows per complex FFT: the inverse DFT of Xa + i Xb (both Hermitian) is
-    // xa + i xb, and the forward DFT Z of ta + i tb gives Ta = (Z_k + conj Z_-k) / 2 and
-    // Tb = (Z_k - conj Z_-k) / 2i.
-    auto step2 = [&](int mode, double lam) -> double {
-        for (int i = tid; i < RP * nh; i += blockDim.x) {
-            const int yl = i / nh, kx = i % nh;
-            const int o = kx / P, kl = kx - o * P;
-            const double2 *rc = cluster.map_shared_rank(colbuf, o);
-            rowbuf[(size_t)yl * nh + kx] = rc[(size_t)kl * n + (y0 + yl)];
+    // partial sums: written before a barrier, read after it; generations alternate.  Every warp
+    // adds all CTAs' partials itself.
+    auto put_part = [&](int gen, double p0, double p1) {
+        p0 = warp_sum(p0);
+        p1 = warp_sum(p1);
+        if ((t & 31) == 0) {
+            red[t >> 5][0] = p0;
+            red[t >> 5][1] = p1;
         }
         __syncthreads();
-        const double lt = lam * A.tau;
-        double acc = 0.0;
-        double2 *x = wscr + (size_t)warp * n;
-        for (int yp = warp; 2 * yp < RP; yp += FLAT_WARPS) {
-            const int ya = 2 * yp;
-            double2 *ba = rowbuf + (size_t)ya * nh, *bb = ba + nh;
-            for (int kx = lane; kx < n; kx += 32) {
-                double2 va, vb;
-                if (kx < nh) {
-                    va = ba[kx];
-                    vb = bb[kx];
-                } else {
-                    va = cconj(ba[n - kx]);
-                    vb = cconj(bb[n - kx]);
-                }
-                x[kx] = make_double2(va.x - vb.y, va.y + vb.x);
-            }
-            __syncwarp();
-            warp_fft(x, logn, +1, tw);  // real part: row ya, imaginary part: row ya + 1
-            for (int xx = lane; xx < n; xx += 32) {
-                double tt[2];
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const double s = (h ? x[xx].y : x[xx].x) * sx;
-                    const int pi = (ya + h) * n + xx;
-                    double t = s;
-                    if (mode == FS_ITER) {
-                        const double nv = nupix[pi], rv = rpix[pi], id = invden[pi];
-                        t = s + lt * (rv - nv * s) * id;
-                        acc += (nv * s * s - 2.0 * rv * s) * id;
-                    } else if (mode == FS_PROLOGUE) {
-                        t = rpix[pi];
-                    } else if (mode == FS_FLUCT_SRC) {
-                        const double rv = sqrt(nupix[pi]) * A.g1[(size_t)y0 * n + pi] + s;
-                        rpix[pi] = rv;
-                        t = rv;
-                    } else {  // FS_OUT
-                        A.s_out[(size_t)y0 * n + pi] = s;
-                        const double nv = nupix[pi];
-                        if (nv > 0.0) {
-                            const double e = rpix[pi] - nv * s;
-                            acc += e * e / nv;  // nu (d - s)^2
-                        }
-                    }
-                    tt[h] = t;
-                }
-                x[xx] = make_double2(tt[0], tt[1]);
-            }
-            __syncwarp();
-            if (mode == FS_ITER || mode == FS_PROLOGUE) {
-                warp_fft(x, logn, -1, tw);
-                for (int kx = lane; kx < nh; kx += 32) {
-                    const double2 z = x[kx], zc = cconj(x[(n - kx) & (n - 1)]);
-                    const double2 d = make_double2(0.5 * (z.x - zc.x), 0.5 * (z.y - zc.y));
-                    ba[kx] = cscale(make_double2(0.5 * (z.x + zc.x), 0.5 * (z.y + zc.y)), sx);
-                    bb[kx] = cscale(make_double2(d.y, -d.x), sx);
-                }
-            }
-            __syncwarp();
-        }
-        return acc;
-    };
-
-    // ---- step 3: columns: gather, forward FFT, harmonic blend ----
-    // mode FS_ITER: a = S/(S + lam tau) t_hat; chi2 of a_old; residual if lam == 1
-    // mode FS_PROLOGUE: accumulate |t_hat|^2 (the b norm), a untouched
-    auto step3 = [&](int mode, double lam, double &chi2h, double &res2) {
-        for (int i = tid; i < ncol * n; i += blockDim.x) {
-            const int kl = i / n, y = i % n;
-            const int o = y / RP, yl = y - o * RP;
-            const double2 *rb = cluster.map_shared_rank(rowbuf, o);
-            colbuf[i] = rb[(size_t)yl * nh + (c0 + kl)];
-        }
-        __syncthreads();
-        const bool full = (lam == 1.0);
-        for (int kl = warp; kl < ncol; kl += FLAT_WARPS) {
-            double2 *x = colbuf + (size_t)kl * n;
-            warp_fft(x, logn, -1, tw);
-            const int kx = c0 + kl;
-            const double w = (kx == 0 || 2 * kx == n) ? 1.0 : 2.0;
-            for (int ky = lane; ky < n; ky += 32) {
-                const double2 th = cscale(x[ky], sy);
-                const double S = Scol[(size_t)kl * n + ky];
-                if (mode == FS_PROLOGUE) {
-                    if (S > 0.0) res2 += w * (th.x * th.x + th.y * th.y);
-                    continue;
-                }
-                const double2 ao = acol[(size_t)kl * n + ky];
-                double2 an = make_double2(0.0, 0.0);
-                if (S > 0.0) {
-                    const double si = Sinv[(size_t)kl * n + ky];
-                    an = cscale(th, fcol[(size_t)kl * n + ky]);
-                    chi2h += w * (ao.x * ao.x + ao.y * ao.y) * si;
-                    if (full) {
-                        const double k = si + inv_tau;
-                        const double dx = k * (ao.x - an.x), dy = k * (ao.y - an.y);
-                        res2 += w * (dx * dx + dy * dy);
-                    }
-                }
-                acol[(size_t)kl * n + ky] = an;
-            }
-            __syncwarp();
+        if (t < FLAT_NP) {
+            double q = red[0][t];
+            for (int i = 1; i < (int)(blockDim.x >> 5); ++i) q += red[i][t];
+            __stcg(A.part + ((size_t)(gen & 1) * nh + c) * FLAT_NP + t, q);
         }
     };
-
-    // sum partial triplets over the cluster (same order in every CTA)
-    auto cluster_sum = [&](double out[3]) {
-        out[0] = out[1] = out[2] = 0.0;
-        for (int o = 0; o < (int)cluster.num_blocks(); ++o) {
-            const double *pp = cluster.map_shared_rank(part, o);
-            out[0] += pp[0];
-            out[1] += pp[1];
-            out[2] += pp[2];
+    auto load_part = [&](int gen) {
+        double2 q = make_double2(0.0, 0.0);
+        const double2 *x = reinterpret_cast<const double2 *>(A.part) + (size_t)(gen & 1) * nh;
+        for (int i = t & 31; i < nh; i += 32) {
+            const double2 v = __ldcg(x + i);
+            q.x += v.x;
+            q.y += v.y;
         }
+        return q;
+    };
+    auto gave_up = [&]() {
+        if (t == 0) A.status->stop_reason = 4;
     };
 
-    double tot[3];
+    double2 tot;
     // ---- fluctuation source: r = nu^1/2 g1 + F^-1 (S^-1/2 g2) ----
     if (A.g1) {
-        for (int i = tid; i < ncol * n; i += blockDim.x) {
-            const int kl = i / n, ky = i % n;
-            const double S = Scol[i];
-            const double f = S > 0.0 ? rsqrt(S) : 0.0;
-            acol[i] = cscale(A.g2[(size_t)ky * nh + c0 + kl], f);
+        double2 v = make_double2(0.0, 0.0);
+        if (mode && S > 0.0) v = cscale(A.g2[(size_t)t * nh + c], rsqrt(S) / dn);
+        columns_out(v);
+        if (!barrier()) return gave_up();
+        const double2 s = rows_in(rows_load());
+        if (row) {
+            ra = sqrt(na) * A.g1[(size_t)ya * n + t] + s.x;
+            rb = sqrt(nb) * A.g1[(size_t)yb * n + t] + s.y;
         }
-        __syncthreads();
-        step1();
-        cluster.sync();
-        step2(FS_FLUCT_SRC, 1.0);
-        __syncthreads();
-        for (int i = tid; i < P * n; i += blockDim.x) acol[i] = make_double2(0.0, 0.0);
-        cluster.sync();
     }
     // ---- prologue: |b| = |F r| ----
+    rows_out(ra, rb);
+    if (!barrier()) return gave_up();
     {
-        step2(FS_PROLOGUE, 1.0);
-        cluster.sync();
-        double ch = 0.0, rs = 0.0;
-        step3(FS_PROLOGUE, 1.0, ch, rs);
-        block_reduce3(0.0, 0.0, rs);
-        cluster.sync();
-        cluster_sum(tot);
+        const double2 v = columns_in();
+        const double b2 = S > 0.0 ? wk * (v.x * v.x + v.y * v.y) : 0.0;
+        put_part(1, 0.0, b2);
     }
-    const double bnorm = sqrt(tot[2]);
-    cluster.sync();
 
     // ---- iterations ----
+    // (the sums of iteration k - 1 are read behind the first barrier of iteration k, which step 1
+    // of iteration k does not wait for; k = 0 reads |b|)
     int k = 0, lev = 0, level_iters = 0, have_prev = 0, converged = 0, stop_reason = 0;
-    double prev = 0.0, last_res = NAN, best = INFINITY;
-    for (;;) {
-        double lam;
+    double prev = 0.0, last_res = NAN, best = INFINITY, bnorm = 0.0, lam = NAN, cur_lam = NAN;
+    for (;; ++k) {
+        columns_out(a);
+        if (!barrier()) return gave_up();
+        tot = load_part(k + 1);
+        const double2 z = rows_load();  // in flight while the schedule is decided
+        tot.x = warp_sum(tot.x);
+        tot.y = warp_sum(tot.y);
+        if (k == 0) {
+            bnorm = sqrt(tot.y) / (2.0 * dn);
+        } else {  // absorb iteration k - 1, which ran at lam
+            const double chi2 = tot.x;
+            const bool full = lam == 1.0;
+            const double resid = full ? sqrt(tot.y) / bnorm : NAN;
+            if (c == 0 && t == 0 && k - 1 < A.tr_cap) {
+                A.tr_lam[k - 1] = lam;
+                A.tr_chi2[k - 1] = chi2;
+                A.tr_res[k - 1] = resid;
+            }
+            if (full) {
+                last_res = resid;
+                if (!isfinite(resid) || (k > 50 && resid > 1e3 * best)) {
+                    stop_reason = 3;
+                    break;
+                }
+                best = fmin(best, resid);
+            }
+            if (!A.replay) {
+                bool advanced = false;
+                if (full) {
+                    if (resid < A.tol) {
+                        converged = 1;
+                        stop_reason = 1;
+                        break;
+                    }
+                } else {
+                    ++level_iters;
+                    const bool plateau = have_prev && fabs(chi2 - prev) < A.eta * A.sigma;
+                    if (plateau || level_iters >= A.level_cap) {
+                        lev = min(lev + 1, A.nlevels - 1);
+                        level_iters = 0;
+                        have_prev = 0;
+                        advanced = true;
+                    }
+                }
+                if (!advanced) {
+                    prev = chi2;
+                    have_prev = 1;
+                }
+            }
+        }
         if (A.replay) {
             if (k >= A.nreplay) break;
             lam = A.replay[k];
         } else {
-            if (k >= A.maxiter) { stop_reason = 2; break; }
+            if (k >= A.maxiter) {
+                stop_reason = 2;
+                break;
+            }
             lam = A.levels[lev];
         }
-        if (!(lam == cur_lam)) set_level(lam);
-        step1();
-        cluster.sync();
-        const double pc = step2(FS_ITER, lam);
-        cluster.sync();
-        double ch = 0.0, rs = 0.0;
-        step3(FS_ITER, lam, ch, rs);
-        block_reduce3(pc, ch, rs);
-        cluster.sync();
-        cluster_sum(tot);
-        const double chi2 = tot[0] + tot[1];
-        const bool full = lam == 1.0;
-        const double resid = full ? sqrt(tot[2]) / bnorm : NAN;
-        if (c == 0 && tid == 0 && k < A.tr_cap) {
-            A.tr_lam[k] = lam;
-            A.tr_chi2[k] = chi2;
-            A.tr_res[k] = resid;
+        const double lt = lam * A.tau;
+        if (!(lam == cur_lam)) {  // FP64 divisions once per cooling level, not once per iteration
+            const double lm1t = (lam - 1.0) * A.tau;
+            ia = 1.0 / (1.0 + lm1t * na);
+            ib = 1.0 / (1.0 + lm1t * nb);
+            la = lt * ia;
+            lb = lt * ib;
+            f = S > 0.0 ? S / (S + lt) / (2.0 * dn * dn) : 0.0;
+            cur_lam = lam;
         }
-        ++k;
-        if (full) {
-            last_res = resid;
-            if (!isfinite(resid) || (k > 50 && resid > 1e3 * best)) { stop_reason = 3; break; }
-            best = fmin(best, resid);
-        }
-        if (A.replay) continue;
-        if (lam == 1.0) {
-            if (resid < A.tol) { converged = 1; stop_reason = 1; break; }
-        } else {
-            ++level_iters;
-            const bool plateau = have_prev && fabs(chi2 - prev) < A.eta * A.sigma;
-            if (plateau || level_iters >= A.level_cap) {
-                lev = min(lev + 1, A.nlevels - 1);
-                level_iters = 0;
-                have_prev = 0;
-                continue;
+        const double2 s = rows_in(z);
+        // Eq. 3 and its chi^2 term (nu s^2 - 2 r s) id = -s (e + r) id with e = r - nu s
+        const double ea = ra - na * s.x, eb = rb - nb * s.y;
+        rows_out(s.x + la * ea, s.y + lb * eb);
+        // sums that need no exchange before the second barrier, while its first arrivals wait
+        double ch = S > 0.0 ? wk * ((a.x * a.x + a.y * a.y) * si) : 0.0, rs = 0.0;
+        ch -= s.x * ((ea + ra) * ia) + s.y * ((eb + rb) * ib);
+        if (!barrier()) return gave_up();
+        const double2 th = columns_in();
+        if (S > 0.0) {
+            const double2 an = cscale(th, f);
+            if (lam == 1.0) {
+                const double dx = kr * (a.x - an.x), dy = kr * (a.y - an.y);
+                rs = wk * (dx * dx + dy * dy);
             }
+            a = an;
         }
-        prev = chi2;
-        have_prev = 1;
+        put_part(k, ch, rs);
     }
     if (A.replay && isfinite(last_res) && last_res < A.tol) converged = 1;
-    // ---- output: s = F^-1 a, chi^2(s, 1) ----
-    cluster.sync();
-    step1();
-    cluster.sync();
-    const double pc = step2(FS_OUT, 1.0);
-    double chh = 0.0;
-    for (int i = tid; i < ncol * n; i += blockDim.x) {
-        const int kl = i / n, ky = i % n;
-        const int kx = c0 + kl;
-        const double2 a = acol[i];
-        if (A.alm_out) A.alm_out[(size_t)ky * nh + kx] = a;
-        const double S = Scol[i];
-        const double w = (kx == 0 || 2 * kx == n) ? 1.0 : 2.0;
-        if (S > 0.0) chh += w * (a.x * a.x + a.y * a.y) / S;
+    // ---- output: s = F^-1 a (its columns are in x1), chi^2(s, 1) ----
+    const double2 s = rows_in(rows_load());
+    double pc = wk * ((a.x * a.x + a.y * a.y) * si);
+    if (row) {
+        A.s_out[(size_t)ya * n + t] = s.x;
+        A.s_out[(size_t)yb * n + t] = s.y;
+        const double ea = ra - na * s.x, eb = rb - nb * s.y;
+        if (na > 0.0) pc += ea * ea / na;  // nu (d - s)^2
+        if (nb > 0.0) pc += eb * eb / nb;
     }
-    block_reduce3(pc, chh, 0.0);
-    cluster.sync();
-    cluster_sum(tot);
-    if (c == 0 && tid == 0) {
+    if (mode && A.alm_out) A.alm_out[(size_t)t * nh + c] = cscale(a, dn);
+    put_part(k, pc, 0.0);
+    if (!barrier()) return gave_up();
+    if (c != 0) return;
+    tot = load_part(k);
+    tot.x = warp_sum(tot.x);
+    if (t == 0) {
         A.status->iters = k;
         A.status->converged = converged;
         A.status->levels = lev + 1;
         A.status->stop_reason = stop_reason;
         A.status->final_resid = last_res;
-        A.status->chi2_final = tot[0] + tot[1];
+        A.status->chi2_final = tot.x;
         A.status->bnorm = bnorm;
     }
-    cluster.sync();  // keep every CTA's shared memory alive until all remote reads are done
 }
 
-// nu = N^-1 (0 where masked), r = nu d; tau = min N and count over observed pixels
-__global__ void k_flat_setup(long long npix, const double *__restrict__ d, const double *__restrict__ nv,
-                             const uint8_t *__restrict__ mask, double *__restrict__ r, double *__restrict__ nu,
-                             double *__restrict__ out /* [min, count, flag] */)
+// nu = N^-1 (0 where masked), r = nu d; per CTA the minimum of N and the count over observed
+// pixels and whether an input is invalid, combined on the host (one CTA's FP64 divisions took
+// 80 us at n = 128)
+__global__ void __launch_bounds__(256) k_flat_setup(int npix, const double *__restrict__ d,
+                                                    const double *__restrict__ nv, const uint8_t *__restrict__ mask,
+                                                    double *__restrict__ r, double *__restrict__ nu,
+                                                    double *__restrict__ out /* per CTA [min, count, flag] */)
 {
-    __shared__ double smin[32], scnt[32], sfl[32];
+    __shared__ double smin[8], scnt[8], sfl[8];
     double mn = INFINITY, cnt = 0, fl = 0;
-    for (long long i = threadIdx.x; i < npix; i += blockDim.x) {
+    const int i = blockIdx.x * 256 + threadIdx.x;
+    if (i < npix) {
         const bool obs = mask ? mask[i] != 0 : true;
         double rv = 0.0, nuv = 0.0;
         if (obs) {
@@ -463,8 +438,8 @@ __global__ void k_flat_setup(long long npix, const double *__restrict__ d, const
             else {
                 nuv = 1.0 / N;
                 rv = dv / N;
-                mn = fmin(mn, N);
-                cnt += 1;
+                mn = N;
+                cnt = 1;
             }
         }
         r[i] = rv;
@@ -483,71 +458,63 @@ __global__ void k_flat_setup(long long npix, const double *__restrict__ d, const
     __syncthreads();
     if (threadIdx.x == 0) {
         double a = INFINITY, b = 0, f = 0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
+        for (int w = 0; w < 8; ++w) {
             a = fmin(a, smin[w]);
             b += scnt[w];
             f = fmax(f, sfl[w]);
         }
-        out[0] = a;
-        out[1] = b;
-        out[2] = f;
+        out[3 * blockIdx.x] = a;
+        out[3 * blockIdx.x + 1] = b;
+        out[3 * blockIdx.x + 2] = f;
     }
 }
 
-// Cluster size of one solve of an n x n grid: FLAT_CS_MAX CTAs (half the columns and rows of
-// each CTA, on twice the SMs) where the device co-schedules such a cluster with this kernel's
-// shared memory and n >= 32 (the packed row FFTs need two rows per CTA), FLAT_CS otherwise.
-// Decided once per device, after the kernel's shared-memory limit is set.
-int flat_cluster_size(int n)
+constexpr int FLAT_SETUP_CTAS = FLAT_MAXN * FLAT_MAXN / 256;
+
+// launches the setup; h: host, 3 * FLAT_SETUP_CTAS entries, valid after the stream synchronises (tmp: device)
+wf_status flat_setup(int n, const double *d, const double *noise_var, const uint8_t *mask, double *r, double *nu,
+                     double *tmp, double *h, cudaStream_t stream)
 {
-    if (n < 2 * FLAT_CS_MAX) return FLAT_CS;
-    static std::mutex mu;
-    static int cache[64] = {};
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) {
-        cudaGetLastError();
-        return FLAT_CS;
-    }
-    std::lock_guard<std::mutex> lock(mu);
-    if (cache[dev]) return cache[dev];
-    int cs = FLAT_CS;
-    if (cudaFuncSetAttribute(k_flat_solve, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
-        const int nm = FLAT_MAXN, nhm = nm / 2 + 1;
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(FLAT_CS_MAX);
-        cfg.blockDim = dim3(FLAT_THREADS);
-        cfg.dynamicSmemBytes = flat_smem(nm, (nhm + FLAT_CS_MAX - 1) / FLAT_CS_MAX, nm / FLAT_CS_MAX, nhm);
-        cudaLaunchAttribute at;
-        at.id = cudaLaunchAttributeClusterDimension;
-        at.val.clusterDim.x = FLAT_CS_MAX;
-        at.val.clusterDim.y = 1;
-        at.val.clusterDim.z = 1;
-        cfg.attrs = &at;
-        cfg.numAttrs = 1;
-        int ncl = 0;
-        if (cudaOccupancyMaxActiveClusters(&ncl, k_flat_solve, &cfg) == cudaSuccess && ncl >= 1) cs = FLAT_CS_MAX;
-    }
-    cudaGetLastError();  // an unsupported size leaves the portable one
-    cache[dev] = cs;
-    return cs;
+    const int npix = n * n, g = (npix + 255) / 256;
+    k_flat_setup<<<g, 256, 0, stream>>>(npix, d, noise_var, mask, r, nu, tmp);
+    WF_CUDA(cudaGetLastError());
+    WF_CUDA(cudaMemcpyAsync(h, tmp, (size_t)3 * g * sizeof(double), cudaMemcpyDeviceToHost, stream));
+    return WF_OK;
 }
 
-// one solve: a single cluster of cs CTAs
-wf_status flat_launch(const FlatArgs &A, int cs, size_t smem, cudaStream_t stream)
+// [min, count, flag] of the whole map into h[0..2]
+void flat_setup_combine(int n, double *h)
 {
+    for (int i = 1; i < (n * n + 255) / 256; ++i) {
+        h[0] = std::fmin(h[0], h[3 * i]);
+        h[1] += h[3 * i + 1];
+        h[2] = std::fmax(h[2], h[3 * i + 2]);
+    }
+}
+
+// one solve: a cooperative launch of n/2 + 1 CTAs (the barriers need them co-resident)
+wf_status flat_launch(const FlatArgs &A, cudaStream_t stream)
+{
+    WF_CUDA(cudaMemsetAsync(A.bar, 0, sizeof(unsigned), stream));
+    WF_CUDA(cudaMemsetAsync(A.status, 0, sizeof(FlatStatus), stream));
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(cs);
-    cfg.blockDim = dim3(FLAT_THREADS);
-    cfg.dynamicSmemBytes = smem;
+    cfg.gridDim = dim3(A.nh);
+    cfg.blockDim = dim3(std::max(32, A.n));
     cfg.stream = stream;
     cudaLaunchAttribute at;
-    at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim.x = cs;
-    at.val.clusterDim.y = 1;
-    at.val.clusterDim.z = 1;
+    at.id = cudaLaunchAttributeCooperative;
+    at.val.cooperative = 1;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
     WF_CUDA(cudaLaunchKernelEx(&cfg, k_flat_solve, A));
+    return WF_OK;
+}
+
+wf_status flat_result(const FlatStatus &fs)
+{
+    if (fs.stop_reason == 4) return set_error(WF_ETIMEOUT, "a bounded wait at a grid barrier gave up");
+    if (fs.stop_reason == 3) return set_error(WF_EDIVERGE, "residual grew (%.3e)", fs.final_resid);
+    if (fs.stop_reason == 2) return set_error(WF_ENOCONV, "iteration cap reached (residual %.3e)", fs.final_resid);
     return WF_OK;
 }
 
@@ -562,8 +529,6 @@ wf_status flat_create(wf_plan p)
     if (!f) return set_error(WF_ENOMEM, "host allocation");
     p->flat = f;
     f->n = n;
-    f->logn = 0;
-    while ((1 << f->logn) < n) ++f->logn;
     f->nh = n / 2 + 1;
     p->npix = (long long)n * n;
     p->nalm = (long long)n * f->nh;
@@ -573,18 +538,7 @@ wf_status flat_create(wf_plan p)
     if ((st = plan_alloc(p, (void **)&f->nu, p->npix * 8)) != WF_OK) return st;
     if ((st = plan_alloc(p, (void **)&f->levels, 64 * 8)) != WF_OK) return st;
     if ((st = plan_alloc(p, (void **)&f->status, sizeof(FlatStatus))) != WF_OK) return st;
-    if ((st = plan_alloc(p, (void **)&p->ws.redu, 16 * 8)) != WF_OK) return st;
-    // the attribute is per function, shared by every plan: set it for the largest grid
-    // (n = FLAT_MAXN) so that a smaller plan never lowers it under a larger one
-    {
-        const int nm = FLAT_MAXN, nhm = nm / 2 + 1, Pm = (nhm + FLAT_CS - 1) / FLAT_CS, RPm = nm / FLAT_CS;
-        const size_t smax = flat_smem(nm, Pm, RPm, nhm);
-        WF_CUDA(cudaFuncSetAttribute(k_flat_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smax));
-    }
-    f->cs = flat_cluster_size(n);
-    f->P = (f->nh + f->cs - 1) / f->cs;
-    f->RP = n / f->cs;
-    f->smem = flat_smem(n, f->P, f->RP, f->nh);
+    if ((st = plan_alloc(p, (void **)&f->xch, flat_scratch_bytes(n))) != WF_OK) return st;
     return WF_OK;
 }
 
@@ -621,12 +575,12 @@ wf_status flat_solve(wf_plan p, const double *d, const double *noise_var, const 
     }();
     const int n = f->n, nh = f->nh;
     Prof pr(p, info, p->opt.profile != 0);
-    k_flat_setup<<<1, 1024, 0, p->stream>>>(p->npix, fluct ? nullptr : d, noise_var, mask, f->r, f->nu, p->ws.redu);
+    double h[3 * FLAT_SETUP_CTAS];
+    if (wf_status ls = flat_setup(n, fluct ? nullptr : d, noise_var, mask, f->r, f->nu, (double *)f->xch, h, p->stream))
+        return ls;
     WF_COUNT_LAUNCH(p);
-    WF_CUDA(cudaGetLastError());
-    double h[3];
-    WF_CUDA(cudaMemcpyAsync(h, p->ws.redu, sizeof h, cudaMemcpyDeviceToHost, p->stream));
     WF_CUDA(cudaStreamSynchronize(p->stream));
+    flat_setup_combine(n, h);
     if (h[2] != 0.0) return set_error(WF_EINVAL, "noise variance must be finite and > 0 (and d finite) on observed pixels");
     if (h[1] == 0.0) return set_error(WF_EINVAL, "every pixel is masked");
     const double tau = h[0];
@@ -676,10 +630,8 @@ wf_status flat_solve(wf_plan p, const double *d, const double *noise_var, const 
 
     FlatArgs A{};
     A.n = n;
-    A.logn = f->logn;
     A.nh = nh;
-    A.P = f->P;
-    A.RP = f->RP;
+    flat_set_scratch(A, f->xch, n);
     A.r = f->r;
     A.nu = f->nu;
     A.S = S;
@@ -703,7 +655,7 @@ wf_status flat_solve(wf_plan p, const double *d, const double *noise_var, const 
     A.tr_cap = f->tr_cap;
     A.status = f->status;
     pr.begin(WF_K_FLAT);
-    if (wf_status ls = flat_launch(A, f->cs, f->smem, p->stream)) return ls;
+    if (wf_status ls = flat_launch(A, p->stream)) return ls;
     WF_COUNT_LAUNCH(p);
     pr.end();
     FlatStatus fs;
@@ -734,9 +686,7 @@ wf_status flat_solve(wf_plan p, const double *d, const double *noise_var, const 
             }
         }
     }
-    if (fs.stop_reason == 3) return set_error(WF_EDIVERGE, "residual grew (%.3e)", fs.final_resid);
-    if (fs.stop_reason == 2) return set_error(WF_ENOCONV, "iteration cap reached (residual %.3e)", fs.final_resid);
-    return WF_OK;
+    return flat_result(fs);
 }
 
 wf_status flat_alm2map(wf_plan p, const double *alm, double *map)
@@ -760,7 +710,7 @@ wf_status flat_map2alm(wf_plan p, const double *map, double *alm)
 // inverse-noise maps, the lambda levels, the status block and the per-
 // iteration traces) in one file-scope device array instead of plan memory.
 // Limits: n <= 128 (a power of two >= 16) and at most 20000 iterations;
-// the array is 0.71 MiB and stays resident on every device that loads the
+// the array is 0.97 MiB and stays resident on every device that loads the
 // library.  In host code the array's symbol is not a device address: every
 // call looks up its address on the current device with cudaGetSymbolAddress,
 // so no address outlives the context it belongs to (a cudaDeviceReset between
@@ -778,10 +728,11 @@ constexpr size_t NA_R = 0;
 constexpr size_t NA_NU = NA_R + NA_PIX * sizeof(double);
 constexpr size_t NA_LEV = NA_NU + NA_PIX * sizeof(double);
 constexpr size_t NA_RAD = NA_LEV + NOALLOC_LEVELS * sizeof(double);
-constexpr size_t NA_REDU = NA_RAD + 32 * sizeof(double);
-constexpr size_t NA_STATUS = NA_REDU + 16 * sizeof(double);
+constexpr size_t NA_STATUS = NA_RAD + 32 * sizeof(double);
 constexpr size_t NA_TRACE = NA_STATUS + 256;
-constexpr size_t NA_BYTES = NA_TRACE + 3 * (size_t)NOALLOC_MAXITER * sizeof(double);
+constexpr size_t NA_XCH = NA_TRACE + 3 * (size_t)NOALLOC_MAXITER * sizeof(double);
+constexpr size_t NA_BYTES = NA_XCH + 2 * (NOALLOC_MAXN / 2 + 1) * (size_t)NOALLOC_MAXN * sizeof(double2) +
+                            2 * (NOALLOC_MAXN / 2 + 1) * (size_t)FLAT_NP * sizeof(double) + 256;
 
 // max S over the half-plane modes whose rounded |k| equals 2^j, j = 1..15
 // (-1 where no mode has that radius): the priors the flat schedule needs.
@@ -855,20 +806,19 @@ extern "C" wf_status wf_flat_solve_noalloc(int n, const double *d, const double 
     wf_status st = noalloc_base(&base);
     if (st != WF_OK) return st;
     double *r = (double *)(base + NA_R), *nu = (double *)(base + NA_NU), *lev_d = (double *)(base + NA_LEV);
-    double *rad = (double *)(base + NA_RAD), *redu = (double *)(base + NA_REDU);
+    double *rad = (double *)(base + NA_RAD);
     FlatStatus *status = (FlatStatus *)(base + NA_STATUS);
     double *tr = (double *)(base + NA_TRACE);
     const long long npix = (long long)n * n;
     const int nh = n / 2 + 1;
 
-    k_flat_setup<<<1, 1024, 0, stream>>>(npix, d, noise_var, mask, r, nu, redu);
-    WF_CUDA(cudaGetLastError());
+    double h[3 * FLAT_SETUP_CTAS], smax[17];
+    if (wf_status ls = flat_setup(n, d, noise_var, mask, r, nu, (double *)(base + NA_XCH), h, stream)) return ls;
     k_flat_radial_max<<<1, 256, 0, stream>>>(n, S, rad);
     WF_CUDA(cudaGetLastError());
-    double h[3], smax[17];
-    WF_CUDA(cudaMemcpyAsync(h, redu, sizeof h, cudaMemcpyDeviceToHost, stream));
     WF_CUDA(cudaMemcpyAsync(smax, rad, sizeof smax, cudaMemcpyDeviceToHost, stream));
     WF_CUDA(cudaStreamSynchronize(stream));
+    flat_setup_combine(n, h);
     if (h[2] != 0.0) return set_error(WF_EINVAL, "noise variance must be finite and > 0 (and d finite) on observed pixels");
     if (h[1] == 0.0) return set_error(WF_EINVAL, "every pixel is masked");
     if (smax[16] != 0.0)
@@ -891,10 +841,8 @@ extern "C" wf_status wf_flat_solve_noalloc(int n, const double *d, const double 
 
     FlatArgs A{};
     A.n = n;
-    A.logn = 0;
-    while ((1 << A.logn) < n) ++A.logn;
     A.nh = nh;
-    // (the cluster size is chosen below, once the kernel's shared-memory limit is set)
+    flat_set_scratch(A, base + NA_XCH, n);
     A.r = r;
     A.nu = nu;
     A.S = S;
@@ -913,17 +861,7 @@ extern "C" wf_status wf_flat_solve_noalloc(int n, const double *d, const double 
     A.tr_res = tr + 2 * NOALLOC_MAXITER;
     A.tr_cap = NOALLOC_MAXITER;
     A.status = status;
-    {
-        // the dynamic shared-memory limit is per function: set it for the largest grid this
-        // entry point takes (n = NOALLOC_MAXN), on every call (a plan may have changed it)
-        const int nm = NOALLOC_MAXN, nhm = nm / 2 + 1, Pm = (nhm + FLAT_CS - 1) / FLAT_CS, RPm = nm / FLAT_CS;
-        const size_t smax = flat_smem(nm, Pm, RPm, nhm);
-        WF_CUDA(cudaFuncSetAttribute(k_flat_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smax));
-    }
-    const int cs = flat_cluster_size(n);
-    A.P = (nh + cs - 1) / cs;
-    A.RP = n / cs;
-    if (wf_status ls = flat_launch(A, cs, flat_smem(n, A.P, A.RP, nh), stream)) return ls;
+    if (wf_status ls = flat_launch(A, stream)) return ls;
     FlatStatus fs;
     WF_CUDA(cudaMemcpyAsync(&fs, status, sizeof fs, cudaMemcpyDeviceToHost, stream));
     WF_CUDA(cudaStreamSynchronize(stream));
@@ -952,7 +890,5 @@ extern "C" wf_status wf_flat_solve_noalloc(int n, const double *d, const double 
                 for (int i = 0; i < nt; ++i) info->L_trace[i] = -1;
         }
     }
-    if (fs.stop_reason == 3) return set_error(WF_EDIVERGE, "residual grew (%.3e)", fs.final_resid);
-    if (fs.stop_reason == 2) return set_error(WF_ENOCONV, "iteration cap reached (residual %.3e)", fs.final_resid);
-    return WF_OK;
+    return flat_result(fs);
 }
