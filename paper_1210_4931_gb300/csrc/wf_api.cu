@@ -1895,7 +1895,8 @@ long long hp_estimate_bytes(int nside, int lmax, wf_precision prec, bool staging
     const long long nalm = (long long)(lmax + 1) * (lmax + 2) / 2, ns = (long long)(lmax + 1) * np;
     const long long es = f32 ? 4 : 8, ec = 2 * es;
     long long b = 0;
-    b += nalm * 16 + np * 16 + (lmax + 1) * 8 + ns * (4 + 16);  // A64, c64, x, st, log2 c, seeds
+    b += nalm * 16 + np * (16 + 32) + (lmax + 1) * 8 + ns * (4 + 16);  // A64, c64, x, st, xw64, log2 c, seeds
+    if (!f32) b += nalm * 16;                                            // sums of the FP64 analysis
     // x32, w32, xw, FP32 seeds; two-step tables, partial sums of the analysis (per (m, k))
     if (f32) b += np * 24 + ns * 12 + (nalm / 2 + 2 * lmax + 8) * (8 + 8 + 32 + 32) + (lmax + 1) * 8;
     if (tc_prec(prec)) b += nalm * 8 + ns * 12;                  // A32, B32 and one-step seeds

@@ -130,6 +130,8 @@ struct HpTables {
     int *ls = nullptr;
     double *s0_64 = nullptr, *s1_64 = nullptr;
     double *x64 = nullptr;
+    double4 *xw64 = nullptr;   // per pair: x^2 rounded, 8 (x^2 - that), x, 1/x
+    double2 *acc64 = nullptr;  // FP64 plans: sums of the analysis, zero between launches
     double *st64 = nullptr;  // sin(theta) per pair
     // mixed precision: x and w = 1 - x per pair (FP32); ring variables and 1/x per pair and the
     // two-step tables of the belt and cap forms per (m, k) (wf_legendre.cu); first k and starting

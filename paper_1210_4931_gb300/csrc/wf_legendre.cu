@@ -175,64 +175,128 @@ __global__ void k_to_T(const double *__restrict__ in, T *__restrict__ out, long 
 }
 
 // ---------------------------------------------------------------------------
-// FP64 synthesis: CTA per (m, block of pairs); thread per pair.
-// lcut > 0: the FP64 block of the mixed path, l < lcm_of(lcut, m), output
-// into Gout with row stride gstride.
+// FP64 transforms.  FP64 runs at 1/64 of the FP32 rate (a warp instruction holds its
+// scheduler's FP64 unit for 64 cycles), so what counts is the FP64 operations per (l, ring
+// pair) and that all 608 schedulers have work.
+//
+// Both directions take one warp per (group of 32 ring pairs, m) and advance two l at once
+// (k = (l - m)/2) with the odd values carried as x mu, which saves the product A_l x on the
+// way from odd to even:
+//     E_k = mu_{m+2k},  O_k = x mu_{m+2k+1},
+//     E_{k+1} = A_{2k+2} O_k - E_k,  O_{k+1} = (A_{2k+3} X) E_{k+1} - O_k,
+// with X = x^2 rounded; X's rounding error d, which would move the ring, is made up for in
+// every fourth step by O += 4 (2 d) E, with the limit 2 of A.  3.6 operations per (l, pair)
+// with the contraction (4 before).  The odd sum is divided by x at the end (analysis: its
+// input is).  A, c and a_lm pass through shared memory in blocks of 32 l, the next block's
+// loads in flight over the present one.
+//
+// One CTA per m before: its 256 threads left up to half the schedulers idle behind m = 0 where
+// the ring pairs are few.  Synthesis at nside 256, lmax 512
+// 0.606 -> 0.390 ms (its FP64 operations take 0.38); at nside 100, lmax 200, 46 -> 35 us and the
+// analysis 87 -> 60 + 6 us.
+//
+// lcut > 0: the FP64 block of the mixed path, l < lcm_of(lcut, m), output into G with row
+// stride gstride.
 // ---------------------------------------------------------------------------
+constexpr int F64_BLK = 32;  // l per block of the tables
+
+struct F64Pair {
+    int k0, kmin, kmaxs;  // first k of this lane's pair; the warp's least and largest first k
+    double s0, s1;        // mu_{m+2k0}, x mu_{m+2k0+1}
+    double4 xw;           // X, 8 (x^2 - X), x, 1/x (0 for x = 0)
+};
+
+__device__ __forceinline__ F64Pair f64_pair(int m, int Lm, int npairs, int p, const int *__restrict__ ls_tab,
+                                            const double *__restrict__ s0_tab, const double *__restrict__ s1_tab,
+                                            const double4 *__restrict__ xw)
+{
+    F64Pair P{BIG, 0, -1, 0.0, 0.0, make_double4(0.0, 0.0, 0.0, 0.0)};
+    if (p < npairs) {
+        const size_t sidx = (size_t)m * npairs + p;
+        const int ls = ls_tab[sidx];
+        if (ls <= Lm) {
+            P.k0 = (ls - m) >> 1;
+            P.xw = xw[p];
+            P.s0 = s0_tab[sidx];
+            P.s1 = P.xw.z * s1_tab[sidx];
+        }
+    }
+    P.kmin = __reduce_min_sync(0xffffffffu, P.k0);
+    P.kmaxs = __reduce_max_sync(0xffffffffu, P.k0 == BIG ? -1 : P.k0);
+    return P;
+}
+
+// (E_k, O_k) to k + 1; FIX: with the correction of X, in every fourth step
+template <bool FIX>
+__device__ __forceinline__ void f64_advance(double2 A /* A_{2k+2}, A_{2k+3} */, const double4 &xw, double &E, double &O)
+{
+    E = fma(A.x, O, -E);
+    O = fma(A.y * xw.x, E, -O);
+    if (FIX) O = fma(xw.y, E, O);
+}
+
 // TG: element type of the output (FP32 for the FP64 block of the mixed path,
 // whose ring pass adds it to the FP32 coefficients in FP32 anyway: converting
 // here keeps the 1/64-rate conversions off the ring kernel).
-template <typename T, typename TG>
-__global__ void __launch_bounds__(LEG_THREADS) k_legsyn(int lmax, int L, int npairs, int lcut,
-                                                        const double2 *__restrict__ alm, const T *__restrict__ A,
-                                                        const double *__restrict__ c64,
-                                                        const int *__restrict__ ls_tab, const T *__restrict__ s0_tab,
-                                                        const T *__restrict__ s1_tab, const T *__restrict__ xp,
-                                                        cx<TG> *__restrict__ G, int gstride)
+template <typename TG>
+__global__ void __launch_bounds__(32) k_legsyn(int lmax, int L, int npairs, int lcut, const double2 *__restrict__ alm,
+                                               const double *__restrict__ A, const double *__restrict__ c64,
+                                               const int *__restrict__ ls_tab, const double *__restrict__ s0_tab,
+                                               const double *__restrict__ s1_tab, const double4 *__restrict__ xw,
+                                               cx<TG> *__restrict__ G, int gstride)
 {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int m = blockIdx.y;
+    __shared__ double2 sac[F64_BLK];    // c a_lm
+    __shared__ double2 sA[F64_BLK / 2];
+    const int m = blockIdx.y, lane = threadIdx.x;
+    const int p = (gridDim.x - 1 - blockIdx.x) * 32 + lane;  // the equator (most work) first
     const int Lm = lcut > 0 ? min(L, lcm_of(lcut, m) - 1) : L;
     const int nl = Lm - m + 1;
     const long long base = mbase(lmax, m);
-    cx<T> *sac = reinterpret_cast<cx<T> *>(smem_raw);
-    T *sA = reinterpret_cast<T *>(sac + (nl + 2));
-    for (int i = threadIdx.x; i < nl + 2; i += blockDim.x) {
-        if (i < nl) {
-            const double2 a = alm[base + i];
-            const double cc = c64[base + i];
-            sac[i] = mk<T>((T)(a.x * cc), (T)(a.y * cc));
-            sA[i] = A[base + i];
-        } else {
-            sac[i] = mk<T>(0, 0);
-            sA[i] = 0;
+    const F64Pair P = f64_pair(m, Lm, npairs, p, ls_tab, s0_tab, s1_tab, xw);
+    double er = 0.0, ei = 0.0, orr = 0.0, oi = 0.0;
+    double E = 0.0, O = 0.0;
+    double2 na;
+    double nc, nA;
+    auto fetch = [&](int j) {
+        na = j < nl ? alm[base + j] : make_double2(0.0, 0.0);
+        nc = j < nl ? c64[base + j] : 0.0;
+        nA = j + 2 < nl ? A[base + j + 2] : 0.0;
+    };
+    int kc = P.kmin & ~3;
+    const int nk = (nl + 1) >> 1;
+    if (P.kmin != BIG) fetch(2 * kc + lane);
+    auto block4 = [&](int k, bool start) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            if (start && kc + k + i == P.k0) {
+                E = P.s0;
+                O = P.s1;
+            }
+            const double2 a0 = sac[2 * (k + i)], a1 = sac[2 * (k + i) + 1], c = sA[k + i];
+            er = fma(a0.x, E, er);
+            ei = fma(a0.y, E, ei);
+            orr = fma(a1.x, O, orr);
+            oi = fma(a1.y, O, oi);
+            if (i == 3) f64_advance<true>(c, P.xw, E, O);
+            else f64_advance<false>(c, P.xw, E, O);
         }
-    }
-    __syncthreads();
-    for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < npairs; p += gridDim.x * blockDim.x) {
-        const size_t sidx = (size_t)m * npairs + p;
-        const int ls = ls_tab[sidx];
-        T er = 0, ei = 0, orr = 0, oi = 0;
-        if (ls <= Lm) {
-            const T x = xp[p];
-            T mu0 = s0_tab[sidx], mu1 = s1_tab[sidx];
-            int i = ls - m;
-            cx<T> a0 = sac[i], a1 = sac[i + 1];
-            er = a0.x * mu0;
-            ei = a0.y * mu0;
-            orr = a1.x * mu1;
-            oi = a1.y * mu1;
-            for (i += 2; i < nl; i += 2) {
-                mu0 = fma(sA[i] * x, mu1, -mu0);
-                a0 = sac[i];
-                er = fma(a0.x, mu0, er);
-                ei = fma(a0.y, mu0, ei);
-                mu1 = fma(sA[i + 1] * x, mu0, -mu1);
-                a1 = sac[i + 1];
-                orr = fma(a1.x, mu1, orr);
-                oi = fma(a1.y, mu1, oi);
+    };
+    if (P.kmin != BIG)
+        for (; kc < nk; kc += F64_BLK / 2) {
+            __syncwarp();
+            sac[lane] = cscale(na, nc);
+            reinterpret_cast<double *>(sA)[lane] = nA;
+            __syncwarp();
+            fetch(2 * (kc + F64_BLK / 2) + lane);
+            const int kn = min(F64_BLK / 2, nk - kc);  // (a block of four runs up to three k past the end, on zeros)
+            for (int k = 0; k < kn; k += 4) {
+                if (kc + k <= P.kmaxs) block4(k, true);
+                else block4(k, false);
             }
         }
+    if (p < npairs) {
+        orr *= P.xw.w;
+        oi *= P.xw.w;
         cx<TG> *g = G + ((size_t)p * gstride + m) * 2;
         g[0] = mk<TG>((TG)(er + orr), (TG)(ei + oi));
         g[1] = mk<TG>((TG)(er - orr), (TG)(ei - oi));
@@ -361,98 +425,81 @@ __device__ __forceinline__ void blend_epilogue(int lmax, int L, int m, long long
     if (mode == LEG_BLEND) blend_sums(v, m, part, red);
 }
 
-// ---------------------------------------------------------------------------
-// FP64 analysis: CTA per m; warp per 32 pairs; register chunks of CH values
-// of l reduced across the warp, added into FP64 shared accumulators.
-// TF is the storage type of F (FP64 plans: double; FP64 block of the mixed
-// path: float).
-// ---------------------------------------------------------------------------
-template <typename T, typename TF, int CH, bool SPLIT>
-__global__ void __launch_bounds__(LEG_THREADS) k_legana(int lmax, int L, int npairs, int lcut,
-                                                        const cx<TF> *__restrict__ F, const T *__restrict__ A,
-                                                        const int *__restrict__ ls_tab, const T *__restrict__ s0_tab,
-                                                        const T *__restrict__ s1_tab, const T *__restrict__ xp,
-                                                        const double *__restrict__ c64, int mode, double omega,
-                                                        BlendArgs ba, const double2 *__restrict__ a_old,
-                                                        double2 *__restrict__ out, double *__restrict__ part)
+// FP64 analysis: chunks of 16 l in registers, reduced across the warp (one addition per value),
+// times c_l added to acc (zero before).  TF is the storage type of F (FP64 plans: double; FP64
+// block of the mixed path: float).
+template <typename TF>
+__global__ void __launch_bounds__(32) k_legana(int lmax, int L, int npairs, int lcut, const cx<TF> *__restrict__ F,
+                                               const double *__restrict__ A, const int *__restrict__ ls_tab,
+                                               const double *__restrict__ s0_tab, const double *__restrict__ s1_tab,
+                                               const double4 *__restrict__ xw, const double *__restrict__ c64,
+                                               double2 *__restrict__ acc)
 {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ double red[4][LEG_THREADS / 32];
-    const int m = blockIdx.x;
+    constexpr int CH = 16;
+    __shared__ double2 sA[F64_BLK / 2];
+    const int m = blockIdx.y, lane = threadIdx.x;
+    const int p = (gridDim.x - 1 - blockIdx.x) * 32 + lane;
     const int Lm = lcut > 0 ? min(L, lcm_of(lcut, m) - 1) : L;
     const int nl = Lm - m + 1;
-    const int nlp = nl + CH + 2;
     const long long base = mbase(lmax, m);
-    double2 *acc = reinterpret_cast<double2 *>(smem_raw);
-    T *sA = reinterpret_cast<T *>(acc + nlp);
-    for (int i = threadIdx.x; i < nlp; i += blockDim.x) {
-        acc[i] = make_double2(0.0, 0.0);
-        sA[i] = (i < nl) ? A[base + i] : (T)0;
+    const F64Pair P = f64_pair(m, Lm, npairs, p, ls_tab, s0_tab, s1_tab, xw);
+    if (P.kmin == BIG) return;
+    double2 FE = make_double2(0.0, 0.0), FO = FE;
+    if (P.k0 != BIG) {
+        const cx<TF> *f = F + ((size_t)p * (lmax + 1) + m) * 2;
+        const cx<TF> fn = f[0], fs = f[1];
+        FE = make_double2((double)fn.x + (double)fs.x, (double)fn.y + (double)fs.y);
+        FO = make_double2(((double)fn.x - (double)fs.x) * P.xw.w, ((double)fn.y - (double)fs.y) * P.xw.w);
     }
-    __syncthreads();
-
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    const int ngroups = (npairs + 31) / 32;
-    // SPLIT: the ring pairs of one m are shared by gridDim.y CTAs
-    const int gpc = SPLIT ? (ngroups + gridDim.y - 1) / gridDim.y : ngroups;
-    const int g0 = SPLIT ? blockIdx.y * gpc : 0;
-    const int g1 = min(ngroups, g0 + gpc);
-    for (int grp = g0 + warp; grp < g1; grp += nwarps) {
-        const int p = grp * 32 + lane;
-        const size_t sidx = (size_t)m * npairs + p;
-        int ls = (p < npairs) ? ls_tab[sidx] : BIG;
-        if (ls > Lm) ls = BIG;
-        const int lmin = __reduce_min_sync(0xffffffffu, ls);
-        if (lmin > Lm) continue;
-        cx<T> FE = mk<T>(0, 0), FO = mk<T>(0, 0);
-        T x = 0, s0 = 0, s1 = 0;
-        if (ls <= Lm) {
-            const cx<TF> *f = F + ((size_t)p * (lmax + 1) + m) * 2;
-            const cx<TF> fn = f[0], fs = f[1];
-            FE = mk<T>((T)fn.x + (T)fs.x, (T)fn.y + (T)fs.y);
-            FO = mk<T>((T)fn.x - (T)fs.x, (T)fn.y - (T)fs.y);
-            x = xp[p];
-            s0 = s0_tab[sidx];
-            s1 = s1_tab[sidx];
-        }
-        T mua = 0, mub = 0;
-        for (int l0 = lmin; l0 <= Lm; l0 += CH) {
-            T vr[CH], vi[CH];
+    double E = 0.0, O = 0.0;
+    int kc = P.kmin & ~3;
+    const int nk = (nl + 1) >> 1;
+    double nA = 2 * kc + lane + 2 < nl ? A[base + 2 * kc + lane + 2] : 0.0;
+    for (; kc < nk; kc += F64_BLK / 2) {
+        __syncwarp();
+        reinterpret_cast<double *>(sA)[lane] = nA;
+        __syncwarp();
+        const int jn = 2 * kc + F64_BLK + lane + 2;
+        nA = jn < nl ? A[base + jn] : 0.0;
+        for (int k = 0; k < min(F64_BLK / 2, nk - kc); k += CH / 2) {
+            double vr[CH], vi[CH];
+            const bool start = kc + k <= P.kmaxs;
 #pragma unroll
-            for (int i = 0; i < CH; i += 2) {
-                const int j = l0 - m + i;
-                T v0 = fma(sA[j] * x, mub, -mua);
-                T v1 = fma(sA[j + 1] * x, v0, -mub);
-                if (l0 + i == ls) { v0 = s0; v1 = s1; }
-                vr[i] = v0 * FE.x;
-                vi[i] = v0 * FE.y;
-                vr[i + 1] = v1 * FO.x;
-                vi[i + 1] = v1 * FO.y;
-                mua = v0;
-                mub = v1;
-            }
-            warp_reduce_scatter<T, CH>(vr, vi, lane);
-            constexpr int sh = 5 - Log2<CH>::v;
-            if ((lane & ((1 << sh) - 1)) == 0) {
-                const int l = l0 + (lane >> sh);
-                if (l <= Lm) {
-                    atomicAdd(&acc[l - m].x, (double)vr[0]);
-                    atomicAdd(&acc[l - m].y, (double)vi[0]);
+            for (int i = 0; i < CH / 2; ++i) {
+                if (start && kc + k + i == P.k0) {
+                    E = P.s0;
+                    O = P.s1;
                 }
+                vr[2 * i] = E * FE.x;
+                vi[2 * i] = E * FE.y;
+                vr[2 * i + 1] = O * FO.x;
+                vi[2 * i + 1] = O * FO.y;
+                if ((i & 3) == 3) f64_advance<true>(sA[k + i], P.xw, E, O);
+                else f64_advance<false>(sA[k + i], P.xw, E, O);
             }
+            // c_l for this lane's l, in flight over the reduction
+            const int j = 2 * (kc + k) + (lane >> 1);
+            const double cc = j < nl ? c64[base + j] : 0.0;
+            warp_reduce_scatter<double, CH>(vr, vi, lane);
+            if (j < nl) atomicAdd(lane & 1 ? &acc[base + j].y : &acc[base + j].x, cc * (lane & 1 ? vi[0] : vr[0]));
         }
     }
-    __syncthreads();
-    if (SPLIT) {  // adjoint only: add this CTA's share into the (zeroed) output
-        for (int j = threadIdx.x; j < nl; j += blockDim.x) {
-            const double cc = c64[base + j];
-            atomicAdd(&out[base + j].x, cc * acc[j].x);
-            atomicAdd(&out[base + j].y, cc * acc[j].y);
-        }
-        return;
-    }
-    auto val = [&](int j) { return cscale(acc[j], c64[base + j]); };
-    blend_epilogue(lmax, Lm, m, base, mode, ba, val, a_old, out, part, red);
+}
+
+// Eq. (4) epilogue of the FP64 analysis, a CTA per m; clears the sums for the next launch
+__global__ void __launch_bounds__(128) k_ana64_epilogue(int lmax, int L, int mode, BlendArgs ba,
+                                                        const double2 *__restrict__ a_old, double2 *__restrict__ out,
+                                                        double *__restrict__ part, double2 *__restrict__ acc)
+{
+    __shared__ double red[4][LEG_THREADS / 32];
+    const int m = blockIdx.x;
+    const long long base = mbase(lmax, m);
+    auto val = [&](int j) {
+        const double2 v = acc[base + j];
+        acc[base + j] = make_double2(0.0, 0.0);
+        return v;
+    };
+    blend_epilogue(lmax, L, m, base, mode, ba, val, a_old, out, part, red);
 }
 
 // ---------------------------------------------------------------------------
@@ -1372,12 +1419,6 @@ __global__ void __launch_bounds__(128) k_ana_epilogue(const MxTables t, int mode
 // ---------------------------------------------------------------------------
 // launches
 // ---------------------------------------------------------------------------
-template <typename T>
-size_t syn_smem(int L) { return (size_t)(L + 3) * (sizeof(cx<T>) + sizeof(T)) + 16; }
-
-template <typename T, int CH>
-size_t ana_smem(int L) { return (size_t)(L + 1 + CH + 2) * (sizeof(double2) + sizeof(T)) + 16; }
-
 size_t syn_mx_smem(int L) { return (size_t)((L + 1) / 2 + 5) * (sizeof(float4) + sizeof(float2)) + 16; }
 
 template <typename TG>
@@ -1386,52 +1427,35 @@ wf_status launch_syn64(wf_plan p, const double2 *alm, int L, int lcut, cx<TG> *G
     const HpTables &t = p->tab;
     const int Lgrid = lcut > 0 ? std::min(L, lcut - 1) : L;
     if (Lgrid < 0) return WF_OK;
-    const int gx = (p->npairs + 4 * LEG_THREADS - 1) / (4 * LEG_THREADS);
-    dim3 grid(gx, Lgrid + 1);
-    const size_t sm = syn_smem<double>(lcut > 0 ? std::min(L, lcut + 1) : L);
-    if (wf_status st = raise_smem_limit((const void *)k_legsyn<double, TG>, sm)) return st;
-    k_legsyn<double, TG><<<grid, LEG_THREADS, sm, s>>>(p->lmax, L, p->npairs, lcut, alm, t.A64, t.c64, t.ls,
-                                                            t.s0_64, t.s1_64, t.x64, G, gstride);
+    k_legsyn<TG><<<dim3((p->npairs + 31) / 32, Lgrid + 1), 32, 0, s>>>(p->lmax, L, p->npairs, lcut, alm, t.A64, t.c64,
+                                                                       t.ls, t.s0_64, t.s1_64, t.xw64, G, gstride);
     WF_COUNT_LAUNCH(p);
     WF_CUDA(cudaGetLastError());
     return WF_OK;
 }
 
-template <typename TF>
-wf_status launch_ana64(wf_plan p, int L, int lcut, const void *F, LegMode mode, const BlendArgs &ba,
-                       const double2 *a_old, double2 *out, cudaStream_t s)
+wf_status launch_ana64(wf_plan p, int L, const double2 *F, LegMode mode, const BlendArgs &ba, const double2 *a_old,
+                       double2 *out, cudaStream_t s)
 {
-    constexpr int CH = 16;
     const HpTables &t = p->tab;
-    const int Lgrid = lcut > 0 ? std::min(L, lcut - 1) : L;
-    if (Lgrid < 0) return WF_OK;
-    const size_t sm = ana_smem<double, CH>(lcut > 0 ? std::min(L, lcut + 1) : L);
-    if (wf_status st = raise_smem_limit((const void *)k_legana<double, TF, CH, false>, sm)) return st;
-    k_legana<double, TF, CH, false><<<Lgrid + 1, LEG_THREADS, sm, s>>>(
-        p->lmax, L, p->npairs, lcut, (const cx<TF> *)F, t.A64, t.ls, t.s0_64, t.s1_64, t.x64, t.c64, (int)mode,
-        p->omega, ba, a_old, out, p->ws.part_harm);
+    k_legana<double><<<dim3((p->npairs + 31) / 32, L + 1), 32, 0, s>>>(
+        p->lmax, L, p->npairs, 0, F, t.A64, t.ls, t.s0_64, t.s1_64, t.xw64, t.c64, t.acc64);
+    WF_COUNT_LAUNCH(p);
+    k_ana64_epilogue<<<L + 1, 128, 0, s>>>(p->lmax, L, (int)mode, ba, a_old, out, p->ws.part_harm, t.acc64);
     WF_COUNT_LAUNCH(p);
     WF_CUDA(cudaGetLastError());
     return WF_OK;
 }
 
-// FP64 block of the mixed analysis (adjoint, l < lcm(lcut, m)): the block is
-// triangular in m, so one CTA per m would leave m = 0 as the critical path;
-// each m is split over ring-pair chunks whose shares are added atomically.
+// FP64 block of the mixed analysis (adjoint, l < lcm(lcut, m))
 wf_status launch_ana64_low(wf_plan p, int L, int lcut, const float2 *F, double2 *out, cudaStream_t s)
 {
-    constexpr int CH = 16;
     const HpTables &t = p->tab;
     const int nm = std::min(L, lcut - 1) + 1;
     if (nm <= 0) return WF_OK;
     WF_CUDA(cudaMemsetAsync(out, 0, (size_t)mbase(p->lmax, nm) * sizeof(double2), s));
-    const size_t sm = ana_smem<double, CH>(std::min(L, lcut + 1));
-    if (wf_status st = raise_smem_limit((const void *)k_legana<double, float, CH, true>, sm)) return st;
-    const int nchunk = std::max(1, std::min(16, p->npairs / 512));
-    BlendArgs none;
-    k_legana<double, float, CH, true><<<dim3(nm, nchunk), LEG_THREADS, sm, s>>>(
-        p->lmax, L, p->npairs, lcut, F, t.A64, t.ls, t.s0_64, t.s1_64, t.x64, t.c64, (int)LEG_ADJOINT, p->omega, none,
-        nullptr, out, nullptr);
+    k_legana<float><<<dim3((p->npairs + 31) / 32, nm), 32, 0, s>>>(p->lmax, L, p->npairs, lcut, F, t.A64, t.ls, t.s0_64,
+                                                                   t.s1_64, t.xw64, t.c64, out);
     WF_COUNT_LAUNCH(p);
     WF_CUDA(cudaGetLastError());
     return WF_OK;
@@ -1595,6 +1619,17 @@ wf_status hp_build_legendre_tables(wf_plan p, const std::vector<double> &xpair, 
     if ((st = plan_alloc(p, (void **)&t.A64, nalm * sizeof(double))) != WF_OK) return st;
     if ((st = plan_alloc(p, (void **)&t.x64, np * sizeof(double))) != WF_OK) return st;
     if ((st = plan_alloc(p, (void **)&dst64, np * sizeof(double))) != WF_OK) return st;
+    if ((st = plan_alloc(p, (void **)&t.xw64, np * sizeof(double4))) != WF_OK) return st;
+    if (!f32) {
+        if ((st = plan_alloc(p, (void **)&t.acc64, nalm * sizeof(double2))) != WF_OK) return st;
+        WF_CUDA(cudaMemsetAsync(t.acc64, 0, nalm * sizeof(double2), p->stream));
+    }
+    std::vector<double4> xw64(np);
+    for (int i = 0; i < np; ++i) {
+        const double x = xpair[i], X = x * x;
+        xw64[i] = make_double4(X, 8.0 * std::fma(x, x, -X), x, i + 1 < np ? 1.0 / x : 0.0);  // the equator's odd values vanish
+    }
+    if ((st = to_device(p, t.xw64, xw64.data(), np * sizeof(double4))) != WF_OK) return st;
     t.st64 = dst64;
     if ((st = plan_alloc(p, (void **)&dlog2c, (lmax + 1) * sizeof(double))) != WF_OK) return st;
     const long long ns = (long long)(lmax + 1) * np;
@@ -1671,11 +1706,6 @@ wf_status hp_build_legendre_tables(wf_plan p, const std::vector<double> &xpair, 
         const void *syn[] = {(const void *)k_legsyn_mx<2>, (const void *)k_legsyn_mx<4>, (const void *)k_legsyn_mx<8>};
         for (const void *f : syn)
             if ((st = raise_smem_limit(f, syn_mx_smem(lmax))) != WF_OK) return st;
-        if ((st = raise_smem_limit((const void *)k_legsyn<double, float>, syn_smem<double>(lmax))) != WF_OK)
-            return st;
-        if ((st = raise_smem_limit((const void *)k_legana<double, float, 16, true>, ana_smem<double, 16>(lmax))) !=
-            WF_OK)
-            return st;
         if ((st = raise_smem_limit((const void *)k_lowsyn_df, (size_t)(lmax + 2) * sizeof(float4))) != WF_OK)
             return st;
         if ((st = raise_smem_limit((const void *)k_lowana_df, (size_t)((np + 31) & ~31) * sizeof(float4))) != WF_OK)
@@ -1687,11 +1717,6 @@ wf_status hp_build_legendre_tables(wf_plan p, const std::vector<double> &xpair, 
     } else {
         if ((st = raise_smem_limit((const void *)k_legsyn_df, syn_df_smem(lmax))) != WF_OK) return st;
         if ((st = raise_smem_limit((const void *)k_legana_df, ana_df_smem(lmax))) != WF_OK) return st;
-        if ((st = raise_smem_limit((const void *)k_legsyn<double, double>, syn_smem<double>(lmax))) != WF_OK)
-            return st;
-        if ((st = raise_smem_limit((const void *)k_legana<double, double, 16, false>, ana_smem<double, 16>(lmax))) !=
-            WF_OK)
-            return st;
     }
     WF_CUDA(cudaStreamSynchronize(p->stream));
     return WF_OK;
@@ -1757,7 +1782,7 @@ wf_status hp_legendre_adjoint_buf(wf_plan p, int L, const double2 *F, double2 *o
     if (p->prec != WF_PREC_FP64) return set_error(WF_EUNSUPPORTED, "explicit-buffer transforms need an FP64 plan");
     WF_CUDA(cudaMemsetAsync(out, 0, p->nalm * sizeof(double2), p->stream));
     BlendArgs none;
-    return launch_ana64<double>(p, L, 0, F, LEG_ADJOINT, none, nullptr, out, p->stream);
+    return launch_ana64(p, L, F, LEG_ADJOINT, none, nullptr, out, p->stream);
 }
 
 // Mixed precision: the FP64 low-l block (FP64 pipe, few CTAs) runs on the
@@ -1937,7 +1962,7 @@ wf_status hp_legendre_analysis(wf_plan p, int L, LegMode mode, const BlendArgs &
     }
     if (p->prec == WF_PREC_FP64)
         return p->df_legendre ? launch_ana_df(p, L, mode, ba, a_old, out)
-                              : launch_ana64<double>(p, L, 0, p->ws.F, mode, ba, a_old, out, p->stream);
+                              : launch_ana64(p, L, (const double2 *)p->ws.F, mode, ba, a_old, out, p->stream);
     const int lc = t.lc_mx;
     if (lc <= 0) return launch_ana_mx(p, L, mode, ba, nullptr, a_old, out);
     // sequential: the FP32 epilogue of m < lc reads the block's result
