@@ -1364,14 +1364,6 @@ __global__ void __launch_bounds__(32, NP == 8 ? 17 : 16) k_legana_mx(const MxTab
     else mx_analysis<NP, true>(t, m, 2 * ngroups - 1 - g, F, &psum[nks + kb].x, S, nk);
 }
 
-// (double)f for finite f in integer arithmetic: the conversion instruction runs at the FP64 rate
-__device__ __forceinline__ double widen(float f)
-{
-    const unsigned u = __float_as_uint(f), a = u & 0x7fffffffu;
-    if (a < 0x00800000u || a >= 0x7f800000u) return (double)f;  // zero, denormal, infinity, NaN
-    return __hiloint2double((int)((u & 0x80000000u) | ((a >> 3) + 0x38000000u)), (int)(a << 29));
-}
-
 // Eq. (4) epilogue of the mixed analysis, a CTA per m; clears the sums for the next launch.  Run
 // by the last warp at its m inside the kernel above it took 14 % of that kernel (one warp's
 // chain of loads per m, nside 768).
