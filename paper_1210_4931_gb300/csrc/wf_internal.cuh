@@ -55,8 +55,8 @@ template <typename C, typename S> __host__ __device__ __forceinline__ C cscale(C
 __device__ __forceinline__ double widen(float f)
 {
     const unsigned u = __float_as_uint(f), a = u & 0x7fffffffu;
-    if (a < 0x00800000u || a >= 0x7f800000u) return (double)f;  // zero, denormal, infinity, NaN
-    return __hiloint2double((int)((u & 0x80000000u) | ((a >> 3) + 0x38000000u)), (int)(a << 29));
+    if (a - 0x00800000u >= 0x7f000000u && a != 0u) return (double)f;  // denormal, infinity, NaN
+    return a == 0u ? __hiloint2double((int)u, 0) : __hiloint2double((int)((u & 0x80000000u) | ((a >> 3) + 0x38000000u)), (int)(a << 29));
 }
 
 // (float)v, rounded to nearest even, in integer arithmetic

@@ -338,26 +338,6 @@ template <> struct Log2<8> { static constexpr int v = 3; };
 template <> struct Log2<16> { static constexpr int v = 4; };
 template <> struct Log2<32> { static constexpr int v = 5; };
 
-__device__ __forceinline__ void block_reduce4(double (&v)[4], double (*red)[LEG_THREADS / 32])
-{
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-#pragma unroll
-        for (int o = 16; o >= 1; o >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
-        if (lane == 0) red[k][warp] = v[k];
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            double x = 0.0;
-            for (int w = 0; w < (int)(blockDim.x >> 5); ++w) x += red[k][w];
-            v[k] = x;
-        }
-    }
-}
-
 // Eq. (4) epilogue shared by both precisions: t_hat = Omega (c acc + low),
 // a_new = S/(S + lam tau_h) t_hat, chi^2 of a_old, lambda = 1 residual.
 __global__ void k_epi_table(EpiArgs a)
@@ -382,13 +362,14 @@ __device__ __forceinline__ void blend_one(int l, int L, long long idx, int mode,
     }
     // per-l factors tabulated once per launch (no FP64 division per a_lm)
     const double4 e = ba.epi[l];
+    const bool on = __double2hiint(e.w) != 0;  // 1 or 0
     const double2 ao = a_old[idx];
     double2 an = make_double2(0.0, 0.0);
-    if (l <= L && e.w > 0.0) {
+    if (l <= L && on) {
         an.x = e.x * b.x;
         an.y = e.x * b.y;
     }
-    if (e.w > 0.0) {
+    if (on) {
         v.chi2 += (ao.x * ao.x + ao.y * ao.y) * e.y;
         if (ba.want_norms) {
             const double an2 = (an.x * an.x + an.y * an.y) * e.y;
@@ -397,32 +378,48 @@ __device__ __forceinline__ void blend_one(int l, int L, long long idx, int mode,
         }
         if (ba.want_resid) {
             const double dx = e.z * (ao.x - an.x), dy = e.z * (ao.y - an.y);
-            v.res2 += dx * dx + dy * dy;
+            v.res2 = fma(dx, dx, fma(dy, dy, v.res2));
         }
     }
     out[idx] = an;
 }
 
-__device__ __forceinline__ void blend_sums(const BlendSums &s, int m, double *__restrict__ part,
-                                           double (*red)[LEG_THREADS / 32])
+// the CTA's sums into part[4 m ..]: a warp per sum that is wanted (NT >= 128 threads).  (Every
+// warp reducing all four by shuffles took more FP64 operations than the blend itself at lmax 1024.)
+template <int NT>
+__device__ __forceinline__ void blend_sums(const BlendSums &s, int m, const BlendArgs &ba, double *__restrict__ part,
+                                           double (*red)[NT])
 {
-    double v[4] = {s.chi2, s.res2, s.hnew, s.qnew};
-    block_reduce4(v, red);
-    if (threadIdx.x == 0)
+    const int t = threadIdx.x, k = t >> 5, lane = t & 31;
+    red[0][t] = s.chi2;
+    if (ba.want_resid) red[1][t] = s.res2;
+    if (ba.want_norms) {
+        red[2][t] = s.hnew;
+        red[3][t] = s.qnew;
+    }
+    __syncthreads();
+    if (k >= 4) return;
+    double x = 0.0;
+    if (k == 0 || (k == 1 ? ba.want_resid : ba.want_norms)) {
+        x = red[k][lane];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) part[4 * m + k] = m ? 2.0 * v[k] : v[k];
+        for (int i = 32; i < NT; i += 32) x += red[k][i + lane];
+#pragma unroll
+        for (int o = 16; o >= 1; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    }
+    if (lane == 0) part[4 * m + k] = m ? 2.0 * x : x;
 }
 
 // val(j): c_lm times the ring sum at l = m + j
-template <typename VAL>
+template <int NT, typename VAL>
 __device__ __forceinline__ void blend_epilogue(int lmax, int L, int m, long long base, int mode, const BlendArgs &ba,
                                                VAL val, const double2 *__restrict__ a_old, double2 *__restrict__ out,
-                                               double *__restrict__ part, double (*red)[LEG_THREADS / 32])
+                                               double *__restrict__ part, double (*red)[NT])
 {
     BlendSums v;
     for (int j = threadIdx.x; j <= lmax - m; j += blockDim.x)
         blend_one(m + j, L, base + j, mode, ba, m + j <= L ? val(j) : make_double2(0.0, 0.0), a_old, out, v);
-    if (mode == LEG_BLEND) blend_sums(v, m, part, red);
+    if (mode == LEG_BLEND) blend_sums(v, m, ba, part, red);
 }
 
 // FP64 analysis: chunks of 16 l in registers, reduced across the warp (one addition per value),
@@ -491,7 +488,7 @@ __global__ void __launch_bounds__(128) k_ana64_epilogue(int lmax, int L, int mod
                                                         const double2 *__restrict__ a_old, double2 *__restrict__ out,
                                                         double *__restrict__ part, double2 *__restrict__ acc)
 {
-    __shared__ double red[4][LEG_THREADS / 32];
+    __shared__ double red[4][128];
     const int m = blockIdx.x;
     const long long base = mbase(lmax, m);
     auto val = [&](int j) {
@@ -858,7 +855,6 @@ __global__ void __launch_bounds__(LEG_THREADS, 2) k_legana_df(int lmax, int L, i
 {
     constexpr int CH = 8;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ double red[4][LEG_THREADS / 32];
     __shared__ int next_group;
     const int m = blockIdx.x;
     const int nl = L - m + 1;
@@ -969,7 +965,7 @@ __global__ void __launch_bounds__(LEG_THREADS, 2) k_legana_df(int lmax, int L, i
     }
     __syncthreads();
     auto val = [&](int j) { return cscale(acc[j], c64[base + j]); };
-    blend_epilogue(lmax, L, m, base, mode, ba, val, a_old, out, part, red);
+    blend_epilogue(lmax, L, m, base, mode, ba, val, a_old, out, part, reinterpret_cast<double (*)[LEG_THREADS]>(stage));
 }
 
 // ---------------------------------------------------------------------------
@@ -1372,7 +1368,7 @@ __global__ void __launch_bounds__(128) k_ana_epilogue(const MxTables t, int mode
                                                       const double2 *__restrict__ a_old, double2 *__restrict__ out,
                                                       double *__restrict__ part, float4 *__restrict__ psum)
 {
-    __shared__ double red[4][LEG_THREADS / 32];
+    __shared__ double red[4][128];
     const int m = blockIdx.x, nk = ((t.L - m + 1) >> 1) + 1;
     const long long base = mbase(t.lmax, m), kb = kbase(t.lmax, m);
     const long long nks = kbase(t.lmax, t.lmax + 1) + 2;
@@ -1403,7 +1399,7 @@ __global__ void __launch_bounds__(128) k_ana_epilogue(const MxTables t, int mode
         blend_one(l, t.L, i, mode, ba, e, a_old, out, v);
         if (l < t.lmax) blend_one(l + 1, t.L, i + 1, mode, ba, o, a_old, out, v);
     }
-    if (mode == LEG_BLEND) blend_sums(v, m, part, red);
+    if (mode == LEG_BLEND) blend_sums(v, m, ba, part, red);
     __syncthreads();
     for (int k = threadIdx.x; k < nk; k += blockDim.x) sb[k] = sc[k] = make_float4(0.f, 0.f, 0.f, 0.f);
 }
