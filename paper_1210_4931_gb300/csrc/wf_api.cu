@@ -1942,7 +1942,7 @@ long long hp_estimate_bytes(int nside, int lmax, wf_precision prec, bool staging
         b += 3 * (lmax + 1) * 32 + 2 * std::max(2LL * (lmax + 2), 8LL * 152) * 8;  // blend table, partials
         if (f32) {
             b += 9 * npix * 4;                                       // FP32 r, nu
-            b += nalm * (8 + 16 + 2 * 16);                           // c, mu-form table, FP64-block (E, B)
+            b += nalm * (8 + 16 + 2 * 16 + 16);                      // c, mu-form table, FP64-block (E, B), sums
             b += ns * (4 + 16);                                      // FP32 seeds
             b += 2 * np * lcap * 2 * 8;                              // FP64-block ring coefficients
         }

@@ -143,6 +143,7 @@ struct PolState {
     float4 *ac32 = nullptr;    // tensor-core plans: c (Re A, Im A, Re C, Im C) in FP32, the spin-2 B operand's source
     float2 *GQlow = nullptr, *GUlow = nullptr;  // FP64 block's ring coefficients [pair][m < lc][hemisphere]
     double2 *Elow = nullptr, *Blow = nullptr;   // FP64 block's (E, B)
+    float4 *psum = nullptr;    // per a_lm: YP, YM sums of the FP32 analysis, zero between launches
     int lc = -1, low_cap = 0;
 };
 

@@ -28,6 +28,7 @@
 #include <climits>
 #include <cmath>
 #include <cstring>
+#include <type_traits>
 #include <vector>
 
 #include "wf_internal.cuh"
@@ -37,7 +38,8 @@ namespace wf {
 namespace {
 
 constexpr int PM_THREADS = 256;
-constexpr int PM_CH = 8;  // values of l per analysis chunk
+constexpr int PM_CH = 4;     // values of l per analysis chunk
+constexpr int PM_TBLK = 32;  // l per block of the analysis table
 constexpr float PM_X_DIFF = 0.4f;
 constexpr int PM_BIG = INT_MAX / 2;
 
@@ -360,212 +362,189 @@ __global__ void __launch_bounds__(PM_THREADS) k_legsyn_pol_mx(int lmax, int L, i
     }
 }
 
-// warp reduce-scatter of CH values per lane: afterwards lane groups of
-// 32 / CH lanes hold the sum over the warp of one value (the l of the chunk
-// given by lane >> (5 - log2 CH))
-template <int CH>
-__device__ __forceinline__ void pm_rscatter(float (&vr)[CH], float (&vi)[CH], int lane)
-{
-#pragma unroll
-    for (int r = 0; r < 5; ++r) {
-        const int off = 16 >> r;
-        const int n = CH >> r;
-        if (n >= 2) {
-            const int half = n / 2;
-            const bool up = (lane & off) != 0;
-#pragma unroll
-            for (int i = 0; i < half; ++i) {
-                const float sr = up ? vr[i] : vr[i + half];
-                const float kr = up ? vr[i + half] : vr[i];
-                const float si = up ? vi[i] : vi[i + half];
-                const float ki = up ? vi[i + half] : vi[i];
-                vr[i] = kr + __shfl_xor_sync(0xffffffffu, sr, off);
-                vi[i] = ki + __shfl_xor_sync(0xffffffffu, si, off);
-            }
-        } else {
-            vr[0] += __shfl_xor_sync(0xffffffffu, vr[0], off);
-            vi[0] += __shfl_xor_sync(0xffffffffu, vi[0], off);
-        }
-    }
-}
-
 // ring coefficients of one pack: G+ = FQ + i FU and G- = FQ - i FU of the
 // north (N) and south (S) rings, real and imaginary parts
 struct PmRing {
     float2 pNr, pNi, pSr, pSi, qNr, qNi, qSr, qSi;
 };
 
+// shared memory of one analysis warp: a table block, and two stages of a chunk's sums over the
+// lane's pairs (row: l of the chunk; YP, YM re and im)
+struct PmAnaShared {
+    float4 tab[PM_TBLK];
+    float4 stage[2][PM_CH * 32];
+};
+
+// one warp's ring pairs at one m, j = l - m from j0 (a multiple of four): dst[4 j ..] += YP, YM
 template <bool DIFF, int NP>
-__device__ __forceinline__ void pm_ana_run(const PmPairs<NP> &P, int m, int L, int lmin_w, int lmaxs_w,
-                                           const float4 *__restrict__ sT, const PmRing (&G)[NP / 2], float2 *accP,
-                                           float2 *accM, int lane)
+__device__ __forceinline__ void pm_ana_run(const PmPairs<NP> &P, int m, int nl, int j0, int lmaxs,
+                                           const float4 *__restrict__ tab, const PmRing (&G)[NP / 2], PmAnaShared &S,
+                                           float *dst, int lane)
 {
     constexpr int NPK = NP / 2;
     float2 Spa[NPK], Spb[NPK], Sqa[NPK], Sqb[NPK], Vp0[NPK], Vp1[NPK], Vq0[NPK], Vq1[NPK];
 #pragma unroll
     for (int pk = 0; pk < NPK; ++pk) Spa[pk] = Spb[pk] = Sqa[pk] = Sqb[pk] = dup(0.f);
-    for (int l0 = lmin_w; l0 <= L; l0 += PM_CH) {
-        float2 YPr[PM_CH], YPi[PM_CH], YMr[PM_CH], YMi[PM_CH];
-        const bool inj = l0 <= lmaxs_w;
+    auto fetch = [&](int j) { return j < nl ? tab[j] : make_float4(0.f, 0.f, 0.f, 0.f); };
+    int j = j0, buf = 0;
+    float4 next = fetch((j0 & ~(PM_TBLK - 1)) + lane);
+    // lane (r, q) = (lane / 8, lane % 8) adds row r of lanes 4q .. 4q + 3 (in an order that keeps the
+    // eight lanes of a phase on distinct banks); three shuffles then leave component q & 3 summed
+    // over the warp
+    const int rr = lane >> 3, rq = lane & 7, rc = rq >> 1, rrow = 32 * rr + 4 * rq;
+    auto finish = [&](int jc, float4 v) {
+        const bool odd = rq & 2, im = rq & 1;
+        float a = odd ? v.z : v.x, b = odd ? v.w : v.y;
+        a += __shfl_xor_sync(0xffffffffu, odd ? v.x : v.z, 2);
+        b += __shfl_xor_sync(0xffffffffu, odd ? v.y : v.w, 2);
+        float c = im ? b : a;
+        c += __shfl_xor_sync(0xffffffffu, im ? a : b, 1);
+        c += __shfl_xor_sync(0xffffffffu, c, 4);
+        if (rq < 4 && jc + rr < nl) atomicAdd(dst + 4 * (jc + rr) + rq, c);
+    };
+    auto chunk = [&](auto inject) {
+        constexpr bool INJ = decltype(inject)::value;
+        if ((j & (PM_TBLK - 1)) == 0 || j == j0) {
+            __syncwarp();
+            S.tab[lane] = next;
+            __syncwarp();
+            next = fetch((j & ~(PM_TBLK - 1)) + PM_TBLK + lane);
+        }
+        const float4 *tj = S.tab + (j & (PM_TBLK - 1));
+        float4 *stage = S.stage[buf] + lane;
+        const float4 *prev = S.stage[buf ^ 1] + rrow;
+        float4 v;
 #pragma unroll
         for (int i = 0; i < PM_CH; i += 2) {
-            const int j = l0 - m + i;
-            const float4 t0 = sT[j], t1 = sT[j + 1];
-            if (inj) pm_step<DIFF, true, NP>(P, l0 + i, t0, t1, Spa, Spb, Sqa, Sqb, Vp0, Vp1, Vq0, Vq1);
-            else pm_step<DIFF, false, NP>(P, l0 + i, t0, t1, Spa, Spb, Sqa, Sqb, Vp0, Vp1, Vq0, Vq1);
-            YPr[i] = YPi[i] = YMr[i] = YMi[i] = YPr[i + 1] = YPi[i + 1] = YMr[i + 1] = YMi[i + 1] = dup(0.f);
+            const float4 w0 = prev[i ^ rc], w1 = prev[(i + 1) ^ rc];
+            pm_step<DIFF, INJ, NP>(P, m + j + i, tj[i], tj[i + 1], Spa, Spb, Sqa, Sqb, Vp0, Vp1, Vq0, Vq1);
+            float2 pr[2], pi[2], mr[2], mi[2];
 #pragma unroll
-            for (int pk = 0; pk < NPK; ++pk) {
-                const PmRing &g = G[pk];
+            for (int k = 0; k < NPK; ++k) {
+                const PmRing &g = G[k];
                 // even l (sigma = +1): YP += mu+ G+N + mu- G+S, YM += mu- G-N + mu+ G-S
-                YPr[i] = __ffma2_rn(Vp0[pk], g.pNr, __ffma2_rn(Vq0[pk], g.pSr, YPr[i]));
-                YPi[i] = __ffma2_rn(Vp0[pk], g.pNi, __ffma2_rn(Vq0[pk], g.pSi, YPi[i]));
-                YMr[i] = __ffma2_rn(Vq0[pk], g.qNr, __ffma2_rn(Vp0[pk], g.qSr, YMr[i]));
-                YMi[i] = __ffma2_rn(Vq0[pk], g.qNi, __ffma2_rn(Vp0[pk], g.qSi, YMi[i]));
+                pr[0] = k ? __ffma2_rn(Vp0[k], g.pNr, pr[0]) : __fmul2_rn(Vp0[k], g.pNr);
+                pi[0] = k ? __ffma2_rn(Vp0[k], g.pNi, pi[0]) : __fmul2_rn(Vp0[k], g.pNi);
+                mr[0] = k ? __ffma2_rn(Vq0[k], g.qNr, mr[0]) : __fmul2_rn(Vq0[k], g.qNr);
+                mi[0] = k ? __ffma2_rn(Vq0[k], g.qNi, mi[0]) : __fmul2_rn(Vq0[k], g.qNi);
+                pr[0] = __ffma2_rn(Vq0[k], g.pSr, pr[0]);
+                pi[0] = __ffma2_rn(Vq0[k], g.pSi, pi[0]);
+                mr[0] = __ffma2_rn(Vp0[k], g.qSr, mr[0]);
+                mi[0] = __ffma2_rn(Vp0[k], g.qSi, mi[0]);
                 // odd l (sigma = -1)
-                YPr[i + 1] = __ffma2_rn(Vp1[pk], g.pNr, __ffma2_rn(neg2(Vq1[pk]), g.pSr, YPr[i + 1]));
-                YPi[i + 1] = __ffma2_rn(Vp1[pk], g.pNi, __ffma2_rn(neg2(Vq1[pk]), g.pSi, YPi[i + 1]));
-                YMr[i + 1] = __ffma2_rn(Vq1[pk], g.qNr, __ffma2_rn(neg2(Vp1[pk]), g.qSr, YMr[i + 1]));
-                YMi[i + 1] = __ffma2_rn(Vq1[pk], g.qNi, __ffma2_rn(neg2(Vp1[pk]), g.qSi, YMi[i + 1]));
+                pr[1] = k ? __ffma2_rn(Vp1[k], g.pNr, pr[1]) : __fmul2_rn(Vp1[k], g.pNr);
+                pi[1] = k ? __ffma2_rn(Vp1[k], g.pNi, pi[1]) : __fmul2_rn(Vp1[k], g.pNi);
+                mr[1] = k ? __ffma2_rn(Vq1[k], g.qNr, mr[1]) : __fmul2_rn(Vq1[k], g.qNr);
+                mi[1] = k ? __ffma2_rn(Vq1[k], g.qNi, mi[1]) : __fmul2_rn(Vq1[k], g.qNi);
+                pr[1] = __ffma2_rn(neg2(Vq1[k]), g.pSr, pr[1]);
+                pi[1] = __ffma2_rn(neg2(Vq1[k]), g.pSi, pi[1]);
+                mr[1] = __ffma2_rn(neg2(Vp1[k]), g.qSr, mr[1]);
+                mi[1] = __ffma2_rn(neg2(Vp1[k]), g.qSi, mi[1]);
             }
-        }
-        float pr[PM_CH], pi[PM_CH], mr[PM_CH], mi[PM_CH];
 #pragma unroll
-        for (int i = 0; i < PM_CH; ++i) {
-            pr[i] = YPr[i].x + YPr[i].y;
-            pi[i] = YPi[i].x + YPi[i].y;
-            mr[i] = YMr[i].x + YMr[i].y;
-            mi[i] = YMi[i].x + YMi[i].y;
+            for (int h = 0; h < 2; ++h)
+                stage[32 * (i + h)] = make_float4(pr[h].x + pr[h].y, pi[h].x + pi[h].y, mr[h].x + mr[h].y, mi[h].x + mi[h].y);
+            v = i ? make_float4(v.x + w0.x, v.y + w0.y, v.z + w0.z, v.w + w0.w) : w0;
+            v = make_float4(v.x + w1.x, v.y + w1.y, v.z + w1.z, v.w + w1.w);
         }
-        pm_rscatter<PM_CH>(pr, pi, lane);
-        pm_rscatter<PM_CH>(mr, mi, lane);
-        constexpr int sh = 2;  // 32 lanes, 8 values: each l ends in 4 lanes
-        if ((lane & ((1 << sh) - 1)) == 0) {
-            const int l = l0 + (lane >> sh);
-            if (l <= L) {
-                atomicAdd(&accP[l - m].x, pr[0]);
-                atomicAdd(&accP[l - m].y, pi[0]);
-                atomicAdd(&accM[l - m].x, mr[0]);
-                atomicAdd(&accM[l - m].y, mi[0]);
-            }
-        }
+        if (j != j0) finish(j - PM_CH, v);
+        __syncwarp();
+        buf ^= 1;
+        j += PM_CH;
+    };
+    while (j < nl && m + j <= lmaxs) chunk(std::true_type{});
+    while (j < nl) chunk(std::false_type{});
+    const float4 *prev = S.stage[buf ^ 1] + rrow;
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int i = 0; i < PM_CH; ++i) {
+        const float4 w = prev[i ^ rc];
+        v = make_float4(v.x + w.x, v.y + w.y, v.z + w.z, v.w + w.w);
     }
+    finish(j - PM_CH, v);
 }
 
-// analysis: CTA per m; warps take groups of 32 x NP ring pairs from a shared
-// counter; chunks of PM_CH values of l are summed over the packs in
-// registers, reduced across the warp and added into FP32 shared
-// accumulators; the epilogue scales by c_l, adds the FP64 block (l < lcm(lc, m))
-// and writes E, B in FP64 (zero outside 2 <= l <= L).  Two CTAs per SM (128
-// registers, a 96-byte spill) measured 17 % faster at nside 1024 than one CTA
-// at 160 registers; chunks of 4 l (118 registers, no spill) and 2 or 8 pairs
-// per lane were slower.
+// analysis: one warp per (group of 32 x NP ring pairs, m); chunks of four l are summed over the
+// lane's pairs in registers, across the warp through shared memory and into psum by FP32
+// reductions in L2.  Bound by the FP32 FMA pipe (12 to 14 operations per (l, pair)).  A CTA per m
+// that took its groups from a counter before: barriers between warps of unequal work, 36 shuffles
+// and 56 selects per 8 l, FP32 atomics in shared memory (compare-and-swap loops).
+// nside 512, lmax 1024 0.219 -> 0.191 + 0.014 ms (the sums alone would take 0.18).  Two pairs per
+// lane 0.208, eight 0.197 to 0.202 ms; 12 warps per SM instead of 16 0.191.
 template <int NP>
-__global__ void __launch_bounds__(PM_THREADS, 2) k_legana_pol_mx(int lmax, int L, int npairs, int lc,
-                                                              const float2 *__restrict__ FQ,
-                                                              const float2 *__restrict__ FU,
-                                                              const float4 *__restrict__ tab,
-                                                              const double *__restrict__ c,
-                                                              const int *__restrict__ ls_tab,
-                                                              const float4 *__restrict__ seed,
-                                                              const float *__restrict__ xp,
-                                                              const float *__restrict__ wp,
-                                                              const double2 *__restrict__ Elow,
-                                                              const double2 *__restrict__ Blow,
-                                                              double2 *__restrict__ Eo, double2 *__restrict__ Bo)
+__global__ void __launch_bounds__(32, 16) k_legana_pol_mx(int lmax, int L, int npairs, const float2 *__restrict__ FQ,
+                                                          const float2 *__restrict__ FU, const float4 *__restrict__ tab,
+                                                          const int *__restrict__ ls_tab, const float4 *__restrict__ seed,
+                                                          const float *__restrict__ xp, const float *__restrict__ wp,
+                                                          float4 *__restrict__ psum)
 {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ int next_group;
-    const int m = blockIdx.x;
-    const int nl = L - m + 1;
-    const int nlp = nl + PM_CH + 2;
+    __shared__ PmAnaShared S;
+    const int m = blockIdx.y, lane = threadIdx.x, nl = L - m + 1;
     const long long base = pmb(lmax, m);
-    float4 *sT = reinterpret_cast<float4 *>(smem_raw);
-    float2 *accP = reinterpret_cast<float2 *>(sT + nlp);
-    float2 *accM = accP + nlp;
-    for (int i = threadIdx.x; i < nlp; i += blockDim.x) {
-        sT[i] = (i < nl) ? tab[base + i] : make_float4(0.f, 0.f, 0.f, 0.f);
-        accP[i] = accM[i] = make_float2(0.f, 0.f);
-    }
-    if (threadIdx.x == 0) next_group = 0;
-    __syncthreads();
-    const int lane = threadIdx.x & 31;
-    const int per_group = 32 * NP;
-    const int ngroups = (npairs + per_group - 1) / per_group;
-    const size_t pstride = (size_t)(lmax + 1) * 2;
-    for (;;) {
-        int grp = 0;
-        if (lane == 0) grp = atomicAdd(&next_group, 1);
-        grp = __shfl_sync(0xffffffffu, grp, 0);
-        if (grp >= ngroups) break;
-        // equator first: the work per pair grows towards the equator (more l above the
-        // first kept one), so handing out the largest groups first shortens the tail at the
-        // barrier before the epilogue
-        const int p0 = (ngroups - 1 - grp) * per_group + lane * NP;
-        PmPairs<NP> P;
-        pm_load_pairs<NP>(P, m, L, npairs, p0, ls_tab, seed, xp, wp);
-        // one recurrence form per warp: the shuffles need warp-uniform control flow
-        P.diff = __shfl_sync(0xffffffffu, P.diff ? 1 : 0, 0) != 0;
-        const int lmin_w = __reduce_min_sync(0xffffffffu, P.lmin);
-        const int lmaxs_w = __reduce_max_sync(0xffffffffu, P.lmaxs);  // one seeding range per warp
-        if (lmin_w > L) continue;
-        float g[8][NP];
+    const int p0 = (gridDim.x - 1 - blockIdx.x) * 32 * NP + lane * NP;  // the equator (most work) first
+    PmPairs<NP> P;
+    pm_load_pairs<NP>(P, m, L, npairs, p0, ls_tab, seed, xp, wp);
+    // one recurrence form per warp: the shuffles need warp-uniform control flow
+    P.diff = __shfl_sync(0xffffffffu, P.diff ? 1 : 0, 0) != 0;
+    const int lmin = __reduce_min_sync(0xffffffffu, P.lmin);
+    const int lmaxs = __reduce_max_sync(0xffffffffu, P.lmaxs);  // one seeding range per warp
+    if (lmin > L) return;
+    PmRing G[NP / 2];
 #pragma unroll
-        for (int k = 0; k < NP; ++k) {
-#pragma unroll
-            for (int q = 0; q < 8; ++q) g[q][k] = 0.f;
-            if (P.ls[k] != PM_BIG) {
-                const size_t o = (size_t)(p0 + k) * pstride + 2 * (size_t)m;
-                const float2 qn = FQ[o], qs = FQ[o + 1], un = FU[o], us = FU[o + 1];
-                g[0][k] = qn.x - un.y;  // G+ north
-                g[1][k] = qn.y + un.x;
-                g[2][k] = qs.x - us.y;  // G+ south
-                g[3][k] = qs.y + us.x;
-                g[4][k] = qn.x + un.y;  // G- north
-                g[5][k] = qn.y - un.x;
-                g[6][k] = qs.x + us.y;  // G- south
-                g[7][k] = qs.y - us.x;
-            }
+    for (int k = 0; k < NP; ++k) {
+        float4 q = make_float4(0.f, 0.f, 0.f, 0.f), u = q;  // north re, im, south re, im
+        if (P.ls[k] != PM_BIG) {
+            const size_t o = ((size_t)(p0 + k) * (lmax + 1) + m) * 2;
+            q = *reinterpret_cast<const float4 *>(FQ + o);
+            u = *reinterpret_cast<const float4 *>(FU + o);
         }
-        PmRing G[NP / 2];
-#pragma unroll
-        for (int pk = 0; pk < NP / 2; ++pk) {
-            G[pk].pNr = make_float2(g[0][2 * pk], g[0][2 * pk + 1]);
-            G[pk].pNi = make_float2(g[1][2 * pk], g[1][2 * pk + 1]);
-            G[pk].pSr = make_float2(g[2][2 * pk], g[2][2 * pk + 1]);
-            G[pk].pSi = make_float2(g[3][2 * pk], g[3][2 * pk + 1]);
-            G[pk].qNr = make_float2(g[4][2 * pk], g[4][2 * pk + 1]);
-            G[pk].qNi = make_float2(g[5][2 * pk], g[5][2 * pk + 1]);
-            G[pk].qSr = make_float2(g[6][2 * pk], g[6][2 * pk + 1]);
-            G[pk].qSi = make_float2(g[7][2 * pk], g[7][2 * pk + 1]);
-        }
-        if (P.diff) pm_ana_run<true, NP>(P, m, L, lmin_w, lmaxs_w, sT, G, accP, accM, lane);
-        else pm_ana_run<false, NP>(P, m, L, lmin_w, lmaxs_w, sT, G, accP, accM, lane);
+        PmRing &g = G[k >> 1];
+        const int h = k & 1;
+        put(g.pNr, h, q.x - u.y);  // G+
+        put(g.pNi, h, q.y + u.x);
+        put(g.pSr, h, q.z - u.w);
+        put(g.pSi, h, q.w + u.z);
+        put(g.qNr, h, q.x + u.y);  // G-
+        put(g.qNi, h, q.y - u.x);
+        put(g.qSr, h, q.z + u.w);
+        put(g.qSi, h, q.w - u.z);
     }
-    __syncthreads();
-    const bool low = Elow && m < lc;
-    const int llim = low ? lcm_of(lc, m) : 0;
-    for (int j = threadIdx.x; j <= lmax - m; j += blockDim.x) {
-        const int l = m + j;
-        double2 e = make_double2(0.0, 0.0), b = e;
-        if (l >= 2 && l <= L) {
-            if (l < llim) {
-                e = Elow[base + j];
-                b = Blow[base + j];
-            } else {
-                const double cc = c[base + j];
-                const double ypr = accP[j].x, ypi = accP[j].y, ymr = accM[j].x, ymi = accM[j].y;
-                e = make_double2(-cc * (ypr + ymr), -cc * (ypi + ymi));
-                b = make_double2(-cc * (ypi - ymi), cc * (ypr - ymr));
-            }
+    float *dst = &psum[base].x;
+    const int j0 = (lmin - m) & ~(PM_CH - 1);
+    if (P.diff) pm_ana_run<true, NP>(P, m, nl, j0, lmaxs, tab + base, G, S, dst, lane);
+    else pm_ana_run<false, NP>(P, m, nl, j0, lmaxs, tab + base, G, S, dst, lane);
+}
+
+// E, B in FP64 (zero outside 2 <= l <= L) from the sums, scaled by c_l, and the FP64 block
+// (l < lcm(lc, m)); clears the sums for the next launch
+__global__ void __launch_bounds__(128) k_ana_pol_epilogue(int lmax, int L, int lc, const double *__restrict__ c,
+                                                          const double2 *__restrict__ Elow,
+                                                          const double2 *__restrict__ Blow, double2 *__restrict__ Eo,
+                                                          double2 *__restrict__ Bo, float4 *__restrict__ psum)
+{
+    const int m = blockIdx.y, j = blockIdx.x * blockDim.x + threadIdx.x, l = m + j;
+    if (l > lmax) return;
+    const long long i = pmb(lmax, m) + j;
+    const int llim = Elow && m < lc ? lcm_of(lc, m) : 0;
+    double2 e = make_double2(0.0, 0.0), b = e;
+    if (l <= L) {
+        const float4 y = psum[i];
+        psum[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (l >= 2 && l < llim) {
+            e = Elow[i];
+            b = Blow[i];
+        } else if (l >= 2) {
+            const double cc = c[i];
+            const double ypr = widen(y.x), ypi = widen(y.y), ymr = widen(y.z), ymi = widen(y.w);
+            e = make_double2(-cc * (ypr + ymr), -cc * (ypi + ymi));
+            b = make_double2(-cc * (ypi - ymi), cc * (ypr - ymr));
         }
-        Eo[base + j] = e;
-        Bo[base + j] = b;
     }
+    Eo[i] = e;
+    Bo[i] = b;
 }
 
 template <int NP> size_t syn_pm_smem(int L, int m0) { return (size_t)2 * (L - m0 + 3) * sizeof(float4) + 16; }
-size_t ana_pm_smem(int L) { return (size_t)(L + 1 + PM_CH + 2) * (sizeof(float4) + 2 * sizeof(float2)) + 16; }
 
 constexpr int SYN_NP = 4;  // ring pairs per thread (synthesis)
 constexpr int ANA_NP = 4;  // ring pairs per lane (analysis)
@@ -615,14 +594,15 @@ wf_status hp_pol_create_mx(wf_plan p)
     if ((st = plan_alloc(p, (void **)&s->seed, ns * sizeof(float4))) != WF_OK) return st;
     if ((st = plan_alloc(p, (void **)&s->Elow, nalm * sizeof(double2))) != WF_OK) return st;
     if ((st = plan_alloc(p, (void **)&s->Blow, nalm * sizeof(double2))) != WF_OK) return st;
+    if ((st = plan_alloc(p, (void **)&s->psum, nalm * sizeof(float4))) != WF_OK) return st;
+    WF_CUDA(cudaMemsetAsync(s->psum, 0, nalm * sizeof(float4), p->stream));
     if ((st = to_device(p, s->c, c.data(), nalm * sizeof(double))) != WF_OK) return st;
     if ((st = to_device(p, s->tab, tab.data(), nalm * sizeof(float4))) != WF_OK) return st;
     if (tc_prec(p->prec) && (st = plan_alloc(p, (void **)&s->ac32, nalm * sizeof(float4))) != WF_OK) return st;
     s->lc = -1;
     if ((st = hp_pol_set_low_block(p, 0)) != WF_OK) return st;
-    const size_t syn_max = syn_pm_smem<SYN_NP>(lmax, 0), ana_max = ana_pm_smem(lmax);
+    const size_t syn_max = syn_pm_smem<SYN_NP>(lmax, 0);
     if ((st = raise_smem_limit((const void *)k_legsyn_pol_mx<SYN_NP>, syn_max)) != WF_OK) return st;
-    if ((st = raise_smem_limit((const void *)k_legana_pol_mx<ANA_NP>, ana_max)) != WF_OK) return st;
     return WF_OK;
 }
 
@@ -686,9 +666,13 @@ wf_status hp_pol_legendre_analysis_mx(wf_plan p, int L, double2 *E, double2 *B)
     if (low && (st = hp_pol_legendre_analysis_low(p, L, s->lc, (const float2 *)s->FQ, (const float2 *)s->FU,
                                                   s->Elow, s->Blow)) != WF_OK)
         return st;
-    k_legana_pol_mx<ANA_NP><<<L + 1, PM_THREADS, ana_pm_smem(L), p->stream>>>(
-        p->lmax, L, p->npairs, s->lc, (const float2 *)s->FQ, (const float2 *)s->FU, s->tab, s->c, s->ls_mx, s->seed,
-        t.x32, t.w32, low ? s->Elow : nullptr, low ? s->Blow : nullptr, E, B);
+    const int per_warp = 32 * ANA_NP;
+    k_legana_pol_mx<ANA_NP><<<dim3((p->npairs + per_warp - 1) / per_warp, L + 1), 32, 0, p->stream>>>(
+        p->lmax, L, p->npairs, (const float2 *)s->FQ, (const float2 *)s->FU, s->tab, s->ls_mx, s->seed, t.x32, t.w32,
+        s->psum);
+    WF_COUNT_LAUNCH(p);
+    k_ana_pol_epilogue<<<dim3((p->lmax + 128) / 128, L + 1), 128, 0, p->stream>>>(p->lmax, L, s->lc, s->c, low ? s->Elow : nullptr,
+                                                     low ? s->Blow : nullptr, E, B, s->psum);
     WF_COUNT_LAUNCH(p);
     WF_CUDA(cudaGetLastError());
     if (L < p->lmax) {
