@@ -546,8 +546,8 @@ __device__ __forceinline__ void df_add(float &ahi, float &alo, float bhi, float 
 // FP64 value split into (hi, lo) floats
 __device__ __forceinline__ float2 df_split(double v)
 {
-    const float hi = (float)v;
-    return make_float2(hi, (float)(v - (double)hi));
+    const float hi = narrow(v);
+    return make_float2(hi, narrow(v - widen(hi)));
 }
 
 __host__ __device__ inline int low_rows(int lmax, int lc, int m) { return min(lcm_of(lc, m), lmax + 1) - m; }
@@ -749,223 +749,186 @@ __device__ __forceinline__ void df_sub(float ah, float al, float bh, float bl, f
     sl = __fsub_rn(e, __fsub_rn(sh, s));
 }
 
-// one recurrence step mu_l = A_l x mu_{l-1} - mu_{l-2} in double-float
-__device__ __forceinline__ void df_step(float2 Al, float xh, float xl, float m1h, float m1l, float &m0h, float &m0l)
+// (E_k, O_k) to k + 1 in double-float, odd values carried as x mu as in the FP64 kernels
+// (A = (A_{2k+2} hi, lo, A_{2k+3} hi, lo), X = x^2): 17 operations per l, 19 with x in each step
+__device__ __forceinline__ void df_advance(float4 A, float2 X, float2 &E, float2 &O)
 {
-    float th, tl, uh, ul;
-    df_mul(Al.x, Al.y, xh, xl, th, tl);
-    df_mul(th, tl, m1h, m1l, uh, ul);
-    df_sub(uh, ul, m0h, m0l, m0h, m0l);
+    float uh, ul, ch, cl;
+    df_mul(A.x, A.y, O.x, O.y, uh, ul);
+    df_sub(uh, ul, E.x, E.y, E.x, E.y);
+    df_mul(A.z, A.w, X.x, X.y, ch, cl);
+    df_mul(ch, cl, E.x, E.y, uh, ul);
+    df_sub(uh, ul, O.x, O.y, O.x, O.y);
 }
 
-__device__ __forceinline__ double df_val(float h, float l) { return (double)h + (double)l; }
+__device__ __forceinline__ double df_val(float h, float l) { return widen(h) + widen(l); }
 
-// synthesis: CTA per (m, block of pairs), thread per pair, as the FP64 kernel
+// synthesis: CTA per (m, block of pairs, the equator first), thread per pair.  nside 512, lmax 1024
+// 0.927 -> 0.697 ms: a CTA that took four blocks of an m in turn left all CTAs resident at once and
+// the SMs unevenly loaded; the two-step form and conversions on the bits are the rest.
 __global__ void __launch_bounds__(LEG_THREADS) k_legsyn_df(int lmax, int L, int npairs,
                                                            const double2 *__restrict__ alm, const double *__restrict__ A,
                                                            const double *__restrict__ c64,
                                                            const int *__restrict__ ls_tab,
                                                            const double *__restrict__ s0_tab,
                                                            const double *__restrict__ s1_tab,
-                                                           const double *__restrict__ xp, double2 *__restrict__ G)
+                                                           const double4 *__restrict__ xw, double2 *__restrict__ G)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int m = blockIdx.y;
-    const int nl = L - m + 1;
+    const int nl = L - m + 1, nk = (nl + 1) >> 1;
     const long long base = mbase(lmax, m);
     float4 *sac = reinterpret_cast<float4 *>(smem_raw);  // c a_lm as (re hi, re lo, im hi, im lo)
-    float2 *sA = reinterpret_cast<float2 *>(sac + (nl + 2));
-    for (int i = threadIdx.x; i < nl + 2; i += blockDim.x) {
+    float4 *sA = sac + 2 * nk;                           // per k: A_{2k+2} and A_{2k+3} as (hi, lo)
+    for (int i = threadIdx.x; i < 2 * nk; i += blockDim.x) {
         float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        float2 a = make_float2(0.f, 0.f);
         if (i < nl) {
-            const double2 q = alm[base + i];
-            const double cc = c64[base + i];
-            const float2 re = df_split(q.x * cc), im = df_split(q.y * cc);
+            const double2 q = cscale(alm[base + i], c64[base + i]);
+            const float2 re = df_split(q.x), im = df_split(q.y);
             v = make_float4(re.x, re.y, im.x, im.y);
-            a = df_split(A[base + i]);
         }
         sac[i] = v;
-        sA[i] = a;
+        reinterpret_cast<float2 *>(sA)[i] = i + 2 < nl ? df_split(A[base + i + 2]) : make_float2(0.f, 0.f);
     }
     __syncthreads();
-    for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < npairs; p += gridDim.x * blockDim.x) {
-        const size_t sidx = (size_t)m * npairs + p;
-        const int ls = ls_tab[sidx];
-        float erh = 0.f, erl = 0.f, eih = 0.f, eil = 0.f, orh = 0.f, orl = 0.f, oih = 0.f, oil = 0.f;
-        if (ls <= L) {
-            const float2 x = df_split(xp[p]), s0 = df_split(s0_tab[sidx]), s1 = df_split(s1_tab[sidx]);
-            float m0h = s0.x, m0l = s0.y, m1h = s1.x, m1l = s1.y;
-            int i = ls - m;
-            float4 a0 = sac[i], a1 = sac[i + 1];
-            df_fma(erh, erl, a0.x, a0.y, m0h, m0l);
-            df_fma(eih, eil, a0.z, a0.w, m0h, m0l);
-            df_fma(orh, orl, a1.x, a1.y, m1h, m1l);
-            df_fma(oih, oil, a1.z, a1.w, m1h, m1l);
-            for (i += 2; i < nl; i += 2) {
-                df_step(sA[i], x.x, x.y, m1h, m1l, m0h, m0l);
-                a0 = sac[i];
-                df_fma(erh, erl, a0.x, a0.y, m0h, m0l);
-                df_fma(eih, eil, a0.z, a0.w, m0h, m0l);
-                df_step(sA[i + 1], x.x, x.y, m0h, m0l, m1h, m1l);
-                a1 = sac[i + 1];
-                df_fma(orh, orl, a1.x, a1.y, m1h, m1l);
-                df_fma(oih, oil, a1.z, a1.w, m1h, m1l);
-            }
+    const int p = (gridDim.x - 1 - blockIdx.x) * LEG_THREADS + threadIdx.x;
+    if (p >= npairs) return;
+    const size_t sidx = (size_t)m * npairs + p;
+    const int ls = ls_tab[sidx];
+    float erh = 0.f, erl = 0.f, eih = 0.f, eil = 0.f, orh = 0.f, orl = 0.f, oih = 0.f, oil = 0.f;
+    const double4 x = xw[p];
+    if (ls <= L) {
+        const float2 X = df_split(x.x);
+        float2 E = df_split(s0_tab[sidx]), O = df_split(x.z * s1_tab[sidx]);
+        for (int k = (ls - m) >> 1; k < nk; ++k) {
+            const float4 a0 = sac[2 * k], a1 = sac[2 * k + 1];
+            df_fma(erh, erl, a0.x, a0.y, E.x, E.y);
+            df_fma(eih, eil, a0.z, a0.w, E.x, E.y);
+            df_fma(orh, orl, a1.x, a1.y, O.x, O.y);
+            df_fma(oih, oil, a1.z, a1.w, O.x, O.y);
+            df_advance(sA[k], X, E, O);
         }
-        const double er = df_val(erh, erl), ei = df_val(eih, eil), orr = df_val(orh, orl), oi = df_val(oih, oil);
-        double2 *g = G + ((size_t)p * (lmax + 1) + m) * 2;
-        g[0] = make_double2(er + orr, ei + oi);
-        g[1] = make_double2(er - orr, ei - oi);
     }
+    const double er = df_val(erh, erl), ei = df_val(eih, eil);
+    const double orr = x.w * df_val(orh, orl), oi = x.w * df_val(oih, oil);
+    double2 *g = G + ((size_t)p * (lmax + 1) + m) * 2;
+    g[0] = make_double2(er + orr, ei + oi);
+    g[1] = make_double2(er - orr, ei - oi);
 }
 
-// analysis: CTA per m; a warp covers 32 lanes x DFP ring pairs taken dynamically,
-// equator first; chunks of 8 values of l are summed over the lane's pairs in
-// double-float, across the warp through a swizzled shared stage (as in the mixed
-// analysis, with (hi, lo) of the real and imaginary parts per slot and double-float
-// additions), and added into FP64 shared accumulators.
+// analysis: one warp per (group of 32 x DFP ring pairs, m); chunks of 8 values of l are summed
+// over the lane's pairs in double-float, across the warp through a swizzled shared stage (with
+// (hi, lo) of the real and imaginary parts per slot and double-float additions), and times c_l
+// added in FP64 to acc (zero before).  nside 512, lmax 1024 0.888 -> 0.818 ms (a CTA per m before:
+// warps without a group waited at the barrier before the epilogue).  Bound by FP32 issue, four
+// warps per scheduler.  The loop over k stays rolled: unrolled four times with a second copy for
+// the starting steps it took 1.03 ms (instruction fetch).  Twenty warps per SM at 96 registers:
+// 0.91 ms; two pairs per lane: 0.98.
 constexpr int DFP = 4;
 
-template <bool INJ>
-__device__ __forceinline__ void df_ana_pair_step(int l, const int (&ls)[DFP], const float2 (&s0)[DFP],
-                                                 const float2 (&s1)[DFP], const float2 (&x)[DFP], float2 A0, float2 A1,
-                                                 float2 (&m0)[DFP], float2 (&m1)[DFP])
-{
-#pragma unroll
-    for (int k = 0; k < DFP; ++k) {
-        df_step(A0, x[k].x, x[k].y, m1[k].x, m1[k].y, m0[k].x, m0[k].y);
-        df_step(A1, x[k].x, x[k].y, m0[k].x, m0[k].y, m1[k].x, m1[k].y);
-        if (INJ && l == ls[k]) {
-            m0[k] = s0[k];
-            m1[k] = s1[k];
-        }
-    }
-}
-
-__global__ void __launch_bounds__(LEG_THREADS, 2) k_legana_df(int lmax, int L, int npairs,
-                                                           const double2 *__restrict__ F, const double *__restrict__ A,
-                                                           const int *__restrict__ ls_tab,
-                                                           const double *__restrict__ s0_tab,
-                                                           const double *__restrict__ s1_tab,
-                                                           const double *__restrict__ xp,
-                                                           const double *__restrict__ c64, int mode, double omega,
-                                                           BlendArgs ba, const double2 *__restrict__ a_old,
-                                                           double2 *__restrict__ out, double *__restrict__ part)
+__global__ void __launch_bounds__(32, 16) k_legana_df(int lmax, int L, int npairs, const double2 *__restrict__ F,
+                                                      const double *__restrict__ A, const int *__restrict__ ls_tab,
+                                                      const double *__restrict__ s0_tab,
+                                                      const double *__restrict__ s1_tab,
+                                                      const double4 *__restrict__ xw, const double *__restrict__ c64,
+                                                      double2 *__restrict__ acc)
 {
     constexpr int CH = 8;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ int next_group;
-    const int m = blockIdx.x;
+    __shared__ float4 sA[F64_BLK / 2];  // per k: A_{2k+2} and A_{2k+3} as (hi, lo)
+    __shared__ float4 wst[CH * 32];     // 8 rows x 32 lanes of (re hi, lo, im hi, lo)
+    const int m = blockIdx.y, lane = threadIdx.x;
     const int nl = L - m + 1;
-    const int nlp = nl + CH + 2;
     const long long base = mbase(lmax, m);
-    double2 *acc = reinterpret_cast<double2 *>(smem_raw);
-    float4 *sAA = reinterpret_cast<float4 *>(acc + nlp);   // (A_l hi, lo, A_l+1 hi, lo) from l - m = 0, even
-    float4 *stage = sAA + (nlp + 1) / 2;                      // per warp: 8 rows x 32 lanes of (re hi, lo, im hi, lo)
-    for (int i = threadIdx.x; i < nlp; i += blockDim.x) acc[i] = make_double2(0.0, 0.0);
-    for (int i = threadIdx.x; i < (nlp + 1) / 2; i += blockDim.x) {
-        const int j = 2 * i;
-        const float2 a0 = j < nl ? df_split(A[base + j]) : make_float2(0.f, 0.f);
-        const float2 a1 = j + 1 < nl ? df_split(A[base + j + 1]) : make_float2(0.f, 0.f);
-        sAA[i] = make_float4(a0.x, a0.y, a1.x, a1.y);
-    }
-    if (threadIdx.x == 0) next_group = 0;
-    __syncthreads();
-    const int lane = threadIdx.x & 31;
-    float4 *wst = stage + (threadIdx.x >> 5) * 256;
-    const int per_group = 32 * DFP;
-    const int ngroups = (npairs + per_group - 1) / per_group;
-    const size_t pstride = (size_t)(lmax + 1) * 2;
-    for (;;) {
-        int grp = 0;
-        if (lane == 0) grp = atomicAdd(&next_group, 1);
-        grp = __shfl_sync(0xffffffffu, grp, 0);
-        if (grp >= ngroups) break;
-        const int p0 = (ngroups - 1 - grp) * per_group + lane * DFP;
-        int ls[DFP];
-        float2 s0[DFP], s1[DFP], x[DFP], m0[DFP], m1[DFP], fer[DFP], fei[DFP], forr[DFP], foi[DFP];
-        int lmin = BIG, lmaxs = -1;
+    const int p0 = (gridDim.x - 1 - blockIdx.x) * 32 * DFP + lane * DFP;  // the equator (most work) first
+    int k0[DFP], kmin = BIG, kmaxs = -1;
+    float2 s0[DFP], s1[DFP], X[DFP], E[DFP], O[DFP], fer[DFP], fei[DFP], forr[DFP], foi[DFP];
 #pragma unroll
-        for (int k = 0; k < DFP; ++k) {
-            const int p = p0 + k;
-            ls[k] = BIG;
-            s0[k] = s1[k] = x[k] = m0[k] = m1[k] = make_float2(0.f, 0.f);
-            fer[k] = fei[k] = forr[k] = foi[k] = make_float2(0.f, 0.f);
-            if (p < npairs) {
-                const size_t sidx = (size_t)m * npairs + p;
-                const int l0 = ls_tab[sidx];
-                if (l0 <= L) {
-                    ls[k] = l0;
-                    s0[k] = df_split(s0_tab[sidx]);
-                    s1[k] = df_split(s1_tab[sidx]);
-                    x[k] = df_split(xp[p]);
-                    const double2 *f = F + (size_t)p * pstride + 2 * (size_t)m;
-                    const double2 fn = f[0], fs = f[1];
-                    fer[k] = df_split(fn.x + fs.x);
-                    fei[k] = df_split(fn.y + fs.y);
-                    forr[k] = df_split(fn.x - fs.x);
-                    foi[k] = df_split(fn.y - fs.y);
-                    lmin = min(lmin, l0);
-                    lmaxs = max(lmaxs, l0);
-                }
+    for (int i = 0; i < DFP; ++i) {
+        const int p = p0 + i;
+        k0[i] = BIG;
+        s0[i] = s1[i] = X[i] = E[i] = O[i] = make_float2(0.f, 0.f);
+        fer[i] = fei[i] = forr[i] = foi[i] = make_float2(0.f, 0.f);
+        if (p < npairs) {
+            const size_t sidx = (size_t)m * npairs + p;
+            const int ls = ls_tab[sidx];
+            if (ls <= L) {
+                const double4 x = xw[p];
+                k0[i] = (ls - m) >> 1;
+                s0[i] = df_split(s0_tab[sidx]);
+                s1[i] = df_split(x.z * s1_tab[sidx]);
+                X[i] = df_split(x.x);
+                const double2 *f = F + ((size_t)p * (lmax + 1) + m) * 2;
+                const double2 fn = f[0], fs = f[1];
+                fer[i] = df_split(fn.x + fs.x);
+                fei[i] = df_split(fn.y + fs.y);
+                forr[i] = df_split((fn.x - fs.x) * x.w);
+                foi[i] = df_split((fn.y - fs.y) * x.w);
+                kmin = min(kmin, k0[i]);
+                kmaxs = max(kmaxs, k0[i]);
             }
         }
-        const int lmin_w = __reduce_min_sync(0xffffffffu, lmin);
-        const int lmaxs_w = __reduce_max_sync(0xffffffffu, lmaxs);
-        if (lmin_w > L) continue;
-        for (int l0 = lmin_w; l0 <= L; l0 += CH) {
-            const bool inj = l0 <= lmaxs_w;
-#pragma unroll
-            for (int i = 0; i < CH; i += 2) {
-                const float4 aa = sAA[(l0 - m + i) >> 1];  // l0 - m is even
-                if (inj) df_ana_pair_step<true>(l0 + i, ls, s0, s1, x, make_float2(aa.x, aa.y), make_float2(aa.z, aa.w), m0, m1);
-                else df_ana_pair_step<false>(l0 + i, ls, s0, s1, x, make_float2(aa.x, aa.y), make_float2(aa.z, aa.w), m0, m1);
-                float r0h = 0.f, r0l = 0.f, i0h = 0.f, i0l = 0.f, r1h = 0.f, r1l = 0.f, i1h = 0.f, i1l = 0.f;
-#pragma unroll
-                for (int k = 0; k < DFP; ++k) {
-                    df_fma(r0h, r0l, fer[k].x, fer[k].y, m0[k].x, m0[k].y);
-                    df_fma(i0h, i0l, fei[k].x, fei[k].y, m0[k].x, m0[k].y);
-                    df_fma(r1h, r1l, forr[k].x, forr[k].y, m1[k].x, m1[k].y);
-                    df_fma(i1h, i1l, foi[k].x, foi[k].y, m1[k].x, m1[k].y);
-                }
-                wst[stage_slot(i, lane)] = make_float4(r0h, r0l, i0h, i0l);
-                wst[stage_slot(i + 1, lane)] = make_float4(r1h, r1l, i1h, i1l);
-            }
+    }
+    kmin = __reduce_min_sync(0xffffffffu, kmin);
+    kmaxs = __reduce_max_sync(0xffffffffu, kmaxs);
+    if (kmin == BIG) return;
+    const int nk = (nl + 1) >> 1;
+    int k = kmin & ~(CH / 2 - 1);
+    auto fetch = [&](int kb) { return 2 * kb + lane + 2 < nl ? A[base + 2 * kb + lane + 2] : 0.0; };
+    double nA = fetch(k & ~(F64_BLK / 2 - 1));
+    while (k < nk) {
+        if ((k & (F64_BLK / 2 - 1)) == 0 || k == (kmin & ~(CH / 2 - 1))) {
             __syncwarp();
-            {
-                const int i = lane >> 2, q = lane & 3;
-                const float4 *row = wst + 32 * i + 8 * q;
-                const int c = q + 4 * (i & 1);
-                float4 v = row[c];
-                float rh = v.x, rl = v.y, ih = v.z, il = v.w;
+            reinterpret_cast<float2 *>(sA)[lane] = df_split(nA);
+            __syncwarp();
+            nA = fetch((k & ~(F64_BLK / 2 - 1)) + F64_BLK / 2);
+        }
+#pragma unroll 1
+        for (int j = 0; j < CH / 2; ++j) {
+            if (k + j <= kmaxs) {
 #pragma unroll
-                for (int j = 1; j < 8; ++j) {
-                    v = row[j ^ c];
-                    df_add(rh, rl, v.x, v.y);
-                    df_add(ih, il, v.z, v.w);
-                }
-#pragma unroll
-                for (int o = 1; o <= 2; o <<= 1) {
-                    const float a = __shfl_xor_sync(0xffffffffu, rh, o), b = __shfl_xor_sync(0xffffffffu, rl, o);
-                    const float cc = __shfl_xor_sync(0xffffffffu, ih, o), d = __shfl_xor_sync(0xffffffffu, il, o);
-                    df_add(rh, rl, a, b);
-                    df_add(ih, il, cc, d);
-                }
-                if (q == 0) {
-                    const int l = l0 + i;
-                    if (l <= L) {
-                        atomicAdd(&acc[l - m].x, df_val(rh, rl));
-                        atomicAdd(&acc[l - m].y, df_val(ih, il));
+                for (int i = 0; i < DFP; ++i)
+                    if (k + j == k0[i]) {
+                        E[i] = s0[i];
+                        O[i] = s1[i];
                     }
-                }
             }
-            __syncwarp();
+            const float4 a = sA[(k & (F64_BLK / 2 - 1)) + j];
+            float r0h = 0.f, r0l = 0.f, i0h = 0.f, i0l = 0.f, r1h = 0.f, r1l = 0.f, i1h = 0.f, i1l = 0.f;
+#pragma unroll
+            for (int i = 0; i < DFP; ++i) {
+                df_fma(r0h, r0l, fer[i].x, fer[i].y, E[i].x, E[i].y);
+                df_fma(i0h, i0l, fei[i].x, fei[i].y, E[i].x, E[i].y);
+                df_fma(r1h, r1l, forr[i].x, forr[i].y, O[i].x, O[i].y);
+                df_fma(i1h, i1l, foi[i].x, foi[i].y, O[i].x, O[i].y);
+                df_advance(a, X[i], E[i], O[i]);
+            }
+            wst[stage_slot(2 * j, lane)] = make_float4(r0h, r0l, i0h, i0l);
+            wst[stage_slot(2 * j + 1, lane)] = make_float4(r1h, r1l, i1h, i1l);
         }
+        __syncwarp();
+        const int i = lane >> 2, q = lane & 3;
+        const float4 *row = wst + 32 * i + 8 * q;
+        const int c = q + 4 * (i & 1);
+        float4 v = row[c];
+        float rh = v.x, rl = v.y, ih = v.z, il = v.w;
+#pragma unroll
+        for (int j = 1; j < 8; ++j) {
+            v = row[j ^ c];
+            df_add(rh, rl, v.x, v.y);
+            df_add(ih, il, v.z, v.w);
+        }
+#pragma unroll
+        for (int o = 1; o <= 2; o <<= 1) {
+            const float a = __shfl_xor_sync(0xffffffffu, rh, o), b = __shfl_xor_sync(0xffffffffu, rl, o);
+            const float cc = __shfl_xor_sync(0xffffffffu, ih, o), d = __shfl_xor_sync(0xffffffffu, il, o);
+            df_add(rh, rl, a, b);
+            df_add(ih, il, cc, d);
+        }
+        const int j = 2 * k + i;
+        if (q < 2 && j < nl) atomicAdd(q ? &acc[base + j].y : &acc[base + j].x, c64[base + j] * (q ? df_val(ih, il) : df_val(rh, rl)));
+        __syncwarp();
+        k += CH / 2;
     }
-    __syncthreads();
-    auto val = [&](int j) { return cscale(acc[j], c64[base + j]); };
-    blend_epilogue(lmax, L, m, base, mode, ba, val, a_old, out, part, reinterpret_cast<double (*)[LEG_THREADS]>(stage));
 }
 
 // ---------------------------------------------------------------------------
@@ -1481,20 +1444,14 @@ wf_status launch_lowana_df(wf_plan p, int L, const float2 *F, double2 *out, cuda
 }
 
 // double-float transforms of a sweep sub-plan (FP64 plan, G and F in FP64)
-size_t syn_df_smem(int L) { return (size_t)(L + 3) * (sizeof(float4) + sizeof(float2)) + 16; }
-size_t ana_df_smem(int L)
-{
-    const size_t nlp = (size_t)L + 1 + 8 + 2;
-    return nlp * sizeof(double2) + ((nlp + 1) / 2) * sizeof(float4) + (size_t)LEG_THREADS * 8 * sizeof(float4) + 32;
-}
+size_t syn_df_smem(int L) { return (size_t)((L + 2) / 2) * 3 * sizeof(float4); }
 
 wf_status launch_syn_df(wf_plan p, const double2 *alm, int L)
 {
     const HpTables &t = p->tab;
-    const int gx = (p->npairs + 4 * LEG_THREADS - 1) / (4 * LEG_THREADS);
-    const size_t sm = syn_df_smem(L);
-    k_legsyn_df<<<dim3(gx, L + 1), LEG_THREADS, sm, p->stream>>>(p->lmax, L, p->npairs, alm, t.A64, t.c64, t.ls, t.s0_64,
-                                                                 t.s1_64, t.x64, (double2 *)p->ws.G);
+    const dim3 grid((p->npairs + LEG_THREADS - 1) / LEG_THREADS, L + 1);
+    k_legsyn_df<<<grid, LEG_THREADS, syn_df_smem(L), p->stream>>>(p->lmax, L, p->npairs, alm, t.A64, t.c64, t.ls, t.s0_64,
+                                                                  t.s1_64, t.xw64, (double2 *)p->ws.G);
     WF_COUNT_LAUNCH(p);
     WF_CUDA(cudaGetLastError());
     return WF_OK;
@@ -1503,10 +1460,11 @@ wf_status launch_syn_df(wf_plan p, const double2 *alm, int L)
 wf_status launch_ana_df(wf_plan p, int L, LegMode mode, const BlendArgs &ba, const double2 *a_old, double2 *out)
 {
     const HpTables &t = p->tab;
-    const size_t sm = ana_df_smem(L);
-    k_legana_df<<<L + 1, LEG_THREADS, sm, p->stream>>>(p->lmax, L, p->npairs, (const double2 *)p->ws.F, t.A64, t.ls,
-                                                       t.s0_64, t.s1_64, t.x64, t.c64, (int)mode, p->omega, ba, a_old,
-                                                       out, p->ws.part_harm);
+    const dim3 grid((p->npairs + 32 * DFP - 1) / (32 * DFP), L + 1);
+    k_legana_df<<<grid, 32, 0, p->stream>>>(p->lmax, L, p->npairs, (const double2 *)p->ws.F, t.A64, t.ls, t.s0_64,
+                                            t.s1_64, t.xw64, t.c64, t.acc64);
+    WF_COUNT_LAUNCH(p);
+    k_ana64_epilogue<<<L + 1, 128, 0, p->stream>>>(p->lmax, L, (int)mode, ba, a_old, out, p->ws.part_harm, t.acc64);
     WF_COUNT_LAUNCH(p);
     WF_CUDA(cudaGetLastError());
     return WF_OK;
@@ -1704,7 +1662,6 @@ wf_status hp_build_legendre_tables(wf_plan p, const std::vector<double> &xpair, 
         }
     } else {
         if ((st = raise_smem_limit((const void *)k_legsyn_df, syn_df_smem(lmax))) != WF_OK) return st;
-        if ((st = raise_smem_limit((const void *)k_legana_df, ana_df_smem(lmax))) != WF_OK) return st;
     }
     WF_CUDA(cudaStreamSynchronize(p->stream));
     return WF_OK;
