@@ -445,6 +445,8 @@ __device__ double eigmin3(const Sym3 &s)
     return q + 2.0 * pp * cos(phi + 2.0 * M_PI / 3.0);
 }
 
+__device__ __forceinline__ bool nonzero(double v) { return (__double_as_longlong(v) << 1) != 0; }
+
 // v > 0 (infinity included), by its bits
 __device__ __forceinline__ bool positive(double v)
 {
@@ -703,15 +705,16 @@ __device__ __forceinline__ void pinv_te(const Prior &S, double &it, double &ie, 
 {
     const double det = S.tt * S.ee - S.te * S.te;
     if (S.tt > 0.0 && S.ee > 0.0 && det > 0.0) {
-        it = S.ee / det;
-        ie = S.tt / det;
-        ix = -S.te / det;
+        const double id = inverse(det);
+        it = S.ee * id;
+        ie = S.tt * id;
+        ix = -S.te * id;
     } else {
-        it = S.tt > 0.0 ? 1.0 / S.tt : 0.0;
-        ie = S.ee > 0.0 ? 1.0 / S.ee : 0.0;
+        it = S.tt > 0.0 ? inverse(S.tt) : 0.0;
+        ie = S.ee > 0.0 ? inverse(S.ee) : 0.0;
         ix = 0.0;
     }
-    ib = S.bb > 0.0 ? 1.0 / S.bb : 0.0;
+    ib = S.bb > 0.0 ? inverse(S.bb) : 0.0;
 }
 
 // sum w a^H S^+ a (mode 0) or sum w |P b|^2 with P the projector on the range of S (mode 1), per m
@@ -727,16 +730,16 @@ __global__ void k_pol_alm_norm(int lmax, const double *__restrict__ C, const dou
         const long long k = base + (l - m);
         const double2 aT = a[k], aE = a[nalm + k], aB = a[2 * nalm + k];
         const Prior S = prior(C, lmax, l);
-        double it, ie, ix, ib;
-        pinv_te(S, it, ie, ix, ib);
         if (mode == 0) {
+            double it, ie, ix, ib;
+            pinv_te(S, it, ie, ix, ib);
             const double re = it * (aT.x * aT.x + aT.y * aT.y) + ie * (aE.x * aE.x + aE.y * aE.y) +
                               2.0 * ix * (aT.x * aE.x + aT.y * aE.y) + ib * (aB.x * aB.x + aB.y * aB.y);
-            acc += wm * re;
+            acc += re;
         } else {
             // projector: identity on the active components (a singular TE block has one active axis)
             const bool t = S.tt > 0.0, e = S.ee > 0.0, b = S.bb > 0.0;
-            acc += wm * ((t ? aT.x * aT.x + aT.y * aT.y : 0.0) + (e ? aE.x * aE.x + aE.y * aE.y : 0.0) +
+            acc += ((t ? aT.x * aT.x + aT.y * aT.y : 0.0) + (e ? aE.x * aE.x + aE.y * aE.y : 0.0) +
                          (b ? aB.x * aB.x + aB.y * aB.y : 0.0));
         }
     }
@@ -746,7 +749,7 @@ __global__ void k_pol_alm_norm(int lmax, const double *__restrict__ C, const dou
     if (threadIdx.x == 0) {
         double s = 0.0;
         for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[w];
-        part[m] = s;
+        part[m] = wm * s;
     }
 }
 
@@ -799,14 +802,14 @@ __global__ void k_hblend_pol(int lmax, int L, long long nalm, const double4 *__r
         }
         const double2 oT = a_old[k], oE = a_old[nalm + k], oB = a_old[2 * nalm + k];
         const double it = T1.y, ie = T1.z, ix = T1.w, ib = T2.x;
-        chi += wm * (it * (oT.x * oT.x + oT.y * oT.y) + ie * (oE.x * oE.x + oE.y * oE.y) +
+        chi += (it * (oT.x * oT.x + oT.y * oT.y) + ie * (oE.x * oE.x + oE.y * oE.y) +
                      2.0 * ix * (oT.x * oE.x + oT.y * oE.y) + ib * (oB.x * oB.x + oB.y * oB.y));
         if (want_resid) {
             const double2 dT = dsub(oT, nT), dE = dsub(oE, nE), dB = dsub(oB, nB);
             const double2 rT = make_double2(T2.y * dT.x + ix * dE.x, T2.y * dT.y + ix * dE.y);
             const double2 rE = make_double2(ix * dT.x + T2.z * dE.x, ix * dT.y + T2.z * dE.y);
             const double2 rB = make_double2(T2.w * dB.x, T2.w * dB.y);
-            res += wm * (rT.x * rT.x + rT.y * rT.y + rE.x * rE.x + rE.y * rE.y + rB.x * rB.x + rB.y * rB.y);
+            res += (rT.x * rT.x + rT.y * rT.y + rE.x * rE.x + rE.y * rE.y + rB.x * rB.x + rB.y * rB.y);
         }
         a_new[k] = nT;
         a_new[nalm + k] = nE;
@@ -827,8 +830,8 @@ __global__ void k_hblend_pol(int lmax, int L, long long nalm, const double4 *__r
             s0 += red[0][w];
             s1 += red[1][w];
         }
-        part[2 * m] = s0;
-        part[2 * m + 1] = s1;
+        part[2 * m] = wm * s0;
+        part[2 * m + 1] = wm * s1;
     }
 }
 
@@ -900,8 +903,9 @@ __global__ void k_pix_chi2_pol(long long npix, const double *__restrict__ d, con
          p += (long long)gridDim.x * blockDim.x) {
         const Sym3 nu = load6(nu6, npix, p);
         // unobserved components (zero rows of nu) may hold anything in d, NaN included
-        const double e[3] = {nu.a != 0.0 ? d[p] - s[p] : 0.0, nu.b != 0.0 ? d[npix + p] - s[npix + p] : 0.0,
-                             nu.c != 0.0 ? d[2 * npix + p] - s[2 * npix + p] : 0.0};
+        // (tests on the bits: an FP64 comparison takes as long as a product)
+        const double e[3] = {nonzero(nu.a) ? d[p] - s[p] : 0.0, nonzero(nu.b) ? d[npix + p] - s[npix + p] : 0.0,
+                             nonzero(nu.c) ? d[2 * npix + p] - s[2 * npix + p] : 0.0};
         double ne[3];
         mv3(nu, e, ne);
         acc += e[0] * ne[0] + e[1] * ne[1] + e[2] * ne[2];
