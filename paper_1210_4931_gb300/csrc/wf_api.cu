@@ -695,6 +695,8 @@ wf_status hp_adjoint_T(wf_plan p, const void *map_T, int L, double2 *out)
 //   begin -> { pick -> launch -> (stream sync) -> absorb } -> end
 // on the plan's stream; the batch solver runs the same phases for several
 // plans, with the launches of one step of all of them captured in one graph.
+constexpr long long AHEAD_MAX_WORK = 1LL << 28;  // (l, m, ring pair) triples, FP64 ones counted 64 times
+
 struct HpRun {
     wf_plan p = nullptr;
     const double *d = nullptr, *nv = nullptr, *C_ell = nullptr, *g1 = nullptr, *g2 = nullptr;
@@ -724,6 +726,8 @@ struct HpRun {
     double lam = 1.0, chi2_bound = NAN;  // the current iteration
     int L = 0;
     bool corr = false, corr_pending = false;  // correction form (mixed_correction): on / due at the next launch
+    int ahead = -1;  // band limit of the synthesis of the iterate that is enqueued already (-1: none)
+    long long ahead_launches = 0;  // its kernels, counted when an iteration uses it
     Prof pr;
 };
 
@@ -968,6 +972,7 @@ wf_status hp_launch(HpRun &R)
     wf_status st;
     if (R.corr_pending) {
         R.corr_pending = false;
+        R.ahead = -1;  // the iterate changes
         if ((st = hp_enter_correction(R)) != WF_OK) return st;
     }
     pr.iter_begin();
@@ -1016,7 +1021,9 @@ wf_status hp_launch(HpRun &R)
         WF_CUDA(cudaGetLastError());
     } else {
         pr.begin(WF_K_LEG_SYN);
-        if ((st = hp_legendre_synthesis(p, p->ws.a, R.L)) != WF_OK) return st;
+        if (R.ahead == R.L) p->kcnt[WF_K_LEG_SYN] += R.ahead_launches;
+        else if ((st = hp_legendre_synthesis(p, p->ws.a, R.L)) != WF_OK) return st;
+        R.ahead = -1;
         pr.end();
         // one ring kernel: fold, inverse DFT, Eq. 3 and the forward DFT of t, which never
         // leaves shared memory (its time is reported under the ring synthesis)
@@ -1067,6 +1074,26 @@ wf_status hp_launch(HpRun &R)
     if (R.copy_back)
         WF_CUDA(cudaMemcpyAsync(p->ws.a, p->ws.a_new, p->nalm * sizeof(double2), cudaMemcpyDeviceToDevice, p->stream));
     return WF_OK;
+}
+
+// Band limit of the next iteration's synthesis if it is worth enqueueing before this iteration's
+// sums reach the host, else -1.  The GPU idles for 10 to 15 us while the host waits for the sums,
+// decides and launches; the synthesis depends on the decision only through L.  A known schedule
+// tells L; otherwise the present L is a guess that fails when a level changes L (once in tens of
+// iterations) or the solve ends, and then costs one synthesis: taken up to the size where that
+// costs as much as the guesses between two failures gain: 25 iterations at nside 128 take 1.55 ms
+// with it, 1.76 without (8 us a synthesis, 8 us gained per iteration); 7 FP64 iterations at nside
+// 100 1.43 against 1.45; at nside 512 a synthesis takes 47 us.
+int hp_ahead(const HpRun &R)
+{
+    wf_plan p = R.p;
+    if (R.rigorous || R.corr || R.copy_back || R.o.profile || p->pol) return -1;
+    const int next = R.k + 1;
+    const bool known = R.replay && !R.a_init;
+    if (next >= (R.replay ? R.nrep : R.o.maxiter)) return -1;
+    const int L = R.replay ? std::min(std::max(p->replay_L[next], 0), R.lmax) : R.L;
+    const long long work = (long long)(L + 1) * (L + 1) / 2 * p->npairs * (p->prec == WF_PREC_FP64 ? 64 : 1);
+    return known || work <= AHEAD_MAX_WORK ? L : -1;
 }
 
 // after the iteration's sums reached the host: trace, residual, schedule;
@@ -1283,8 +1310,22 @@ wf_status hp_solve(wf_plan p, const double *d, const double *nv, const uint8_t *
     if (st != WF_OK) return st;
     while (hp_pick(R)) {
         if ((st = hp_launch(R)) != WF_OK) return st;
-        WF_CUDA(cudaStreamSynchronize(p->stream));
+        const int ahead = hp_ahead(R);
+        if (ahead >= 0) {
+            WF_CUDA(cudaEventRecord(p->sums_ev, p->stream));
+            const long long n0 = p->kcnt[WF_K_LEG_SYN];
+            p->kfam = WF_K_LEG_SYN;
+            st = hp_legendre_synthesis(p, p->ws.a_new, ahead);
+            p->kfam = WF_K_OTHER;
+            R.ahead_launches = p->kcnt[WF_K_LEG_SYN] - n0;
+            p->kcnt[WF_K_LEG_SYN] = n0;
+            if (st != WF_OK) return st;
+            WF_CUDA(cudaEventSynchronize(p->sums_ev));
+        } else {
+            WF_CUDA(cudaStreamSynchronize(p->stream));
+        }
         if (!hp_absorb(R)) break;
+        R.ahead = ahead;
     }
     return hp_end(R);
 }
@@ -1872,6 +1913,7 @@ wf_status hp_create(wf_plan p)
         WF_CUDA(cudaEventCreateWithFlags(&p->fork_ev, cudaEventDisableTiming));
         WF_CUDA(cudaEventCreateWithFlags(&p->join_ev, cudaEventDisableTiming));
     }
+    WF_CUDA(cudaEventCreateWithFlags(&p->sums_ev, cudaEventDisableTiming));
     wf_status st;
     if ((st = hp_build_legendre_tables(p, xp, stp)) != WF_OK) return st;
     if ((st = hp_build_ring_tables(p)) != WF_OK) return st;
@@ -2058,6 +2100,7 @@ void wf_plan_destroy(wf_plan p)
     if (p->pol) hp_pol_destroy(p);
     if (p->sub) wf_plan_destroy(p->sub);
     if (p->aux) cudaStreamDestroy(p->aux);
+    if (p->sums_ev) cudaEventDestroy(p->sums_ev);
     if (p->fork_ev) cudaEventDestroy(p->fork_ev);
     if (p->join_ev) cudaEventDestroy(p->join_ev);
     if (p->events_ready)

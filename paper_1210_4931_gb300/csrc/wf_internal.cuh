@@ -246,6 +246,7 @@ struct wf_plan_s {
     bool tc_deferred = false;        // tensor-core plan in a batch step: its synthesis ran in the group launch
     cudaStream_t aux = nullptr;      // mixed precision: stream of the FP64 low-l block
     cudaEvent_t fork_ev = nullptr, join_ev = nullptr;
+    cudaEvent_t sums_ev = nullptr;   // an iteration's sums are in ws.h_scal
     long long kcnt[WF_NK] = {};  // kernels launched on this plan, by family (WF_K_*)
     int kfam = WF_K_OTHER;       // family the next launches are counted under
 };
