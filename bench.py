@@ -1011,7 +1011,7 @@ def _pcts(x):
 
 def run_config1(args):
     """Flat 128 x 128 periodic grid, FP64, one map: the whole solve (cooling from lambda 100 to 1
-    and lambda = 1 down to tol) is one persistent 8-CTA cluster kernel.  A step is one solve."""
+    and lambda = 1 down to tol) is one cooperative launch.  A step is one solve."""
     import torch
 
     import paper_1210_4931_gb300 as wf

@@ -300,7 +300,8 @@ long long wf_plan_estimate_bytes(const wf_geometry *g, int lmax, wf_precision pr
  * this plan's own buffers at the full band and keeps the fastest; reps timed
  * launches per variant (<= 0: 3).  FP64 and flat plans: no effect.  Overwrites
  * the plan's iterate buffers (call it between solves).  wf_plan_tiles reports
- * the current choice (defaults 4 and 8). */
+ * the current choice (4 and 8 where none was made: each launch then takes the
+ * tile that suits its size). */
 wf_status wf_plan_autotune(wf_plan p, int reps);
 wf_status wf_plan_tiles(wf_plan p, int *syn_pairs, int *ana_pairs);
 /* Move the plan to another CUDA stream (waits for work queued on the old one). */

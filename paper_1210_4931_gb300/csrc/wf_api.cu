@@ -1050,6 +1050,10 @@ wf_status hp_launch(HpRun &R)
     ba.want_resid = full ? 1 : 0;
     ba.want_norms = R.rigorous ? 1 : 0;
     ba.epi_ready = R.rigorous ? 0 : 1;
+    ba.pix = p->ws.part_pix;
+    ba.npix = p->npairs;
+    ba.sums_out = p->ws.h_scal;
+    ba.sums_count = p->ws.count;
     const double2 *a_old = p->ws.a;
     if (R.corr) {
         // the epilogue's residual compares its output B delta_k with delta_k - d0, i.e.
@@ -1061,16 +1065,6 @@ wf_status hp_launch(HpRun &R)
     if ((st = hp_legendre_analysis(p, L, LEG_BLEND, ba, a_old, p->ws.a_new)) != WF_OK) return st;
     pr.end();
     if (R.corr && (st = alm_axpy(p, p->ws.a_new, p->ws.cd0, 1.0, p->ws.a_new)) != WF_OK) return st;
-    SumSpec sp{};
-    sp.in[0] = p->ws.part_pix;
-    sp.n[0] = p->npairs;
-    sp.stride[0] = 1;
-    for (int q = 0; q < 4; ++q) {
-        sp.in[1 + q] = p->ws.part_harm + q;
-        sp.n[1 + q] = L + 1;
-        sp.stride[1 + q] = 4;
-    }
-    if ((st = sums_enqueue(p, sp, 5)) != WF_OK) return st;
     if (R.copy_back)
         WF_CUDA(cudaMemcpyAsync(p->ws.a, p->ws.a_new, p->nalm * sizeof(double2), cudaMemcpyDeviceToDevice, p->stream));
     return WF_OK;
@@ -1934,6 +1928,8 @@ wf_status hp_create(wf_plan p)
     const int npart = std::max(p->npairs, std::max(256, 4 * p->nsm));
     if ((st = plan_alloc(p, (void **)&p->ws.part_pix, npart * sizeof(double))) != WF_OK) return st;
     if ((st = plan_alloc(p, (void **)&p->ws.part_harm, 4 * (p->lmax + 2) * sizeof(double))) != WF_OK) return st;
+    if ((st = plan_alloc(p, (void **)&p->ws.count, sizeof(unsigned))) != WF_OK) return st;
+    WF_CUDA(cudaMemsetAsync(p->ws.count, 0, sizeof(unsigned), p->stream));
     if ((st = plan_alloc(p, (void **)&p->ws.epi, (p->lmax + 1) * sizeof(double4))) != WF_OK) return st;
     return WF_OK;
 }

@@ -166,6 +166,7 @@ struct Workspace {
     int *flag = nullptr;          // device flags (invalid input)
     int *tc_err = nullptr;        // tensor-core kernels: set when a bounded wait gave up
     double *redu = nullptr;       // reduction scratch
+    unsigned *count = nullptr;    // CTAs of the blend that have finished, zero between launches
     // mixed plans in correction form (wf_options.mixed_correction), allocated on first use:
     // the iterate x0 at the switch, d0 = G(x0) - x0, delta - d0, and a zero FP32 source map
     double2 *cx0 = nullptr, *cd0 = nullptr, *caold = nullptr;
@@ -311,6 +312,13 @@ struct BlendArgs {
     int want_resid = 0;
     int want_norms = 0;  // x^T S^-1 x and x^T S^-2 x of the result (the chi^2-bound schedule's; else 0)
     int epi_ready = 0;   // the ring pass of this iteration has filled ws.epi (EpiArgs)
+    // sums over the whole blend by its last CTA (null: none): the ring pairs' partials, chi^2,
+    // residual^2 and the two norms into sums_out (5; host memory the device can write);
+    // sums_count is zero between launches
+    const double *pix = nullptr;
+    int npix = 0;
+    double *sums_out = nullptr;
+    unsigned *sums_count = nullptr;
 };
 // per-l factors of the harmonic blend (Eq. 4) and of the chi^2 / residual sums, l <= lmax
 struct EpiArgs {

@@ -384,13 +384,27 @@ __device__ __forceinline__ void blend_one(int l, int L, long long idx, int mode,
     out[idx] = an;
 }
 
-// the CTA's sums into part[4 m ..]: a warp per sum that is wanted (NT >= 128 threads).  (Every
-// warp reducing all four by shuffles took more FP64 operations than the blend itself at lmax 1024.)
-template <int NT>
+// the CTA's sums into part[4 m ..]: a warp per sum that is wanted (128 threads); the last CTA adds
+// up the partials of all (fixed order).  Every warp reducing all four by shuffles took more FP64
+// operations than the blend itself at lmax 1024.  Totals by a launch of its own: 25 iterations at
+// nside 128 1.55 ms, 1.51 here; 16 at nside 512 (with a sweep) 7.56 and 7.49 ms.
+constexpr int EPI_THREADS = 128;
+
 __device__ __forceinline__ void blend_sums(const BlendSums &s, int m, const BlendArgs &ba, double *__restrict__ part,
-                                           double (*red)[NT])
+                                           double (*red)[EPI_THREADS])
 {
-    const int t = threadIdx.x, k = t >> 5, lane = t & 31;
+    __shared__ int last;
+    const int t = threadIdx.x, w = t >> 5, lane = t & 31;
+    auto wanted = [&](int k) { return k == 0 || (k == 1 ? ba.want_resid : ba.want_norms); };
+    // the sum of row k, in every lane of the warp that asks
+    auto row_sum = [&](int k) {
+        double x = red[k][lane];
+#pragma unroll
+        for (int i = 32; i < EPI_THREADS; i += 32) x += red[k][i + lane];
+#pragma unroll
+        for (int o = 16; o >= 1; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+        return x;
+    };
     red[0][t] = s.chi2;
     if (ba.want_resid) red[1][t] = s.res2;
     if (ba.want_norms) {
@@ -398,23 +412,41 @@ __device__ __forceinline__ void blend_sums(const BlendSums &s, int m, const Blen
         red[3][t] = s.qnew;
     }
     __syncthreads();
-    if (k >= 4) return;
-    double x = 0.0;
-    if (k == 0 || (k == 1 ? ba.want_resid : ba.want_norms)) {
-        x = red[k][lane];
-#pragma unroll
-        for (int i = 32; i < NT; i += 32) x += red[k][i + lane];
-#pragma unroll
-        for (int o = 16; o >= 1; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    const double x = wanted(w) ? row_sum(w) : 0.0;
+    if (lane == 0) {
+        __stcg(&part[4 * m + w], m ? 2.0 * x : x);
+        __threadfence();
     }
-    if (lane == 0) part[4 * m + k] = m ? 2.0 * x : x;
+    if (!ba.sums_out) return;
+    __syncthreads();
+    if (t == 0) last = atomicAdd(ba.sums_count, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    for (int k = 0; k < 4; ++k) {
+        if (!wanted(k)) continue;
+        double v = 0.0;
+#pragma unroll 4
+        for (int i = t; i < (int)gridDim.x; i += EPI_THREADS) v += __ldcg(&part[4 * i + k]);
+        red[k][t] = v;
+    }
+    double v = 0.0;
+#pragma unroll 4
+    for (int i = t; i < ba.npix; i += EPI_THREADS) v += __ldcg(&ba.pix[i]);
+    red[4][t] = v;
+    __syncthreads();
+    for (int k = w; k < 5; k += EPI_THREADS / 32) {
+        const double y = k == 4 || wanted(k) ? row_sum(k) : 0.0;
+        if (lane == 0) ba.sums_out[k == 4 ? 0 : 1 + k] = y;
+    }
+    if (t == 0) *ba.sums_count = 0;
 }
 
 // val(j): c_lm times the ring sum at l = m + j
-template <int NT, typename VAL>
+template <typename VAL>
 __device__ __forceinline__ void blend_epilogue(int lmax, int L, int m, long long base, int mode, const BlendArgs &ba,
                                                VAL val, const double2 *__restrict__ a_old, double2 *__restrict__ out,
-                                               double *__restrict__ part, double (*red)[NT])
+                                               double *__restrict__ part, double (*red)[EPI_THREADS])
 {
     BlendSums v;
     for (int j = threadIdx.x; j <= lmax - m; j += blockDim.x)
@@ -484,11 +516,11 @@ __global__ void __launch_bounds__(32) k_legana(int lmax, int L, int npairs, int 
 }
 
 // Eq. (4) epilogue of the FP64 analysis, a CTA per m; clears the sums for the next launch
-__global__ void __launch_bounds__(128) k_ana64_epilogue(int lmax, int L, int mode, BlendArgs ba,
+__global__ void __launch_bounds__(EPI_THREADS) k_ana64_epilogue(int lmax, int L, int mode, BlendArgs ba,
                                                         const double2 *__restrict__ a_old, double2 *__restrict__ out,
                                                         double *__restrict__ part, double2 *__restrict__ acc)
 {
-    __shared__ double red[4][128];
+    __shared__ double red[5][EPI_THREADS];
     const int m = blockIdx.x;
     const long long base = mbase(lmax, m);
     auto val = [&](int j) {
@@ -1326,12 +1358,12 @@ __global__ void __launch_bounds__(32, NP == 8 ? 17 : 16) k_legana_mx(const MxTab
 // Eq. (4) epilogue of the mixed analysis, a CTA per m; clears the sums for the next launch.  Run
 // by the last warp at its m inside the kernel above it took 14 % of that kernel (one warp's
 // chain of loads per m, nside 768).
-__global__ void __launch_bounds__(128) k_ana_epilogue(const MxTables t, int mode, BlendArgs ba,
+__global__ void __launch_bounds__(EPI_THREADS) k_ana_epilogue(const MxTables t, int mode, BlendArgs ba,
                                                       const double2 *__restrict__ low,
                                                       const double2 *__restrict__ a_old, double2 *__restrict__ out,
                                                       double *__restrict__ part, float4 *__restrict__ psum)
 {
-    __shared__ double red[4][128];
+    __shared__ double red[5][EPI_THREADS];
     const int m = blockIdx.x, nk = ((t.L - m + 1) >> 1) + 1;
     const long long base = mbase(t.lmax, m), kb = kbase(t.lmax, m);
     const long long nks = kbase(t.lmax, t.lmax + 1) + 2;
@@ -1392,7 +1424,7 @@ wf_status launch_ana64(wf_plan p, int L, const double2 *F, LegMode mode, const B
     k_legana<double><<<dim3((p->npairs + 31) / 32, L + 1), 32, 0, s>>>(
         p->lmax, L, p->npairs, 0, F, t.A64, t.ls, t.s0_64, t.s1_64, t.xw64, t.c64, t.acc64);
     WF_COUNT_LAUNCH(p);
-    k_ana64_epilogue<<<L + 1, 128, 0, s>>>(p->lmax, L, (int)mode, ba, a_old, out, p->ws.part_harm, t.acc64);
+    k_ana64_epilogue<<<L + 1, EPI_THREADS, 0, s>>>(p->lmax, L, (int)mode, ba, a_old, out, p->ws.part_harm, t.acc64);
     WF_COUNT_LAUNCH(p);
     WF_CUDA(cudaGetLastError());
     return WF_OK;
@@ -1464,7 +1496,7 @@ wf_status launch_ana_df(wf_plan p, int L, LegMode mode, const BlendArgs &ba, con
     k_legana_df<<<grid, 32, 0, p->stream>>>(p->lmax, L, p->npairs, (const double2 *)p->ws.F, t.A64, t.ls, t.s0_64,
                                             t.s1_64, t.xw64, t.c64, t.acc64);
     WF_COUNT_LAUNCH(p);
-    k_ana64_epilogue<<<L + 1, 128, 0, p->stream>>>(p->lmax, L, (int)mode, ba, a_old, out, p->ws.part_harm, t.acc64);
+    k_ana64_epilogue<<<L + 1, EPI_THREADS, 0, p->stream>>>(p->lmax, L, (int)mode, ba, a_old, out, p->ws.part_harm, t.acc64);
     WF_COUNT_LAUNCH(p);
     WF_CUDA(cudaGetLastError());
     return WF_OK;
@@ -1821,7 +1853,7 @@ wf_status launch_ana_mx_t(wf_plan p, int L, LegMode mode, const BlendArgs &ba, c
     const MxTables t = mx_tables(p, L);
     k_legana_mx<NP><<<dim3(2 * ng, L + 1), 32, 0, p->stream>>>(t, ng, (const float2 *)p->ws.F, p->tab.psum);
     WF_COUNT_LAUNCH(p);
-    k_ana_epilogue<<<L + 1, 128, 0, p->stream>>>(t, (int)mode, ba, low, a_old, out, p->ws.part_harm, p->tab.psum);
+    k_ana_epilogue<<<L + 1, EPI_THREADS, 0, p->stream>>>(t, (int)mode, ba, low, a_old, out, p->ws.part_harm, p->tab.psum);
     WF_COUNT_LAUNCH(p);
     WF_CUDA(cudaGetLastError());
     return WF_OK;
