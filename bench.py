@@ -432,10 +432,10 @@ def run_ours(args):
     # the measured FP32 FMA rate of this GPU (packed f32x2 FMAs, as the kernels issue them)
     peak_meas = {"packed": wf.wf_probe_fp32_fma(True), "scalar": wf.wf_probe_fp32_fma(False)}
     peak = max(peak_meas.values())
-    # DRAM bytes (read + write) of one full-band k_legsyn_mx<8> + k_legana_mx<8, 8> pair at nside 2048,
-    # lmax 4096, from a one-pass ncu capture of these kernels (666.1 + 738.0 MB); other sizes or tiles
-    # were not captured
-    traffic = 1404146432 if (nside, lmax, tuple(tiles), args.precision) == (2048, 4096, (8, 8), "mixed") else None
+    # DRAM bytes (read + write) of one full-band k_legsyn_mx<8> + k_legana_mx<8> + k_ana_epilogue at
+    # nside 2048, lmax 4096, from a one-pass ncu capture of these kernels (924.8 + 641.7 + 702.2 MB);
+    # other sizes or tiles were not captured
+    traffic = 2268670000 if (nside, lmax, tuple(tiles), args.precision) == (2048, 4096, (8, 8), "mixed") else None
     roof = {"bound": "alu", "kernel": "legendre synthesis + analysis (k_legsyn, k_legana)",
             "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak, "traffic": traffic,
             "traffic_basis": "DRAM bytes of one full-band synthesis + analysis pair (ncu dram__bytes_read.sum + "

@@ -809,7 +809,6 @@ extern "C" wf_status wf_flat_solve_noalloc(int n, const double *d, const double 
     double *rad = (double *)(base + NA_RAD);
     FlatStatus *status = (FlatStatus *)(base + NA_STATUS);
     double *tr = (double *)(base + NA_TRACE);
-    const long long npix = (long long)n * n;
     const int nh = n / 2 + 1;
 
     double h[3 * FLAT_SETUP_CTAS], smax[17];

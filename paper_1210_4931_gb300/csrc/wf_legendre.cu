@@ -333,11 +333,6 @@ __device__ __forceinline__ void warp_reduce_scatter(T (&vr)[CH], T (&vi)[CH], in
     }
 }
 
-template <int CH> struct Log2;
-template <> struct Log2<8> { static constexpr int v = 3; };
-template <> struct Log2<16> { static constexpr int v = 4; };
-template <> struct Log2<32> { static constexpr int v = 5; };
-
 // Eq. (4) epilogue shared by both precisions: t_hat = Omega (c acc + low),
 // a_new = S/(S + lam tau_h) t_hat, chi^2 of a_old, lambda = 1 residual.
 __global__ void k_epi_table(EpiArgs a)
@@ -454,10 +449,12 @@ __device__ __forceinline__ void blend_epilogue(int lmax, int L, int m, long long
     if (mode == LEG_BLEND) blend_sums(v, m, ba, part, red);
 }
 
-// FP64 analysis: chunks of 16 l in registers, reduced across the warp (one addition per value),
-// times c_l added to acc (zero before).  TF is the storage type of F (FP64 plans: double; FP64
-// block of the mixed path: float).
-template <typename TF>
+// FP64 analysis: chunks of 16 l in registers, summed over a lane's NP ring pairs, reduced across
+// the warp (one addition per value), times c_l added to acc (zero before).  Two pairs per lane
+// halve the reduction per pair, 3.6 + 2/NP operations per (l, pair), where there are ring pairs
+// for it (ANA64_MIN_PAIRS).  TF is the storage type of F (FP64 plans: double; FP64 block of the
+// mixed path: float).
+template <typename TF, int NP>
 __global__ void __launch_bounds__(32) k_legana(int lmax, int L, int npairs, int lcut, const cx<TF> *__restrict__ F,
                                                const double *__restrict__ A, const int *__restrict__ ls_tab,
                                                const double *__restrict__ s0_tab, const double *__restrict__ s1_tab,
@@ -467,21 +464,31 @@ __global__ void __launch_bounds__(32) k_legana(int lmax, int L, int npairs, int 
     constexpr int CH = 16;
     __shared__ double2 sA[F64_BLK / 2];
     const int m = blockIdx.y, lane = threadIdx.x;
-    const int p = (gridDim.x - 1 - blockIdx.x) * 32 + lane;
+    const int p0 = (gridDim.x - 1 - blockIdx.x) * 32 * NP + lane;
     const int Lm = lcut > 0 ? min(L, lcm_of(lcut, m) - 1) : L;
     const int nl = Lm - m + 1;
     const long long base = mbase(lmax, m);
-    const F64Pair P = f64_pair(m, Lm, npairs, p, ls_tab, s0_tab, s1_tab, xw);
-    if (P.kmin == BIG) return;
-    double2 FE = make_double2(0.0, 0.0), FO = FE;
-    if (P.k0 != BIG) {
-        const cx<TF> *f = F + ((size_t)p * (lmax + 1) + m) * 2;
-        const cx<TF> fn = f[0], fs = f[1];
-        FE = make_double2((double)fn.x + (double)fs.x, (double)fn.y + (double)fs.y);
-        FO = make_double2(((double)fn.x - (double)fs.x) * P.xw.w, ((double)fn.y - (double)fs.y) * P.xw.w);
+    F64Pair P[NP];
+    double2 FE[NP], FO[NP];
+    double E[NP], O[NP];
+    int kmin = BIG, kmaxs = -1;
+#pragma unroll
+    for (int q = 0; q < NP; ++q) {
+        const int p = p0 + 32 * q;
+        P[q] = f64_pair(m, Lm, npairs, p, ls_tab, s0_tab, s1_tab, xw);
+        kmin = min(kmin, P[q].kmin);
+        kmaxs = max(kmaxs, P[q].kmaxs);
+        E[q] = O[q] = 0.0;
+        FE[q] = FO[q] = make_double2(0.0, 0.0);
+        if (P[q].k0 != BIG) {
+            const cx<TF> *f = F + ((size_t)p * (lmax + 1) + m) * 2;
+            const cx<TF> fn = f[0], fs = f[1];
+            FE[q] = make_double2((double)fn.x + (double)fs.x, (double)fn.y + (double)fs.y);
+            FO[q] = make_double2(((double)fn.x - (double)fs.x) * P[q].xw.w, ((double)fn.y - (double)fs.y) * P[q].xw.w);
+        }
     }
-    double E = 0.0, O = 0.0;
-    int kc = P.kmin & ~3;
+    if (kmin == BIG) return;
+    int kc = kmin & ~3;
     const int nk = (nl + 1) >> 1;
     double nA = 2 * kc + lane + 2 < nl ? A[base + 2 * kc + lane + 2] : 0.0;
     for (; kc < nk; kc += F64_BLK / 2) {
@@ -492,19 +499,22 @@ __global__ void __launch_bounds__(32) k_legana(int lmax, int L, int npairs, int 
         nA = jn < nl ? A[base + jn] : 0.0;
         for (int k = 0; k < min(F64_BLK / 2, nk - kc); k += CH / 2) {
             double vr[CH], vi[CH];
-            const bool start = kc + k <= P.kmaxs;
+            const bool start = kc + k <= kmaxs;
 #pragma unroll
             for (int i = 0; i < CH / 2; ++i) {
-                if (start && kc + k + i == P.k0) {
-                    E = P.s0;
-                    O = P.s1;
+#pragma unroll
+                for (int q = 0; q < NP; ++q) {
+                    if (start && kc + k + i == P[q].k0) {
+                        E[q] = P[q].s0;
+                        O[q] = P[q].s1;
+                    }
+                    vr[2 * i] = q ? fma(E[q], FE[q].x, vr[2 * i]) : E[q] * FE[q].x;
+                    vi[2 * i] = q ? fma(E[q], FE[q].y, vi[2 * i]) : E[q] * FE[q].y;
+                    vr[2 * i + 1] = q ? fma(O[q], FO[q].x, vr[2 * i + 1]) : O[q] * FO[q].x;
+                    vi[2 * i + 1] = q ? fma(O[q], FO[q].y, vi[2 * i + 1]) : O[q] * FO[q].y;
+                    if ((i & 3) == 3) f64_advance<true>(sA[k + i], P[q].xw, E[q], O[q]);
+                    else f64_advance<false>(sA[k + i], P[q].xw, E[q], O[q]);
                 }
-                vr[2 * i] = E * FE.x;
-                vi[2 * i] = E * FE.y;
-                vr[2 * i + 1] = O * FO.x;
-                vi[2 * i + 1] = O * FO.y;
-                if ((i & 3) == 3) f64_advance<true>(sA[k + i], P.xw, E, O);
-                else f64_advance<false>(sA[k + i], P.xw, E, O);
             }
             // c_l for this lane's l, in flight over the reduction
             const int j = 2 * (kc + k) + (lane >> 1);
@@ -1417,12 +1427,18 @@ wf_status launch_syn64(wf_plan p, const double2 *alm, int L, int lcut, cx<TG> *G
     return WF_OK;
 }
 
+// ring pairs from which the FP64 analysis takes two per lane; one / two (us): nside 48 29 / 43, 100
+// 68 / 77, 128 128 / 124, 192 356 / 315, 256 665 / 592, 512 4515 / 3619
+constexpr int ANA64_MIN_PAIRS = 256;
+
 wf_status launch_ana64(wf_plan p, int L, const double2 *F, LegMode mode, const BlendArgs &ba, const double2 *a_old,
                        double2 *out, cudaStream_t s)
 {
     const HpTables &t = p->tab;
-    k_legana<double><<<dim3((p->npairs + 31) / 32, L + 1), 32, 0, s>>>(
-        p->lmax, L, p->npairs, 0, F, t.A64, t.ls, t.s0_64, t.s1_64, t.xw64, t.c64, t.acc64);
+    const int np = p->npairs >= ANA64_MIN_PAIRS ? 2 : 1;
+    const dim3 grid((p->npairs + 32 * np - 1) / (32 * np), L + 1);
+    auto kernel = np == 2 ? k_legana<double, 2> : k_legana<double, 1>;
+    kernel<<<grid, 32, 0, s>>>(p->lmax, L, p->npairs, 0, F, t.A64, t.ls, t.s0_64, t.s1_64, t.xw64, t.c64, t.acc64);
     WF_COUNT_LAUNCH(p);
     k_ana64_epilogue<<<L + 1, EPI_THREADS, 0, s>>>(p->lmax, L, (int)mode, ba, a_old, out, p->ws.part_harm, t.acc64);
     WF_COUNT_LAUNCH(p);
@@ -1437,7 +1453,7 @@ wf_status launch_ana64_low(wf_plan p, int L, int lcut, const float2 *F, double2 
     const int nm = std::min(L, lcut - 1) + 1;
     if (nm <= 0) return WF_OK;
     WF_CUDA(cudaMemsetAsync(out, 0, (size_t)mbase(p->lmax, nm) * sizeof(double2), s));
-    k_legana<float><<<dim3((p->npairs + 31) / 32, nm), 32, 0, s>>>(p->lmax, L, p->npairs, lcut, F, t.A64, t.ls, t.s0_64,
+    k_legana<float, 1><<<dim3((p->npairs + 31) / 32, nm), 32, 0, s>>>(p->lmax, L, p->npairs, lcut, F, t.A64, t.ls, t.s0_64,
                                                                    t.s1_64, t.xw64, t.c64, out);
     WF_COUNT_LAUNCH(p);
     WF_CUDA(cudaGetLastError());

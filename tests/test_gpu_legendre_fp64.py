@@ -1,7 +1,8 @@
 """FP64 Legendre transforms at the edges of their split: ring pairs just below, at and above a
-warp (npairs = 2 nside), band limits around a table block of 32 l, a band limit below the plan's,
-both directions against the oracle (1e-10 of the largest value, the FP64 bound of the other
-tests), and the analysis twice in a row (its sums start from zero each time)."""
+warp (npairs = 2 nside) and 256 (two pairs per lane from there on in the analysis), band limits
+around a table block of 32 l, a band limit below the plan's, both directions against the oracle
+(1e-10 of the largest value, the FP64 bound of the other tests), and the analysis twice in a row
+(its sums start from zero each time)."""
 import numpy as np
 import pytest
 
@@ -13,7 +14,8 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("nside,lmax,L", [(1, 2, 2), (2, 4, 3), (15, 30, 30), (16, 31, 31), (16, 32, 30), (17, 33, 33),
-                                          (24, 48, 47), (33, 64, 64), (40, 80, 65), (64, 128, 128)])
+                                          (24, 48, 47), (33, 64, 64), (40, 80, 65), (64, 128, 128), (127, 33, 33),
+                                          (128, 40, 39), (145, 60, 60)])
 def test_fp64_legendre_edges(nside, lmax, L):
     import torch
 
