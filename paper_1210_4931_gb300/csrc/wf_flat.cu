@@ -17,9 +17,9 @@
 // Hermitian) is xa + i xb, and the forward DFT Z of ta + i tb gives
 // Ta = (Z_k + conj Z_-k) / 2 and Tb = (Z_k - conj Z_-k) / 2i.
 //
-// What bounds it: FP64 runs at 1/64 of the FP32 rate (a warp instruction takes 64 cycles
-// of its scheduler's FP64 unit), so an iteration wants many SMs: one FFT per SM, one
-// value per thread on all four schedulers, 32 FP64 operations per thread and FFT.  The
+// What bounds it: FP64 runs at 1/64 of the FP32 rate (two lanes per clock and SM), so an
+// iteration wants many SMs: one FFT per SM, one value per thread, 32 FP64 operations per
+// thread and FFT.  The
 // rest is two grid barriers and their exchanges through L2.  A cluster of 16 CTAs (the
 // largest) with four to five FFTs each in one warp took 42.5 us per iteration of the
 // 128 x 128 grid, 18 to 21 us of it FP64 issue, three cluster barriers;

@@ -15,11 +15,11 @@
 // poles at large m); below that l every term is < 2^-80 and is dropped.
 //
 // Two precisions:
-//   FP64     k_legsyn<double>, k_legana<double,...>: one ring pair per thread.
+//   FP64     k_legsyn<TG>, k_legana<TF, NP>: one ring pair per lane, two in large analyses.
 //   mixed    k_legsyn_mx<NP>, k_legana_mx<NP>: FP32 recurrence and
 //            contraction, NP ring pairs per thread (synthesis) or per lane
 //            (analysis) in packed f32x2 lanes (__ffma2_rn), in the two-step
-//            forms of the belt and the polar cap described at MxPart below.
+//            forms of the belt and the polar cap described above MxTables below.
 //            The block l < l_c, where the messenger iteration's contraction
 //            margin tau_h / S_l is below the FP32 error, runs through the FP64
 //            kernels instead (the FP32 recurrence restarts at l_c from FP64
@@ -175,9 +175,8 @@ __global__ void k_to_T(const double *__restrict__ in, T *__restrict__ out, long 
 }
 
 // ---------------------------------------------------------------------------
-// FP64 transforms.  FP64 runs at 1/64 of the FP32 rate (a warp instruction holds its
-// scheduler's FP64 unit for 64 cycles), so what counts is the FP64 operations per (l, ring
-// pair) and that all 608 schedulers have work.
+// FP64 transforms.  FP64 runs at 1/64 of the FP32 rate (two lanes per clock and SM), so what
+// counts is the FP64 operations per (l, ring pair) and that all SMs have work.
 //
 // Both directions take one warp per (group of 32 ring pairs, m) and advance two l at once
 // (k = (l - m)/2) with the odd values carried as x mu, which saves the product A_l x on the
@@ -190,8 +189,8 @@ __global__ void k_to_T(const double *__restrict__ in, T *__restrict__ out, long 
 // input is).  A, c and a_lm pass through shared memory in blocks of 32 l, the next block's
 // loads in flight over the present one.
 //
-// One CTA per m before: its 256 threads left up to half the schedulers idle behind m = 0 where
-// the ring pairs are few.  Synthesis at nside 256, lmax 512
+// One CTA per m before: the SMs waited for those that had m = 0 and its neighbours where the
+// ring pairs are few.  Synthesis at nside 256, lmax 512
 // 0.606 -> 0.390 ms (its FP64 operations take 0.38); at nside 100, lmax 200, 46 -> 35 us and the
 // analysis 87 -> 60 + 6 us.
 //
