@@ -454,13 +454,14 @@ __device__ __forceinline__ bool positive(double v)
 }
 
 // a lower bound of eigmin3 in FP32: Gershgorin's, less 1e-5 of the trace for the roundings here
-// and there; NaN or infinite where FP32 cannot hold the entries
+// and there; of no use (-infinity, or NaN where FP32 overflows) where the trace is so small that
+// entries may be FP32 subnormals, whose rounding is fixed and not relative to them
 __device__ __forceinline__ float eig_bound(const Sym3 &s)
 {
     const float a = narrow(s.a), b = narrow(s.b), c = narrow(s.c);
     const float d = fabsf(narrow(s.d)), e = fabsf(narrow(s.e)), f = fabsf(narrow(s.f));
-    const float g = fminf(a - (d + e), fminf(b - (d + f), c - (e + f)));
-    return g - 1e-5f * (a + b + c);
+    const float g = fminf(a - (d + e), fminf(b - (d + f), c - (e + f))), t = a + b + c;
+    return t > 1e-30f ? g - 1e-5f * t : -INFINITY;
 }
 
 // all three eigenvalues, descending (same trigonometric solution)
