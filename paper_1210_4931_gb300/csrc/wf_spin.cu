@@ -445,6 +445,13 @@ __device__ double eigmin3(const Sym3 &s)
     return q + 2.0 * pp * cos(phi + 2.0 * M_PI / 3.0);
 }
 
+// v / det with id = 1 / det at hand, which overflows for a determinant below 5.6e-309 where the
+// quotient need not (a beam takes the product of two spectra there)
+__device__ __forceinline__ double over(double v, double det, double id)
+{
+    return finite_bits(id) ? v * id : v / det;
+}
+
 __device__ __forceinline__ bool nonzero(double v) { return (__double_as_longlong(v) << 1) != 0; }
 
 // v > 0 (infinity included), by its bits
@@ -582,9 +589,9 @@ __global__ void __launch_bounds__(256) k_setup_pol(long long npix, const double 
                     ok = ok && finite_bits(N.c) && finite_bits(N.f) && positive_finite(N.b) && positive(det);
                     if (ok) {
                         const double id = inverse(det), h = 0.5 * (N.b - N.c);
-                        nu.b = N.c * id;
-                        nu.c = N.b * id;
-                        nu.f = -N.f * id;
+                        nu.b = over(N.c, det, id);
+                        nu.c = over(N.b, det, id);
+                        nu.f = -over(N.f, det, id);
                         tl = __double_as_longlong(0.5 * (N.b + N.c) - sqrt(h * h + N.f * N.f));
                     }
                 }
@@ -707,9 +714,9 @@ __device__ __forceinline__ void pinv_te(const Prior &S, double &it, double &ie, 
     const double det = S.tt * S.ee - S.te * S.te;
     if (S.tt > 0.0 && S.ee > 0.0 && det > 0.0) {
         const double id = inverse(det);
-        it = S.ee * id;
-        ie = S.tt * id;
-        ix = -S.te * id;
+        it = over(S.ee, det, id);
+        ie = over(S.tt, det, id);
+        ix = -over(S.te, det, id);
     } else {
         it = S.tt > 0.0 ? inverse(S.tt) : 0.0;
         ie = S.ee > 0.0 ? inverse(S.ee) : 0.0;
