@@ -181,16 +181,18 @@ __global__ void __launch_bounds__(FLAT_MAXN) k_flat_solve(const FlatArgs A)
     const bool mode = t < n, row = mode && c < n / 2;
     const int ya = 2 * c, yb = 2 * c + 1;
     const double inv_tau = 1.0 / A.tau, dn = (double)n, wk = (c == 0 || 2 * c == n) ? 1.0 : 2.0;
+    const double wkn = wk * dn * dn;  // weight of a mode's squares, for a over n
     unsigned arrivals = 0;
     for (int i = t; i < n; i += blockDim.x) {
         double sn, cs;
         sincospi(-2.0 * i / n, &sn, &cs);
         tw[i] = make_double2(cs, sn);
     }
-    // this thread's mode (ky = t, kx = c); a is kept over n, so that neither FFT needs its 1/n
+    // this thread's mode (ky = t, kx = c); a is kept over n, so that neither FFT needs its 1/n.  The
+    // n^2 of the squares stays out of 1 / S, which may be next to the largest FP64 number
     const double S = mode ? A.S[(size_t)t * nh + c] : 0.0;
-    const double si = S > 0.0 ? dn * dn / S : 0.0;                     // chi^2 of a: |a / n|^2 n^2 / S
-    const double kr = S > 0.0 ? dn * (1.0 / S + inv_tau) : 0.0;        // residual
+    const double si = S > 0.0 ? 1.0 / S : 0.0;                         // chi^2
+    const double kr = S > 0.0 ? si + inv_tau : 0.0;                    // residual
     double2 a = make_double2(0.0, 0.0);
     double f = 0.0;                                                    // S / (S + lam tau) / (2 n^2)
     // its two pixels (rows ya, yb; x = t)
@@ -291,7 +293,7 @@ __global__ void __launch_bounds__(FLAT_MAXN) k_flat_solve(const FlatArgs A)
     rows_out(ra, rb);
     if (!barrier()) return gave_up();
     {
-        const double2 v = columns_in();
+        const double2 v = cscale(columns_in(), 0.5 / dn);
         const double b2 = S > 0.0 ? wk * (v.x * v.x + v.y * v.y) : 0.0;
         put_part(1, 0.0, b2);
     }
@@ -309,7 +311,7 @@ __global__ void __launch_bounds__(FLAT_MAXN) k_flat_solve(const FlatArgs A)
         tot.x = warp_sum(tot.x);
         tot.y = warp_sum(tot.y);
         if (k == 0) {
-            bnorm = sqrt(tot.y) / (2.0 * dn);
+            bnorm = sqrt(tot.y);
         } else {  // absorb iteration k - 1, which ran at lam
             const double chi2 = tot.x;
             const bool full = lam == 1.0;
@@ -376,7 +378,7 @@ __global__ void __launch_bounds__(FLAT_MAXN) k_flat_solve(const FlatArgs A)
         const double ea = ra - na * s.x, eb = rb - nb * s.y;
         rows_out(s.x + la * ea, s.y + lb * eb);
         // sums that need no exchange before the second barrier, while its first arrivals wait
-        double ch = S > 0.0 ? wk * ((a.x * a.x + a.y * a.y) * si) : 0.0, rs = 0.0;
+        double ch = S > 0.0 ? wkn * ((a.x * a.x + a.y * a.y) * si) : 0.0, rs = 0.0;
         ch -= s.x * ((ea + ra) * ia) + s.y * ((eb + rb) * ib);
         if (!barrier()) return gave_up();
         const double2 th = columns_in();
@@ -384,7 +386,7 @@ __global__ void __launch_bounds__(FLAT_MAXN) k_flat_solve(const FlatArgs A)
             const double2 an = cscale(th, f);
             if (lam == 1.0) {
                 const double dx = kr * (a.x - an.x), dy = kr * (a.y - an.y);
-                rs = wk * (dx * dx + dy * dy);
+                rs = wkn * (dx * dx + dy * dy);
             }
             a = an;
         }
@@ -393,7 +395,7 @@ __global__ void __launch_bounds__(FLAT_MAXN) k_flat_solve(const FlatArgs A)
     if (A.replay && isfinite(last_res) && last_res < A.tol) converged = 1;
     // ---- output: s = F^-1 a (its columns are in x1), chi^2(s, 1) ----
     const double2 s = rows_in(rows_load());
-    double pc = wk * ((a.x * a.x + a.y * a.y) * si);
+    double pc = wkn * ((a.x * a.x + a.y * a.y) * si);
     if (row) {
         A.s_out[(size_t)ya * n + t] = s.x;
         A.s_out[(size_t)yb * n + t] = s.y;
