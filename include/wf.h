@@ -171,7 +171,10 @@ typedef struct {
     double *resid_trace;    /* optional, relative residual (NaN where lambda > 1 or L < lmax) */
     double *iter_ms_trace;  /* optional, device time of iteration k in ms (CUDA events; HEALPix) */
     int trace_cap;
-    long long launches;                 /* kernels this call launched */
+    long long launches;                 /* kernels the solve's iterations and its setup and output used.  A single
+                                           solve may enqueue the next iteration's synthesis before the schedule has
+                                           decided; one that the decision discards is not counted here or in
+                                           kernel_launches (the counts are those of the same solve in a batch) */
     double kernel_ms[WF_NK];            /* device time per kernel family (wf_options.profile) */
     long long kernel_launches[WF_NK];   /* launches per kernel family */
 } wf_info;
