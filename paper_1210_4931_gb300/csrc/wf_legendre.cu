@@ -1877,7 +1877,12 @@ wf_status launch_ana_mx_t(wf_plan p, int L, LegMode mode, const BlendArgs &ba, c
 wf_status launch_ana_mx(wf_plan p, int L, LegMode mode, const BlendArgs &ba, const double2 *low, const double2 *a_old,
                         double2 *out)
 {
-    switch (mx_tile(p, L, p->tile_ana, p->tile_ana_set, ANA_MIN_WARPS, ANA_MIN_WARPS)) {
+    int tile = mx_tile(p, L, p->tile_ana, p->tile_ana_set, ANA_MIN_WARPS, ANA_MIN_WARPS);
+    // Two warps that add to zeroed sums give the same bits in either order, three do not: up to nside
+    // 256 the default keeps to two groups of a part's ring pairs, and runs repeat exactly (adjoint, tiles
+    // 2 / 4: nside 160, lmax 320 51.8 / 54.0 us; 192, 384 55.4 / 56.8; 227, 454 62.4 / 61.4; 256, 256 50.9 / 50.9)
+    if (!p->tile_ana_set && tile == 2 && p->nside > 128 && p->nside <= 256) tile = 4;
+    switch (tile) {
     case 2: return launch_ana_mx_t<2>(p, L, mode, ba, low, a_old, out);
     case 4: return launch_ana_mx_t<4>(p, L, mode, ba, low, a_old, out);
     default: return launch_ana_mx_t<8>(p, L, mode, ba, low, a_old, out);
