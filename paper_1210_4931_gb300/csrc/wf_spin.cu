@@ -452,14 +452,6 @@ __device__ __forceinline__ double over(double v, double det, double id)
     return finite_bits(id) ? v * id : v / det;
 }
 
-__device__ __forceinline__ bool nonzero(double v) { return (__double_as_longlong(v) << 1) != 0; }
-
-// v > 0 (infinity included), by its bits
-__device__ __forceinline__ bool positive(double v)
-{
-    return (unsigned long long)(__double_as_longlong(v) - 1) < 0x7ff0000000000000ULL;
-}
-
 // a lower bound of eigmin3 in FP32: Gershgorin's, less 1e-5 of the trace for the roundings here
 // and there; of no use (-infinity, or NaN where FP32 overflows) where the trace is so small that
 // entries may be FP32 subnormals, whose rounding is fixed and not relative to them
