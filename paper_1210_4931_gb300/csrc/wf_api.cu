@@ -1956,9 +1956,8 @@ long long hp_estimate_bytes(int nside, int lmax, wf_precision prec, bool staging
     for (int k = 1; k <= nside; ++k) {
         const long long n = 4LL * k;
         roots += 2 * n;
-        bool direct = false;
-        const int b2 = ring_fft_log((int)n, &direct);
-        if (!direct) V += (1LL << b2) + k;  // filter and chirp
+        int logF = 0;
+        if (ring_kind((int)n, &logF) == RING_BLUESTEIN) V += (1LL << logF) + k;  // filter and chirp
     }
     b += (roots + V + RING_TW) * ec + np * ((long long)sizeof(RingTab) + 4) + 64;
     // workspace

@@ -53,13 +53,13 @@ template <typename C, typename S> __host__ __device__ __forceinline__ C cscale(C
 // ---------------------------------------------------------------------------
 // ring table (one entry per north/south ring pair)
 // ---------------------------------------------------------------------------
-enum RingKind : int { RING_POW2 = 1, RING_BLUESTEIN = 2 };
+enum RingKind : int { RING_SHORT = 0, RING_POW2 = 1, RING_BLUESTEIN = 2 };
 
 struct RingTab {
     int n;             // pixels in each ring of the pair
     int q;             // first-pixel longitude is q pi / n (q = 0 or 1)
     int kind;          // RingKind
-    int logF;          // log2 of the FFT length N of its four length-n/4 DFTs (n/4, or 2^b >= n/2 - 1)
+    int logF;          // log2 of the FFT length N of its four length-n/4 DFTs (n/4, or 2^b >= n/2 - 1; short: 0)
     unsigned inv;      // ceil(2^32 / n): m / n = umulhi(m, inv) for the m of a band limit
     long long offN;    // first pixel of the north ring
     long long offS;    // first pixel of the south ring, -1 for the equator
@@ -69,6 +69,7 @@ struct RingTab {
 };
 
 constexpr int LEG_THREADS = 256;
+constexpr int RING_SHORT_K = 8;      // quarter rings up to here take direct sums (4 k threads of one warp)
 constexpr int RING_MAX_K = 2048;     // longest quarter ring (nside) of the ring kernel's FFTs
 constexpr int RING_TW = 2 * 4096 - 32;  // twiddles of the FFT lengths 32 .. 4096
 
@@ -318,7 +319,7 @@ wf_status hp_pol_tc_synthesis(wf_plan p, int ncols, const double2 *const *E, con
 
 // ring transforms (wf_ring.cu)
 wf_status hp_build_ring_tables(wf_plan p);
-int ring_fft_log(int n, bool *direct);
+RingKind ring_kind(int n, int *logF);
 // RS_BLEND_ANA: the blended ring goes straight into the forward DFT and the unfold to F
 enum RingSynMode { RS_BLEND = 0, RS_MAP = 1, RS_SYN = 2, RS_BLEND_ANA = 3 };
 wf_status hp_ring_synthesis(wf_plan p, int L, RingSynMode mode, double lam, double tau, double *out_map);

@@ -16,6 +16,7 @@
 // directions touches the pixels q, q + k, q + 2k, q + 3k of one thread: in the
 // messenger step a thread combines its four pixels, blends them (Eq. 3) and
 // splits them again in registers.  The four length-k DFTs run
+//   k <= 8              as direct sums;
 //   k = 2^b >= 16       as FFTs of length N = k;
 //   otherwise           by Bluestein's chirp convolution
 //                       X_p = c_p sum_j (x_j c_j) conj(c_{p-j}), c_j = e^{-i pi j^2 / k},
@@ -398,14 +399,40 @@ __device__ __noinline__ void sub_dfts(cx<T> *zb, cx<T> *exch, int k, bool flip, 
     }
 }
 
+// The same for k <= 8 by direct sums, one value per thread of the first warp; root: e^{i pi t / 4k}.
+// What bounds a grid of such rings alone (nside <= 8) is the chain of one pair: as a Bluestein FFT
+// of length 16 a DFT is one thread's, some 600 FP64 operations in a row.  Synthesis / adjoint in FP64
+// (whole calls) at nside 2 35.9 / 46.5 -> 22.7 / 30.6 us, at nside 8 39.9 / 50.7 -> 27.7 / 36.5 us.
+template <typename T>
+__device__ __noinline__ void short_dfts(cx<T> *zb, int k, bool flip, const cx<T> *__restrict__ root)
+{
+    const int t = threadIdx.x, r = t / k, p = t - r * k;
+    if (t >= 32) return;
+    cx<T> s = mk<T>(0, 0);
+    if (r < 4) {
+        int i = 0;  // j p mod k
+        for (int j = 0; j < k; ++j) {
+            cx<T> w = root[8 * i];
+            if (!flip) w.y = -w.y;
+            s = cadd(s, cmul(zb[pidx(r * k + j)], w));
+            i += p;
+            if (i >= k) i -= k;
+        }
+    }
+    __syncwarp();
+    if (r < 4) zb[pidx(t)] = s;
+}
+
 template <typename T>
 __device__ __forceinline__ void ring_sub_dfts(const RingTab &R, cx<T> *zb, cx<T> *ex, bool flip,
                                               const cx<T> *__restrict__ V, const cx<T> *__restrict__ chirp,
-                                              const cx<T> *__restrict__ tw)
+                                              const cx<T> *__restrict__ tw, const cx<T> *__restrict__ root)
 {
     const cx<T> *v = V + R.vOff, *c = chirp + R.cOff;
     const int k = R.n >> 2;
-    if (R.kind == RING_POW2) {
+    if (R.kind == RING_SHORT) {
+        short_dfts<T>(zb, k, flip, root);
+    } else if (R.kind == RING_POW2) {
         switch (R.logF) {
         case 4: sub_dfts<T, 4, false>(zb, ex, k, flip, v, c, tw); break;
         case 5: sub_dfts<T, 5, false>(zb, ex, k, flip, v, c, tw); break;
@@ -418,7 +445,6 @@ __device__ __forceinline__ void ring_sub_dfts(const RingTab &R, cx<T> *zb, cx<T>
         }
     } else {
         switch (R.logF) {
-        case 4: sub_dfts<T, 4, true>(zb, ex, k, flip, v, c, tw); break;
         case 5: sub_dfts<T, 5, true>(zb, ex, k, flip, v, c, tw); break;
         case 6: sub_dfts<T, 6, true>(zb, ex, k, flip, v, c, tw); break;
         case 7: sub_dfts<T, 7, true>(zb, ex, k, flip, v, c, tw); break;
@@ -641,7 +667,7 @@ __global__ void __launch_bounds__(RING_CTA, MINB) k_ring(const RingArgs<T> A)
     if (syn) {
         fold_ring<T>(A, R, A.G + row, A.Glow ? A.Glow + (size_t)pair * A.glow_stride * 2 : nullptr, south, zb);
         __syncthreads();
-        ring_sub_dfts<T>(R, zb, ex, true, A.V, A.chirp, A.tw);
+        ring_sub_dfts<T>(R, zb, ex, true, A.V, A.chirp, A.tw, root);
     }
     const T lt = A.lam * A.tau, lm1t = (A.lam - (T)1) * A.tau;
     T chi = 0;
@@ -719,7 +745,7 @@ __global__ void __launch_bounds__(RING_CTA, MINB) k_ring(const RingArgs<T> A)
     }
     if (ana) {
         __syncthreads();
-        ring_sub_dfts<T>(R, zb, ex, false, A.V, A.chirp, A.tw);
+        ring_sub_dfts<T>(R, zb, ex, false, A.V, A.chirp, A.tw, root);
         unfold_ring<T>(A, R, zb, south, A.F + row);
     }
 }
@@ -844,12 +870,13 @@ wf_status upload_cx(wf_plan p, void **dst, const std::vector<double2> &src)
 
 }  // namespace
 
-// log2 of the FFT length that serves a ring of n = 4k pixels, and whether k itself is that length
-int ring_fft_log(int n, bool *direct)
+// how the DFTs of a ring of n = 4k pixels are done, and log2 of their FFT length (short rings: 0)
+RingKind ring_kind(int n, int *logF)
 {
     const int k = n / 4;
-    *direct = k >= 16 && is_pow2(k);
-    return *direct ? ilog2(k) : std::max(4, ilog2(2LL * k - 1));
+    const RingKind kind = k <= RING_SHORT_K ? RING_SHORT : is_pow2(k) ? RING_POW2 : RING_BLUESTEIN;
+    *logF = kind == RING_SHORT ? 0 : ilog2(kind == RING_POW2 ? k : 2LL * k - 1);
+    return kind;
 }
 
 wf_status hp_build_ring_tables(wf_plan p)
@@ -894,12 +921,11 @@ wf_status hp_build_ring_tables(wf_plan p)
         t.rootOff = rootOff[n];
         t.vOff = 0;
         t.cOff = 0;
-        bool direct = false;
-        t.logF = ring_fft_log(n, &direct);
-        t.kind = direct ? RING_POW2 : RING_BLUESTEIN;
+        t.kind = ring_kind(n, &t.logF);
+        if (t.kind == RING_SHORT) continue;
         const int N = 1 << t.logF, nt = N / 16;
         exmax = std::max(exmax, N * std::min(4, RING_CTA / nt));
-        if (!direct) {
+        if (t.kind == RING_BLUESTEIN) {
             if (!vOff.count(k)) {
                 vOff[k] = (long long)Vtab.size();
                 std::vector<double2> v(N, make_double2(0.0, 0.0));
