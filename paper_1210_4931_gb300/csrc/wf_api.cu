@@ -1953,13 +1953,15 @@ long long hp_estimate_bytes(int nside, int lmax, wf_precision prec, bool staging
     if (tc_prec(prec)) b += nalm * 8 + ns * 12;                  // A32, B32 and one-step seeds
     // ring tables: roots per distinct length, Bluestein filters and chirps, twiddles
     long long roots = 0, V = 0;
+    int logmax = 0;
     for (int k = 1; k <= nside; ++k) {
         const long long n = 4LL * k;
         roots += 2 * n;
         int logF = 0;
         if (ring_kind((int)n, &logF) == RING_BLUESTEIN) V += (1LL << logF) + k;  // filter and chirp
+        logmax = std::max(logmax, logF);
     }
-    b += (roots + V + RING_TW) * ec + np * ((long long)sizeof(RingTab) + 4) + 64;
+    b += (roots + V + ring_tw_len(logmax)) * ec + np * ((long long)sizeof(RingTab) + 4) + 64;
     // workspace
     b += nalm * 16 * (f32 ? 4 : 3);                              // a, a_new, b (+ b_low)
     b += 2 * np * (lmax + 1) * 2 * ec;                           // G, F

@@ -71,7 +71,8 @@ struct RingTab {
 constexpr int LEG_THREADS = 256;
 constexpr int RING_SHORT_K = 8;      // quarter rings up to here take direct sums (4 k threads of one warp)
 constexpr int RING_MAX_K = 2048;     // longest quarter ring (nside) of the ring kernel's FFTs
-constexpr int RING_TW = 2 * 4096 - 32;  // twiddles of the FFT lengths 32 .. 4096
+// twiddles of the FFT lengths 32 .. 2^logF, one after another
+constexpr int ring_tw_len(int logF) { return logF < 5 ? 0 : (2 << logF) - 32; }
 
 // ---------------------------------------------------------------------------
 // plan

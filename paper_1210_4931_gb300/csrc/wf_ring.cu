@@ -901,7 +901,7 @@ wf_status hp_build_ring_tables(wf_plan p)
     std::vector<RingTab> rt(np);
     std::map<int, long long> rootOff, vOff, cOff;
     std::vector<double2> roots, Vtab, chirp;
-    int exmax = 0;
+    int exmax = 0, logmax = 0;
     for (int pr = 0; pr < np; ++pr) {
         RingTab &t = rt[pr];
         const int i0 = pr;  // north ring, 0-based
@@ -923,6 +923,7 @@ wf_status hp_build_ring_tables(wf_plan p)
         t.cOff = 0;
         t.kind = ring_kind(n, &t.logF);
         if (t.kind == RING_SHORT) continue;
+        logmax = std::max(logmax, t.logF);
         const int N = 1 << t.logF, nt = N / 16;
         exmax = std::max(exmax, N * std::min(4, RING_CTA / nt));
         if (t.kind == RING_BLUESTEIN) {
@@ -949,9 +950,9 @@ wf_status hp_build_ring_tables(wf_plan p)
             t.cOff = cOff[k];
         }
     }
-    // twiddles of every FFT length N = 32 .. 4096: tw[N - 32 + k N/16 + t] = e^{-2 pi i t k / N}
-    std::vector<double2> tw(RING_TW);
-    for (int N = 32; N <= 4096; N *= 2)
+    // twiddles of every FFT length N = 32 .. 2^logmax: tw[N - 32 + k N/16 + t] = e^{-2 pi i t k / N}
+    std::vector<double2> tw(std::max(1, ring_tw_len(logmax)));
+    for (int N = 32; N <= 1 << logmax; N *= 2)
         for (int kk = 0; kk < 16; ++kk)
             for (int t = 0; t < N / 16; ++t) {
                 const double a = -2.0 * M_PI * (double)(t * kk) / (double)N;
