@@ -167,13 +167,6 @@ __global__ void k_restart_seeds(int lmax, int npairs, int lc, int ncap, const do
     seed[idx] = sd;
 }
 
-template <typename T>
-__global__ void k_to_T(const double *__restrict__ in, T *__restrict__ out, long long n)
-{
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        out[i] = (T)in[i];
-}
-
 // ---------------------------------------------------------------------------
 // FP64 transforms.  FP64 runs at 1/64 of the FP32 rate (two lanes per clock and SM), so what
 // counts is the FP64 operations per (l, ring pair) and that all SMs have work.
