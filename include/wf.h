@@ -342,9 +342,11 @@ wf_status wf_probe_fp32_fma(void *cuda_stream, int packed, double *tflops);
  * use.  S must be finite and >= 0 (WF_EINVAL otherwise).  Each call looks up
  * the array's device address on the current device (cudaGetSymbolAddress);
  * nothing is cached between calls.  All calls share
- * the array, so calls that overlap on the GPU race; each call writes what it
- * reads first.  Every copy of the call (status, traces) is ordered on
- * cuda_stream, and the call returns after that stream has synchronised. */
+ * the array, so calls that overlap on the GPU race (with each other's data, and
+ * with the counter of the kernel's barriers: such a call may also end with
+ * WF_ETIMEOUT after its bounded waits); each call writes what it reads first.
+ * Every copy of the call (status, traces) is ordered on cuda_stream, and the
+ * call returns after that stream has synchronised. */
 wf_status wf_flat_solve_noalloc(int n, const double *d, const double *noise_var, const uint8_t *mask,
                                 const double *S, double tol, const wf_options *opt, void *cuda_stream,
                                 double *s_wf, double *alm_out, wf_info *info);

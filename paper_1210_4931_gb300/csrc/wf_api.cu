@@ -485,7 +485,7 @@ __global__ void k_blend(long long npix, const T *__restrict__ r, const T *__rest
     }
 }
 
-int grid_chi2(int nsm) { return std::min(1024, 4 * nsm); }  // CTAs of k_pix_chi2; part_pix holds at least 1024
+int grid_chi2(int nsm) { return std::min(1024, 4 * nsm); }  // CTAs of k_pix_chi2; part_pix holds at least 4 nsm
 int grid_for(long long n, int nsm) { return (int)std::min<long long>((n + 255) / 256, (long long)nsm * 8); }
 
 // reduce the partial sums in a fixed order, a CTA each, into the pinned host
@@ -1070,14 +1070,16 @@ wf_status hp_launch(HpRun &R)
     return WF_OK;
 }
 
-// Band limit of the next iteration's synthesis if it is worth enqueueing before this iteration's
+// Band limit of the next iteration's synthesis if it is to be enqueued before this iteration's
 // sums reach the host, else -1.  The GPU idles for 10 to 15 us while the host waits for the sums,
-// decides and launches; the synthesis depends on the decision only through L.  A known schedule
-// tells L; otherwise the present L is a guess that fails when a level changes L (once in tens of
-// iterations) or the solve ends, and then costs one synthesis: taken up to the size where that
-// costs as much as the guesses between two failures gain: 25 iterations at nside 128 take 1.55 ms
-// with it, 1.76 without (8 us a synthesis, 8 us gained per iteration); 7 FP64 iterations at nside
-// 100 1.43 against 1.45; at nside 512 a synthesis takes 47 us.
+// decides and launches; the synthesis depends on the decision only through L.  A given schedule
+// tells L: always.  A live one keeps L until a level changes it or the solve ends; that guess
+// costs one synthesis when it fails and is taken up to AHEAD_MAX_WORK, where a synthesis takes
+// about 35 us (nside 400).  Live solves to 1e-4 without / with (ms): nside 64 29.7 / 24.3,
+// 128 29.0 / 25.0, 256 35.8 / 32.4, 400 60.0 / 54.6; FP64 nside 64 76.6 / 72.4, 100 90.7 / 87.7; with
+// a level change every two iterations at first, nside 64 86.0 / 69.9, 256 76.4 / 70.5.  The line is on
+// the safe side of where it stops to pay: without it nside 512 would take 63.5 for 67.0 and nside
+// 1024 214.7 for 215.5.
 int hp_ahead(const HpRun &R)
 {
     wf_plan p = R.p;

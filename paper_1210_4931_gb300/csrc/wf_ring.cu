@@ -641,12 +641,13 @@ __device__ __forceinline__ void unfold_ring(const RingArgs<T> &A, const RingTab 
 // 2048 1.28 -> 0.53 ms, nside 512 0.153 -> 0.057 ms, nside 128 0.042 -> 0.019 ms (cold caches);
 // FP64: nside 512 0.93 -> 0.55 ms and nside 100 0.21 -> 0.073 ms, bound by the FP64 pipe.
 //
-// MINB CTAs per SM set the register budget: FP32 at 128 registers (2) or 80 with a small spill
-// (3).  Three are faster where shared memory holds three and there are pairs for them (a map
-// pass at nside 1024 0.131 -> 0.112 ms, a step at nside 512 0.066 -> 0.057 ms), two where it does
-// not (nside 2048: 0.525 against 0.570 ms averaged over a solve) or where one wave holds every
-// pair (nside 128: 18.5 against 20.6 us).  FP64: two at 128 registers against one at 255:
-// nside 100 0.126 -> 0.073 ms, nside 512 0.60 -> 0.55 ms.
+// MINB CTAs per SM set the register budget: FP32 at 128 registers (2) or 80 with some 210 bytes
+// spilled per thread in the Bluestein FFTs of 2048 and 4096 (3).  Three are faster where shared
+// memory holds three and there are pairs for them (a map pass at nside 1024 0.131 -> 0.112 ms, a
+// step at nside 512 0.066 -> 0.057 ms), two where it does not (nside 2048: 0.525 against 0.570 ms
+// averaged over a solve) or where one wave holds every pair (nside 128: 18.5 against 20.6 us).
+// FP64: two at 128 registers against one at 255: nside 100 0.126 -> 0.073 ms, nside 512
+// 0.60 -> 0.55 ms.
 template <typename T, int MINB>
 __global__ void __launch_bounds__(RING_CTA, MINB) k_ring(const RingArgs<T> A)
 {
