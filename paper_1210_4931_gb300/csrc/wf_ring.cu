@@ -402,7 +402,7 @@ __device__ __noinline__ void sub_dfts(cx<T> *zb, cx<T> *exch, int k, bool flip, 
 // The same for k <= 8 by direct sums, one value per thread of the first warp; root: e^{i pi t / 4k}.
 // What bounds a grid of such rings alone (nside <= 8) is the chain of one pair: as a Bluestein FFT
 // of length 16 a DFT is one thread's, some 600 FP64 operations in a row.  Synthesis / adjoint in FP64
-// (whole calls) at nside 2 35.9 / 46.5 -> 22.7 / 30.6 us, at nside 8 39.9 / 50.7 -> 27.7 / 36.5 us.
+// (whole calls) at nside 2 35.9 / 46.5 -> 22.1 / 30.8 us, at nside 8 39.9 / 50.7 -> 27.1 / 37.0 us.
 template <typename T>
 __device__ __noinline__ void short_dfts(cx<T> *zb, int k, bool flip, const cx<T> *__restrict__ root)
 {
@@ -410,13 +410,19 @@ __device__ __noinline__ void short_dfts(cx<T> *zb, int k, bool flip, const cx<T>
     if (t >= 32) return;
     cx<T> s = mk<T>(0, 0);
     if (r < 4) {
+        cx<T> w[RING_SHORT_K];
         int i = 0;  // j p mod k
-        for (int j = 0; j < k; ++j) {
-            cx<T> w = root[8 * i];
-            if (!flip) w.y = -w.y;
-            s = cadd(s, cmul(zb[pidx(r * k + j)], w));
+#pragma unroll
+        for (int j = 0; j < RING_SHORT_K; ++j) {  // every load in flight before the sum
+            w[j] = root[8 * i];
             i += p;
             if (i >= k) i -= k;
+        }
+#pragma unroll
+        for (int j = 0; j < RING_SHORT_K; ++j) {
+            if (j == k) break;
+            if (!flip) w[j].y = -w[j].y;
+            s = cadd(s, cmul(zb[pidx(r * k + j)], w[j]));
         }
     }
     __syncwarp();
